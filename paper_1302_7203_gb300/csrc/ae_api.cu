@@ -151,6 +151,14 @@ static int solve_common(ae::Kind kind, int n, const double *d, const double *z, 
     }
     S.wbuf = (double2 *)wb;
     S.wstride = wstride;
+    void *fb = nullptr;                     // the fixed-point path's data
+    e = cudaMallocAsync(&fb, ae::fast_bytes(n), st);
+    if (e != cudaSuccess) {
+        cudaFreeAsync(wb, st);
+        cudaFreeAsync(base, st);
+        return cuda_fail(e);
+    }
+    S.f = ae::carve_fast(fb, n);
     int status = AE_OK;
     bool solved = true;
     if (part) {
@@ -200,6 +208,8 @@ static int solve_common(ae::Kind kind, int n, const double *d, const double *z, 
             else if (cnt[ae::C_CAPPED]) status = AE_ERR_NOCONV;
         }
     }
+    e = cudaFreeAsync(fb, st);
+    if (e != cudaSuccess && status == AE_OK) status = cuda_fail(e);
     e = cudaFreeAsync(wb, st);
     if (e != cudaSuccess && status == AE_OK) status = cuda_fail(e);
     e = cudaFreeAsync(base, st);

@@ -234,11 +234,61 @@ static size_t layout(uintptr_t base, int n, Scratch *S) {
     T.pos0 = (int *)take(sizeof(int) * nn);
     T.wbuf = nullptr;
     T.wstride = 0;
+    T.f = FastPtrs{};
     if (S) *S = T;
     return (size_t)(p - start);
 }
 
 // bytes to request: the layout from a 256-aligned base, plus room to align
+// (fixed-point path, carved the same way from its own block)
+static size_t fast_layout(uintptr_t base, int n, FastPtrs *F) {
+    const size_t n1 = n > 1 ? (size_t)n : 1, nn = (size_t)n;
+    uintptr_t p = (base + 255) & ~(uintptr_t)255;
+    auto take = [&](size_t bytes) {
+        uintptr_t q = p;
+        p += (bytes + 255) & ~(size_t)255;
+        return (void *)q;
+    };
+    using u64 = unsigned long long;
+    FastPtrs T;
+    T.p = (double *)take(8 * n1);
+    T.plo = (double *)take(8 * n1);
+    T.P = (u64 *)take(8 * n1);
+    T.z = (u64 *)take(8 * n1);
+    T.ez = (int *)take(4 * n1);
+    T.rp = (double *)take(8 * n1);
+    T.rP = (u64 *)take(8 * n1);
+    T.mu = (double *)take(8 * nn);
+    T.mulo = (double *)take(8 * nn);
+    T.lhi = (double *)take(8 * nn);
+    T.N = (double *)take(8 * nn);
+    T.M2u = (double *)take(8 * nn);
+    T.lmod = (u64 *)take(8 * nn);
+    T.K1 = (int *)take(4 * nn);
+    T.K2 = (int *)take(4 * nn);
+    T.er = (int *)take(4 * nn);
+    T.s1 = (long long *)take(8 * nn);
+    T.s3 = (long long *)take(8 * nn);
+    T.s5 = (long long *)take(8 * nn);
+    T.s2 = (u64 *)take(8 * nn);
+    T.s4 = (u64 *)take(8 * nn);
+    T.n1 = (int *)take(4 * nn);
+    T.n2 = (int *)take(4 * nn);
+    T.st = (int *)take(4 * nn);
+    T.old = (int *)take(4 * nn);
+    T.more = (int *)take(4 * nn);
+    if (F) *F = T;
+    return (size_t)(p - base);
+}
+
+size_t fast_bytes(int n) { return fast_layout(0, n, nullptr) + 256; }
+
+FastPtrs carve_fast(void *base, int n) {
+    FastPtrs F;
+    fast_layout((uintptr_t)base, n, &F);
+    return F;
+}
+
 size_t arrow_scratch_bytes(int n) { return layout(0, n, nullptr) + 256; }
 
 Scratch carve_scratch(void *base, int n) {
@@ -256,8 +306,7 @@ Scratch carve_scratch(void *base, int n) {
 static int eig_grid(int n) {
     static int per_sm = 0;
     if (!per_sm) {
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_eig<KIND_ARROW, KIND_ARROW>,
-                                                      256, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_eig<KIND_ARROW>, 256, 0);
         if (per_sm <= 0) per_sm = 1;
     }
     const int want = (n + 7) / 8;
@@ -293,7 +342,7 @@ cudaError_t launch_solve(Kind kind, int n, const double *d, const double *z, dou
     }
     k_reduce<<<1, 1024, 0, st>>>(n1, key, spk, S.perm, S);
     SolveOpts so{ro.max_iter, ro.precision, ro.finish, ro.bgate, ro.kb_max};
-    VecArgs va{n, n1, key, spk, z, zrow, alpha, sgn, out, (S.wbuf && out.V) ? 1 : 0};
+    VecArgs va{n, n1, key, spk, z, zrow, kind == KIND_DPR1 ? rho : alpha, sgn, out};
     const int grid = eig_grid(n);
     switch (kind) {
         case KIND_ARROW:
@@ -345,7 +394,7 @@ cudaError_t launch_arrow_part(int n, const double *d, const double *z, double al
     *count = (h[C_K1] - h[C_K0]) + (h[C_U1] - h[C_U0]);
     if (!out.lambda || *count > cap) return cudaSuccess;   // size query, or no room
     const SolveOpts so{ro.max_iter, ro.precision, ro.finish, ro.bgate, ro.kb_max};
-    const VecArgs va{n, n1, d, z, z, nullptr, alpha, 1.0, out, (S.wbuf && out.V) ? 1 : 0};
+    const VecArgs va{n, n1, d, z, z, nullptr, alpha, 1.0, out};
     launch_pipeline<KIND_ARROW, KIND_ARROW>(n, eig_grid(n), S, so, ro, va, st);
     if (ro.ev[4]) cudaEventRecord(ro.ev[4], st);
     return cudaGetLastError();

@@ -1,12 +1,17 @@
 // ae_batch.cu -- many arrowheads of uneven order solved together.
 //
 // All instances go through the same pipeline as arrow_eig, but each stage is
-// ONE persistent launch over every instance:
-//   k_batch_prep      one CTA per instance: checks, order, reduction, FP32 copies
-//   k_batch_eig       global work queue of (instance, eigenpair) units; a unit
-//                     is 32/W eigenpairs of one instance solved by W-lane teams
-//                     (W = 8, 16 or 32, chosen per order bucket by the tuner)
-//   k_batch_fix_*     remedy decisions over all eigenpairs, one CTA per remedy
+// ONE launch over every instance:
+//   k_batch_prep      one CTA per instance: checks, order, reduction, FP32 and
+//                     fixed-point copies
+//   k_fopen, k_feval, k_fstep, k_fold, k_ffix, k_fcols (ae_fast.cuh) on units of
+//                     32, 8 or 1 eigenpairs of one instance (SrcMany)
+//   k_batch_eig       the FP64 solver instead, for options the fixed-point path
+//                     does not serve: global work queue of (instance, eigenpair)
+//                     units; a unit is 32/W eigenpairs of one instance solved by
+//                     W-lane teams (W = 8, 16 or 32, chosen per order bucket by
+//                     the tuner)
+//   k_batch_fix_*     remedy decisions over all eigenpairs, a warp per FP64 remedy
 //   k_batch_place / k_batch_vectors / k_batch_status
 // A plan (ae_batch_create) owns the descriptor table and the scratch of every
 // instance and captures the whole sequence in a CUDA graph that
@@ -25,6 +30,7 @@
 #include <string>
 #include <vector>
 
+#include "ae_fast.cuh"
 #include "ae_pipeline.cuh"
 
 namespace ae {
@@ -72,12 +78,12 @@ struct BatchInst {
     int n, n1;
     const double *d, *z, *alpha;   // device inputs of this instance
     Scratch S;
-    Outputs out;
+    VecArgs va;                    // (alpha is read from the device, not from here)
     int team;                      // eigenpair team width W
 };
 
 struct BatchCtl {
-    int tick_eig, tick_fix, nfix, tick_vec;
+    int tick_eig, tick_fix, nfix, nold, tick_old, nmore[2];
 };
 
 // index i with off[i] <= t < off[i+1]
@@ -91,6 +97,47 @@ __device__ __forceinline__ int find_inst(const long long *off, int count, long l
     return lo;
 }
 
+// the instances of a batch, for the kernels of ae_fast.cuh
+struct SrcMany {
+    const BatchInst *__restrict__ I;
+    int count;
+    const long long *__restrict__ eoff, *__restrict__ off8, *__restrict__ off32;
+    BatchCtl *ctl;
+    int2 *old, *fix, *more;
+    double2 *wbuf;
+    long long wstride;
+    __device__ bool unit(long long u, int per, int &i, int &first) const {
+        const long long *off = per == 8 ? off8 : off32;
+        if (u >= off[count]) return false;
+        i = find_inst(off, count, u);
+        first = (int)(u - off[i]) * per;
+        return true;
+    }
+    __device__ bool item(long long t, int &i, int &idx) const {
+        if (t >= eoff[count]) return false;
+        i = find_inst(eoff, count, t);
+        idx = (int)(t - eoff[i]);
+        return true;
+    }
+    __device__ const Scratch &scr(int i) const { return I[i].S; }
+    __device__ const VecArgs &vec(int i) const { return I[i].va; }
+    __device__ void push_old(int i, int k) const {
+        old[atomicAdd(&ctl->nold, 1)] = make_int2(i, k);
+    }
+    __device__ int old_count() const { return ctl->nold; }
+    __device__ int2 old_at(int w) const { return old[w]; }
+    __device__ int *old_ticket() const { return &ctl->tick_old; }
+    __device__ void push_more(int ph, int i, int k) const {
+        more[atomicAdd(&ctl->nmore[ph], 1)] = make_int2(i, k);
+    }
+    __device__ int more_count(int ph) const { return ctl->nmore[ph]; }
+    __device__ int2 more_at(int w) const { return more[w]; }
+    __device__ void push_fix(int i, int k, bool, int) const {
+        fix[atomicAdd(&ctl->nfix, 1)] = make_int2(i, k);
+    }
+    __device__ double2 *slice(long long w) const { return wbuf ? wbuf + w * wstride : nullptr; }
+};
+
 // ---------------------------------------------------------------------------
 // kernels
 // ---------------------------------------------------------------------------
@@ -101,12 +148,10 @@ __global__ void __launch_bounds__(1024) k_batch_prep(const BatchInst *__restrict
     const BatchInst &B = I[blockIdx.x];
     const Scratch &S = B.S;
     const int n1 = B.n1;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *ctl = BatchCtl{0, 0, 0, 0};
+    if (blockIdx.x == 0 && threadIdx.x == 0) *ctl = BatchCtl{};
     if (threadIdx.x < C_COUNT) S.cnt[threadIdx.x] = 0;
     if (threadIdx.x < C64_COUNT) S.cnt64[threadIdx.x] = 0ull;
     if (threadIdx.x == 0) sflags = 0;
-    // -1: no column written by the remedy pass (see k_batch_fix_solve)
-    for (int k = threadIdx.x; k < B.n; k += blockDim.x) S.pos0[k] = -1;
     __syncthreads();
     int flags = 0;
     for (int r = threadIdx.x; r < n1; r += blockDim.x) {
@@ -148,6 +193,9 @@ __global__ void __launch_bounds__(1024) k_batch_prep(const BatchInst *__restrict
     reduce_block(n1, B.d, B.z, S.perm, S);
     __syncthreads();
     post_block<KIND_ARROW>(n1, B.d, B.z, nullptr, *B.alpha, 0.0, S);
+    __syncthreads();
+    if (S.f.p)
+        for (int t = threadIdx.x; t < n1; t += blockDim.x) fprep_item<KIND_ARROW>(S, B.va, t);
 }
 
 // buf: this warp's 4 slices of stored (delta_j, c_j) pairs, `stride` apart
@@ -160,28 +208,11 @@ __device__ __forceinline__ void batch_unit(const BatchInst &B, long long unit_in
     const int k = (int)(unit_in_inst * EPW) + g;
     const auto R = PolesOf<KIND_ARROW>::make(B.S, m);
     double2 *tb = buf ? buf + g * stride : nullptr;
-    // the solve, then (with vectors and a stored-pair slice) the column at its
-    // position as the single-instance k_eig writes it
-    auto run = [&](const auto &T) {
-        eig_item<KIND_ARROW>(R, T, B.S, k, o, tb);
-        if (B.out.V && tb) {
-            T.sync();
-            if (T.rank == 0) {
-                place_item(B.S, k);
-                B.S.pos0[k] = B.S.pos[k];
-            }
-            T.sync();
-            // (the stored differences only for whole-warp teams: narrower ones
-            // would add a sync per step to the divergent teams of one warp)
-            vector_item<KIND_ARROW>(B.n, B.n1, B.d, B.z, B.z, nullptr, *B.alpha, 1.0, B.S,
-                                    B.out, k, T, (double *)tb, true, W == 32);
-        }
-    };
     if constexpr (W == 32) {
-        if (k <= m) run(WarpTeam{lane});
+        if (k <= m) eig_item<KIND_ARROW>(R, WarpTeam{lane}, B.S, k, o, tb);
     } else {
         const unsigned mask = ((1u << W) - 1u) << (lane & ~(W - 1));
-        if (k <= m) run(SubWarpTeam<W>{lane & (W - 1), mask});
+        if (k <= m) eig_item<KIND_ARROW>(R, SubWarpTeam<W>{lane & (W - 1), mask}, B.S, k, o, tb);
     }
 }
 
@@ -211,25 +242,19 @@ __global__ void __launch_bounds__(256, 3) k_batch_eig(const BatchInst *__restric
 }
 
 __global__ void k_batch_fix_decide(const BatchInst *__restrict__ I, int count,
-                                   const long long *__restrict__ eoff, int2 *fixlist,
-                                   BatchCtl *ctl, double knu_max) {
+                                   const long long *__restrict__ eoff, double knu_max) {
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= eoff[count]) return;
     const int i = find_inst(eoff, count, t);
-    const int k = (int)(t - eoff[i]);
-    if (fix_decide_item(KIND_ARROW, I[i].S, k, knu_max)) fixlist[atomicAdd(&ctl->nfix, 1)] = {i, k};
+    fix_decide_item(KIND_ARROW, I[i].S, (int)(t - eoff[i]), knu_max);
 }
 
-// One warp per remedied eigenpair (remedies are many in a batch of small
-// instances), on the warp's first stored-pair slice; the warp also rewrites the
-// remedied column, which k_batch_vectors then skips unless the final placement
-// moved it.
+// One warp per remedied eigenpair that k_ffix left to the FP64 solver.
 __global__ void __launch_bounds__(256) k_batch_fix_solve(const BatchInst *__restrict__ I,
                                                          const int2 *fixlist, BatchCtl *ctl,
                                                          SolveOpts o, double2 *wbuf,
                                                          long long wstride) {
     const int lane = threadIdx.x & 31;
-    const WarpTeam T{lane};
     const long long gw = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     double2 *buf = wbuf ? wbuf + gw * 4 * wstride : nullptr;
     for (;;) {
@@ -238,20 +263,9 @@ __global__ void __launch_bounds__(256) k_batch_fix_solve(const BatchInst *__rest
         w = __shfl_sync(FULL, w, 0);
         if (w >= ctl->nfix) break;
         const int2 ik = fixlist[w];
-        const BatchInst &B = I[ik.x];
-        const Scratch &S = B.S;
+        const Scratch &S = I[ik.x].S;
         const auto R = PolesOf<KIND_ARROW>::make(S, S.cnt[C_M]);
-        const bool kept = fix_solve_item<KIND_ARROW>(R, T, S, ik.y, o, buf);
-        __syncwarp();
-        if (B.out.V && buf) {
-            if (lane == 0) {
-                place_item(S, ik.y);
-                S.pos0[ik.y] = S.pos[ik.y];
-            }
-            __syncwarp();
-            vector_item<KIND_ARROW>(B.n, B.n1, B.d, B.z, B.z, nullptr, *B.alpha, 1.0, S, B.out,
-                                    ik.y, T, (double *)buf, true, kept);
-        }
+        fix_solve_item<KIND_ARROW>(R, WarpTeam{lane}, S, ik.y, o, buf);
         __syncwarp();
     }
 }
@@ -264,24 +278,24 @@ __global__ void k_batch_place(const BatchInst *__restrict__ I, int count,
     place_item(I[i].S, (int)(t - eoff[i]));
 }
 
+// 8 items a CTA: scalar outputs by a thread each, and the columns k_fcols does
+// not write by the CTA
 __global__ void __launch_bounds__(256) k_batch_vectors(const BatchInst *__restrict__ I, int count,
-                                                       const long long *__restrict__ eoff,
-                                                       BatchCtl *ctl) {
-    const int lane = threadIdx.x & 31;
-    const long long total = eoff[count];
-    for (;;) {
-        long long t = 0;
-        if (lane == 0) t = atomicAdd(&ctl->tick_vec, 1);
-        t = __shfl_sync(FULL, t, 0);
-        if (t >= total) break;
-        const int i = find_inst(eoff, count, t);
-        const BatchInst &B = I[i];
-        const int item = (int)(t - eoff[i]);
-        const bool cols = !(item <= B.S.cnt[C_M] && B.S.pos0[item] >= 0 &&
-                            B.S.pos[item] == B.S.pos0[item]);
-        vector_item<KIND_ARROW>(B.n, B.n1, B.d, B.z, B.z, nullptr, *B.alpha, 1.0, B.S, B.out,
-                                item, WarpTeam{lane}, nullptr, cols);
-        __syncwarp();
+                                                       const long long *__restrict__ off8) {
+    __shared__ double red[16];
+    const long long u = blockIdx.x;
+    const int i = find_inst(off8, count, u);
+    const BatchInst &B = I[i];
+    const VecArgs &va = B.va;
+    const int i0 = (int)(u - off8[i]) * 8, ncomp = B.S.cnt[C_M] + 1;
+    if (threadIdx.x < 8 && i0 + (int)threadIdx.x < B.n)
+        scalar_item<KIND_ARROW>(B.n, B.d, 1.0, B.S, va.out, i0 + threadIdx.x);
+    if (!va.out.V) return;
+    for (int item = i0; item < i0 + 8 && item < B.n; ++item) {
+        if (item < ncomp && B.S.f.p && B.S.f.st[item] == FST_DONE) continue;
+        vector_item<KIND_ARROW>(B.n, B.n1, B.d, B.z, B.z, nullptr, 0.0, 1.0, B.S, va.out, item,
+                                CtaTeam<8>{(int)threadIdx.x, red, 0});
+        __syncthreads();
     }
 }
 
@@ -406,8 +420,12 @@ struct Plan {
     double2 *wbuf = nullptr;     // 4 slices of stored pairs per warp of k_batch_eig
     long long wstride = 0;
     BatchInst *d_inst = nullptr;
-    long long *d_eoff = nullptr, *d_uoff = nullptr;
-    int2 *d_fix = nullptr;
+    // prefix tables: eigenpairs, FP64 team units, units of 8 and of 32 eigenpairs
+    // (count + 1 entries each, one after another)
+    long long *d_eoff = nullptr, *d_uoff = nullptr, *d_off8 = nullptr, *d_off32 = nullptr;
+    long long n8 = 0, n32 = 0;   // units in all
+    int2 *d_fix = nullptr, *d_old = nullptr, *d_more = nullptr;
+    bool fast = true, vectors = false;
     BatchCtl *d_ctl = nullptr;
     void *scratch = nullptr;
     int *status = nullptr;
@@ -417,20 +435,65 @@ struct Plan {
     std::vector<BatchInst> host;
 };
 
+// bytes of one instance's scratch and fixed-point data
+static size_t inst_bytes(int n) {
+    return ((arrow_scratch_bytes(n) + 255) & ~(size_t)255) + ((fast_bytes(n) + 255) & ~(size_t)255);
+}
+static Scratch carve_inst(char *base, int n, bool fast) {
+    Scratch S = carve_scratch(base, n);
+    if (fast) S.f = carve_fast(base + ((arrow_scratch_bytes(n) + 255) & ~(size_t)255), n);
+    return S;
+}
+
+// the prefix tables of `count` instances of orders ns[i] and team widths W[i]
+static std::vector<long long> prefix_tables(int count, const int *ns, const int *W, Plan &P) {
+    std::vector<long long> t(4 * (size_t)(count + 1), 0);
+    long long *e = t.data(), *u = e + count + 1, *a = u + count + 1, *b = a + count + 1;
+    for (int i = 0; i < count; ++i) {
+        const long long n = ns[i], epw = 32 / W[i];
+        e[i + 1] = e[i] + n;
+        u[i + 1] = u[i] + (n + epw - 1) / epw;
+        a[i + 1] = a[i] + (n + 7) / 8;
+        b[i + 1] = b[i] + (n + 31) / 32;
+    }
+    P.total_n = e[count];
+    P.n8 = a[count];
+    P.n32 = b[count];
+    return t;
+}
+static void set_tables(Plan &P, long long *d) {
+    P.d_eoff = d;
+    P.d_uoff = d + (P.count + 1);
+    P.d_off8 = d + 2 * (size_t)(P.count + 1);
+    P.d_off32 = d + 3 * (size_t)(P.count + 1);
+}
+
 static void enqueue(const Plan &P, cudaStream_t st) {
-    const int sms = sm_count_b();
+    const unsigned g = (unsigned)((P.total_n + 255) / 256), g1 = (unsigned)((P.total_n + 63) / 64);
+    const unsigned gm = (unsigned)std::min<long long>(P.total_n, 4 * sm_count_b());
+    const SrcMany src{P.d_inst, P.count, P.d_eoff, P.d_off8, P.d_off32, P.d_ctl, P.d_old, P.d_fix, P.d_more,
+                      P.wbuf, 4 * P.wstride};
     k_batch_prep<<<P.count, 1024, 0, st>>>(P.d_inst, P.d_ctl);
-    k_batch_eig<<<batch_eig_grid(), 256, 0, st>>>(P.d_inst, P.count, P.d_uoff, P.d_ctl, P.so,
-                                                  P.wbuf, P.wstride);
-    const unsigned g = (unsigned)((P.total_n + 255) / 256);
+    if (P.fast) {
+        k_fopen<KIND_ARROW><<<(unsigned)P.n32, 256, 0, st>>>(src, P.so);
+        k_feval<<<(unsigned)P.n8, 256, 0, st>>>(src);
+        k_fstep<KIND_ARROW><<<g1, 64, 0, st>>>(src, P.so, 0);
+        k_fmore<KIND_ARROW><<<gm, 256, 0, st>>>(src, P.so, 0, 0);
+        k_fold<KIND_ARROW><<<batch_eig_grid(), 256, 0, st>>>(src, P.so);
+    } else {
+        k_batch_eig<<<batch_eig_grid(), 256, 0, st>>>(P.d_inst, P.count, P.d_uoff, P.d_ctl, P.so,
+                                                      P.wbuf, P.wstride);
+    }
     if (P.ro.fixup) {
-        k_batch_fix_decide<<<g, 256, 0, st>>>(P.d_inst, P.count, P.d_eoff, P.d_fix, P.d_ctl,
-                                              P.ro.knu_max);
+        k_batch_fix_decide<<<g, 256, 0, st>>>(P.d_inst, P.count, P.d_eoff, P.ro.knu_max);
+        k_ffix<KIND_ARROW><<<g1, 64, 0, st>>>(src);
+        if (P.fast) k_fmore<KIND_ARROW><<<gm, 256, 0, st>>>(src, P.so, 1, 0);
         k_batch_fix_solve<<<batch_eig_grid(), 256, 0, st>>>(P.d_inst, P.d_fix, P.d_ctl, P.so,
                                                              P.wbuf, P.wstride);
     }
     k_batch_place<<<g, 256, 0, st>>>(P.d_inst, P.count, P.d_eoff);
-    k_batch_vectors<<<sms * 16, 256, 0, st>>>(P.d_inst, P.count, P.d_eoff, P.d_ctl);
+    if (P.fast && P.vectors) k_fcols<KIND_ARROW><<<(unsigned)P.n8, 256, 0, st>>>(src);
+    k_batch_vectors<<<(unsigned)P.n8, 256, 0, st>>>(P.d_inst, P.count, P.d_off8);
     if (P.status) k_batch_status<<<(P.count + 255) / 256, 256, 0, st>>>(P.d_inst, P.count, P.status);
 }
 
@@ -438,16 +501,37 @@ static void free_plan(Plan *P) {
     if (!P) return;
     if (P->exec) cudaGraphExecDestroy(P->exec);
     cudaFree(P->d_inst);
-    cudaFree(P->d_eoff);
-    cudaFree(P->d_uoff);
+    cudaFree(P->d_eoff);         // (the other tables lie behind it)
     cudaFree(P->d_fix);
+    cudaFree(P->d_old);
+    cudaFree(P->d_more);
     cudaFree(P->d_ctl);
     cudaFree(P->scratch);
     cudaFree(P->wbuf);
     delete P;
 }
 
-// Build the descriptor table and scratch; `force_team` > 0 overrides the tuner.
+// an instance's descriptor (alpha lives on the device)
+static BatchInst make_inst(int n, const double *d, const double *z, const double *alpha,
+                           double *lambda, double *V, const Scratch &S, int team) {
+    BatchInst B;
+    B.n = n;
+    B.n1 = n - 1;
+    B.d = d;
+    B.z = z;
+    B.alpha = alpha;
+    B.S = S;
+    Outputs out{};
+    out.lambda = lambda;
+    out.V = V;
+    out.ldv = n;
+    B.va = VecArgs{n, n - 1, d, z, z, nullptr, 0.0, 1.0, out};
+    B.team = team;
+    return B;
+}
+
+// Build the descriptor table and scratch; `force_team` > 0 overrides the tuner
+// and takes the FP64 solver (the tuner times it).
 static cudaError_t build_plan(Plan *P, int count, const long long *n_off, const long long *v_off,
                               const double *d_all, const double *z_all, const double *alpha_all,
                               double *lambda_all, double *V_all, int *status_all,
@@ -456,58 +540,47 @@ static cudaError_t build_plan(Plan *P, int count, const long long *n_off, const 
     P->status = status_all;
     P->ro = ro;
     P->so = SolveOpts{ro.max_iter, ro.precision, ro.finish, ro.bgate, ro.kb_max};
+    P->fast = force_team <= 0 && ro.max_iter >= kMinIterCap;
+    P->vectors = V_all != nullptr;
     std::vector<size_t> soff(count + 1, 0);
+    std::vector<int> ns(count), W(count);
     for (int i = 0; i < count; ++i) {
-        const int n = (int)(n_off[i + 1] - n_off[i]);
-        soff[i + 1] = soff[i] + ((arrow_scratch_bytes(n) + 255) & ~(size_t)255);
+        ns[i] = (int)(n_off[i + 1] - n_off[i]);
+        W[i] = force_team > 0 ? force_team : team_for(ns[i]);
+        soff[i + 1] = soff[i] + inst_bytes(ns[i]);
     }
-    P->total_n = n_off[count];
+    const std::vector<long long> tab = prefix_tables(count, ns.data(), W.data(), *P);
+    const size_t items = (size_t)(P->total_n > 0 ? P->total_n : 1);
+    long long *d_tab = nullptr;
     cudaError_t e;
     if ((e = cudaMalloc(&P->scratch, soff[count] + 256))) return e;
     if ((e = cudaMalloc(&P->d_inst, sizeof(BatchInst) * count))) return e;
-    if ((e = cudaMalloc(&P->d_eoff, sizeof(long long) * (count + 1)))) return e;
-    if ((e = cudaMalloc(&P->d_uoff, sizeof(long long) * (count + 1)))) return e;
-    if ((e = cudaMalloc(&P->d_fix, sizeof(int2) * (size_t)(P->total_n > 0 ? P->total_n : 1))))
-        return e;
+    if ((e = cudaMalloc(&d_tab, sizeof(long long) * tab.size()))) return e;
+    set_tables(*P, d_tab);
+    if ((e = cudaMalloc(&P->d_fix, sizeof(int2) * items))) return e;
+    if ((e = cudaMalloc(&P->d_old, sizeof(int2) * items))) return e;
+    if ((e = cudaMalloc(&P->d_more, sizeof(int2) * items))) return e;
     if ((e = cudaMalloc(&P->d_ctl, sizeof(BatchCtl)))) return e;
     long long nmax = 1;
-    for (int i = 0; i < count; ++i) nmax = std::max(nmax, n_off[i + 1] - n_off[i]);
+    for (int i = 0; i < count; ++i) nmax = std::max<long long>(nmax, ns[i]);
     P->wstride = (nmax + 1) & ~1LL;
     if ((e = cudaMalloc(&P->wbuf, sizeof(double2) * P->wstride * 4 *
                                       (size_t)batch_eig_grid() * 8)))
         return e;
     P->host.resize(count);
-    std::vector<long long> uoff(count + 1, 0);
     long long vo = 0;
     for (int i = 0; i < count; ++i) {
-        const int n = (int)(n_off[i + 1] - n_off[i]);
-        BatchInst &B = P->host[i];
-        B.n = n;
-        B.n1 = n - 1;
-        B.d = d_all + (n_off[i] - i);
-        B.z = z_all + (n_off[i] - i);
-        B.alpha = alpha_all + i;
-        B.S = carve_scratch((char *)P->scratch + soff[i], n);
-        B.out.lambda = lambda_all + n_off[i];
+        const int n = ns[i];
         const long long vi = v_off ? v_off[i] : vo;
-        B.out.V = V_all ? V_all + vi : nullptr;
-        B.out.ldv = n;
-        B.out.U = nullptr;
-        B.out.ldu = 0;
-        B.out.shift = B.out.mu = nullptr;
-        B.out.dg_b = B.out.dg_Kb = B.out.dg_Knu = nullptr;
-        B.out.dg_iters = B.out.dg_flags = nullptr;
-        B.team = force_team > 0 ? force_team : team_for(n);
+        P->host[i] = make_inst(n, d_all + (n_off[i] - i), z_all + (n_off[i] - i), alpha_all + i,
+                               lambda_all + n_off[i], V_all ? V_all + vi : nullptr,
+                               carve_inst((char *)P->scratch + soff[i], n, P->fast), W[i]);
         vo += (long long)n * n;
-        uoff[i + 1] = uoff[i] + (n + (32 / B.team) - 1) / (32 / B.team);
     }
     if ((e = cudaMemcpyAsync(P->d_inst, P->host.data(), sizeof(BatchInst) * count,
                              cudaMemcpyHostToDevice, st)))
         return e;
-    if ((e = cudaMemcpyAsync(P->d_eoff, n_off, sizeof(long long) * (count + 1),
-                             cudaMemcpyHostToDevice, st)))
-        return e;
-    if ((e = cudaMemcpyAsync(P->d_uoff, uoff.data(), sizeof(long long) * (count + 1),
+    if ((e = cudaMemcpyAsync(d_tab, tab.data(), sizeof(long long) * tab.size(),
                              cudaMemcpyHostToDevice, st)))
         return e;
     return cudaStreamSynchronize(st);
@@ -521,7 +594,7 @@ static cudaError_t build_plan(Plan *P, int count, const long long *n_off, const 
 // tables, remedy list, control block, corners, per-instance scratch and the
 // stored-pair slices; every part 256-byte aligned.
 struct ReqBatchLayout {
-    size_t inst, eoff, uoff, fix, ctl, alpha, scratch, wbuf, total;
+    size_t inst, tab, fix, old, more, ctl, alpha, scratch, wbuf, total;
     long long wstride;
     std::vector<size_t> soff;
 };
@@ -534,14 +607,15 @@ static ReqBatchLayout req_batch_layout(int count, const int *ns) {
     for (int i = 0; i < count; ++i) {
         total_n += ns[i];
         nmax = std::max<long long>(nmax, ns[i]);
-        L.soff[i + 1] = L.soff[i] + up(arrow_scratch_bytes(ns[i]));
+        L.soff[i + 1] = L.soff[i] + inst_bytes(ns[i]);
     }
     L.wstride = (nmax + 1) & ~1LL;
     size_t p = 0;
     L.inst = p; p += up(sizeof(BatchInst) * count);
-    L.eoff = p; p += up(sizeof(long long) * (count + 1));
-    L.uoff = p; p += up(sizeof(long long) * (count + 1));
+    L.tab = p;  p += up(sizeof(long long) * 4 * (count + 1));
     L.fix = p;  p += up(sizeof(int2) * (size_t)(total_n > 0 ? total_n : 1));
+    L.old = p;  p += up(sizeof(int2) * (size_t)(total_n > 0 ? total_n : 1));
+    L.more = p; p += up(sizeof(int2) * (size_t)(total_n > 0 ? total_n : 1));
     L.ctl = p;  p += up(sizeof(BatchCtl));
     L.alpha = p; p += up(sizeof(double) * count);
     L.scratch = p; p += L.soff[count];
@@ -554,10 +628,10 @@ size_t req_batch_bytes(int count, const int *ns) { return req_batch_layout(count
 
 // Solve `count` arrowhead requests (orders ns, inputs d[i], z[i] with corner
 // alpha[i], outputs lam[i] and V[i] with ld = n) with the batched stages on
-// `st`, using the device block `block` of req_batch_bytes() bytes.  Every
-// eigenpair is solved by a 32-lane team, so each result has the bits the
-// single-instance solve gives (remedies, solved by a warp here and by a team
-// as wide as one wave allows there, agree within the tolerance).  cnt[i]
+// `st`, using the device block `block` of req_batch_bytes() bytes.  Each
+// result has the bits the single-instance solve gives (remedies the FP64
+// solver takes, by a warp here and by a team as wide as one wave allows there,
+// agree within the tolerance).  cnt[i]
 // receives the device address of instance i's counters (C_COUNT ints).
 cudaError_t launch_req_batch(int count, const int *ns, const double *const *d,
                              const double *const *z, const double *alpha, double *const *lam,
@@ -569,40 +643,30 @@ cudaError_t launch_req_batch(int count, const int *ns, const double *const *d,
     P.count = count;
     P.ro = ro;
     P.so = SolveOpts{ro.max_iter, ro.precision, ro.finish, ro.bgate, ro.kb_max};
+    P.fast = ro.max_iter >= kMinIterCap;
     P.d_inst = (BatchInst *)(b + L.inst);
-    P.d_eoff = (long long *)(b + L.eoff);
-    P.d_uoff = (long long *)(b + L.uoff);
     P.d_fix = (int2 *)(b + L.fix);
+    P.d_old = (int2 *)(b + L.old);
+    P.d_more = (int2 *)(b + L.more);
     P.d_ctl = (BatchCtl *)(b + L.ctl);
     P.wbuf = (double2 *)(b + L.wbuf);
     P.wstride = L.wstride;
     double *d_alpha = (double *)(b + L.alpha);
     std::vector<BatchInst> host(count);
-    std::vector<long long> eoff(count + 1, 0), uoff(count + 1, 0);
+    const std::vector<int> W(count, 32);
+    const std::vector<long long> tab = prefix_tables(count, ns, W.data(), P);
+    set_tables(P, (long long *)(b + L.tab));
     for (int i = 0; i < count; ++i) {
-        BatchInst &B = host[i];
-        B.n = ns[i];
-        B.n1 = ns[i] - 1;
-        B.d = d[i];
-        B.z = z[i];
-        B.alpha = d_alpha + i;
-        B.S = carve_scratch(b + L.scratch + L.soff[i], ns[i]);
-        B.out = Outputs{};
-        B.out.lambda = lam[i];
-        B.out.V = V ? V[i] : nullptr;
-        B.out.ldv = ns[i];
-        B.team = 32;
-        eoff[i + 1] = eoff[i] + ns[i];
-        uoff[i + 1] = uoff[i] + ns[i];
-        cnt[i] = B.S.cnt;
+        double *Vi = V ? V[i] : nullptr;
+        P.vectors |= Vi != nullptr;
+        host[i] = make_inst(ns[i], d[i], z[i], d_alpha + i, lam[i], Vi,
+                            carve_inst(b + L.scratch + L.soff[i], ns[i], P.fast), 32);
+        cnt[i] = host[i].S.cnt;
     }
-    P.total_n = eoff[count];
     // (pageable sources: each copy is staged before the call returns)
     cudaError_t e = cudaMemcpyAsync(P.d_inst, host.data(), sizeof(BatchInst) * count,
                                     cudaMemcpyHostToDevice, st);
-    if (!e) e = cudaMemcpyAsync(P.d_eoff, eoff.data(), sizeof(long long) * (count + 1),
-                                cudaMemcpyHostToDevice, st);
-    if (!e) e = cudaMemcpyAsync(P.d_uoff, uoff.data(), sizeof(long long) * (count + 1),
+    if (!e) e = cudaMemcpyAsync(P.d_eoff, tab.data(), sizeof(long long) * tab.size(),
                                 cudaMemcpyHostToDevice, st);
     if (!e) e = cudaMemcpyAsync(d_alpha, alpha, sizeof(double) * count, cudaMemcpyHostToDevice,
                                 st);

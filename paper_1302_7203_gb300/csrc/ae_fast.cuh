@@ -1,0 +1,1448 @@
+// ae_fast.cuh -- all eigenpairs of a reduced arrowhead by a few O(n) passes in
+// fixed point (ae_fixed.cuh), one thread per eigenpair for everything scalar.
+//
+// The secular function f(lambda) = alpha - lambda - sum_j zeta_j^2 / (p_j - lambda)
+// (the shifted inverse's Pick function F of Algorithm 3 is f divided by
+// zeta_i^2 / mu^2 up to sign) is evaluated at lambda = p_i + mu with every
+// difference exact and every term good to ~2^-59, against 2^-53 a rounding in
+// FP64: that covers what the paper's doubled-precision b buys wherever the
+// terms' cancellation against the pole's own term stays below 2^5 (kErrTerm).
+// Beyond it f is summed in 128 bits (~2^-80), and wherever a range test fails
+// the eigenpair takes the FP64 / double-double solver (k_fold, ae_solver.cuh).
+//
+//   k_fprep   poles, spikes and rows in scaled and fixed-point form
+//   k_fopen   FP32: midpoint test (Algorithm 1), K_b (Algorithm 5's gate
+//             counters), model steps to |error| < 2^-16 of the distance to the
+//             nearest pole; a warp holds 4 eigenpairs, so that a pole read
+//             from L1/L2 serves 4
+//   k_feval   fixed point: f and its next four derivatives' sums in one pass
+//   k_fstep   one thread per eigenpair: the zero from the quartic expansion
+//             (relative error eps^4 at a step eps of the pole distance), the
+//             vector's norm from the same sums, else a model step
+//   k_fmore   the few (1-4 %) whose opening was too far off or whose terms
+//             cancel too much: further evaluations, a CTA each, with f summed
+//             in 128 bits
+//   k_fold    the FP64 solver for what is left, a CTA per eigenpair
+//   k_ffix    remedies (Remarks 1, 2): the zero is already known beyond double
+//             precision, so moving it to the remedy's shift is a subtraction;
+//             checked, else k_fmore evaluates f at the zero in 128 bits first,
+//             and what that does not settle is left to k_fix_solve
+//   k_fcols   columns: one difference, one reciprocal and two products a
+//             component, normalised in the same step and written once
+#pragma once
+#include "ae_fixed.cuh"
+#include "ae_pipeline.cuh"
+
+namespace ae {
+
+// states of a computed eigenpair in the fast path
+enum { FST_EVAL = 0, FST_DONE = 1, FST_OLD = 2, FST_MORE = 3 };
+
+// A zero's offset mu is taken from an evaluation whose error is below 2^-54 of
+// it.  Two errors count, both over f' |mu|: the terms' and sums', 2^-59 (in
+// 128 bits 2^-80) of sum |zeta^2/(p - lambda)|, and that of the differences'
+// unit, 2^-105 of sum zeta^2/(p - lambda)^2 (the differences formed in
+// double-double left out).  Hence the weights of the two sums against f' |mu|:
+constexpr double kErrTerm = 0x1p-5, kErrTermWide = 0x1p-25, kErrUnit = 0x1p-50;
+// largest step, relative to the distance to the nearest pole, that the quartic
+// expansion closes: (2^-14)^4 = 2^-56
+constexpr double kStepMax = 0x1p-14;
+constexpr int kMoreRounds = 4;
+// iteration caps below this are meant to stop a solve: the FP64 solver takes them
+constexpr int kMinIterCap = 100;
+
+__device__ __forceinline__ unsigned long long shr64(unsigned long long v, unsigned s) {
+    unsigned long long r;
+    asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(s));   // 0 from 64 on
+    return r;
+}
+__device__ __forceinline__ unsigned hi32(double x) { return (unsigned)__double2hiint(x); }
+__device__ __forceinline__ unsigned bexp(double x) { return (hi32(x) << 1) >> 21; }
+
+// ---------------------------------------------------------------------------
+// where the kernels find their instances
+// ---------------------------------------------------------------------------
+struct SrcOne {          // one instance, by value
+    Scratch S;
+    VecArgs va;
+    __device__ bool unit(long long u, int per, int &i, int &first) const {
+        i = 0;
+        first = (int)u * per;
+        return true;
+    }
+    __device__ bool item(long long t, int &i, int &idx) const {
+        i = 0;
+        idx = (int)t;
+        return t < va.n;
+    }
+    __device__ const Scratch &scr(int) const { return S; }
+    __device__ const VecArgs &vec(int) const { return va; }
+    __device__ void push_old(int, int k) const { S.f.old[atomicAdd(S.cnt + C_NOLD, 1)] = k; }
+    __device__ int old_count() const { return S.cnt[C_NOLD]; }
+    __device__ int2 old_at(int w) const { return make_int2(0, S.f.old[w]); }
+    __device__ int *old_ticket() const { return S.cnt + C_OLDTK; }
+    // eigenpairs for k_fmore: phase 0 after k_fstep, phase 1 after k_ffix (the
+    // list of phase 0 is done with by then)
+    __device__ void push_more(int ph, int, int k) const {
+        S.f.more[atomicAdd(S.cnt + C_NMORE + ph, 1)] = k;
+    }
+    __device__ int more_count(int ph) const { return S.cnt[C_NMORE + ph]; }
+    __device__ int2 more_at(int w) const { return make_int2(0, S.f.more[w]); }
+    __device__ void push_fix(int, int k, bool front, int n) const {
+        if (front) S.fixlist[atomicAdd(S.cnt + C_NFIX, 1)] = k;
+        else S.fixlist[n - 1 - atomicAdd(S.cnt + C_NFIX2, 1)] = k;
+    }
+    __device__ double2 *slice(long long w) const {
+        return S.wbuf ? S.wbuf + w * S.wstride : nullptr;
+    }
+};
+
+// eigenpairs [lo, hi) of the reduced arrowhead that this solve computes (a
+// part also solves the eigenpair on each side of its range)
+__device__ __forceinline__ void fast_range(const Scratch &S, int &lo, int &hi) {
+    lo = 0;
+    hi = S.cnt[C_M] + 1;
+    if (S.cnt[C_PART]) {
+        lo = S.cnt[C_K0] > 0 ? S.cnt[C_K0] - 1 : 0;
+        hi = S.cnt[C_KHI];
+    }
+}
+
+// power of two that scales the poles below 1/2 (see k_fprep)
+template <Kind K>
+__device__ __forceinline__ int fast_scale(const Scratch &S) {
+    const int e = ilogb(S.prm[P_DS]);
+    return K == KIND_TSVD ? 2 * e - 3 : e - 2;
+}
+
+__device__ __forceinline__ double pow2(int e) {          // 2^e, -1022 <= e <= 1023
+    return __longlong_as_double((long long)(1023 + e) << 52);
+}
+
+// ---------------------------------------------------------------------------
+// k_fprep
+// ---------------------------------------------------------------------------
+// pole (or row) value in scaled double-double: d, or d^2 for the SVD
+template <Kind K>
+__device__ __forceinline__ dd fast_pole(double d, int es) {
+    if (K == KIND_TSVD) {
+        const double s = d * pow2((es + 3) / 2);
+        const dd q = two_prod(s, s);
+        return dd{q.hi * 0.125, q.lo * 0.125};
+    }
+    return dd{ldexp(d, es), 0.0};
+}
+
+// One thread per pole and row.  Whatever falls outside the ranges the fixed-
+// point passes are made for sets CF_NOFAST, and the whole instance is solved
+// by the FP64 solver.
+template <Kind K>
+__device__ __forceinline__ void fprep_item(const Scratch &S, const VecArgs &va, int t) {
+    const int m = S.cnt[C_M];
+    bool bad = false;
+    const int es = fast_scale<K>(S);
+    const int e0 = K == KIND_TSVD ? (es + 3) / 2 : es;
+    if (m < 2 || es < -480 || es > 480 || e0 < -480 || e0 > 480) {
+        if (t == 0) atomicOr(S.cnt + C_FLAGS, CF_NOFAST);
+        return;
+    }
+    if (t < m) {
+        const dd p = fast_pole<K>(S.pd[t], es);
+        S.f.p[t] = p.hi;
+        S.f.plo[t] = p.lo;
+        S.f.P[t] = fix_mod(p.hi) + fix_mod(p.lo);
+        bad |= !(fabs(p.hi) < 0.5) || (p.hi != 0.0 && fabs(p.hi) < 0x1p-900);
+        // zeta^2 as a 64-bit significand and exponent (scaled by 4^es)
+        const double z2 = S.pz2[t], zl = S.pz2lo[t];
+        const int e = (int)bexp(z2) - 1023;
+        bad |= !(e > -900 && e < 900);
+        if (!bad) {
+            const unsigned long long b = (unsigned long long)__double_as_longlong(z2);
+            unsigned long long Z = ((b & 0xfffffffffffffull) | 0x10000000000000ull) << 11;
+            Z += (unsigned long long)__double2ll_rn(ldexp(zl, 63 - e));
+            if (!(Z >> 63)) Z = ~0ull;               // a low part that rounds below 2^63, or over
+            S.f.z[t] = Z;
+            S.f.ez[t] = e + 2 * es;
+        }
+    }
+    if (t < va.n1) {
+        const dd p = fast_pole<K>(va.key[t], es);
+        S.f.rp[t] = p.hi;
+        S.f.rP[t] = fix_mod(p.hi) + fix_mod(p.lo);
+    }
+    if (t == 0) bad |= !(fabs(ldexp(S.prm[P_ALPHA_HI], es)) < 0x1p300);
+    if (bad) atomicOr(S.cnt + C_FLAGS, CF_NOFAST);
+}
+
+// ---------------------------------------------------------------------------
+// the evaluation point of an eigenpair
+// ---------------------------------------------------------------------------
+// lambda = sigma + mu as its rounded value and its fixed-point form.  Beyond
+// |lambda| = 5/2 (an outermost eigenvalue far from all poles) the rounded
+// value IS the point, mu absorbs the difference, and no tails are taken.
+__device__ __forceinline__ bool set_point(const Scratch &S, int k, dd sg, dd mu) {
+    dd l = two_sum(sg.hi, mu.hi);
+    l.lo += sg.lo + mu.lo;
+    l = fast_two_sum(l.hi, l.lo);
+    const bool notail = !(fabs(l.hi) < 2.5);
+    if (notail) {
+        mu = dd_add(dd{l.hi, 0.0}, dd_neg(sg));
+        l.lo = 0.0;
+    }
+    S.f.mu[k] = mu.hi;
+    S.f.mulo[k] = mu.lo;
+    S.f.lhi[k] = l.hi;
+    S.f.lmod[k] = fix_mod(l.hi) + fix_mod(l.lo);
+    return isfinite(l.hi);
+}
+
+// Differences whose biased exponent lies in [lo, lo + span) are formed as
+// fl(p - lambda) with the modular tail (tails != 0) or without one (a point
+// beyond 5/2); the others as (p - sigma) - mu in double-double: those small
+// against lambda or the unit, and a DPR1's last pole, which is no pole of the
+// arrowhead and may lie far outside the others or next to such a point.
+struct DiffRange {
+    unsigned lo, span;
+    int tails;            // mask of the tail
+};
+__device__ __forceinline__ DiffRange diff_range(double lhi) {
+    const unsigned e = bexp(lhi);
+    const unsigned a = e > 6u ? e - 6u : 0u;
+    if (!(fabs(lhi) < 2.5)) return {a, 4096u, 0};
+    const unsigned lo = a > kFixMinExp ? a : kFixMinExp;
+    return {lo, 1025u - lo, -1};
+}
+
+// |p - lambda| where it is small against lambda or against the unit: value
+// and tail (2^-23 of its last place)
+__device__ __forceinline__ double near_diff(dd p, dd sg, dd mu, int &tl) {
+    const dd dl = dd_add(p, dd_neg(sg));
+    const dd D = dd_add(dl, dd_neg(mu));
+    const double t = ldexp(D.hi < 0.0 ? -D.lo : D.lo, 23 + 52 + 1023 - (int)bexp(D.hi));
+    tl = (int)t;
+    return D.hi;
+}
+
+// sigma (the shift pole, or another shift) in scaled double-double
+template <Kind K>
+__device__ __forceinline__ dd fast_sigma(const Scratch &S, int k, int es) {
+    const int i = S.es_pole[k];
+    if (i >= 0) return dd{S.f.p[i], S.f.plo[i]};
+    return dd{ldexp(S.es_sigma[k], es), 0.0};
+}
+
+// ---------------------------------------------------------------------------
+// k_fopen
+// ---------------------------------------------------------------------------
+// Sums over the warp of four values, one per eigenpair: lane group g = lane/8
+// ends with the sum of v[g] (6 shuffles instead of 20).
+__device__ __forceinline__ float reduce4(const float (&v)[4], int lane) {
+    const bool h = lane & 16, q = lane & 8;
+    float a = h ? v[2] : v[0], b = h ? v[3] : v[1];
+    const float sa = h ? v[0] : v[2], sb = h ? v[1] : v[3];
+    a += __shfl_xor_sync(FULL, sa, 16);
+    b += __shfl_xor_sync(FULL, sb, 16);
+    float k = q ? b : a;
+    const float s = q ? a : b;
+    k += __shfl_xor_sync(FULL, s, 8);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) k += __shfl_xor_sync(FULL, k, o);
+    return k;
+}
+__device__ __forceinline__ float reduce4max(const float (&v)[4], int lane) {
+    const bool h = lane & 16, q = lane & 8;
+    float a = h ? v[2] : v[0], b = h ? v[3] : v[1];
+    const float sa = h ? v[0] : v[2], sb = h ? v[1] : v[3];
+    a = fmaxf(a, __shfl_xor_sync(FULL, sa, 16));
+    b = fmaxf(b, __shfl_xor_sync(FULL, sb, 16));
+    float k = q ? b : a;
+    const float s = q ? a : b;
+    k = fmaxf(k, __shfl_xor_sync(FULL, s, 8));
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) k = fmaxf(k, __shfl_xor_sync(FULL, k, o));
+    return k;
+}
+
+__device__ __forceinline__ float sqrt_f32(float x) {
+    float r;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// Zero of the model Phi(mu) ~ A + B / (dn - mu) = w / mu fitted to (Phi, Phi')
+// at u, as |mu|: with e = |dn| the distance to the interval's other pole (0:
+// none, then Phi is linear), s the side, everything scaled by a power of two
+// so that squares stay in range.  (The one-pole model of the Newton finish,
+// written in mu = 1/x.)
+__device__ __forceinline__ float model_root(float s, float Phi, float dPhi, float u, float e,
+                                            float w) {
+    const float mu = fabsf(u);
+    if (e > 0.f) {
+        const float g = e - mu;
+        float B = dPhi * g * g;
+        float A = s * Phi - dPhi * g;
+        float X = fmaf(A, e, B);
+        const float big = fmaxf(fmaxf(fabsf(X), B), w);
+        const float c = __uint_as_float((254u << 23) - (__float_as_uint(big) & 0x7f800000u));
+        X *= c; B *= c; A *= c; w *= c;
+        const float b = X + w;
+        const float h = X - w;
+        const float rt = sqrt_f32(fmaf(4.f * w, B, h * h));
+        return b >= 0.f ? __fdividef(2.f * w * e, b + rt) : __fdividef(b - rt, 2.f * A);
+    }
+    const float A = s * Phi - dPhi * mu;             // A + B m = w / m
+    const float B = dPhi;
+    const float rt = sqrt_f32(fmaf(4.f * B, w, A * A));
+    return A >= 0.f ? __fdividef(2.f * w, A + rt) : __fdividef(rt - A, 2.f * B);
+}
+
+template <Kind K, class Src>
+__global__ void __launch_bounds__(256) k_fopen(const __grid_constant__ Src src, SolveOpts o) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int inst, first;
+    if (!src.unit(blockIdx.x, 32, inst, first)) return;
+    const Scratch &S = src.scr(inst);
+    const int m = S.cnt[C_M];
+    int klo, khi;
+    fast_range(S, klo, khi);
+    const int k0 = klo + first + 4 * wid;
+    if (k0 >= khi) return;
+    const int g = lane >> 3;                          // this lane group's eigenpair
+    const int k = k0 + g;
+    const bool have = k < khi;
+    if ((S.cnt[C_FLAGS] & CF_NOFAST) || m < 2) {
+        if (have && (lane & 7) == 0) {
+            S.f.st[k] = FST_OLD;
+            src.push_old(inst, k);
+        }
+        return;
+    }
+    const auto R = PolesOf<K>::make(S, m);
+    const int kc = have ? k : khi - 1;
+    const bool lowx = kc == 0, upx = kc == m;         // outermost eigenvalues
+    const double Ld = R.f32_scale();
+    const double g1 = R.zs / Ld;                      // scales f to the FP32 sums
+    const float gam = (float)(g1 / Ld);
+    float sh, sl, mf, tf[4], af[4], bf[4], df[4];
+    // ---- the sign of f at the midpoint of the eigenvalue's interval ----
+    int i = lowx ? 0 : upx ? m - 1 : kc, side = lowx ? +1 : -1;
+    const double sk = R.pole(i);
+    const double middle = (lowx || upx) ? 0.0 : 0.5 * R.shifted(kc - 1, sk, kc);
+    R.f32_shift(sk, i, sh, sl);
+    mf = (float)(middle * Ld);
+    float tm, am, bm, dm;
+    {
+        float she[4], sle[4], mfe[4];
+        bool bad[4] = {false, false, false, false};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            she[e] = __shfl_sync(FULL, sh, 8 * e);
+            sle[e] = __shfl_sync(FULL, sl, 8 * e);
+            mfe[e] = __shfl_sync(FULL, mf, 8 * e);
+            tf[e] = af[e] = bf[e] = df[e] = 0.f;
+        }
+        for (int j = lane; j < m; j += 32) {
+            const float z = R.z2f(j);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                float gg;
+                const float D = R.shifted_f32_mag(j, she[e], sle[e], gg) - mfe[e];
+                bad[e] |= !(fabsf(D) >= fmaf(gg, 0x1p-20f, 0x1p-100f));
+                const float r = rcp_f32(D);
+                const float t = z * r;
+                tf[e] += t;
+                af[e] += fabsf(t);
+                bf[e] += fabsf(r);
+                df[e] = fmaf(t, r, df[e]);
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            if (bad[e]) bf[e] = INFINITY;
+        tm = reduce4(tf, lane);
+        am = reduce4(af, lane);
+        bm = reduce4(bf, lane);
+        dm = reduce4(df, lane);
+    }
+    bool ok = true, mid64 = false;
+    int passes = 0;
+    if (!lowx && !upx) {
+        // (the bound is select_shift's)
+        const double a = R.a_dd(sk, i).hi - middle;
+        const double f = Ld / R.zs;
+        const double L = (double)((m + 31) / 32);
+        const double F32 = a - f * (double)tm;
+        const double ET = 2.0 * (L + 24.0) * 0x1p-24 * (2.0 * (double)am) +
+                          0x1p-148 * ((double)bm + (double)m);
+        const double M = f * ET * (1.0 + 0x1p-20) + (L + 16.0) * 0x1p-52 * fabs(a);
+        mid64 = !(isfinite(F32) && fabs(F32) > M * (1.0 + 0x1p-40));
+        // (left open: either side serves -- the zero is moved to the nearer
+        // pole once it is known, k_fstep)
+        if (F32 < 0.0) side = +1;
+        else { i = kc - 1; side = -1; }
+        ++passes;
+        // poles that FP32 pairs cannot tell apart here
+        ok &= middle > 0x1p-32 * fabs(sk);
+    }
+    // ---- the chosen pole: model steps ----
+    const double sig = R.pole(i);
+    R.f32_shift(sig, i, sh, sl);
+    const int jn = side > 0 ? i - 1 : i + 1;          // the interval's other pole
+    const float en = (jn >= 0 && jn < m) ? (float)(fabs(R.shifted(jn, sig, i)) * Ld) : 0.f;
+    const double a64 = R.a_dd(sig, i).hi;
+    const float Af = (float)(a64 * g1);
+    const float w = R.z2f(i);
+    const float s = (float)side;
+    const int jb = side > 0 ? i + 1 : i - 1;          // the pole behind it
+    if (jb >= 0 && jb < m) ok &= fabs(R.shifted(jb, sig, i)) > 0x1p-32 * fabs(sig);
+    ok &= w > 0x1p-100f && fabsf(Af) < 0x1p100f && gam < 0x1p60f;
+    float rm = 0.f;
+    if (!lowx && !upx) {
+        // from the midpoint: own term taken out (|mf| from either pole)
+        const float um = s * mf;
+        const float to = -w / um;                     // w / (0 - um)
+        const float Phi = -Af + gam * um + (tm - to);
+        const float dPhi = gam + fmaxf(dm - w / (mf * mf), 0.f);
+        rm = model_root(s, Phi, dPhi, um, en, w);
+    }
+    float u = 0.f, ul = 0.f, wsum = 0.f, wmax = 0.f, num = 0.f, Tabs = 0.f, dsum = 0.f;
+    bool done = false;
+    const bool gersh = o.finish == 0;
+    for (int it = 0; it < 9; ++it) {
+        float she[4], sle[4], ue[4], wi[4], sd[4], ws[4], wx[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            she[e] = __shfl_sync(FULL, sh, 8 * e);
+            sle[e] = __shfl_sync(FULL, sl, 8 * e);
+            ue[e] = __shfl_sync(FULL, u, 8 * e);
+            tf[e] = af[e] = df[e] = 0.f;
+        }
+        if (it == 0 && gersh) {
+            // with Algorithm 3's bracket: sum and extreme of the Gershgorin
+            // quantities |w_j| = zeta_j / (|delta_j| zeta_i)
+            const float iw = rcp_f32(sqrt_f32(w));
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                wi[e] = __shfl_sync(FULL, iw, 8 * e);
+                sd[e] = __shfl_sync(FULL, s, 8 * e);
+                ws[e] = wx[e] = 0.f;
+            }
+            for (int j = lane; j < m; j += 32) {
+                const float z = R.z2f(j), q = sqrt_f32(z);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float D = R.shifted_f32(j, she[e], sle[e]);
+                    const float r = D == 0.f ? 0.f : rcp_f32(D);
+                    const float t = z * r;
+                    tf[e] += t;
+                    af[e] += fabsf(t);
+                    df[e] = fmaf(t, r, df[e]);
+                    const float aw = q * fabsf(r) * wi[e];
+                    ws[e] += aw;
+                    wx[e] = fmaxf(wx[e], fmaf(sd[e], r, aw));
+                }
+            }
+            wsum = reduce4(ws, lane);
+            wmax = reduce4max(wx, lane);
+        } else {
+            for (int j = lane; j < m; j += 32) {
+                const float z = R.z2f(j);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float D = R.shifted_f32(j, she[e], sle[e]);
+                    const float rr = rcp_f32(D - ue[e]);
+                    const float r = D == 0.f ? 0.f : rr;     // not the shift pole's own
+                    const float t = z * r;
+                    tf[e] += t;
+                    af[e] += fabsf(t);
+                    df[e] = fmaf(t, r, df[e]);
+                }
+            }
+        }
+        const float t = reduce4(tf, lane);
+        const float a = reduce4(af, lane);
+        const float d = reduce4(df, lane);
+        if (!done) {
+            ++passes;
+            const float Phi = -Af + gam * u + t, dPhi = gam + d;
+            if (it == 0) {
+                num = Phi;
+                Tabs = a;
+                dsum = d;
+                // between the zeros of the models at the pole and at the midpoint
+                const float r0 = model_root(s, Phi, dPhi, 0.f, en, w);
+                u = (!lowx && !upx) ? s * 0.5f * (r0 + rm) : s * r0;
+            } else {
+                const float mn = model_root(s, Phi, dPhi, u, en, w);
+                const float mo = fabsf(u);
+                const float rho = en > 0.f ? fminf(mn, en - mn) : mn;
+                if (!(mn > 0.f) || (en > 0.f && !(mn < en))) { ok = false; done = true; }
+                else if (fabsf(mn - mo) <= 0x1p-8f * rho) {
+                    ul = s * mn;
+                    Tabs = a + __fdividef(w, mn);     // (num keeps the pole's own sums)
+                    dsum = d;
+                    done = true;
+                }
+                u = s * mn;
+            }
+        }
+        if (it == 0) {
+            // Algorithm 5's gate quantities, for its counters (Eq. K2: P + Q over |P - Q|)
+            float kb = __fdividef(Tabs + fabsf(Af), fabsf(num));
+            bm = kb;
+            am = wsum;
+            tm = wmax;
+        }
+        if (__all_sync(FULL, done || !ok)) break;
+    }
+    ok &= done && isfinite(ul) && ul != 0.f && isfinite(Tabs) && Tabs > 0.f && isfinite(dsum);
+    if (!have || (lane & 7) != 0) return;
+    int flags = 0;
+    if (o.precision == 1) {
+        atomicAdd(S.cnt64 + C64_F32, (unsigned long long)passes);
+        if (mid64) flags |= AE_FLAG_MID64;             // (counted when solved)
+    }
+    if (o.bgate) {
+        const double zi = R.zabs(i);
+        if (R.zsum - zi > (double)(m + 1) * zi && !((double)bm <= o.kb_max)) {
+            flags |= AE_FLAG_DDB;
+        }
+    }
+    S.es_flags[k] = flags;
+    S.es_pole[k] = i;
+    S.es_Knu[k] = 1.0;
+    S.es_b[k] = (double)num / (double)w * R.f32_scale();
+    S.es_Kb[k] = (double)bm;
+    S.es_iters[k] = 0;
+    const int es = fast_scale<K>(S);
+    const int eL = ilogb(Ld), ezs = ilogb(R.zs);
+    const double mu = ldexp((double)ul, es - eL);
+    if (gersh) {
+        // steps of Algorithm 3 from its Gershgorin bracket (1/mu inside it) to
+        // the width 2 eps |1/mu|; after an FP32 bracket, from that one's width
+        const float iw = rcp_f32(sqrt_f32(w));
+        const float b = s * num / w;                   // (in units of 1/D)
+        const float left = en > 0.f ? rcp_f32(en) : 0.f;
+        const float wz = iw * sqrt_f32(gam);           // 1/zeta_i
+        const float right = fmaxf(fmaxf(tm, wz), b + am + wz);
+        const float W = (right - left) * fabsf(ul);
+        int N = isfinite(W) && W > 0.f ? (int)ceilf(log2f(W) + 51.f) : 62;
+        N = N < 1 ? 1 : N;
+        if (o.precision == 1 && N > 32) N = 32;
+        S.es_iters[k] = N;
+    }
+    const dd sg = {S.f.p[i], S.f.plo[i]};
+    ok &= set_point(S, k, sg, dd{mu, 0.0});
+    // bounds of the sums: sum |t| < 2^K1, sum zeta^2/D^2 < 2^K2 (the pole's own
+    // term by its exponent: it can exceed FP32's range), |D| >= 2^er
+    const float mn = fabsf(ul);
+    S.f.K1[k] = ilogbf(Tabs * 1.02f) + 1 + eL + es - ezs;
+    S.f.K2[k] = max(dsum > 0.f ? ilogbf(dsum * 1.04f) + 1 : -200,
+                    ilogbf(__fdividef(w, mn) * 1.04f) + 1 - ilogbf(mn)) + 1 + 2 * eL - ezs;
+    S.f.er[k] = ilogbf(0.98f * (en > 0.f ? fminf(mn, en - mn) : mn)) + es - eL;
+    S.f.st[k] = ok ? FST_EVAL : FST_OLD;
+    if (!ok) src.push_old(inst, k);
+}
+
+// ---------------------------------------------------------------------------
+// k_feval
+// ---------------------------------------------------------------------------
+// Five sums over the poles at each eigenpair's point: zeta^2/(p - lambda)^r for
+// r = 1..5, a warp per eigenpair, the 8 warps of a CTA sharing tiles of poles in
+// shared memory.  Bound by issue slots: ~90 a term (FP64: one subtraction, 64
+// clocks of that pipe, behind them); the r = 4, 5 sums are skipped, warp by
+// warp, where no lane's term reaches 2^-44 of their bound.
+constexpr int kTile = 256;
+
+template <class Src>
+__global__ void __launch_bounds__(256, 3) k_feval(const __grid_constant__ Src src) {
+    __shared__ double tp[2][kTile];
+    __shared__ unsigned long long tP[2][kTile], tz[2][kTile];
+    __shared__ int te[2][kTile];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int inst, first;
+    if (!src.unit(blockIdx.x, 8, inst, first)) return;
+    const Scratch &S = src.scr(inst);
+    int klo, khi;
+    fast_range(S, klo, khi);
+    if (klo + first >= khi) return;
+    const int k = klo + first + wid;
+    const bool act = k < khi && S.f.st[k] == FST_EVAL;
+    if (!__syncthreads_or(act)) return;
+    const int m = S.cnt[C_M];
+    const int ka = act ? k : klo + first;
+    const double lhi = S.f.lhi[ka];
+    const unsigned long long L = S.f.lmod[ka];
+    const DiffRange dr = diff_range(lhi);
+    const int K1 = S.f.K1[ka], K2 = S.f.K2[ka], er = S.f.er[ka];
+    const int c1 = K1 - 1023, c2 = K2 - K1 + 1 - 1023, c3 = 2 - er - 1023, c4 = 1 - er - 1023;
+    unsigned long long a1 = 0, a2 = 0, a3 = 0, a4 = 0, a5 = 0;
+    int n1 = 0, n2 = 0;
+    bool flip = true;
+    auto load = [&](int t, double &p, unsigned long long &P, unsigned long long &z, int &e) {
+        const int j = t * kTile + threadIdx.x;
+        p = 4.0; P = 0; z = 0; e = -8192;               // padding: terms of 0
+        if (j < m) {
+            p = S.f.p[j];
+            P = S.f.P[j];
+            z = S.f.z[j];
+            e = S.f.ez[j];
+        }
+    };
+    const int tiles = (m + kTile - 1) / kTile;
+    double lp;
+    unsigned long long lP, lz;
+    int le;
+    load(0, lp, lP, lz, le);
+    for (int t = 0; t < tiles; ++t) {
+        const int bsel = t & 1;
+        tp[bsel][threadIdx.x] = lp;
+        tP[bsel][threadIdx.x] = lP;
+        tz[bsel][threadIdx.x] = lz;
+        te[bsel][threadIdx.x] = le;
+        __syncthreads();
+        if (t + 1 < tiles) load(t + 1, lp, lP, lz, le);
+        if (!act) continue;
+        const int left = m - t * kTile;
+        const int nc = left >= kTile ? kTile / 32 : (left + 31) / 32;
+#pragma unroll 1
+        for (int c = 0; c < nc; ++c) {
+            const int x = c * 32 + lane;
+            const int j0 = t * kTile + c * 32;
+            double D = tp[bsel][x] - lhi;
+            int tl;
+            unsigned dh = hi32(D), dl = (unsigned)__double2loint(D);
+            unsigned eb = (dh << 1) >> 21;
+            const int j = j0 + lane;
+            if (eb - dr.lo >= dr.span && j < m) {
+                const dd pj = {tp[bsel][x], S.f.plo[j]};
+                const int i = S.es_pole[ka];
+                const dd sg = {S.f.p[i], S.f.plo[i]};
+                D = near_diff(pj, sg, dd{S.f.mu[ka], S.f.mulo[ka]}, tl);
+                dh = hi32(D);
+                dl = (unsigned)__double2loint(D);
+                eb = (dh << 1) >> 21;
+            } else {
+                tl = tail_of(tP[bsel][x] - L, dh, dl, eb) & dr.tails;
+            }
+            const unsigned seed = hi32(rcp_seed(__hiloint2double(
+                (int)((dh & 0xfffffu) | 0x3ff00000u), 0)));
+            const unsigned long long Rr = recip63<true>(dh, dl, tl, seed);
+            unsigned long long q = mul_hi3(tz[bsel][x], Rr);       // 2^62 of the term
+            const unsigned s1 = (unsigned)(c1 + (int)eb - te[bsel][x]);
+            unsigned long long v1 = shr64(q, s1);
+            const int u1 = s1 < 62u;
+            q = mul_hi3(q, Rr);
+            const unsigned s2 = s1 + eb + c2;
+            a2 += shr64(q, s2);
+            n2 += s2 < 60u;
+            q = mul_hi3(q, Rr);
+            const unsigned s3 = s2 + eb + c3;
+            unsigned long long v3 = shr64(q, s3);
+            unsigned long long v5 = 0;
+            const unsigned s4 = s3 + eb + c4;
+            if (__any_sync(FULL, (int)s4 < 44)) {
+                q = (unsigned long long)(unsigned)(q >> 32) * (unsigned)(Rr >> 32);
+                a4 += shr64(q, s4);
+                const unsigned s5 = s4 + eb + c4;
+                q = (unsigned long long)(unsigned)(q >> 32) * (unsigned)(Rr >> 32);
+                v5 = shr64(q, s5);
+            }
+            if (k >= j0 && k < j0 + 32) {
+                // the poles change sides of lambda in this chunk: sums of odd
+                // order end as (below) - (above)
+                const bool above = j < k;
+                a1 = (above ? 0ull - v1 : v1) - a1;
+                a3 = (above ? 0ull - v3 : v3) - a3;
+                a5 = (above ? 0ull - v5 : v5) - a5;
+                n1 = (above ? -u1 : u1) - n1;
+                flip = false;
+            } else {
+                a1 += v1;
+                a3 += v3;
+                a5 += v5;
+                n1 += u1;
+            }
+        }
+    }
+    if (!act) return;
+    if (flip) {
+        a1 = 0ull - a1;
+        a3 = 0ull - a3;
+        a5 = 0ull - a5;
+        n1 = -n1;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        a1 += __shfl_xor_sync(FULL, a1, o);
+        a2 += __shfl_xor_sync(FULL, a2, o);
+        a3 += __shfl_xor_sync(FULL, a3, o);
+        a4 += __shfl_xor_sync(FULL, a4, o);
+        a5 += __shfl_xor_sync(FULL, a5, o);
+    }
+    n1 = __reduce_add_sync(FULL, n1);
+    n2 = __reduce_add_sync(FULL, n2);
+    if (lane == 0) {
+        S.f.s1[k] = (long long)a1;
+        S.f.s2[k] = a2;
+        S.f.s3[k] = (long long)a3;
+        S.f.s4[k] = a4;
+        S.f.s5[k] = (long long)a5;
+        S.f.n1[k] = n1;
+        S.f.n2[k] = n2;
+    }
+}
+
+// ---------------------------------------------------------------------------
+// k_fstep
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ dd dd_of_ll(long long v) {
+    const double h = (double)v;
+    return fast_two_sum(h, (double)(v - (long long)h));
+}
+
+// the counters of a solved eigenpair, added up over the warp's lanes that
+// share its instance
+__device__ __forceinline__ void fast_stats(const Scratch &S, int inst, int iters, int deriv,
+                                           double Kb, bool ddb, bool any) {
+    const unsigned act = __ballot_sync(FULL, any);
+    if (!any) return;
+    const unsigned grp = __match_any_sync(act, inst);
+    const int it = __reduce_add_sync(grp, iters);
+    const int de = __reduce_add_sync(grp, deriv);
+    const int mx = __reduce_max_sync(grp, iters);
+    const int dd_ = __reduce_add_sync(grp, ddb ? 1 : 0);
+    const unsigned kb = __reduce_max_sync(grp, isfinite(Kb) && Kb >= 0.0
+                                                  ? __float_as_uint((float)Kb) : 0u);
+    if ((threadIdx.x & 31) == __ffs(grp) - 1) {
+        atomicAdd(S.cnt64 + C64_ITERS, (unsigned long long)it);
+        if (de) atomicAdd(S.cnt64 + C64_DERIV, (unsigned long long)de);
+        atomicMax(S.cnt + C_MAXIT, mx);
+        if (dd_) atomicAdd(S.cnt + C_DDB, dd_);
+        atomic_max_nonneg(S.cnt64 + C64_MAXKB, (double)__uint_as_float(kb));
+    }
+}
+
+// Sums of an evaluation at sigma + mu: M1 = (below - above), M_r = sum zeta^2 /
+// (p - lambda)^r for r >= 2, in scaled units.
+struct FastSums {
+    dd M1;
+    double M2, M3, M4, M5;
+};
+
+// The zero from an evaluation, by one thread.  cterm: the weight of the terms'
+// error (kErrTerm...); M2u: the sum the unit's error counts over (negative:
+// M2 less the pole's own term, always formed in double-double when small).
+// Returns FST_DONE with
+// the result stored (when no round is left FST_OLD), or FST_MORE with the next
+// point set: the model's zero, or the zero found where only its accuracy is
+// wanting.
+template <Kind K>
+__device__ int fast_advance(const Scratch &S, int k, const FastSums &q, double cterm, double M2u) {
+    const int m = S.cnt[C_M];
+    const int es = fast_scale<K>(S);
+    int i = S.es_pole[k];
+    const dd sg = {S.f.p[i], S.f.plo[i]};
+    const dd mu = {S.f.mu[k], S.f.mulo[k]};
+    const int K1 = S.f.K1[k], K2 = S.f.K2[k];
+    const double N = 1.0 + q.M2;
+    // f = (alpha - sigma - mu) + (sum below - sum above)
+    const double sc = pow2(es);
+    dd a = dd{S.prm[P_ALPHA_HI] * sc, S.prm[P_ALPHA_LO] * sc};
+    a = dd_add(a, dd_neg(sg));
+    a = dd_add(a, dd_neg(mu));
+    const double f = dd_add(a, q.M1).hi;
+    // distances to the interval's poles
+    const bool up = mu.hi > 0.0;
+    const int jn = up ? i - 1 : i + 1;
+    const bool other = jn >= 0 && jn < m;
+    dd dn = {0.0, 0.0};
+    double rho = fabs(mu.hi);
+    if (other) {
+        dn = dd_add(dd{S.f.p[jn], S.f.plo[jn]}, dd_neg(sg));
+        rho = fmin(rho, fabs(dn.hi - mu.hi));
+    }
+    const double iN = rcp(N);
+    double d = f * iN;
+    if (!(isfinite(d) && N >= 1.0)) return FST_OLD;
+    if (fabs(d) <= kStepMax * rho) {
+        // d = f / (N + M3 d + M4 d^2 + M5 d^3): each turn gains a factor |d|/rho
+#pragma unroll
+        for (int r = 0; r < 4; ++r) d = f * rcp(N + d * (q.M3 + d * (q.M4 + d * q.M5)));
+        const double Nf = N + d * (2.0 * q.M3 + d * (3.0 * q.M4 + d * (4.0 * q.M5)));
+        // lambda = sigma + mu + d
+        dd mf = two_sum(mu.hi, d);
+        mf.lo += mu.lo;
+        mf = fast_two_sum(mf.hi, mf.lo);
+        if (!(Nf >= 1.0)) return FST_OLD;
+        if (M2u < 0.0) {
+            const double z2 = S.pz2[i] * sc * sc;
+            M2u = fmax(q.M2 - (z2 / mu.hi) / mu.hi, 0.0) + 0x1p-40 * q.M2;
+        }
+        if (!(pow2(K1) * cterm + M2u * kErrUnit <= Nf * fabs(mf.hi))) {
+            set_point(S, k, sg, mf);
+            return FST_MORE;
+        }
+        // the nearer pole is the shift (the upper one where they tie, as the
+        // midpoint test has it)
+        if (other) {
+            const dd alt = dd_add(mf, dd_neg(dn));
+            const double x = fabs(mf.hi), y = fabs(alt.hi);
+            if (y < x || (y == x && up)) {
+                i = jn;
+                mf = alt;
+            }
+        }
+        if (mf.hi > 0.0 ? k != i : k != i + 1) return FST_OLD;   // outside its interval
+        const double sigma = PolesOf<K>::make(S, m).pole(i);
+        const double muu = mf.hi * pow2(-es);
+        if (!(fabs(muu) >= 0x1p-1000)) return FST_OLD;
+        S.es_pole[k] = i;
+        S.es_sigma[k] = sigma;
+        S.es_mu[k] = muu;
+        S.es_lam[k] = sigma + muu;
+        S.f.N[k] = Nf;
+        S.f.M2u[k] = M2u;
+        set_point(S, k, dd{S.f.p[i], S.f.plo[i]}, mf);
+        S.f.mu[k] = mf.hi;           // (set_point may have moved it to the rounded lambda)
+        S.f.mulo[k] = mf.lo;
+        return FST_DONE;
+    }
+    // the model's zero, in double; a short step is the Newton step
+    double mn;
+    const double s = up ? 1.0 : -1.0, x = fabs(mu.hi);
+    if (fabs(d) <= 0x1p-10 * rho) {
+        mn = s * (mu.hi + d);
+    } else {
+        const double z2 = S.pz2[i] * sc * sc, t = z2 / mu.hi;
+        const double Phi = t - f, dPhi = fmax(N - t / mu.hi, 1.0);
+        if (other) {
+            const double e = fabs(dn.hi), g = e - x;
+            const double B = dPhi * g * g, A = s * Phi - dPhi * g, X = A * e + B;
+            const double b = X + z2, h = X - z2, rt = sqrt(h * h + 4.0 * z2 * B);
+            mn = b >= 0.0 ? 2.0 * z2 * e / (b + rt) : (b - rt) / (2.0 * A);
+        } else {
+            const double A = s * Phi - dPhi * x, rt = sqrt(A * A + 4.0 * dPhi * z2);
+            mn = A >= 0.0 ? 2.0 * z2 / (A + rt) : (rt - A) / (2.0 * dPhi);
+        }
+    }
+    // at most a quarter of the distance to the nearest pole, so that the sums'
+    // bounds grow by less than 4/3 and 16/9
+    const double lim = 0.25 * rho;
+    mn = fmin(fmax(mn, x - lim), x + lim);
+    if (!(isfinite(mn) && mn > 0.0) || !set_point(S, k, sg, dd{s * mn, 0.0})) return FST_OLD;
+    S.f.K1[k] = K1 + 1;
+    S.f.K2[k] = K2 + 1;
+    S.f.er[k] -= 1;
+    return FST_MORE;
+}
+
+// Eigenpair k moved to its remedy's shift (other pole, the eigenvalue itself,
+// 0, or a DPR1's last pole) when the zero is known well enough for what that
+// shift is meant to keep: the error of f over f' against |lambda|, the
+// distance to the nearest pole and the new offset.  False: not moved.
+template <Kind K>
+__device__ bool fast_remedy(const Scratch &S, int k, double cterm) {
+    const int es = fast_scale<K>(S), m = S.cnt[C_M];
+    const int rem = S.es_flags[k];
+    const dd sg = fast_sigma<K>(S, k, es);
+    const dd mu = {S.f.mu[k], S.f.mulo[k]};
+    const double sc = pow2(es);
+    int i = -1;
+    dd s2;
+    double sv;
+    if (rem & AE_FLAG_NEARZERO) {
+        sv = 0.0;
+        s2 = dd{0.0, 0.0};
+    } else if (rem & AE_FLAG_OTHERPOLE) {
+        i = S.es_fixpole[k];
+        s2 = dd{S.f.p[i], S.f.plo[i]};
+        sv = S.pv[i];
+    } else {
+        sv = S.es_fixshift[k];
+        s2 = dd{sv * sc, 0.0};
+    }
+    const dd mu2 = dd_add(dd_add(sg, dd_neg(s2)), mu);
+    const double lam = dd_add(s2, mu2).hi;
+    double need = fmin(fabs(mu.hi), fabs(lam));
+    for (int j = k - 1; j <= k; ++j)
+        if (j >= 0 && j < m) {
+            const dd dj = dd_add(sg, dd_neg(dd{S.f.p[j], S.f.plo[j]}));
+            need = fmin(need, fabs(dd_add(dj, mu).hi));
+        }
+    // (the offset itself counts from a pole, the DPR1's last one included)
+    if (i >= 0 || (K == KIND_DPR1 && sv == S.prm[P_PLAST])) need = fmin(need, fabs(mu2.hi));
+    const double muu = mu2.hi * pow2(-es), l2 = sv + muu;
+    const auto R = PolesOf<K>::make(S, m);
+    const double lo = k < m ? R.pole(k) : (K == KIND_DPR1 ? S.prm[P_PLAST] : -INFINITY);
+    const double hi = k > 0 ? R.pole(k - 1) : INFINITY;
+    if (!(pow2(S.f.K1[k]) * cterm + S.f.M2u[k] * kErrUnit <= S.f.N[k] * need && isfinite(mu2.hi) && l2 >= lo &&
+          l2 <= hi && (i < 0 || muu != 0.0)))
+        return false;
+    S.es_pole[k] = i;
+    S.es_sigma[k] = sv;
+    S.es_mu[k] = muu;
+    S.es_lam[k] = l2;
+    set_point(S, k, s2, mu2);
+    S.f.mu[k] = mu2.hi;
+    S.f.mulo[k] = mu2.lo;
+    return true;
+}
+
+// the counters and iteration count of a solved eigenpair
+__device__ __forceinline__ void fast_count(const Scratch &S, int k, const SolveOpts &o, int diag,
+                                           int rounds, int &iters, int &deriv, double &Kb,
+                                           bool &ddb) {
+    iters = o.finish == 0 ? S.es_iters[k] : rounds;
+    deriv = o.finish == 0 ? 0 : rounds;
+    S.es_iters[k] = iters;
+    Kb = diag ? 0.0 : S.es_Kb[k];
+    ddb = !diag && (S.es_flags[k] & AE_FLAG_DDB);
+    if (S.es_flags[k] & AE_FLAG_MID64) atomicAdd(S.cnt + C_MID64, 1);
+}
+
+// One thread per eigenpair: the zero from k_feval's sums, or on to k_fmore.
+template <Kind K, class Src>
+__global__ void __launch_bounds__(64) k_fstep(const __grid_constant__ Src src, SolveOpts o,
+                                              int diag) {
+    int inst = 0, idx = 0, klo = 0, khi = 0, k = 0;
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    bool act = src.item(t, inst, idx);
+    const Scratch &S = src.scr(inst);
+    if (act) {
+        fast_range(S, klo, khi);
+        k = klo + idx;
+        act = k < khi && S.f.st[k] == FST_EVAL;
+    }
+    int iters = 0, deriv = 0;
+    double Kb = 0.0;
+    bool ddb = false, fin = false;
+    if (act) {
+        const int K1 = S.f.K1[k], K2 = S.f.K2[k], er = S.f.er[k];
+        const int K3 = K2 - er, K4 = K3 - er, K5 = K4 - er;
+        FastSums q;
+        const dd v = dd_add(dd_of_ll(S.f.s1[k]), dd{0.5 * (double)S.f.n1[k], 0.0});
+        const double us = ldexp(1.0, K1 - 62);
+        q.M1 = dd{v.hi * us, v.lo * us};
+        q.M2 = ldexp((double)S.f.s2[k] + 0.5 * (double)S.f.n2[k], K2 - 60);
+        q.M3 = -ldexp((double)S.f.s3[k], K3 - 57);
+        q.M4 = ldexp((double)S.f.s4[k], K4 - 55);
+        q.M5 = -ldexp((double)S.f.s5[k], K5 - 53);
+        const int st = fast_advance<K>(S, k, q, kErrTerm, -1.0);
+        S.f.st[k] = st;
+        if (st == FST_OLD) src.push_old(inst, k);
+        else if (st == FST_MORE) src.push_more(0, inst, k);
+        else {
+            fast_count(S, k, o, diag, 1, iters, deriv, Kb, ddb);
+            fin = true;
+        }
+    }
+    fast_stats(S, inst, iters, deriv, Kb, ddb, fin);
+}
+
+// ---------------------------------------------------------------------------
+// k_fmore
+// ---------------------------------------------------------------------------
+// |p - lambda| as its rounded value (returned) and m 2^127, m in [1, 2) the
+// whole difference's significand
+__device__ __forceinline__ unsigned __int128 wide_mant(double D, unsigned __int128 tail) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(D);
+    const unsigned long long Dm = (b & 0xfffffffffffffull) | 0x10000000000000ull;
+    return ((unsigned __int128)Dm << 75) + tail;
+}
+
+// high 128 bits of a b
+__device__ __forceinline__ unsigned __int128 mul_hi128(unsigned __int128 a,
+                                                       unsigned __int128 b) {
+    const unsigned long long al = (unsigned long long)a, ah = (unsigned long long)(a >> 64);
+    const unsigned long long bl = (unsigned long long)b, bh = (unsigned long long)(b >> 64);
+    return (unsigned __int128)ah * bh + __umul64hi(ah, bl) + __umul64hi(al, bh);
+}
+
+// 2^127 / m for the significand m 2^127 = M, from its 63-bit reciprocal R
+__device__ __forceinline__ unsigned __int128 recip127(unsigned __int128 M, unsigned long long R) {
+    if (R >> 63) R = 0x7fffffffffffffffull;
+    const unsigned __int128 V =
+        (unsigned __int128)(unsigned long long)(M >> 64) * R + __umul64hi((unsigned long long)M, R);
+    const __int128 E = (__int128)(((unsigned __int128)1 << 126) - V);      // e 2^126, |e| < 2^-58
+    const __int128 c = (__int128)(long long)(E >> 5) * (__int128)(long long)R;
+    return ((unsigned __int128)R << 64) + (unsigned __int128)(c >> 57);
+}
+
+__device__ __forceinline__ dd dd_of_i128(__int128 v) {
+    const double a = (double)(long long)(v >> 84) * 0x1p84;
+    const double b = (double)((unsigned long long)(v >> 42) & 0x3ffffffffffull) * 0x1p42;
+    const double c = (double)((unsigned long long)v & 0x3ffffffffffull);
+    return dd_add(two_sum(a, b), dd{c, 0.0});
+}
+
+// One CTA per listed eigenpair: evaluations with f in 128 bits (a term to
+// ~2^-85, D's fixed-point unit 2^-106 permitting) and the other sums as
+// k_feval forms them, until the zero is accurate enough.  Phase 1 (after
+// k_ffix): one evaluation at a flagged eigenpair's zero, then its remedy.
+template <Kind K, class Src>
+__global__ void __launch_bounds__(256) k_fmore(const __grid_constant__ Src src, SolveOpts o,
+                                               int phase, int diag) {
+    __shared__ unsigned long long sh1[8], sh1h[8], sh2[8], sh2u[8], sh4[8];
+    __shared__ long long sh3[8], sh5[8];
+    __shared__ int shn[8], verdict;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int cnt = src.more_count(phase);
+    for (int w = blockIdx.x; w < cnt; w += gridDim.x) {
+        const int2 ik = src.more_at(w);
+        const Scratch &S = src.scr(ik.x);
+        const int k = ik.y, m = S.cnt[C_M];
+        int st = FST_MORE;
+        if (phase == 1) {
+            // (an outermost eigenvalue's point is its rounded lambda)
+            if (threadIdx.x == 0)
+                set_point(S, k, dd{S.f.p[S.es_pole[k]], S.f.plo[S.es_pole[k]]},
+                          dd{S.f.mu[k], S.f.mulo[k]});
+            __syncthreads();
+        }
+        for (int round = 0; round < kMoreRounds && st == FST_MORE; ++round) {
+            const double lhi = S.f.lhi[k];
+            const unsigned long long L = S.f.lmod[k];
+            const DiffRange dr = diff_range(lhi);
+            const int K1 = S.f.K1[k], K2 = S.f.K2[k], er = S.f.er[k];
+            const int c1 = K1 - 1023, c2 = K2 - K1 + 1 - 1023, c3 = 2 - er - 1023,
+                      c4 = 1 - er - 1023;
+            __int128 a1 = 0;
+            unsigned long long a2 = 0, a2u = 0, a4 = 0;
+            long long a3 = 0, a5 = 0;
+            int n2 = 0;
+            for (int j = threadIdx.x; j < m; j += 256) {
+                const double p = S.f.p[j];
+                double D = p - lhi;
+                unsigned dh = hi32(D), eb = (dh << 1) >> 21;
+                int tl;
+                unsigned __int128 M;
+                const bool dd_diff = eb - dr.lo >= dr.span;
+                if (dd_diff) {
+                    const int i = S.es_pole[k];
+                    const dd dl = dd_add(dd{p, S.f.plo[j]}, dd_neg(dd{S.f.p[i], S.f.plo[i]}));
+                    const dd Dd = dd_add(dl, dd_neg(dd{S.f.mu[k], S.f.mulo[k]}));
+                    D = Dd.hi;
+                    dh = hi32(D);
+                    eb = (dh << 1) >> 21;
+                    const double lo = ldexp(D < 0.0 ? -Dd.lo : Dd.lo, 62 + 1075 - (int)eb);
+                    const long long li = (long long)lo;          // 2^-62 of D's last place
+                    tl = (int)(li >> 39);
+                    M = wide_mant(D, (unsigned __int128)((__int128)li << 13));
+                } else if (dr.tails) {
+                    const unsigned dl = (unsigned)__double2loint(D);
+                    unsigned long long T = S.f.P[j] - L;
+                    if (dh >> 31) T = 0ull - T;
+                    const unsigned long long Dm =
+                        ((unsigned long long)((dh & 0xfffffu) | 0x100000u) << 32) | dl;
+                    const int sh = (int)eb - (1075 - kFixFrac);
+                    const long long tail = (long long)(T - (Dm << (sh & 63)));
+                    tl = (int)(unsigned)(((unsigned long long)tail << ((55 - sh) & 63)) >> 32);
+                    M = wide_mant(D, (unsigned __int128)((__int128)tail << (75 - sh)));
+                } else {
+                    tl = 0;
+                    M = wide_mant(D, 0);
+                }
+                const unsigned seed = hi32(rcp_seed(__hiloint2double(
+                    (int)((dh & 0xfffffu) | 0x3ff00000u), 0)));
+                const unsigned long long R =
+                    recip63<true>(dh, (unsigned)__double2loint(D), tl, seed);
+                const bool above = j < k;
+                const int ez = S.f.ez[j];
+                // f's term: zeta^2 in double-double over the wide difference
+                {
+                    const double z2 = S.pz2[j];
+                    const int e = (int)bexp(z2) - 1023;
+                    const long long zl = (long long)ldexp(S.pz2lo[j], 115 - e);
+                    const unsigned __int128 Z =
+                        wide_mant(z2, (unsigned __int128)((__int128)zl << 12));
+                    const unsigned __int128 q = mul_hi128(Z, recip127(M, R));
+                    const int s = K1 + 2 - ez + (int)eb - 1023;
+                    const __int128 v = s < 128 ? (__int128)(q >> (s < 0 ? 0 : s)) : (__int128)0;
+                    a1 += above ? -v : v;
+                }
+                unsigned long long q = mul_hi3(S.f.z[j], R);
+                const unsigned s2 = (unsigned)(c1 + (int)eb - ez) + eb + c2;
+                q = mul_hi3(q, R);
+                const unsigned long long v2 = shr64(q, s2);
+                a2 += v2;
+                a2u += dd_diff ? 0ull : v2;
+                n2 += s2 < 60u;
+                q = mul_hi3(q, R);
+                const unsigned s3 = s2 + eb + c3;
+                const long long v3 = (long long)shr64(q, s3);
+                a3 += above ? -v3 : v3;
+                const unsigned s4 = s3 + eb + c4;
+                q = (unsigned long long)(unsigned)(q >> 32) * (unsigned)(R >> 32);
+                a4 += shr64(q, s4);
+                q = (unsigned long long)(unsigned)(q >> 32) * (unsigned)(R >> 32);
+                const long long v5 = (long long)shr64(q, s4 + eb + c4);
+                a5 += above ? -v5 : v5;
+            }
+#pragma unroll
+            for (int s = 16; s > 0; s >>= 1) {
+                const unsigned long long hl = __shfl_xor_sync(FULL, (unsigned long long)a1, s);
+                const unsigned long long hh =
+                    __shfl_xor_sync(FULL, (unsigned long long)((unsigned __int128)a1 >> 64), s);
+                a1 += (__int128)(((unsigned __int128)hh << 64) | hl);
+                a2 += __shfl_xor_sync(FULL, a2, s);
+                a2u += __shfl_xor_sync(FULL, a2u, s);
+                a3 += __shfl_xor_sync(FULL, a3, s);
+                a4 += __shfl_xor_sync(FULL, a4, s);
+                a5 += __shfl_xor_sync(FULL, a5, s);
+            }
+            n2 = __reduce_add_sync(FULL, n2);
+            __syncthreads();
+            if (lane == 0) {
+                shn[wid] = n2;
+                sh1[wid] = (unsigned long long)a1;
+                sh1h[wid] = (unsigned long long)((unsigned __int128)a1 >> 64);
+                sh2[wid] = a2;
+                sh2u[wid] = a2u;
+                sh3[wid] = a3;
+                sh4[wid] = a4;
+                sh5[wid] = a5;
+            }
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                for (int x = 1; x < 8; ++x) {
+                    a1 += (__int128)(((unsigned __int128)sh1h[x] << 64) | sh1[x]);
+                    a2 += sh2[x];
+                    a2u += sh2u[x];
+                    n2 += shn[x];
+                    a3 += sh3[x];
+                    a4 += sh4[x];
+                    a5 += sh5[x];
+                }
+                const int K3 = K2 - er, K4 = K3 - er, K5 = K4 - er;
+                FastSums q;
+                const dd v = dd_of_i128(a1);
+                const double us = ldexp(1.0, K1 - 124);
+                q.M1 = dd{v.hi * us, v.lo * us};
+                q.M2 = ldexp((double)a2 + 0.5 * (double)n2, K2 - 60);
+                q.M3 = -ldexp((double)a3, K3 - 57);
+                q.M4 = ldexp((double)a4, K4 - 55);
+                q.M5 = -ldexp((double)a5, K5 - 53);
+                const double ct = dr.tails ? kErrTermWide : kErrTerm;
+                int v2 = fast_advance<K>(S, k, q, ct, dr.tails ? ldexp((double)a2u, K2 - 60) : 0.0);
+                if (v2 == FST_MORE && round + 1 == kMoreRounds) v2 = FST_OLD;
+                if (phase == 0) {
+                    if (v2 == FST_DONE) {
+                        int iters, deriv;
+                        double Kb;
+                        bool ddb;
+                        fast_count(S, k, o, diag, 2 + round, iters, deriv, Kb, ddb);
+                        EigResult r{};
+                        r.iters = iters;
+                        r.iters_d = deriv;
+                        r.Kb = Kb;
+                        r.flags = ddb ? AE_FLAG_DDB : 0;
+                        record_stats(S, r);
+                    } else if (v2 == FST_OLD) {
+                        src.push_old(ik.x, k);
+                    }
+                    S.f.st[k] = v2;
+                } else if (v2 != FST_MORE) {
+                    atomicAdd(S.cnt64 + C64_ITERS, (unsigned long long)(round + 1));
+                    atomicAdd(S.cnt64 + C64_ITERS_FIX, (unsigned long long)(round + 1));
+                    if (v2 != FST_DONE || !fast_remedy<K>(S, k, ct)) {
+                        S.f.st[k] = FST_OLD;
+                        const bool op = S.es_flags[k] & AE_FLAG_OTHERPOLE;
+                        src.push_fix(ik.x, k, !op, src.vec(ik.x).n);
+                    }
+                }
+                verdict = v2;
+            }
+            __syncthreads();
+            st = verdict;
+        }
+        __syncthreads();
+    }
+}
+
+// ---------------------------------------------------------------------------
+// k_fold: the FP64 solver for the eigenpairs left over
+// ---------------------------------------------------------------------------
+// A CTA of 8 warps each (a few stragglers must not run as long as a warp
+// takes for a whole eigenpair), or a warp each when there are many.
+template <Kind K, class Src>
+__global__ void __launch_bounds__(256) k_fold(const __grid_constant__ Src src, SolveOpts o) {
+    __shared__ double red[16];
+    __shared__ int tick;
+    const int cnt = src.old_count();
+    if (cnt == 0) return;
+    if (cnt < 16 * (int)gridDim.x) {
+        const CtaTeam<8> T{(int)threadIdx.x, red, 0};
+        for (;;) {
+            __syncthreads();
+            if (threadIdx.x == 0) tick = atomicAdd(src.old_ticket(), 1);
+            __syncthreads();
+            if (tick >= cnt) break;
+            const int2 ik = src.old_at(tick);
+            const Scratch &S = src.scr(ik.x);
+            const auto R = PolesOf<K>::make(S, S.cnt[C_M]);
+            eig_item<K>(R, T, S, ik.y, o, src.slice((long long)blockIdx.x * 8));
+        }
+    } else {
+        const int lane = threadIdx.x & 31;
+        for (;;) {
+            int w = 0;
+            if (lane == 0) w = atomicAdd(src.old_ticket(), 1);
+            w = __shfl_sync(FULL, w, 0);
+            if (w >= cnt) break;
+            const int2 ik = src.old_at(w);
+            const Scratch &S = src.scr(ik.x);
+            const auto R = PolesOf<K>::make(S, S.cnt[C_M]);
+            eig_item<K>(R, WarpTeam{lane}, S, ik.y, o,
+                        src.slice(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5));
+            __syncwarp();
+        }
+    }
+}
+
+// b and K_b of Algorithm 2 for callers that ask for the diagnostics, as the
+// FP64 solver forms them (a warp per eigenpair)
+template <Kind K, class Src>
+__global__ void __launch_bounds__(256) k_fdiag(const __grid_constant__ Src src, SolveOpts o) {
+    const int lane = threadIdx.x & 31;
+    const WarpTeam T{lane};
+    int inst, first;
+    if (!src.unit(blockIdx.x, 8, inst, first)) return;
+    const Scratch &S = src.scr(inst);
+    int klo, khi;
+    fast_range(S, klo, khi);
+    const int k = klo + first + (int)(threadIdx.x >> 5);
+    if (k >= khi || S.f.st[k] != FST_DONE) return;
+    const auto R = PolesOf<K>::make(S, S.cnt[C_M]);
+    const int i = S.es_pole[k];
+    double b, Kb;
+    const bool dd2 = shifted_b(R, T, i, o, b, Kb);
+    if (lane == 0) {
+        S.es_b[k] = b;
+        S.es_Kb[k] = Kb;
+        S.es_flags[k] = (S.es_flags[k] & ~AE_FLAG_DDB) | (dd2 ? AE_FLAG_DDB : 0);
+        if (dd2) atomicAdd(S.cnt + C_DDB, 1);
+        if (isfinite(Kb)) atomic_max_nonneg(S.cnt64 + C64_MAXKB, Kb);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// k_ffix: remedies
+// ---------------------------------------------------------------------------
+// The eigenpairs k_fix_decide flagged: moved by a subtraction where that
+// serves, else on to k_fmore, or (those the FP64 solver took) to k_fix_solve.
+template <Kind K, class Src>
+__global__ void __launch_bounds__(64) k_ffix(const __grid_constant__ Src src) {
+    int inst = 0, idx = 0;
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (!src.item(t, inst, idx)) return;
+    const Scratch &S = src.scr(inst);
+    const PartRange P = part_range(S);
+    const int k = P.k0 + idx;
+    if (k >= P.k1) return;
+    const int rem = S.es_flags[k] & (AE_FLAG_NEARZERO | AE_FLAG_OTHERPOLE | AE_FLAG_DPR1SHIFT);
+    if (!rem) return;
+    if (S.f.p && S.f.st[k] == FST_DONE) {
+        if (!fast_remedy<K>(S, k, kErrTerm)) src.push_more(1, inst, k);
+    } else {
+        src.push_fix(inst, k, !(rem & AE_FLAG_OTHERPOLE), src.vec(inst).n);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// k_fcols
+// ---------------------------------------------------------------------------
+// significand (64 bits, top bit set), biased exponent and sign of a double;
+// a zero has significand 0
+struct Mant {
+    unsigned long long m;
+    int e;                // bit 31: the sign, low bits: the biased exponent
+};
+__device__ __forceinline__ Mant mant_of(double x) {
+    unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    const unsigned sg = (unsigned)(b >> 32) & 0x80000000u;
+    int e = (int)((b >> 52) & 0x7ff), off = 0;
+    if (e == 0 && x != 0.0) {
+        b = (unsigned long long)__double_as_longlong(x * 0x1p64);
+        e = (int)((b >> 52) & 0x7ff);
+        off = 64;
+    }
+    Mant r;
+    r.m = e ? ((b & 0xfffffffffffffull) | 0x10000000000000ull) << 11 : 0ull;
+    r.e = (int)(((unsigned)(e - off) & 0xffffu) | sg);
+    return r;
+}
+
+// a G / 2^61 2^(be - 1023) rounded to double, G in (2^61, 2^63], a's
+// significand in [2^63, 2^64); sgn: the sign bit
+__device__ __forceinline__ double pack_prod(unsigned long long a, unsigned long long G, int be,
+                                            unsigned sgn) {
+    const unsigned long long H0 = mul_hi3(a, G);
+    const unsigned h = (unsigned)(H0 >> 32);
+    const int lz = __clz(h);                            // 1..3
+    const unsigned long long H = (H0 << (lz - 1)) + 0x200ull;
+    const int e = be + 2 - lz;
+    const unsigned lo = (unsigned)(H >> 10);
+    unsigned hi = (unsigned)(H >> 42) + ((unsigned)(e - 1) << 20);
+    if (a == 0) return __hiloint2double((int)sgn, 0);
+    if ((unsigned)(e - 1) >= 2045u) {
+        // below the normal range (or above it): in FP64
+        const double v = ldexp((double)(H >> 10), e - 1075);
+        return sgn ? -v : v;
+    }
+    return __hiloint2double((int)(hi | sgn), (int)lo);
+}
+
+// Columns of the eigenpairs the fast path solved, a warp each; the CTA's 8
+// warps share tiles of input rows.  Component a_r / ((d_r - sigma) - mu) /
+// ||x||, for the second matrix (SVD: U, NSYM: Y) or the imaginary part (HERM)
+// with its own multiplier.
+template <Kind VK, class Src>
+__global__ void __launch_bounds__(256, 3) k_fcols(const __grid_constant__ Src src) {
+    constexpr bool CPLX = VK == KIND_HERM;
+    constexpr bool TWO = VK == KIND_HERM || VK == KIND_NSYM || VK == KIND_TSVD;
+    __shared__ double tp[2][kTile];
+    __shared__ unsigned long long tP[2][kTile], ta[2][kTile], tb[2][TWO ? kTile : 1];
+    __shared__ int ea[2][kTile], eb2[2][TWO ? kTile : 1];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int inst, first;
+    if (!src.unit(blockIdx.x, 8, inst, first)) return;
+    const Scratch &S = src.scr(inst);
+    const VecArgs &va = src.vec(inst);
+    const PartRange P = part_range(S);
+    if (!va.out.V || P.k0 + first >= P.k1) return;
+    const int k = P.k0 + first + wid;
+    const bool act = k < P.k1 && S.f.st[k] == FST_DONE;
+    if (!__syncthreads_or(act)) return;
+    const int ka = act ? k : P.k0 + first;
+    const int n1 = va.n1;
+    constexpr Kind RK = VK;                             // pole form of the rows
+    const int es = fast_scale<RK>(S);
+    const double lhi = S.f.lhi[ka];
+    const unsigned long long L = S.f.lmod[ka];
+    const DiffRange dr = diff_range(lhi);
+    // 1 / ||x||: the norm is sqrt(f') but for the DPR1, whose vector (without
+    // the arrowhead's corner) has ||x||^2 = f' / (|rho| (lambda - p_last))
+    double nrm = S.f.N[ka];
+    if (VK == KIND_DPR1) {
+        const dd sg = fast_sigma<RK>(S, ka, es);
+        const dd pl = {ldexp(S.prm[P_PLAST], es), 0.0};
+        const double x = dd_add(dd_add(sg, dd_neg(pl)), dd{S.f.mu[ka], S.f.mulo[ka]}).hi;
+        nrm = nrm / x / ldexp(fabs(va.alpha), es);     // (va.alpha is rho; u is not scaled)
+    }
+    const double inv = 1.0 / sqrt(nrm);
+    const double sv = VK == KIND_TSVD ? sv_of(S, ka) : 1.0;      // the singular value
+    // scaled multipliers: spikes and poles both scale by 2^es (DPR1: see nrm)
+    const Mant mi = mant_of(inv);
+    const int ei = mi.e - 1023 + (VK == KIND_DPR1 ? 0 : es);
+    const Mant mu2 = mant_of(VK == KIND_TSVD ? inv * sv : inv);
+    const int ei2 = mu2.e - 1023 + es;
+    const int pos = out_pos<VK>(S, va.n, va.sgn, ka);
+    const unsigned vsg = (VK == KIND_DPR1 && va.sgn < 0.0) ? 0x80000000u : 0u;
+    double *col = va.out.V + (size_t)pos * va.out.ldv;
+    double *ucol = (TWO && !CPLX && va.out.U) ? va.out.U + (size_t)pos * va.out.ldu : nullptr;
+    double lp;
+    unsigned long long lP;
+    Mant la, lb;
+    auto load = [&](int t) {
+        const int r = t * kTile + threadIdx.x;
+        lp = 4.0; lP = 0; la = lb = Mant{0, 0};
+        if (r < n1) {
+            lp = S.f.rp[r];
+            lP = S.f.rP[r];
+            if (CPLX) {
+                la = mant_of(va.z[2 * r]);
+                lb = mant_of(va.z[2 * r + 1]);
+            } else if (VK == KIND_NSYM) {
+                la = mant_of(va.z[r]);
+                lb = mant_of(va.zrow[r]);
+            } else if (VK == KIND_TSVD) {
+                la = mant_of(va.spk[r]);
+                lb = mant_of(va.z[r]);                 // u_r = s v_r / d_r, spike d_r z_r
+            } else {
+                la = mant_of(va.spk[r]);
+            }
+        }
+    };
+    const int tiles = (n1 + kTile - 1) / kTile;
+    load(0);
+    for (int t = 0; t < tiles; ++t) {
+        const int b = t & 1;
+        tp[b][threadIdx.x] = lp;
+        tP[b][threadIdx.x] = lP;
+        ta[b][threadIdx.x] = la.m;
+        ea[b][threadIdx.x] = la.e;
+        if (TWO) {
+            tb[b][threadIdx.x] = lb.m;
+            eb2[b][threadIdx.x] = lb.e;
+        }
+        __syncthreads();
+        if (t + 1 < tiles) load(t + 1);
+        if (!act) continue;
+        const int left = n1 - t * kTile;
+        const int nc = left >= kTile ? kTile / 32 : (left + 31) / 32;
+#pragma unroll 1
+        for (int c = 0; c < nc; ++c) {
+            const int x = c * 32 + lane;
+            const int r = t * kTile + x;
+            double D = tp[b][x] - lhi;
+            int tl;
+            unsigned dh = hi32(D), dl = (unsigned)__double2loint(D);
+            unsigned ed = (dh << 1) >> 21;
+            if (ed - dr.lo >= dr.span && r < n1) {
+                const dd pr = fast_pole<RK>(va.key[r], es);
+                D = near_diff(pr, fast_sigma<RK>(S, ka, es), dd{S.f.mu[ka], S.f.mulo[ka]}, tl);
+                dh = hi32(D);
+                dl = (unsigned)__double2loint(D);
+                ed = (dh << 1) >> 21;
+            } else {
+                tl = tail_of(tP[b][x] - L, dh, dl, ed) & dr.tails;
+            }
+            const unsigned seed = hi32(rcp_seed(__hiloint2double(
+                (int)((dh & 0xfffffu) | 0x3ff00000u), 0)));
+            const unsigned long long Rr = recip63<false>(dh, dl, tl, seed);
+            const unsigned long long G = mul_hi3(mi.m, Rr);
+            const int e1 = ea[b][x];
+            const unsigned sg = (((unsigned)e1 ^ dh) & 0x80000000u) ^ vsg;
+            const int be = (int)(short)(e1 & 0xffff) - (int)ed + ei + 1023;
+            const double v = pack_prod(ta[b][x], G, be, sg);
+            if (CPLX) {
+                const int e2 = eb2[b][x];
+                const double vi = pack_prod(tb[b][x], G, (int)(short)(e2 & 0xffff) - (int)ed + ei + 1023,
+                                            ((unsigned)e2 ^ dh) & 0x80000000u);
+                if (r < n1) {
+                    col[2 * r] = v;
+                    col[2 * r + 1] = vi;
+                }
+            } else {
+                if (r < n1) col[r] = v;
+                if (TWO && ucol) {
+                    const unsigned long long G2 = VK == KIND_TSVD ? mul_hi3(mu2.m, Rr) : G;
+                    const int e2 = eb2[b][x];
+                    const double vu = pack_prod(tb[b][x], G2,
+                                                (int)(short)(e2 & 0xffff) - (int)ed + ei2 + 1023,
+                                                ((unsigned)e2 ^ dh) & 0x80000000u);
+                    if (r < n1) ucol[r] = vu;
+                }
+            }
+        }
+    }
+    if (act && lane == 0 && VK != KIND_DPR1) {
+        const double vn = -inv;
+        if (CPLX) {
+            col[2 * n1] = vn;
+            col[2 * n1 + 1] = 0.0;
+        } else {
+            col[n1] = vn;
+            if (ucol) ucol[n1] = VK == KIND_TSVD ? va.alpha * vn / sv : vn;
+        }
+    }
+}
+
+template <Kind K>
+__global__ void __launch_bounds__(256) k_fprep(Scratch S, VecArgs va) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < va.n1) fprep_item<K>(S, va, t);
+}
+
+}  // namespace ae

@@ -32,7 +32,11 @@ enum {
     C_U1 = 18,
     C_POS0 = 19,      // output position of the part's first item
     C_KHI = 20,       // end of the eigenpairs k_eig solves (the part's range and its edges)
-    C_COUNT = 21
+    C_NOLD = 21,      // eigenpairs the fixed-point path leaves to the FP64 solver
+    C_OLDTK = 22,     // their work ticket
+    C_NMORE = 23,     // eigenpairs k_fmore evaluates: after k_fstep, after k_ffix
+    C_NMORE1 = 24,
+    C_COUNT = 25
 };
 enum { C64_ITERS = 0, C64_MAXKB = 1, C64_MAXKNU = 2, C64_ITERS_FIX = 3, C64_DERIV = 4,
        C64_F32 = 5,     // O(n) passes in FP32 (midpoint tests, FP32 steps and brackets)
@@ -40,7 +44,8 @@ enum { C64_ITERS = 0, C64_MAXKB = 1, C64_MAXKNU = 2, C64_ITERS_FIX = 3, C64_DERI
        C64_COUNT = 7 };
 
 // k_check flag bits
-enum { CF_UNSORTED = 1, CF_ZERO = 2, CF_BAD = 4, CF_ZEROPOLE = 8 };
+// (CF_NOFAST, from k_fprep: outside the fixed-point path's ranges)
+enum { CF_UNSORTED = 1, CF_ZERO = 2, CF_BAD = 4, CF_ZEROPOLE = 8, CF_NOFAST = 16 };
 
 // problem kinds sharing the pipeline
 // (HERM and NSYM are solved as the real arrowhead with spikes |zeta_r|, resp.
@@ -59,7 +64,27 @@ enum {
     P_COUNT = 8
 };
 
+// Data of the fixed-point path (ae_fast.cuh): poles and rows scaled below 1/2 by
+// a power of two, as doubles and modulo 2^64 in units of 2^-106; spikes^2 as
+// significand and exponent; per eigenpair the evaluation point, the bounds and
+// values of its sums, and its state.  p == null: the path is not used.
+struct FastPtrs {
+    double *p, *plo;                      // reduced poles (double-double)
+    unsigned long long *P, *z;
+    int *ez;
+    double *rp;                           // input rows
+    unsigned long long *rP;
+    double *mu, *mulo, *lhi, *N, *M2u;
+    unsigned long long *lmod;
+    int *K1, *K2, *er;
+    long long *s1, *s3, *s5;
+    unsigned long long *s2, *s4;
+    int *n1, *n2;
+    int *st, *old, *more;
+};
+
 struct Scratch {
+    FastPtrs f;
     int *cnt;
     unsigned long long *cnt64;
     int *perm;      // sorted position -> input row
@@ -96,16 +121,12 @@ struct Outputs {
 };
 
 // What the eigenvector epilogue needs (the transformed inputs the reduction
-// saw, the caller's spikes, the outputs).  fused != 0: the eigenvalue kernel
-// writes each column as soon as its eigenvalue is known, staged in the warp's
-// stored-pair slice, and the vector kernel later only rewrites the columns
-// that the remedies or the final placement changed (and the deflated ones).
+// saw, the caller's spikes, the outputs).
 struct VecArgs {
     int n, n1;
     const double *key, *spk, *z, *zrow;
-    double alpha, sgn;
+    double alpha, sgn;                    // (DPR1: alpha holds rho)
     Outputs out;
-    int fused;
 };
 
 struct RunOpts {
@@ -123,6 +144,9 @@ struct RunOpts {
 int resolve_opts(const ae_opts *o, RunOpts &ro);
 
 size_t arrow_scratch_bytes(int n);
+// the fixed-point path's data for order n, and its pointers into `base`
+size_t fast_bytes(int n);
+FastPtrs carve_fast(void *base, int n);
 // warps of the eigenvalue kernel for order n (the stored-pair buffer holds one
 // slice of n pairs per warp)
 int eig_grid_warps(int n);

@@ -425,9 +425,8 @@ static __device__ int fix_decide_item(Kind kind, const Scratch &S, int k, double
 // Remedy solve of eigenpair k by a team (a CTA in the single-instance pipeline,
 // a warp in the batched one); all of its threads call it.
 // buf: the team's slice of stored pairs (or null).
-// Returns whether the remedy's result was kept (buf then holds its stored pairs).
 template <Kind K, class Team>
-__device__ bool fix_solve_item(const typename PolesOf<K>::type &R, const Team &T, const Scratch &S,
+__device__ void fix_solve_item(const typename PolesOf<K>::type &R, const Team &T, const Scratch &S,
                                int k, const SolveOpts &o, double2 *buf = nullptr) {
     const int m = S.cnt[C_M];
     const int f = S.es_flags[k];
@@ -457,7 +456,6 @@ __device__ bool fix_solve_item(const typename PolesOf<K>::type &R, const Team &T
             S.es_flags[k] = f & ~(AE_FLAG_NEARZERO | AE_FLAG_OTHERPOLE | AE_FLAG_DPR1SHIFT);
         }
     }
-    return ok;
 }
 
 // The items a solve writes: all of them, or one part of a split solve --
@@ -518,28 +516,78 @@ __device__ __forceinline__ void run_column(const Scratch &S, const double *spk, 
     if (lane == 0) col[row] = sign * (Rm1 / Rm);
 }
 
-// Output of item `item` (a computed eigenpair, or a deflated row) by one team:
-// value, optional shift/mu/diagnostics, and its column(s).  `key`/`spk` are the
-// transformed inputs the reduction saw; z is the caller's spike array (SVD:
-// for the left vectors; HERM: the complex spikes; NSYM: the column spikes,
-// zrow the row spikes).
+// output position of item `item` in the caller's arrays (a part's own block;
+// -M's order reversed for a DPR1 with rho < 0)
+template <Kind K>
+__device__ __forceinline__ int out_pos(const Scratch &S, int n, double sgn, int item) {
+    const int pos = S.pos[item] - (S.cnt[C_PART] ? S.cnt[C_POS0] : 0);
+    return K == KIND_DPR1 && sgn < 0.0 ? n - 1 - pos : pos;
+}
+
+// SVD: the singular value of computed eigenpair k, from lambda = d_i^2 + mu
+// (pole shift) or sigma + mu in double-double
+__device__ __forceinline__ double sv_of(const Scratch &S, int k) {
+    const int pi = S.es_pole[k];
+    const double mu = S.es_mu[k];
+    dd l2;
+    if (pi >= 0) {
+        const double di = S.pd[pi];
+        l2 = dd_add(two_prod(di, di), dd{mu, 0.0});
+    } else {
+        l2 = two_sum(S.es_sigma[k], mu);
+    }
+    return dd_sqrt(l2).hi;
+}
+
+// Scalar outputs of item `item` (a computed eigenpair, or a deflated row) by
+// one thread: the value, optional shift / mu, diagnostics.
+template <Kind K>
+__device__ void scalar_item(int n, const double *__restrict__ key, double sgn, const Scratch &S,
+                            const Outputs &out, int item) {
+    const int ncomp = S.cnt[C_M] + 1;
+    const int pos = out_pos<K>(S, n, sgn, item);
+    if (item < ncomp) {
+        const int k = item;
+        const double sig = S.es_sigma[k], mu = S.es_mu[k];
+        double value = S.es_lam[k];
+        if (K == KIND_TSVD) value = sv_of(S, k);
+        else if (K == KIND_DPR1) value = sgn * value;
+        out.lambda[pos] = value;
+        if (out.shift) out.shift[pos] = K == KIND_DPR1 ? sgn * sig : sig;
+        if (out.mu) out.mu[pos] = K == KIND_DPR1 ? sgn * mu : mu;
+        if (out.dg_b) out.dg_b[pos] = S.es_b[k];
+        if (out.dg_Kb) out.dg_Kb[pos] = S.es_Kb[k];
+        if (out.dg_Knu) out.dg_Knu[pos] = S.es_Knu[k];
+        if (out.dg_iters) out.dg_iters[pos] = S.es_iters[k];
+        if (out.dg_flags) out.dg_flags[pos] = S.es_flags[k];
+    } else {
+        const double kv = key[S.drow[item - ncomp]];
+        const double value = K == KIND_DPR1 ? sgn * kv : kv;
+        out.lambda[pos] = value;
+        if (out.shift) out.shift[pos] = value;
+        if (out.mu) out.mu[pos] = 0.0;
+        if (out.dg_b) out.dg_b[pos] = NAN;
+        if (out.dg_Kb) out.dg_Kb[pos] = 0.0;
+        if (out.dg_Knu) out.dg_Knu[pos] = 1.0;
+        if (out.dg_iters) out.dg_iters[pos] = 0;
+        if (out.dg_flags) out.dg_flags[pos] = AE_FLAG_DEFLATED;
+    }
+}
+
+// Column(s) of item `item` by one team in FP64: deflated rows, and eigenpairs
+// the FP64 solver took.  `key`/`spk` are the transformed inputs the reduction
+// saw; z is the caller's spike array (SVD: for the left vectors; HERM: the
+// complex spikes; NSYM: the column spikes, zrow the row spikes).
 // HERM writes U = Phi V (Sec. 6.1) as complex columns, row r at doubles 2r,
 // 2r+1: u_r = zeta_r t_r / ||x|| with t_r = 1/((d_r - sigma) - mu), since
 // Phi_r |zeta_r| = zeta_r.  NSYM writes the right vectors X = Psi V into V and
 // the left ones Y = Psi^{-1} V into U: x_r = zc_r t_r / ||x||, y_r = zr_r t_r
 // / ||x||, since Psi_r sqrt(zc_r zr_r) = zc_r; then y^T x = 1.
-// stage: null (pass 1 keeps its values in the output column) or the team's
-// scratch for RS * n1 doubles (the column is then written once, normalised --
-// what an output in host memory needs).  columns = false writes the scalar
-// outputs only.  pairs: stage is the team's stored-pair slice and still holds
-// the (delta_j, zeta_j^2 / delta_j) of this item's final solve.
 template <Kind K, class Team>
 __device__ void vector_item(int n, int n1, const double *__restrict__ key,
                             const double *__restrict__ spk, const double *__restrict__ z,
                             const double *__restrict__ zrow, double alpha, double sgn,
-                            const Scratch &S, const Outputs &out, int item, const Team &T,
-                            double *stage = nullptr, bool columns = true,
-                            bool pairs = false) {
+                            const Scratch &S, const Outputs &out, int item, const Team &T) {
     const int lane = T.rank;
     constexpr bool CPLX = K == KIND_HERM;
     constexpr bool TWO = K == KIND_NSYM;
@@ -547,42 +595,15 @@ __device__ void vector_item(int n, int n1, const double *__restrict__ key,
     const int m = S.cnt[C_M];
     const int ncomp = m + 1;
     const bool last_row = K != KIND_DPR1;     // arrowhead rows have the x_n = -1 entry
-    int pos = S.pos[item] - (S.cnt[C_PART] ? S.cnt[C_POS0] : 0);   // in this part's block
-    if (K == KIND_DPR1 && sgn < 0.0) pos = n - 1 - pos;   // -M's order reversed
-    double *col = (out.V && columns) ? out.V + (size_t)pos * out.ldv : nullptr;
-    double *ucol = ((K == KIND_TSVD || TWO) && out.U && columns) ? out.U + (size_t)pos * out.ldu
-                                                                   : nullptr;
+    const int pos = out_pos<K>(S, n, sgn, item);
+    double *col = out.V ? out.V + (size_t)pos * out.ldv : nullptr;
+    double *ucol = ((K == KIND_TSVD || TWO) && out.U) ? out.U + (size_t)pos * out.ldu : nullptr;
+    if (!col) return;
     if (item < ncomp) {
         const int k = item;
         const double sig = S.es_sigma[k], mu = S.es_mu[k];
         const int pi = S.es_pole[k];
-        double value = S.es_lam[k];
-        double sv = 0.0;   // SVD: singular value
-        if (K == KIND_TSVD) {
-            // lambda = d_i^2 + mu (pole shift) or sigma + mu, in double-double
-            dd l2;
-            if (pi >= 0) {
-                const double di = S.pd[pi];
-                l2 = dd_add(two_prod(di, di), dd{mu, 0.0});
-            } else {
-                l2 = two_sum(sig, mu);
-            }
-            sv = dd_sqrt(l2).hi;
-            value = sv;
-        } else if (K == KIND_DPR1) {
-            value = sgn * value;
-        }
-        if (lane == 0) {
-            out.lambda[pos] = value;
-            if (out.shift) out.shift[pos] = K == KIND_DPR1 ? sgn * sig : sig;
-            if (out.mu) out.mu[pos] = K == KIND_DPR1 ? sgn * mu : mu;
-            if (out.dg_b) out.dg_b[pos] = S.es_b[k];
-            if (out.dg_Kb) out.dg_Kb[pos] = S.es_Kb[k];
-            if (out.dg_Knu) out.dg_Knu[pos] = S.es_Knu[k];
-            if (out.dg_iters) out.dg_iters[pos] = S.es_iters[k];
-            if (out.dg_flags) out.dg_flags[pos] = S.es_flags[k];
-        }
-        if (!col) return;
+        const double sv = K == KIND_TSVD ? sv_of(S, k) : 0.0;   // the singular value
         // 1/(shifted difference of row r - mu); 0 for a zero spike
         const double unit = unit_reg();
         auto recip = [&](int r) {
@@ -606,7 +627,7 @@ __device__ void vector_item(int n, int n1, const double *__restrict__ key,
         // Pass 1 stores x (HERM, NSYM: the reciprocal t) in the column and sums
         // x^2 in sorted order (so the norm does not depend on the order of the
         // input rows); pass 2 scales in place.
-        double *keep = stage ? stage : col;      // pass-1 values, RS doubles a row
+        double *keep = col;                      // pass-1 values, RS doubles a row
         // two rows a lane at a time, two independent sums (the same order for
         // every kind, so that real spikes give the real solver's bits)
         auto one = [&](int r, double &acc) {
@@ -622,38 +643,12 @@ __device__ void vector_item(int n, int n1, const double *__restrict__ key,
             }
         };
         double s = 0.0, s1 = 0.0;
-        // Sorted input without deflation: row r is reduced pole r, and its
-        // shifted difference d_r - sigma is the one the solve stored (0 for
-        // the shift pole): the same double, loaded instead of recomputed.  The
-        // staged values overwrite the stored pairs of rows up to r (a slot per
-        // row, 2 per pair; the complex stage overwrites row r's own), so each
-        // step's loads come before the team syncs and its stores after.
-        const bool fast = pairs && stage && (K == KIND_ARROW || CPLX || TWO) && m == n1 &&
-                          !(S.cnt[C_FLAGS] & CF_UNSORTED);
-        if (fast) {
-            const double2 *P = reinterpret_cast<const double2 *>(stage);
-            auto one_d = [&](int r, double del, double &acc) {
-                const double t = rcp_o(del - mu, unit);
-                const double x = spk[r] * t;
-                keep[RS * r] = (CPLX || TWO) ? t : x;
-                acc = fma(x, x, acc);
-            };
-            for (int base = 0; base < n1; base += 2 * Team::size) {
-                const int ra = base + lane, rb = ra + Team::size;
-                const double da = ra < n1 ? P[ra].x : 0.0;
-                const double db = rb < n1 ? P[rb].x : 0.0;
-                T.sync();
-                if (ra < n1) one_d(ra, da, s);
-                if (rb < n1) one_d(rb, db, s1);
-            }
-        } else {
-            int q0 = lane;
-            for (; q0 + Team::size < n1; q0 += 2 * Team::size) {
-                one(S.perm[q0], s);
-                one(S.perm[q0 + Team::size], s1);
-            }
-            if (q0 < n1) one(S.perm[q0], s);
+        int q0 = lane;
+        for (; q0 + Team::size < n1; q0 += 2 * Team::size) {
+            one(S.perm[q0], s);
+            one(S.perm[q0 + Team::size], s1);
         }
+        if (q0 < n1) one(S.perm[q0], s);
         s += s1;
         s = T.sum(s) + (last_row ? 1.0 : 0.0);
         double inv, scale = 1.0;
@@ -726,19 +721,6 @@ __device__ void vector_item(int n, int n1, const double *__restrict__ key,
     } else {
         const int u = item - ncomp;
         const int row = S.drow[u];
-        const double kv = key[row];
-        const double value = K == KIND_TSVD ? kv : (K == KIND_DPR1 ? sgn * kv : kv);
-        if (lane == 0) {
-            out.lambda[pos] = value;
-            if (out.shift) out.shift[pos] = value;
-            if (out.mu) out.mu[pos] = 0.0;
-            if (out.dg_b) out.dg_b[pos] = NAN;
-            if (out.dg_Kb) out.dg_Kb[pos] = 0.0;
-            if (out.dg_Knu) out.dg_Knu[pos] = 1.0;
-            if (out.dg_iters) out.dg_iters[pos] = 0;
-            if (out.dg_flags) out.dg_flags[pos] = AE_FLAG_DEFLATED;
-        }
-        if (!col) return;
         for (int r = lane; r < RS * n; r += Team::size) col[r] = 0.0;
         if (TWO && ucol)
             for (int r = lane; r < n; r += Team::size) ucol[r] = 0.0;

@@ -46,6 +46,7 @@ struct Req {
     size_t bytes = 0;           // scratch + results charged to the budget
     bool charged = false;       // bytes are counted in in_use
     void *scratch = nullptr;
+    void *fast = nullptr;       // the fixed-point path's data
     void *wbuf = nullptr;       // stored (delta_j, c_j) pairs of the eigenvalue kernel
     double *result = nullptr;   // lambda | V | U in one block
     double *lam = nullptr, *V = nullptr, *U = nullptr;
@@ -216,12 +217,15 @@ bool ae_server::admit_locked(Req *r) {
     const long long wstride = ((long long)q.n + 1) & ~1LL;
     cudaError_t e = cudaMallocAsync(&r->scratch, ae::arrow_scratch_bytes(q.n), st);
     if (!e) e = cudaMallocAsync(&r->wbuf, wbuf_bytes(q.n), st);
+    if (!e) e = cudaMallocAsync(&r->fast, ae::fast_bytes(q.n), st);
     if (!e) e = cudaMallocAsync((void **)&r->result, sizeof(double) * result_doubles(q), st);
     if (e) {                       // out of device memory now: retry later
         if (r->scratch) cudaFreeAsync(r->scratch, st);
         if (r->wbuf) cudaFreeAsync(r->wbuf, st);
+        if (r->fast) cudaFreeAsync(r->fast, st);
         r->scratch = nullptr;
         r->wbuf = nullptr;
+        r->fast = nullptr;
         r->result = nullptr;
         cudaGetLastError();
         return false;
@@ -233,6 +237,7 @@ bool ae_server::admit_locked(Req *r) {
     ae::Scratch S = ae::carve_scratch(r->scratch, q.n);
     S.wbuf = (double2 *)r->wbuf;
     S.wstride = wstride;
+    S.f = ae::carve_fast(r->fast, q.n);
     ae::Outputs out{};
     out.lambda = r->lam;
     out.V = r->V;
@@ -245,9 +250,11 @@ bool ae_server::admit_locked(Req *r) {
                                 cudaMemcpyDeviceToHost, st);
     if (!e) e = cudaFreeAsync(r->scratch, st);
     if (!e) e = cudaFreeAsync(r->wbuf, st);
+    if (!e) e = cudaFreeAsync(r->fast, st);
     if (!e) e = cudaEventRecord(r->done, st);
     r->scratch = nullptr;
     r->wbuf = nullptr;
+    r->fast = nullptr;
     if (e) {
         r->state = AE_REQ_ERROR;
         r->status = AE_ERR_CUDA;
@@ -360,7 +367,7 @@ int ae_serve_submit(ae_server *s, const ae_request *req, unsigned long long *tic
     if (!isfinite(q.alpha) || (q.kind == AE_KIND_SVD && q.alpha == 0.0)) return -2;
     Req *r = new Req();
     r->in = q;
-    r->bytes = ae::arrow_scratch_bytes(q.n) + wbuf_bytes(q.n) + sizeof(double) * result_doubles(q);
+    r->bytes = ae::arrow_scratch_bytes(q.n) + ae::fast_bytes(q.n) + wbuf_bytes(q.n) + sizeof(double) * result_doubles(q);
     if (cudaEventCreateWithFlags(&r->done, cudaEventDisableTiming) != cudaSuccess ||
         cudaMallocHost((void **)&r->cnt_host, sizeof(int) * ae::C_COUNT) != cudaSuccess) {
         if (r->done) cudaEventDestroy(r->done);

@@ -10,6 +10,7 @@
 
 #include <cuda_runtime.h>
 
+#include "ae_fast.cuh"
 #include "ae_internal.h"
 #include "ae_pipeline.cuh"
 
@@ -18,11 +19,11 @@ namespace ae {
 // ---------------------------------------------------------------------------
 // eigenpairs
 // ---------------------------------------------------------------------------
-// With va.fused, each warp writes eigenpair k's column right after solving it
-// (pass 1 staged in its stored-pair slice, which the solve no longer needs), at
-// the position k + #(deflated values >= lambda_k) that the placement gives.
-template <Kind K, Kind VK>
-__global__ void __launch_bounds__(256, 3) k_eig(Scratch S, SolveOpts o, VecArgs va) {
+// The FP64 solver for all eigenpairs, a warp each: callers that bring no
+// memory for the fixed-point path (arrow_eig_noalloc), and options it does not
+// serve.
+template <Kind K>
+__global__ void __launch_bounds__(256, 3) k_eig(Scratch S, SolveOpts o) {
     const int lane = threadIdx.x & 31;
     const int m = S.cnt[C_M];
     const auto R = PolesOf<K>::make(S, m);
@@ -41,34 +42,21 @@ __global__ void __launch_bounds__(256, 3) k_eig(Scratch S, SolveOpts o, VecArgs 
         k = __shfl_sync(FULL, k, 0);
         if (k >= k_hi) break;
         eig_item<K>(R, T, S, k, o, buf);
-        if (va.fused && (!__ldcg(S.cnt + C_PART) ||
-                         (k >= __ldcg(S.cnt + C_K0) && k < __ldcg(S.cnt + C_K1)))) {
-            __syncwarp();
-            if (lane == 0) {
-                place_item(S, k);
-                S.pos0[k] = S.pos[k];
-            }
-            __syncwarp();
-            vector_item<VK>(va.n, va.n1, va.key, va.spk, va.z, va.zrow, va.alpha, va.sgn, S,
-                            va.out, k, T, (double *)buf, true, true);
-        }
     }
 }
 
-// Remedy decisions: one thread per eigenpair (of the part).  The solves on a
-// DPR1 inverse (Remarks 1, 2(b)), which add a double-double pass, are listed
-// from the front of the n-entry list and the others from its back, so that
-// the remedy kernel deals the costlier ones out first, one per SM in turn.
-static __global__ void k_fix_decide(Kind kind, Scratch S, double knu_max, int n) {
+// Remedy decisions: one thread per eigenpair (of the part).  k_ffix takes
+// them up: the solves on a DPR1 inverse (Remarks 1, 2(b)), which add a
+// double-double pass, are listed from the front of the n-entry list and the
+// others from its back, so that the remedy kernel deals the costlier ones out
+// first, one per SM in turn.
+static __global__ void k_fix_decide(Kind kind, Scratch S, double knu_max) {
     const PartRange P = part_range(S);
     const int k = P.k0 + blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= P.k1) return;
-    const int r = fix_decide_item(kind, S, k, knu_max);
-    if (r == AE_FLAG_OTHERPOLE) S.fixlist[n - 1 - atomicAdd(S.cnt + C_NFIX2, 1)] = k;
-    else if (r) S.fixlist[atomicAdd(S.cnt + C_NFIX, 1)] = k;
+    if (k < P.k1) fix_decide_item(kind, S, k, knu_max);
 }
 
-// remedy w of the list k_fix_decide wrote (front part first, then the back)
+// remedy w of the list k_ffix wrote (front part first, then the back)
 __device__ __forceinline__ int fix_at(const Scratch &S, long long w, int n) {
     const int nf = S.cnt[C_NFIX];
     return w < nf ? S.fixlist[w] : S.fixlist[n - 1 - (int)(w - nf)];
@@ -78,11 +66,10 @@ __device__ __forceinline__ int fix_at(const Scratch &S, long long w, int n) {
 // team g of CTA b takes remedies w = g * grid + b, then w + teams, ... (so that
 // consecutive remedies land on different SMs), each on the stored-pair slice
 // of the team's first warp (the grid never exceeds k_eig's, so the slices
-// exist).  With va.fused the same team rewrites the remedied eigenpair's
-// column (its position recorded in pos0, as k_eig does).
-template <Kind K, Kind VK, int NW>
-__device__ __forceinline__ void fix_solve_teams(const Scratch &S, const SolveOpts &o,
-                                                const VecArgs &va, int nfix, double *red) {
+// exist).
+template <Kind K, int NW>
+__device__ __forceinline__ void fix_solve_teams(const Scratch &S, const SolveOpts &o, int n,
+                                                int nfix, double *red) {
     constexpr int TPC = 8 / NW;                  // teams per CTA of 8 warps
     const int m = S.cnt[C_M];
     const auto R = PolesOf<K>::make(S, m);
@@ -92,18 +79,7 @@ __device__ __forceinline__ void fix_solve_teams(const Scratch &S, const SolveOpt
     double2 *buf = S.wbuf ? S.wbuf + w0 * S.wstride : nullptr;
     for (long long w = (long long)g * gridDim.x + blockIdx.x; w < nfix;
          w += (long long)TPC * gridDim.x) {
-        const int k = fix_at(S, w, va.n);
-        const bool kept = fix_solve_item<K>(R, T, S, k, o, buf);
-        if (va.fused) {
-            T.sync();
-            if (T.rank == 0) {
-                place_item(S, k);
-                S.pos0[k] = S.pos[k];
-            }
-            T.sync();
-            vector_item<VK>(va.n, va.n1, va.key, va.spk, va.z, va.zrow, va.alpha, va.sgn, S,
-                            va.out, k, T, (double *)buf, true, kept);
-        }
+        fix_solve_item<K>(R, T, S, fix_at(S, w, n), o, buf);
         T.sync();                                // before buf and red are reused
     }
 }
@@ -112,23 +88,22 @@ __device__ __forceinline__ void fix_solve_teams(const Scratch &S, const SolveOpt
 // gives every listed eigenpair a team of its own (one wave over the grid);
 // with more remedies than half the grid's warps, one warp each, remedy w on
 // warp w / CTAs of CTA w mod CTAs: spread over all SMs.
-template <Kind K, Kind VK>
-__global__ void __launch_bounds__(256) k_fix_solve(Scratch S, SolveOpts o, VecArgs va) {
+template <Kind K>
+__global__ void __launch_bounds__(256) k_fix_solve(Scratch S, SolveOpts o, int n) {
     __shared__ double red[16];
     const int nfix = S.cnt[C_NFIX] + S.cnt[C_NFIX2];
     const long long nwarps = (long long)gridDim.x * (blockDim.x >> 5);
     if (nfix == 0) return;
     if (nwarps / 8 >= nfix) {
-        fix_solve_teams<K, VK, 8>(S, o, va, nfix, red);
+        fix_solve_teams<K, 8>(S, o, n, nfix, red);
     } else if (nwarps / 4 >= nfix) {
-        fix_solve_teams<K, VK, 4>(S, o, va, nfix, red);
+        fix_solve_teams<K, 4>(S, o, n, nfix, red);
     } else if (nwarps / 2 >= nfix) {
-        fix_solve_teams<K, VK, 2>(S, o, va, nfix, red);
+        fix_solve_teams<K, 2>(S, o, n, nfix, red);
     } else {
         const int m = S.cnt[C_M];
         const auto R = PolesOf<K>::make(S, m);
         const int lane = threadIdx.x & 31;
-        const WarpTeam T{lane};
         const long long gw = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
         double2 *buf = S.wbuf ? S.wbuf + gw * S.wstride : nullptr;
         // (tickets would hand consecutive remedies to the warps of the first
@@ -136,18 +111,8 @@ __global__ void __launch_bounds__(256) k_fix_solve(Scratch S, SolveOpts o, VecAr
         const int wi = threadIdx.x >> 5;
         for (long long w = (long long)wi * gridDim.x + blockIdx.x; w < nfix;
              w += (long long)(blockDim.x >> 5) * gridDim.x) {
-            const int k = fix_at(S, w, va.n);
-            const bool kept = fix_solve_item<K>(R, T, S, k, o, buf);
-            if (va.fused) {
-                __syncwarp();
-                if (lane == 0) {
-                    place_item(S, k);
-                    S.pos0[k] = S.pos[k];
-                }
-                __syncwarp();
-                vector_item<VK>(va.n, va.n1, va.key, va.spk, va.z, va.zrow, va.alpha, va.sgn,
-                                S, va.out, k, T, (double *)buf, true, kept);
-            }
+            fix_solve_item<K>(R, WarpTeam{lane}, S, fix_at(S, w, n), o, buf);
+            __syncwarp();
         }
     }
 }
@@ -164,28 +129,27 @@ static __global__ void k_place(Scratch S) {
     else if (i < nk + P.u1 - P.u0) place_item(S, ncomp + P.u0 + (i - nk));
 }
 
-// All columns, or with va.fused (k_eig and k_fix_solve wrote the computed
-// ones) only those whose final position differs from the one used then, and
-// the deflated ones; the scalar outputs of every item (K_nu and the remedy
-// flags are known only now).  Staged in the warps' stored-pair slices when
-// there are enough of them.
+// 8 items a CTA: their scalar outputs by a thread each, and by the CTA the
+// columns k_fcols does not write -- those of deflated rows and of eigenpairs the
+// FP64 solver took.
 template <Kind K>
 __global__ void __launch_bounds__(256) k_vectors(VecArgs va, Scratch S) {
-    const int lane = threadIdx.x & 31;
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nwarps = (gridDim.x * blockDim.x) >> 5;
+    __shared__ double red[16];
     const int ncomp = S.cnt[C_M] + 1;
     const PartRange P = part_range(S);
     const int nk = P.k1 - P.k0;
     const int nitems = nk + P.u1 - P.u0;
-    const WarpTeam T{lane};
-    double *stage = (S.wbuf && va.fused) ? (double *)(S.wbuf + (long long)warp * S.wstride)
-                                         : nullptr;
-    for (int i = warp; i < nitems; i += nwarps) {
-        const int item = i < nk ? P.k0 + i : ncomp + P.u0 + (i - nk);
-        const bool cols = !(va.fused && item < ncomp) || S.pos[item] != S.pos0[item];
+    auto item_at = [&](int i) { return i < nk ? P.k0 + i : ncomp + P.u0 + (i - nk); };
+    const int i0 = blockIdx.x * 8;
+    if (threadIdx.x < 8 && i0 + (int)threadIdx.x < nitems)
+        scalar_item<K>(va.n, va.key, va.sgn, S, va.out, item_at(i0 + threadIdx.x));
+    if (!va.out.V) return;
+    for (int i = i0; i < i0 + 8 && i < nitems; ++i) {
+        const int item = item_at(i);
+        if (item < ncomp && S.f.p && S.f.st[item] == FST_DONE) continue;
         vector_item<K>(va.n, va.n1, va.key, va.spk, va.z, va.zrow, va.alpha, va.sgn, S, va.out,
-                       item, T, stage, cols);
+                       item, CtaTeam<8>{(int)threadIdx.x, red, 0});
+        __syncthreads();
     }
 }
 
@@ -210,29 +174,42 @@ template <Kind K, Kind VK>
 static void launch_pipeline(int n, int grid, Scratch S, const SolveOpts &so,
                             const RunOpts &ro, const VecArgs &va, cudaStream_t st) {
     const int sms = sm_count();
+    const int gt = (n + 63) / 64, gm = n < 2 * sms ? n : 2 * sms, g8 = (n + 7) / 8, g32 = (n + 31) / 32;
+    if (so.max_iter < kMinIterCap) S.f = FastPtrs{};
+    const SrcOne src{S, va};
+    if (S.f.p && va.n1 > 0) k_fprep<VK><<<(va.n1 + 255) / 256, 256, 0, st>>>(S, va);
     if (ro.ev[1]) cudaEventRecord(ro.ev[1], st);
-    k_eig<K, VK><<<grid, 256, 0, st>>>(S, so, va);
+    if (S.f.p) {
+        const int diag = va.out.dg_b || va.out.dg_Kb || va.out.dg_flags;
+        k_fopen<K><<<g32, 256, 0, st>>>(src, so);
+        k_feval<<<g8, 256, 0, st>>>(src);
+        k_fstep<K><<<gt, 64, 0, st>>>(src, so, diag);
+        k_fmore<K><<<gm, 256, 0, st>>>(src, so, 0, diag);
+        k_fold<K><<<grid, 256, 0, st>>>(src, so);
+        if (diag) k_fdiag<K><<<g8, 256, 0, st>>>(src, so);
+    } else {
+        k_eig<K><<<grid, 256, 0, st>>>(S, so);
+    }
     if (ro.ev[2]) cudaEventRecord(ro.ev[2], st);
     if (ro.fixup) {
-        k_fix_decide<<<(n + 255) / 256, 256, 0, st>>>(K, S, ro.knu_max, n);
+        k_fix_decide<<<(n + 255) / 256, 256, 0, st>>>(K, S, ro.knu_max);
+        k_ffix<K><<<gt, 64, 0, st>>>(src);
+        if (S.f.p) k_fmore<K><<<gm, 256, 0, st>>>(src, so, 1, 0);
         // every CTA resident at once (the remedies are assigned statically)
         static int fix_per_sm = 0;
         if (!fix_per_sm) {
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fix_per_sm, k_fix_solve<K, VK>, 256, 0);
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fix_per_sm, k_fix_solve<K>, 256, 0);
             if (fix_per_sm <= 0) fix_per_sm = 1;
         }
         int fgrid = sms * fix_per_sm;
         fgrid = fgrid < grid ? fgrid : grid;
         fgrid = n < fgrid ? n : fgrid;
-        k_fix_solve<K, VK><<<fgrid, 256, 0, st>>>(S, so, va);
+        k_fix_solve<K><<<fgrid, 256, 0, st>>>(S, so, n);
     }
     if (ro.ev[3]) cudaEventRecord(ro.ev[3], st);
     k_place<<<(n + 255) / 256, 256, 0, st>>>(S);
-    // fused: one warp per stored-pair slice, so every warp can stage
-    int vgrid = (n + 7) / 8;
-    const int vcap = va.fused ? grid : sms * 16;
-    vgrid = vgrid < vcap ? vgrid : vcap;
-    k_vectors<VK><<<vgrid, 256, 0, st>>>(va, S);
+    if (S.f.p && va.out.V) k_fcols<VK><<<g8, 256, 0, st>>>(src);
+    k_vectors<VK><<<g8, 256, 0, st>>>(va, S);
 }
 
 // The pipeline for each kind other than the arrowhead, one translation unit

@@ -1045,6 +1045,49 @@ __device__ __forceinline__ int newton_finish(FD fd, int side, double pole, doubl
 // ---------------------------------------------------------------------------
 // Algorithm 2 + 3 for the shift pole i on `side`, then lambda = sigma + 1/nu.
 // ---------------------------------------------------------------------------
+// Algorithm 2's b for the shift pole i and K_b of Eq. (K2), under Algorithm
+// 5's gate when asked: A gets the pass's sums, with P and Q in double-double
+// unless both gates pass.  Returns whether the gate asked for double-double.
+template <bool GERSH, class P, class Team>
+__device__ __forceinline__ bool gated_pass(const P &R, const Team &T, int i, const SolveOpts &o,
+                                           double wz, double2 *buf, PassA &A) {
+    const double sigma = R.pole(i), zi = R.zabs(i);
+    if (!o.bgate) {
+        A = pass_a<GERSH>(R, T, sigma, i, wz, buf);
+        return false;
+    }
+    A = pass_a<GERSH, false>(R, T, sigma, i, wz, buf);
+    // b in standard precision unless both C2 (i) and C2 (ii) fail -- the spike
+    // ratio sum_{j != i} |zeta_j| / |zeta_i| exceeds the order n and K_b from
+    // the standard sums exceeds kb_max (both multiplied out; NaN or a zero
+    // P - Q included) -- then P and Q again in double-double (Theorem 6)
+    if (R.zsum - zi > (double)(R.m + 1) * zi &&
+        !(A.P.hi + A.Q.hi <= o.kb_max * fabs(A.P.hi - A.Q.hi))) {
+        const PassA D = pass_a<false, true>(R, T, sigma, i, wz);
+        A.P = D.P;
+        A.Q = D.Q;
+        return true;
+    }
+    return false;
+}
+
+// b = (P - Q) / zeta_i^2 in double-double (Theorem 6), rounded once, and K_b
+__device__ __forceinline__ double b_of(const PassA &A, double zi, double &Kb) {
+    const dd num = dd_add(A.P, dd_neg(A.Q));
+    Kb = (A.P.hi + A.Q.hi) / fabs(num.hi);
+    return dd_div(num, two_prod(zi, zi)).hi;
+}
+
+template <class P, class Team>
+__device__ __forceinline__ bool shifted_b(const P &R, const Team &T, int i, const SolveOpts &o,
+                                          double &b, double &Kb) {
+    const double zi = R.zabs(i);
+    PassA A;
+    const bool ddb = gated_pass<false>(R, T, i, o, 1.0 / zi, nullptr, A);
+    b = b_of(A, zi, Kb);
+    return ddb;
+}
+
 template <class P, class Team>
 __device__ EigResult solve_shifted(const P &R, const Team &T, int i, int side,
                                    const SolveOpts &o, double2 *buf = nullptr) {
@@ -1058,30 +1101,10 @@ __device__ EigResult solve_shifted(const P &R, const Team &T, int i, int side,
     const double c = wz * wz;           // 1/zeta_i^2
     const bool newton = o.finish == 1;
     PassA A;
-    if (o.bgate) {
-        // Algorithm 5: b in standard precision unless both C2 (i) and C2 (ii)
-        // fail -- the spike ratio sum_{j != i} |zeta_j| / |zeta_i| exceeds the
-        // order n and K_b of Eq. (K2) from the standard sums exceeds kb_max --
-        // then P and Q again in double-double (Theorem 6)
-        A = newton ? pass_a<false, false>(R, T, sigma, i, wz, buf)
-                   : pass_a<true, false>(R, T, sigma, i, wz, buf);
-        // (both tests multiplied out: ratio = (zsum - zeta_i) / zeta_i > m + 1
-        // and K_b0 = (P + Q) / |P - Q| > kb_max, NaN or a zero P - Q included)
-        if (R.zsum - zi > (double)(R.m + 1) * zi &&
-            !(A.P.hi + A.Q.hi <= o.kb_max * fabs(A.P.hi - A.Q.hi))) {
-            const PassA D = pass_a<false, true>(R, T, sigma, i, wz);
-            A.P = D.P;
-            A.Q = D.Q;
-            res.flags |= 128;                  // AE_FLAG_DDB
-        }
-    } else {
-        A = newton ? pass_a<false>(R, T, sigma, i, wz, buf)
-                   : pass_a<true>(R, T, sigma, i, wz, buf);
-    }
-    // b = (P - Q) / zeta_i^2 in double-double (Theorem 6), rounded once
-    const dd num = dd_add(A.P, dd_neg(A.Q));
-    const double b = dd_div(num, two_prod(zi, zi)).hi;
-    res.Kb = (A.P.hi + A.Q.hi) / fabs(num.hi);
+    if (newton ? gated_pass<false>(R, T, i, o, wz, buf, A)
+               : gated_pass<true>(R, T, i, o, wz, buf, A))
+        res.flags |= 128;                      // AE_FLAG_DDB
+    const double b = b_of(A, zi, res.Kb);
     res.b = b;
     // with a buffer, each term is c_j / (1 - x delta_j) from the stored pair
     // (5 FP64 instructions instead of 7); the value is the same S(x)
