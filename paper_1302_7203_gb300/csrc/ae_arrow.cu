@@ -231,7 +231,7 @@ static size_t layout(uintptr_t base, int n, Scratch *S) {
     T.es_fixpole = (int *)take(sizeof(int) * nn);
     T.fixlist = (int *)take(sizeof(int) * nn);
     T.pos = (int *)take(sizeof(int) * nn);
-    T.pos0 = (int *)take(sizeof(int) * nn);
+    T.cols = (int *)take(sizeof(int) * nn);
     T.wbuf = nullptr;
     T.wstride = 0;
     T.f = FastPtrs{};
@@ -254,16 +254,27 @@ static size_t fast_layout(uintptr_t base, int n, FastPtrs *F) {
     T.p = (double *)take(8 * n1);
     T.plo = (double *)take(8 * n1);
     T.P = (u64 *)take(8 * n1);
+    T.P2 = (u64 *)take(8 * n1);
     T.z = (u64 *)take(8 * n1);
+    T.zh = (u64 *)take(8 * n1);
+    T.zl = (u64 *)take(8 * n1);
     T.ez = (int *)take(4 * n1);
     T.rp = (double *)take(8 * n1);
     T.rP = (u64 *)take(8 * n1);
     T.mu = (double *)take(8 * nn);
     T.mulo = (double *)take(8 * nn);
     T.lhi = (double *)take(8 * nn);
+    T.llo = (double *)take(8 * nn);
     T.N = (double *)take(8 * nn);
+    T.Nlo = (double *)take(8 * nn);
     T.M2u = (double *)take(8 * nn);
     T.lmod = (u64 *)take(8 * nn);
+    T.lmod2 = (u64 *)take(8 * nn);
+    T.cm = (u64 *)take(8 * nn);
+    T.cm2 = (u64 *)take(8 * nn);
+    T.ce = (int *)take(4 * nn);
+    T.ce2 = (int *)take(4 * nn);
+    T.l32 = (int *)take(4 * nn);
     T.K1 = (int *)take(4 * nn);
     T.K2 = (int *)take(4 * nn);
     T.er = (int *)take(4 * nn);
@@ -272,8 +283,8 @@ static size_t fast_layout(uintptr_t base, int n, FastPtrs *F) {
     T.s5 = (long long *)take(8 * nn);
     T.s2 = (u64 *)take(8 * nn);
     T.s4 = (u64 *)take(8 * nn);
-    T.n1 = (int *)take(4 * nn);
-    T.n2 = (int *)take(4 * nn);
+    T.l1 = (long long *)take(8 * nn);
+    T.l2 = (u64 *)take(8 * nn);
     T.st = (int *)take(4 * nn);
     T.old = (int *)take(4 * nn);
     T.more = (int *)take(4 * nn);

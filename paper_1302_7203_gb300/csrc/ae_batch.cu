@@ -12,7 +12,7 @@
 //                     W-lane teams (W = 8, 16 or 32, chosen per order bucket by
 //                     the tuner)
 //   k_batch_fix_*     remedy decisions over all eigenpairs, a warp per FP64 remedy
-//   k_batch_place / k_batch_vectors / k_batch_status
+//   k_fout, k_fcols, k_vectors, k_batch_status
 // A plan (ae_batch_create) owns the descriptor table and the scratch of every
 // instance and captures the whole sequence in a CUDA graph that
 // ae_batch_run replays.
@@ -83,7 +83,7 @@ struct BatchInst {
 };
 
 struct BatchCtl {
-    int tick_eig, tick_fix, nfix, nold, tick_old, nmore[2];
+    int tick_eig, tick_fix, nfix, nold, tick_old, nmore[2], ncol;
 };
 
 // index i with off[i] <= t < off[i+1]
@@ -132,6 +132,12 @@ struct SrcMany {
     }
     __device__ int more_count(int ph) const { return ctl->nmore[ph]; }
     __device__ int2 more_at(int w) const { return more[w]; }
+    // (the remedy list is done with by then)
+    __device__ void push_col(int i, int item) const {
+        fix[atomicAdd(&ctl->ncol, 1)] = make_int2(i, item);
+    }
+    __device__ int col_count() const { return ctl->ncol; }
+    __device__ int2 col_at(int w) const { return fix[w]; }
     __device__ void push_fix(int i, int k, bool, int) const {
         fix[atomicAdd(&ctl->nfix, 1)] = make_int2(i, k);
     }
@@ -267,35 +273,6 @@ __global__ void __launch_bounds__(256) k_batch_fix_solve(const BatchInst *__rest
         const auto R = PolesOf<KIND_ARROW>::make(S, S.cnt[C_M]);
         fix_solve_item<KIND_ARROW>(R, WarpTeam{lane}, S, ik.y, o, buf);
         __syncwarp();
-    }
-}
-
-__global__ void k_batch_place(const BatchInst *__restrict__ I, int count,
-                              const long long *__restrict__ eoff) {
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= eoff[count]) return;
-    const int i = find_inst(eoff, count, t);
-    place_item(I[i].S, (int)(t - eoff[i]));
-}
-
-// 8 items a CTA: scalar outputs by a thread each, and the columns k_fcols does
-// not write by the CTA
-__global__ void __launch_bounds__(256) k_batch_vectors(const BatchInst *__restrict__ I, int count,
-                                                       const long long *__restrict__ off8) {
-    __shared__ double red[16];
-    const long long u = blockIdx.x;
-    const int i = find_inst(off8, count, u);
-    const BatchInst &B = I[i];
-    const VecArgs &va = B.va;
-    const int i0 = (int)(u - off8[i]) * 8, ncomp = B.S.cnt[C_M] + 1;
-    if (threadIdx.x < 8 && i0 + (int)threadIdx.x < B.n)
-        scalar_item<KIND_ARROW>(B.n, B.d, 1.0, B.S, va.out, i0 + threadIdx.x);
-    if (!va.out.V) return;
-    for (int item = i0; item < i0 + 8 && item < B.n; ++item) {
-        if (item < ncomp && B.S.f.p && B.S.f.st[item] == FST_DONE) continue;
-        vector_item<KIND_ARROW>(B.n, B.n1, B.d, B.z, B.z, nullptr, 0.0, 1.0, B.S, va.out, item,
-                                CtaTeam<8>{(int)threadIdx.x, red, 0});
-        __syncthreads();
     }
 }
 
@@ -491,9 +468,11 @@ static void enqueue(const Plan &P, cudaStream_t st) {
         k_batch_fix_solve<<<batch_eig_grid(), 256, 0, st>>>(P.d_inst, P.d_fix, P.d_ctl, P.so,
                                                              P.wbuf, P.wstride);
     }
-    k_batch_place<<<g, 256, 0, st>>>(P.d_inst, P.count, P.d_eoff);
-    if (P.fast && P.vectors) k_fcols<KIND_ARROW><<<(unsigned)P.n8, 256, 0, st>>>(src);
-    k_batch_vectors<<<(unsigned)P.n8, 256, 0, st>>>(P.d_inst, P.count, P.d_off8);
+    k_fout<KIND_ARROW><<<g1, 64, 0, st>>>(src);
+    if (P.vectors) {
+        if (P.fast) k_fcols<KIND_ARROW><<<(unsigned)P.n8, 256, 0, st>>>(src);
+        k_vectors<KIND_ARROW><<<gm, 256, 0, st>>>(src);
+    }
     if (P.status) k_batch_status<<<(P.count + 255) / 256, 256, 0, st>>>(P.d_inst, P.count, P.status);
 }
 

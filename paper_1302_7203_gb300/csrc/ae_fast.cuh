@@ -6,7 +6,7 @@
 // zeta_i^2 / mu^2 up to sign) is evaluated at lambda = p_i + mu with every
 // difference exact and every term good to ~2^-59, against 2^-53 a rounding in
 // FP64: that covers what the paper's doubled-precision b buys wherever the
-// terms' cancellation against the pole's own term stays below 2^5 (kErrTerm).
+// terms' cancellation against the pole's own term stays below 2^7 (kErrTerm).
 // Beyond it f is summed in 128 bits (~2^-80), and wherever a range test fails
 // the eigenpair takes the FP64 / double-double solver (k_fold, ae_solver.cuh).
 //
@@ -38,12 +38,12 @@ namespace ae {
 // states of a computed eigenpair in the fast path
 enum { FST_EVAL = 0, FST_DONE = 1, FST_OLD = 2, FST_MORE = 3 };
 
-// A zero's offset mu is taken from an evaluation whose error is below 2^-54 of
-// it.  Two errors count, both over f' |mu|: the terms' and sums', 2^-59 (in
+// A zero's offset mu is taken from an evaluation whose error is below 2^-52 of
+// it (2^-54 as a rule: the bounds below are worst cases).  Two errors count, both over f' |mu|: the terms' and sums', 2^-59 (in
 // 128 bits 2^-80) of sum |zeta^2/(p - lambda)|, and that of the differences'
 // unit, 2^-105 of sum zeta^2/(p - lambda)^2 (the differences formed in
 // double-double left out).  Hence the weights of the two sums against f' |mu|:
-constexpr double kErrTerm = 0x1p-5, kErrTermWide = 0x1p-25, kErrUnit = 0x1p-50;
+constexpr double kErrTerm = 0x1p-7, kErrTermWide = 0x1p-25, kErrUnit = 0x1p-50;
 // largest step, relative to the distance to the nearest pole, that the quartic
 // expansion closes: (2^-14)^4 = 2^-56
 constexpr double kStepMax = 0x1p-14;
@@ -54,6 +54,19 @@ constexpr int kMinIterCap = 100;
 __device__ __forceinline__ unsigned long long shr64(unsigned long long v, unsigned s) {
     unsigned long long r;
     asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(s));   // 0 from 64 on
+    return r;
+}
+// the 32 bits below the last place of v >> s (s up to 95)
+__device__ __forceinline__ unsigned low32(unsigned long long v, unsigned s) {
+    unsigned long long r;
+    unsigned q;
+    asm("shl.b64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(64u - s));          // 0 from s = 65 on
+    asm("shr.u32 %0, %1, %2;" : "=r"(q) : "r"((unsigned)(v >> 32)), "r"(s - 64u));   // up to 63
+    return (unsigned)(r >> 32) | q;
+}
+__device__ __forceinline__ int sar32(int v, unsigned s) {
+    int r;
+    asm("shr.s32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(s));   // the sign from 32 on
     return r;
 }
 __device__ __forceinline__ unsigned hi32(double x) { return (unsigned)__double2hiint(x); }
@@ -88,6 +101,12 @@ struct SrcOne {          // one instance, by value
     }
     __device__ int more_count(int ph) const { return S.cnt[C_NMORE + ph]; }
     __device__ int2 more_at(int w) const { return make_int2(0, S.f.more[w]); }
+    // columns for k_vectors
+    __device__ void push_col(int, int item) const {
+        S.cols[atomicAdd(S.cnt + C_NCOL, 1)] = item;
+    }
+    __device__ int col_count() const { return S.cnt[C_NCOL]; }
+    __device__ int2 col_at(int w) const { return make_int2(0, S.cols[w]); }
     __device__ void push_fix(int, int k, bool front, int n) const {
         if (front) S.fixlist[atomicAdd(S.cnt + C_NFIX, 1)] = k;
         else S.fixlist[n - 1 - atomicAdd(S.cnt + C_NFIX2, 1)] = k;
@@ -151,6 +170,7 @@ __device__ __forceinline__ void fprep_item(const Scratch &S, const VecArgs &va, 
         S.f.p[t] = p.hi;
         S.f.plo[t] = p.lo;
         S.f.P[t] = fix_mod(p.hi) + fix_mod(p.lo);
+        S.f.P2[t] = fix_mod<kFixFrac2>(p.hi) + fix_mod<kFixFrac2>(p.lo);
         bad |= !(fabs(p.hi) < 0.5) || (p.hi != 0.0 && fabs(p.hi) < 0x1p-900);
         // zeta^2 as a 64-bit significand and exponent (scaled by 4^es)
         const double z2 = S.pz2[t], zl = S.pz2lo[t];
@@ -162,13 +182,19 @@ __device__ __forceinline__ void fprep_item(const Scratch &S, const VecArgs &va, 
             Z += (unsigned long long)__double2ll_rn(ldexp(zl, 63 - e));
             if (!(Z >> 63)) Z = ~0ull;               // a low part that rounds below 2^63, or over
             S.f.z[t] = Z;
+            // and in 128 bits
+            const unsigned __int128 W =
+                ((unsigned __int128)((b & 0xfffffffffffffull) | 0x10000000000000ull) << 75) +
+                (unsigned __int128)((__int128)(long long)ldexp(zl, 115 - e) << 12);
+            S.f.zh[t] = (unsigned long long)(W >> 64);
+            S.f.zl[t] = (unsigned long long)W;
             S.f.ez[t] = e + 2 * es;
         }
     }
     if (t < va.n1) {
         const dd p = fast_pole<K>(va.key[t], es);
         S.f.rp[t] = p.hi;
-        S.f.rP[t] = fix_mod(p.hi) + fix_mod(p.lo);
+        if (K == KIND_TSVD) S.f.rP[t] = fix_mod(p.hi) + fix_mod(p.lo);
     }
     if (t == 0) bad |= !(fabs(ldexp(S.prm[P_ALPHA_HI], es)) < 0x1p300);
     if (bad) atomicOr(S.cnt + C_FLAGS, CF_NOFAST);
@@ -192,7 +218,9 @@ __device__ __forceinline__ bool set_point(const Scratch &S, int k, dd sg, dd mu)
     S.f.mu[k] = mu.hi;
     S.f.mulo[k] = mu.lo;
     S.f.lhi[k] = l.hi;
+    S.f.llo[k] = l.lo;
     S.f.lmod[k] = fix_mod(l.hi) + fix_mod(l.lo);
+    S.f.lmod2[k] = fix_mod<kFixFrac2>(l.hi) + fix_mod<kFixFrac2>(l.lo);
     return isfinite(l.hi);
 }
 
@@ -203,24 +231,29 @@ __device__ __forceinline__ bool set_point(const Scratch &S, int k, dd sg, dd mu)
 // arrowhead and may lie far outside the others or next to such a point.
 struct DiffRange {
     unsigned lo, span;
+    unsigned lo0;         // lo without the unit's limit
     int tails;            // mask of the tail
 };
 __device__ __forceinline__ DiffRange diff_range(double lhi) {
     const unsigned e = bexp(lhi);
-    const unsigned a = e > 6u ? e - 6u : 0u;
-    if (!(fabs(lhi) < 2.5)) return {a, 4096u, 0};
-    const unsigned lo = a > kFixMinExp ? a : kFixMinExp;
-    return {lo, 1025u - lo, -1};
+    const unsigned a = e > kTailSpan ? e - kTailSpan : 0u;
+    if (!(fabs(lhi) < 2.5)) return {a, 4096u, a, 0};
+    const unsigned lo = a > kFixMinExp2 ? a : kFixMinExp2;
+    return {lo, 1025u - lo, a, -1};
 }
 
-// |p - lambda| where it is small against lambda or against the unit: value
-// and tail (2^-23 of its last place)
-__device__ __forceinline__ double near_diff(dd p, dd sg, dd mu, int &tl) {
-    const dd dl = dd_add(p, dd_neg(sg));
-    const dd D = dd_add(dl, dd_neg(mu));
-    const double t = ldexp(D.hi < 0.0 ? -D.lo : D.lo, 23 + 52 + 1023 - (int)bexp(D.hi));
-    tl = (int)t;
-    return D.hi;
+// (p - sigma) - mu in double-double: exact but for roundings of the low parts
+// (the differences do not cancel: |p - lambda| is at least half of |p - sigma|
+// or of |mu|)
+__device__ __forceinline__ dd near_diff(dd p, dd sg, dd mu) {
+    const dd d = two_sum(p.hi, -sg.hi);
+    const dd D = two_sum(d.hi, -mu.hi);
+    return fast_two_sum(D.hi, D.lo + (d.lo + ((p.lo - sg.lo) - mu.lo)));
+}
+// its tail along |D.hi|, in 2^-7 of D's last place
+__device__ __forceinline__ int near_tail(dd D) {
+    const double t = (D.hi < 0.0 ? -D.lo : D.lo) * pow2(7 + 1075 - (int)bexp(D.hi));
+    return __double2int_rd(t);
 }
 
 // sigma (the shift pole, or another shift) in scaled double-double
@@ -540,6 +573,10 @@ __global__ void __launch_bounds__(256) k_fopen(const __grid_constant__ Src src, 
     S.f.K2[k] = max(dsum > 0.f ? ilogbf(dsum * 1.04f) + 1 : -200,
                     ilogbf(__fdividef(w, mn) * 1.04f) + 1 - ilogbf(mn)) + 1 + 2 * eL - ezs;
     S.f.er[k] = ilogbf(0.98f * (en > 0.f ? fminf(mn, en - mn) : mn)) + es - eL;
+    S.f.s1[k] = S.f.s3[k] = S.f.s5[k] = 0;
+    S.f.s2[k] = S.f.s4[k] = 0;
+    S.f.l1[k] = 0;
+    S.f.l2[k] = 0;
     S.f.st[k] = ok ? FST_EVAL : FST_OLD;
     if (!ok) src.push_old(inst, k);
 }
@@ -548,8 +585,9 @@ __global__ void __launch_bounds__(256) k_fopen(const __grid_constant__ Src src, 
 // k_feval
 // ---------------------------------------------------------------------------
 // Five sums over the poles at each eigenpair's point: zeta^2/(p - lambda)^r for
-// r = 1..5, a warp per eigenpair, the 8 warps of a CTA sharing tiles of poles in
-// shared memory.  Bound by issue slots: ~90 a term (FP64: one subtraction, 64
+// r = 1..5, a warp per eigenpair (and segment of the poles, blockIdx.y: the sums
+// are integers, so that segments add up in any order), the 8 warps of a CTA
+// sharing tiles of poles in shared memory.  Bound by issue slots: ~90 a term (FP64: one subtraction, 64
 // clocks of that pipe, behind them); the r = 4, 5 sums are skipped, warp by
 // warp, where no lane's term reaches 2^-44 of their bound.
 constexpr int kTile = 256;
@@ -576,9 +614,14 @@ __global__ void __launch_bounds__(256, 3) k_feval(const __grid_constant__ Src sr
     const DiffRange dr = diff_range(lhi);
     const int K1 = S.f.K1[ka], K2 = S.f.K2[ka], er = S.f.er[ka];
     const int c1 = K1 - 1023, c2 = K2 - K1 + 1 - 1023, c3 = 2 - er - 1023, c4 = 1 - er - 1023;
+    const double one = unit_reg();
     unsigned long long a1 = 0, a2 = 0, a3 = 0, a4 = 0, a5 = 0;
-    int n1 = 0, n2 = 0;
-    bool flip = true;
+    unsigned long long l1 = 0, l2 = 0;       // 32 bits below a1, a2 (summed apart)
+    // this segment's poles: whole tiles
+    const int all_tiles = (m + kTile - 1) / kTile;
+    const int t0 = (int)((long long)blockIdx.y * all_tiles / gridDim.y);
+    const int tiles = (int)((long long)(blockIdx.y + 1) * all_tiles / gridDim.y);
+    bool flip = k >= t0 * kTile;
     auto load = [&](int t, double &p, unsigned long long &P, unsigned long long &z, int &e) {
         const int j = t * kTile + threadIdx.x;
         p = 4.0; P = 0; z = 0; e = -8192;               // padding: terms of 0
@@ -589,12 +632,11 @@ __global__ void __launch_bounds__(256, 3) k_feval(const __grid_constant__ Src sr
             e = S.f.ez[j];
         }
     };
-    const int tiles = (m + kTile - 1) / kTile;
     double lp;
     unsigned long long lP, lz;
     int le;
-    load(0, lp, lP, lz, le);
-    for (int t = 0; t < tiles; ++t) {
+    load(t0, lp, lP, lz, le);
+    for (int t = t0; t < tiles; ++t) {
         const int bsel = t & 1;
         tp[bsel][threadIdx.x] = lp;
         tP[bsel][threadIdx.x] = lP;
@@ -609,7 +651,7 @@ __global__ void __launch_bounds__(256, 3) k_feval(const __grid_constant__ Src sr
         for (int c = 0; c < nc; ++c) {
             const int x = c * 32 + lane;
             const int j0 = t * kTile + c * 32;
-            double D = tp[bsel][x] - lhi;
+            double D = fma(tp[bsel][x], one, -lhi);    // (an FMA: 2.0 lanes a clock, DADD 1.7)
             int tl;
             unsigned dh = hi32(D), dl = (unsigned)__double2loint(D);
             unsigned eb = (dh << 1) >> 21;
@@ -618,10 +660,14 @@ __global__ void __launch_bounds__(256, 3) k_feval(const __grid_constant__ Src sr
                 const dd pj = {tp[bsel][x], S.f.plo[j]};
                 const int i = S.es_pole[ka];
                 const dd sg = {S.f.p[i], S.f.plo[i]};
-                D = near_diff(pj, sg, dd{S.f.mu[ka], S.f.mulo[ka]}, tl);
+                const dd Dd = near_diff(pj, sg, dd{S.f.mu[ka], S.f.mulo[ka]});
+                D = Dd.hi;
+                tl = near_tail(Dd);
                 dh = hi32(D);
                 dl = (unsigned)__double2loint(D);
                 eb = (dh << 1) >> 21;
+            } else if (eb < kFixMinExp && dr.tails) {
+                tl = tail_of<kFixFrac2>(S.f.P2[j < m ? j : 0] - S.f.lmod2[ka], dh, dl, eb);
             } else {
                 tl = tail_of(tP[bsel][x] - L, dh, dl, eb) & dr.tails;
             }
@@ -631,11 +677,11 @@ __global__ void __launch_bounds__(256, 3) k_feval(const __grid_constant__ Src sr
             unsigned long long q = mul_hi3(tz[bsel][x], Rr);       // 2^62 of the term
             const unsigned s1 = (unsigned)(c1 + (int)eb - te[bsel][x]);
             unsigned long long v1 = shr64(q, s1);
-            const int u1 = s1 < 62u;
+            unsigned long long w1 = low32(q, s1);
             q = mul_hi3(q, Rr);
             const unsigned s2 = s1 + eb + c2;
             a2 += shr64(q, s2);
-            n2 += s2 < 60u;
+            l2 += low32(q, s2);
             q = mul_hi3(q, Rr);
             const unsigned s3 = s2 + eb + c3;
             unsigned long long v3 = shr64(q, s3);
@@ -655,13 +701,13 @@ __global__ void __launch_bounds__(256, 3) k_feval(const __grid_constant__ Src sr
                 a1 = (above ? 0ull - v1 : v1) - a1;
                 a3 = (above ? 0ull - v3 : v3) - a3;
                 a5 = (above ? 0ull - v5 : v5) - a5;
-                n1 = (above ? -u1 : u1) - n1;
+                l1 = (above ? 0ull - w1 : w1) - l1;
                 flip = false;
             } else {
                 a1 += v1;
                 a3 += v3;
                 a5 += v5;
-                n1 += u1;
+                l1 += w1;
             }
         }
     }
@@ -670,7 +716,7 @@ __global__ void __launch_bounds__(256, 3) k_feval(const __grid_constant__ Src sr
         a1 = 0ull - a1;
         a3 = 0ull - a3;
         a5 = 0ull - a5;
-        n1 = -n1;
+        l1 = 0ull - l1;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -679,17 +725,17 @@ __global__ void __launch_bounds__(256, 3) k_feval(const __grid_constant__ Src sr
         a3 += __shfl_xor_sync(FULL, a3, o);
         a4 += __shfl_xor_sync(FULL, a4, o);
         a5 += __shfl_xor_sync(FULL, a5, o);
+        l1 += __shfl_xor_sync(FULL, l1, o);
+        l2 += __shfl_xor_sync(FULL, l2, o);
     }
-    n1 = __reduce_add_sync(FULL, n1);
-    n2 = __reduce_add_sync(FULL, n2);
     if (lane == 0) {
-        S.f.s1[k] = (long long)a1;
-        S.f.s2[k] = a2;
-        S.f.s3[k] = (long long)a3;
-        S.f.s4[k] = a4;
-        S.f.s5[k] = (long long)a5;
-        S.f.n1[k] = n1;
-        S.f.n2[k] = n2;
+        atomicAdd((unsigned long long *)S.f.s1 + k, a1);
+        atomicAdd(S.f.s2 + k, a2);
+        atomicAdd((unsigned long long *)S.f.s3 + k, a3);
+        atomicAdd(S.f.s4 + k, a4);
+        atomicAdd((unsigned long long *)S.f.s5 + k, a5);
+        atomicAdd((unsigned long long *)S.f.l1 + k, l1);
+        atomicAdd(S.f.l2 + k, l2);
     }
 }
 
@@ -699,6 +745,15 @@ __global__ void __launch_bounds__(256, 3) k_feval(const __grid_constant__ Src sr
 __device__ __forceinline__ dd dd_of_ll(long long v) {
     const double h = (double)v;
     return fast_two_sum(h, (double)(v - (long long)h));
+}
+
+// M2 from its fixed-point sum and the 32 bits a term below
+__device__ __forceinline__ dd sum2(unsigned long long a, unsigned long long l, int K2) {
+    const double h = (double)a;
+    const double r = (double)(long long)(a - (unsigned long long)h) + (double)l * 0x1p-32;
+    const dd v = fast_two_sum(h, r);
+    const double u = ldexp(1.0, K2 - 60);
+    return dd{v.hi * u, v.lo * u};
 }
 
 // the counters of a solved eigenpair, added up over the warp's lanes that
@@ -726,8 +781,8 @@ __device__ __forceinline__ void fast_stats(const Scratch &S, int inst, int iters
 // Sums of an evaluation at sigma + mu: M1 = (below - above), M_r = sum zeta^2 /
 // (p - lambda)^r for r >= 2, in scaled units.
 struct FastSums {
-    dd M1;
-    double M2, M3, M4, M5;
+    dd M1, M2;
+    double M3, M4, M5;
 };
 
 // The zero from an evaluation, by one thread.  cterm: the weight of the terms'
@@ -745,7 +800,8 @@ __device__ int fast_advance(const Scratch &S, int k, const FastSums &q, double c
     const dd sg = {S.f.p[i], S.f.plo[i]};
     const dd mu = {S.f.mu[k], S.f.mulo[k]};
     const int K1 = S.f.K1[k], K2 = S.f.K2[k];
-    const double N = 1.0 + q.M2;
+    const dd N2 = dd_add(q.M2, dd{1.0, 0.0});
+    const double N = N2.hi;
     // f = (alpha - sigma - mu) + (sum below - sum above)
     const double sc = pow2(es);
     dd a = dd{S.prm[P_ALPHA_HI] * sc, S.prm[P_ALPHA_LO] * sc};
@@ -769,7 +825,9 @@ __device__ int fast_advance(const Scratch &S, int k, const FastSums &q, double c
         // d = f / (N + M3 d + M4 d^2 + M5 d^3): each turn gains a factor |d|/rho
 #pragma unroll
         for (int r = 0; r < 4; ++r) d = f * rcp(N + d * (q.M3 + d * (q.M4 + d * q.M5)));
-        const double Nf = N + d * (2.0 * q.M3 + d * (3.0 * q.M4 + d * (4.0 * q.M5)));
+        // f' there, to more than double: the vector's norm
+        const dd Nd = dd_add(N2, dd{d * (2.0 * q.M3 + d * (3.0 * q.M4 + d * (4.0 * q.M5))), 0.0});
+        const double Nf = Nd.hi;
         // lambda = sigma + mu + d
         dd mf = two_sum(mu.hi, d);
         mf.lo += mu.lo;
@@ -777,9 +835,14 @@ __device__ int fast_advance(const Scratch &S, int k, const FastSums &q, double c
         if (!(Nf >= 1.0)) return FST_OLD;
         if (M2u < 0.0) {
             const double z2 = S.pz2[i] * sc * sc;
-            M2u = fmax(q.M2 - (z2 / mu.hi) / mu.hi, 0.0) + 0x1p-40 * q.M2;
+            // (a difference with that unit is at least 2^-45: the second bound,
+            // for offsets so small that the first one cancels)
+            M2u = fmin(fmax(q.M2.hi - (z2 / mu.hi) / mu.hi, 0.0) + 0x1p-50 * q.M2.hi,
+                       0x1p45 * pow2(K1));
         }
         if (!(pow2(K1) * cterm + M2u * kErrUnit <= Nf * fabs(mf.hi))) {
+            S.f.M2u[k] = M2u;
+            S.f.N[k] = Nf;
             set_point(S, k, sg, mf);
             return FST_MORE;
         }
@@ -802,6 +865,7 @@ __device__ int fast_advance(const Scratch &S, int k, const FastSums &q, double c
         S.es_mu[k] = muu;
         S.es_lam[k] = sigma + muu;
         S.f.N[k] = Nf;
+        S.f.Nlo[k] = Nd.lo;
         S.f.M2u[k] = M2u;
         set_point(S, k, dd{S.f.p[i], S.f.plo[i]}, mf);
         S.f.mu[k] = mf.hi;           // (set_point may have moved it to the rounded lambda)
@@ -921,10 +985,10 @@ __global__ void __launch_bounds__(64) k_fstep(const __grid_constant__ Src src, S
         const int K1 = S.f.K1[k], K2 = S.f.K2[k], er = S.f.er[k];
         const int K3 = K2 - er, K4 = K3 - er, K5 = K4 - er;
         FastSums q;
-        const dd v = dd_add(dd_of_ll(S.f.s1[k]), dd{0.5 * (double)S.f.n1[k], 0.0});
+        const dd v = dd_add(dd_of_ll(S.f.s1[k]), dd{(double)S.f.l1[k] * 0x1p-32, 0.0});
         const double us = ldexp(1.0, K1 - 62);
         q.M1 = dd{v.hi * us, v.lo * us};
-        q.M2 = ldexp((double)S.f.s2[k] + 0.5 * (double)S.f.n2[k], K2 - 60);
+        q.M2 = sum2(S.f.s2[k], S.f.l2[k], K2);
         q.M3 = -ldexp((double)S.f.s3[k], K3 - 57);
         q.M4 = ldexp((double)S.f.s4[k], K4 - 55);
         q.M5 = -ldexp((double)S.f.s5[k], K5 - 53);
@@ -949,6 +1013,15 @@ __device__ __forceinline__ unsigned __int128 wide_mant(double D, unsigned __int1
     const unsigned long long b = (unsigned long long)__double_as_longlong(D);
     const unsigned long long Dm = (b & 0xfffffffffffffull) | 0x10000000000000ull;
     return ((unsigned __int128)Dm << 75) + tail;
+}
+
+// v >> s, 0 from 128 on
+__device__ __forceinline__ unsigned __int128 shr128(unsigned __int128 v, unsigned s) {
+    const unsigned long long lo = (unsigned long long)v, hi = (unsigned long long)(v >> 64);
+    const unsigned t = s & 63;
+    const unsigned long long h = hi >> t, x = t ? hi << (64 - t) : 0ull, l = (lo >> t) | x;
+    const unsigned __int128 a = ((unsigned __int128)h << 64) | l;
+    return s < 64 ? a : s < 128 ? (unsigned __int128)h : (unsigned __int128)0;
 }
 
 // high 128 bits of a b
@@ -985,7 +1058,8 @@ __global__ void __launch_bounds__(256) k_fmore(const __grid_constant__ Src src, 
                                                int phase, int diag) {
     __shared__ unsigned long long sh1[8], sh1h[8], sh2[8], sh2u[8], sh4[8];
     __shared__ long long sh3[8], sh5[8];
-    __shared__ int shn[8], verdict;
+    __shared__ unsigned long long sh2l[8];
+    __shared__ int verdict, verdict_unit;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int cnt = src.more_count(phase);
     for (int w = blockIdx.x; w < cnt; w += gridDim.x) {
@@ -993,6 +1067,7 @@ __global__ void __launch_bounds__(256) k_fmore(const __grid_constant__ Src src, 
         const Scratch &S = src.scr(ik.x);
         const int k = ik.y, m = S.cnt[C_M];
         int st = FST_MORE;
+        bool unit_bad = false;
         if (phase == 1) {
             // (an outermost eigenvalue's point is its rounded lambda)
             if (threadIdx.x == 0)
@@ -1004,31 +1079,34 @@ __global__ void __launch_bounds__(256) k_fmore(const __grid_constant__ Src src, 
             const double lhi = S.f.lhi[k];
             const unsigned long long L = S.f.lmod[k];
             const DiffRange dr = diff_range(lhi);
+            // (a unit's error that one evaluation showed to be too large: every
+            // difference in double-double)
+            const bool all_dd = unit_bad && dr.tails;
             const int K1 = S.f.K1[k], K2 = S.f.K2[k], er = S.f.er[k];
             const int c1 = K1 - 1023, c2 = K2 - K1 + 1 - 1023, c3 = 2 - er - 1023,
                       c4 = 1 - er - 1023;
             __int128 a1 = 0;
             unsigned long long a2 = 0, a2u = 0, a4 = 0;
             long long a3 = 0, a5 = 0;
-            int n2 = 0;
+            unsigned long long l2 = 0;
             for (int j = threadIdx.x; j < m; j += 256) {
                 const double p = S.f.p[j];
                 double D = p - lhi;
                 unsigned dh = hi32(D), eb = (dh << 1) >> 21;
                 int tl;
                 unsigned __int128 M;
-                const bool dd_diff = eb - dr.lo >= dr.span;
+                const bool dd_diff = eb - dr.lo >= dr.span || (dr.tails && eb < kFixMinExp) || all_dd;
                 if (dd_diff) {
                     const int i = S.es_pole[k];
-                    const dd dl = dd_add(dd{p, S.f.plo[j]}, dd_neg(dd{S.f.p[i], S.f.plo[i]}));
-                    const dd Dd = dd_add(dl, dd_neg(dd{S.f.mu[k], S.f.mulo[k]}));
+                    const dd Dd = near_diff(dd{p, S.f.plo[j]}, dd{S.f.p[i], S.f.plo[i]},
+                                            dd{S.f.mu[k], S.f.mulo[k]});
                     D = Dd.hi;
                     dh = hi32(D);
                     eb = (dh << 1) >> 21;
-                    const double lo = ldexp(D < 0.0 ? -Dd.lo : Dd.lo, 62 + 1075 - (int)eb);
-                    const long long li = (long long)lo;          // 2^-62 of D's last place
-                    tl = (int)(li >> 39);
-                    M = wide_mant(D, (unsigned __int128)((__int128)li << 13));
+                    const double lo = (D < 0.0 ? -Dd.lo : Dd.lo) * pow2(51 + 1075 - (int)eb);
+                    const long long li = __double2ll_rd(lo);     // 2^-51 of D's last place
+                    tl = (int)(li >> 44);
+                    M = wide_mant(D, (unsigned __int128)((__int128)li << 24));
                 } else if (dr.tails) {
                     const unsigned dl = (unsigned)__double2loint(D);
                     unsigned long long T = S.f.P[j] - L;
@@ -1037,7 +1115,7 @@ __global__ void __launch_bounds__(256) k_fmore(const __grid_constant__ Src src, 
                         ((unsigned long long)((dh & 0xfffffu) | 0x100000u) << 32) | dl;
                     const int sh = (int)eb - (1075 - kFixFrac);
                     const long long tail = (long long)(T - (Dm << (sh & 63)));
-                    tl = (int)(unsigned)(((unsigned long long)tail << ((55 - sh) & 63)) >> 32);
+                    tl = (int)(tail >> ((sh - 7) & 63));
                     M = wide_mant(D, (unsigned __int128)((__int128)tail << (75 - sh)));
                 } else {
                     tl = 0;
@@ -1051,14 +1129,11 @@ __global__ void __launch_bounds__(256) k_fmore(const __grid_constant__ Src src, 
                 const int ez = S.f.ez[j];
                 // f's term: zeta^2 in double-double over the wide difference
                 {
-                    const double z2 = S.pz2[j];
-                    const int e = (int)bexp(z2) - 1023;
-                    const long long zl = (long long)ldexp(S.pz2lo[j], 115 - e);
                     const unsigned __int128 Z =
-                        wide_mant(z2, (unsigned __int128)((__int128)zl << 12));
+                        ((unsigned __int128)S.f.zh[j] << 64) | S.f.zl[j];
                     const unsigned __int128 q = mul_hi128(Z, recip127(M, R));
-                    const int s = K1 + 2 - ez + (int)eb - 1023;
-                    const __int128 v = s < 128 ? (__int128)(q >> (s < 0 ? 0 : s)) : (__int128)0;
+                    const __int128 v =
+                        (__int128)shr128(q, (unsigned)(K1 + 2 - ez + (int)eb - 1023));
                     a1 += above ? -v : v;
                 }
                 unsigned long long q = mul_hi3(S.f.z[j], R);
@@ -1067,7 +1142,7 @@ __global__ void __launch_bounds__(256) k_fmore(const __grid_constant__ Src src, 
                 const unsigned long long v2 = shr64(q, s2);
                 a2 += v2;
                 a2u += dd_diff ? 0ull : v2;
-                n2 += s2 < 60u;
+                l2 += low32(q, s2);
                 q = mul_hi3(q, R);
                 const unsigned s3 = s2 + eb + c3;
                 const long long v3 = (long long)shr64(q, s3);
@@ -1087,14 +1162,14 @@ __global__ void __launch_bounds__(256) k_fmore(const __grid_constant__ Src src, 
                 a1 += (__int128)(((unsigned __int128)hh << 64) | hl);
                 a2 += __shfl_xor_sync(FULL, a2, s);
                 a2u += __shfl_xor_sync(FULL, a2u, s);
+                l2 += __shfl_xor_sync(FULL, l2, s);
                 a3 += __shfl_xor_sync(FULL, a3, s);
                 a4 += __shfl_xor_sync(FULL, a4, s);
                 a5 += __shfl_xor_sync(FULL, a5, s);
             }
-            n2 = __reduce_add_sync(FULL, n2);
             __syncthreads();
             if (lane == 0) {
-                shn[wid] = n2;
+                sh2l[wid] = l2;
                 sh1[wid] = (unsigned long long)a1;
                 sh1h[wid] = (unsigned long long)((unsigned __int128)a1 >> 64);
                 sh2[wid] = a2;
@@ -1109,7 +1184,7 @@ __global__ void __launch_bounds__(256) k_fmore(const __grid_constant__ Src src, 
                     a1 += (__int128)(((unsigned __int128)sh1h[x] << 64) | sh1[x]);
                     a2 += sh2[x];
                     a2u += sh2u[x];
-                    n2 += shn[x];
+                    l2 += sh2l[x];
                     a3 += sh3[x];
                     a4 += sh4[x];
                     a5 += sh5[x];
@@ -1119,7 +1194,7 @@ __global__ void __launch_bounds__(256) k_fmore(const __grid_constant__ Src src, 
                 const dd v = dd_of_i128(a1);
                 const double us = ldexp(1.0, K1 - 124);
                 q.M1 = dd{v.hi * us, v.lo * us};
-                q.M2 = ldexp((double)a2 + 0.5 * (double)n2, K2 - 60);
+                q.M2 = sum2(a2, l2, K2);
                 q.M3 = -ldexp((double)a3, K3 - 57);
                 q.M4 = ldexp((double)a4, K4 - 55);
                 q.M5 = -ldexp((double)a5, K5 - 53);
@@ -1152,9 +1227,11 @@ __global__ void __launch_bounds__(256) k_fmore(const __grid_constant__ Src src, 
                     }
                 }
                 verdict = v2;
+                verdict_unit = v2 == FST_MORE && S.f.M2u[k] * kErrUnit > 0.25 * S.f.N[k] * fabs(S.f.mu[k]);
             }
             __syncthreads();
             st = verdict;
+            unit_bad |= verdict_unit != 0;
         }
         __syncthreads();
     }
@@ -1293,16 +1370,85 @@ __device__ __forceinline__ double pack_prod(unsigned long long a, unsigned long 
     return __hiloint2double((int)(hi | sgn), (int)lo);
 }
 
+// 1 / sqrt(x) in double-double
+__device__ __forceinline__ dd dd_rsqrt(dd x) {
+    const double r = 1.0 / sqrt(x.hi);
+    const dd t = dd_mul(two_prod(r, r), x);                    // 1 + O(eps)
+    const double e = (1.0 - t.hi) - t.lo;
+    return fast_two_sum(r, 0.5 * r * e);
+}
+
+// a positive double-double as a significand of 64 bits (top bit set) and an
+// exponent
+__device__ __forceinline__ void scale_of(dd x, unsigned long long &m, int &e) {
+    const Mant h = mant_of(x.hi);
+    e = h.e - 1023;
+    m = h.m + (unsigned long long)__double2ll_rn(ldexp(x.lo, 63 - e));
+    if (!(m >> 63)) m = h.m;                                   // (the low part crossed a power of 2)
+}
+
+// One thread per item: its output position and scalar outputs, and for an
+// eigenpair the fast path solved what its column needs -- the scale 1/||x|| (and
+// the second matrix's) as significand and exponent, lambda's tail.  The other
+// items' columns are listed for k_vectors.
+template <Kind VK, class Src>
+__global__ void __launch_bounds__(64) k_fout(const __grid_constant__ Src src) {
+    int inst = 0, idx = 0;
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (!src.item(t, inst, idx)) return;
+    const Scratch &S = src.scr(inst);
+    const VecArgs &va = src.vec(inst);
+    const int ncomp = S.cnt[C_M] + 1;
+    const PartRange P = part_range(S);
+    const int nk = P.k1 - P.k0;
+    if (idx >= nk + P.u1 - P.u0) return;
+    const int item = idx < nk ? P.k0 + idx : ncomp + P.u0 + (idx - nk);
+    place_item(S, item);
+    scalar_item<VK>(va.n, va.key, va.sgn, S, va.out, item);
+    if (!va.out.V) return;
+    if (item >= ncomp || !S.f.p || S.f.st[item] != FST_DONE) {
+        src.push_col(inst, item);
+        return;
+    }
+    const int k = item, es = fast_scale<VK>(S);
+    // the norm is sqrt(f') but for the DPR1, whose vector (without the
+    // arrowhead's corner) has ||x||^2 = f' / (|rho| (lambda - p_last))
+    dd nrm = {S.f.N[k], S.f.Nlo[k]};
+    if (VK == KIND_DPR1) {
+        const dd sg = fast_sigma<VK>(S, k, es);
+        const dd pl = {S.prm[P_PLAST] * pow2(es), 0.0};
+        const dd x = dd_add(dd_add(sg, dd_neg(pl)), dd{S.f.mu[k], S.f.mulo[k]});
+        nrm = dd_div(nrm, dd_mul_d(x, fabs(va.alpha) * pow2(es)));   // (va.alpha is rho; u is
+    }                                                                //  not scaled)
+    // scaled multipliers: spikes and poles both scale by 2^es (DPR1: see nrm)
+    const dd inv = dd_rsqrt(nrm);
+    scale_of(inv, S.f.cm[k], S.f.ce[k]);
+    if (VK != KIND_DPR1) S.f.ce[k] += es;
+    if (VK == KIND_TSVD) {
+        scale_of(dd_mul_d(inv, sv_of(S, k)), S.f.cm2[k], S.f.ce2[k]);
+        S.f.ce2[k] += es;
+    }
+    // lambda's own tail, as an integer of 2^-30 last places of lambda
+    const double lhi = S.f.lhi[k];
+    S.f.l32[k] = fabs(lhi) < 2.5
+                     ? (int)rint(S.f.llo[k] * pow2(min(1075 - (int)bexp(lhi) + 30, 1023)))
+                     : 0;
+}
+
 // Columns of the eigenpairs the fast path solved, a warp each; the CTA's 8
-// warps share tiles of input rows.  Component a_r / ((d_r - sigma) - mu) /
-// ||x||, for the second matrix (SVD: U, NSYM: Y) or the imaginary part (HERM)
-// with its own multiplier.
+// warps share tiles of input rows, blockIdx.y is the segment of rows.
+// Component a_r / ((d_r - sigma) - mu) / ||x||, for the second matrix (SVD: U,
+// NSYM: Y) or the imaginary part (HERM) with its own multiplier.  The difference
+// is fl(d_r - lambda) with lambda's tail taken into its reciprocal (SVD, whose
+// poles d^2 are no doubles: the exact tail): a component's error is that of
+// one subtraction and one rounding.
 template <Kind VK, class Src>
 __global__ void __launch_bounds__(256, 3) k_fcols(const __grid_constant__ Src src) {
     constexpr bool CPLX = VK == KIND_HERM;
     constexpr bool TWO = VK == KIND_HERM || VK == KIND_NSYM || VK == KIND_TSVD;
+    constexpr bool SVD = VK == KIND_TSVD;
     __shared__ double tp[2][kTile];
-    __shared__ unsigned long long tP[2][kTile], ta[2][kTile], tb[2][TWO ? kTile : 1];
+    __shared__ unsigned long long ta[2][kTile], tb[2][TWO ? kTile : 1], tP[2][SVD ? kTile : 1];
     __shared__ int ea[2][kTile], eb2[2][TWO ? kTile : 1];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     int inst, first;
@@ -1316,47 +1462,34 @@ __global__ void __launch_bounds__(256, 3) k_fcols(const __grid_constant__ Src sr
     if (!__syncthreads_or(act)) return;
     const int ka = act ? k : P.k0 + first;
     const int n1 = va.n1;
-    constexpr Kind RK = VK;                             // pole form of the rows
-    const int es = fast_scale<RK>(S);
     const double lhi = S.f.lhi[ka];
-    const unsigned long long L = S.f.lmod[ka];
-    const DiffRange dr = diff_range(lhi);
-    // 1 / ||x||: the norm is sqrt(f') but for the DPR1, whose vector (without
-    // the arrowhead's corner) has ||x||^2 = f' / (|rho| (lambda - p_last))
-    double nrm = S.f.N[ka];
-    if (VK == KIND_DPR1) {
-        const dd sg = fast_sigma<RK>(S, ka, es);
-        const dd pl = {ldexp(S.prm[P_PLAST], es), 0.0};
-        const double x = dd_add(dd_add(sg, dd_neg(pl)), dd{S.f.mu[ka], S.f.mulo[ka]}).hi;
-        nrm = nrm / x / ldexp(fabs(va.alpha), es);     // (va.alpha is rho; u is not scaled)
-    }
-    const double inv = 1.0 / sqrt(nrm);
-    const double sv = VK == KIND_TSVD ? sv_of(S, ka) : 1.0;      // the singular value
-    // scaled multipliers: spikes and poles both scale by 2^es (DPR1: see nrm)
-    const Mant mi = mant_of(inv);
-    const int ei = mi.e - 1023 + (VK == KIND_DPR1 ? 0 : es);
-    const Mant mu2 = mant_of(VK == KIND_TSVD ? inv * sv : inv);
-    const int ei2 = mu2.e - 1023 + es;
+    DiffRange dr = diff_range(lhi);
+    if (!SVD) dr = {dr.lo0, 4096u, dr.lo0, dr.tails};  // (no unit to mind)
+    const int l32 = S.f.l32[ka], el = (int)bexp(lhi) - 23;
+    const unsigned long long L = SVD ? S.f.lmod[ka] : 0ull;
+    const double one = unit_reg();
+    const unsigned long long mi = S.f.cm[ka], mi2 = SVD ? S.f.cm2[ka] : 0ull;
+    const int ei = S.f.ce[ka] + 1023, ei2 = SVD ? S.f.ce2[ka] + 1023 : ei;
     const int pos = out_pos<VK>(S, va.n, va.sgn, ka);
     const unsigned vsg = (VK == KIND_DPR1 && va.sgn < 0.0) ? 0x80000000u : 0u;
     double *col = va.out.V + (size_t)pos * va.out.ldv;
     double *ucol = (TWO && !CPLX && va.out.U) ? va.out.U + (size_t)pos * va.out.ldu : nullptr;
     double lp;
-    unsigned long long lP;
+    unsigned long long lP = 0;
     Mant la, lb;
     auto load = [&](int t) {
         const int r = t * kTile + threadIdx.x;
-        lp = 4.0; lP = 0; la = lb = Mant{0, 0};
+        lp = 4.0; la = lb = Mant{0, 0};
         if (r < n1) {
             lp = S.f.rp[r];
-            lP = S.f.rP[r];
+            if (SVD) lP = S.f.rP[r];
             if (CPLX) {
                 la = mant_of(va.z[2 * r]);
                 lb = mant_of(va.z[2 * r + 1]);
             } else if (VK == KIND_NSYM) {
                 la = mant_of(va.z[r]);
                 lb = mant_of(va.zrow[r]);
-            } else if (VK == KIND_TSVD) {
+            } else if (SVD) {
                 la = mant_of(va.spk[r]);
                 lb = mant_of(va.z[r]);                 // u_r = s v_r / d_r, spike d_r z_r
             } else {
@@ -1364,14 +1497,16 @@ __global__ void __launch_bounds__(256, 3) k_fcols(const __grid_constant__ Src sr
             }
         }
     };
-    const int tiles = (n1 + kTile - 1) / kTile;
-    load(0);
-    for (int t = 0; t < tiles; ++t) {
+    const int all_tiles = (n1 + kTile - 1) / kTile;
+    const int t0 = (int)((long long)blockIdx.y * all_tiles / gridDim.y);
+    const int tiles = (int)((long long)(blockIdx.y + 1) * all_tiles / gridDim.y);
+    load(t0);
+    for (int t = t0; t < tiles; ++t) {
         const int b = t & 1;
         tp[b][threadIdx.x] = lp;
-        tP[b][threadIdx.x] = lP;
         ta[b][threadIdx.x] = la.m;
         ea[b][threadIdx.x] = la.e;
+        if (SVD) tP[b][threadIdx.x] = lP;
         if (TWO) {
             tb[b][threadIdx.x] = lb.m;
             eb2[b][threadIdx.x] = lb.e;
@@ -1381,34 +1516,39 @@ __global__ void __launch_bounds__(256, 3) k_fcols(const __grid_constant__ Src sr
         if (!act) continue;
         const int left = n1 - t * kTile;
         const int nc = left >= kTile ? kTile / 32 : (left + 31) / 32;
-#pragma unroll 1
+#pragma unroll 2
         for (int c = 0; c < nc; ++c) {
             const int x = c * 32 + lane;
             const int r = t * kTile + x;
-            double D = tp[b][x] - lhi;
+            double D = fma(tp[b][x], one, -lhi);       // (an FMA: 2.0 lanes a clock, DADD 1.7)
             int tl;
             unsigned dh = hi32(D), dl = (unsigned)__double2loint(D);
             unsigned ed = (dh << 1) >> 21;
             if (ed - dr.lo >= dr.span && r < n1) {
-                const dd pr = fast_pole<RK>(va.key[r], es);
-                D = near_diff(pr, fast_sigma<RK>(S, ka, es), dd{S.f.mu[ka], S.f.mulo[ka]}, tl);
+                const int es = fast_scale<VK>(S);
+                const dd pr = fast_pole<VK>(va.key[r], es);
+                const dd Dd =
+                    near_diff(pr, fast_sigma<VK>(S, ka, es), dd{S.f.mu[ka], S.f.mulo[ka]});
+                D = Dd.hi;
+                tl = near_tail(Dd);
                 dh = hi32(D);
                 dl = (unsigned)__double2loint(D);
                 ed = (dh << 1) >> 21;
             } else {
-                tl = tail_of(tP[b][x] - L, dh, dl, ed) & dr.tails;
+                // -lambda's tail for p above, + below, in 2^-7 of D's last place
+                tl = SVD ? tail_of(tP[b][x] - L, dh, dl, ed) & dr.tails
+                         : sar32(l32 ^ ~((int)dh >> 31), ed - el);
             }
             const unsigned seed = hi32(rcp_seed(__hiloint2double(
                 (int)((dh & 0xfffffu) | 0x3ff00000u), 0)));
             const unsigned long long Rr = recip63<false>(dh, dl, tl, seed);
-            const unsigned long long G = mul_hi3(mi.m, Rr);
+            const unsigned long long G = mul_hi3(mi, Rr);
             const int e1 = ea[b][x];
             const unsigned sg = (((unsigned)e1 ^ dh) & 0x80000000u) ^ vsg;
-            const int be = (int)(short)(e1 & 0xffff) - (int)ed + ei + 1023;
-            const double v = pack_prod(ta[b][x], G, be, sg);
+            const double v = pack_prod(ta[b][x], G, (int)(short)(e1 & 0xffff) - (int)ed + ei, sg);
             if (CPLX) {
                 const int e2 = eb2[b][x];
-                const double vi = pack_prod(tb[b][x], G, (int)(short)(e2 & 0xffff) - (int)ed + ei + 1023,
+                const double vi = pack_prod(tb[b][x], G, (int)(short)(e2 & 0xffff) - (int)ed + ei,
                                             ((unsigned)e2 ^ dh) & 0x80000000u);
                 if (r < n1) {
                     col[2 * r] = v;
@@ -1417,25 +1557,40 @@ __global__ void __launch_bounds__(256, 3) k_fcols(const __grid_constant__ Src sr
             } else {
                 if (r < n1) col[r] = v;
                 if (TWO && ucol) {
-                    const unsigned long long G2 = VK == KIND_TSVD ? mul_hi3(mu2.m, Rr) : G;
+                    const unsigned long long G2 = SVD ? mul_hi3(mi2, Rr) : G;
                     const int e2 = eb2[b][x];
                     const double vu = pack_prod(tb[b][x], G2,
-                                                (int)(short)(e2 & 0xffff) - (int)ed + ei2 + 1023,
+                                                (int)(short)(e2 & 0xffff) - (int)ed + ei2,
                                                 ((unsigned)e2 ^ dh) & 0x80000000u);
                     if (r < n1) ucol[r] = vu;
                 }
             }
         }
     }
-    if (act && lane == 0 && VK != KIND_DPR1) {
-        const double vn = -inv;
+    if (act && lane == 0 && VK != KIND_DPR1 && blockIdx.y == 0) {
+        const double vn = -dd_rsqrt(dd{S.f.N[ka], S.f.Nlo[ka]}).hi;
         if (CPLX) {
             col[2 * n1] = vn;
             col[2 * n1 + 1] = 0.0;
         } else {
             col[n1] = vn;
-            if (ucol) ucol[n1] = VK == KIND_TSVD ? va.alpha * vn / sv : vn;
+            if (ucol) ucol[n1] = SVD ? va.alpha * vn / sv_of(S, ka) : vn;
         }
+    }
+}
+
+// The columns k_fcols does not write -- those of deflated rows and of
+// eigenpairs the FP64 solver took -- by a CTA each.
+template <Kind VK, class Src>
+__global__ void __launch_bounds__(256) k_vectors(const __grid_constant__ Src src) {
+    __shared__ double red[16];
+    const int cnt = src.col_count();
+    for (int w = blockIdx.x; w < cnt; w += gridDim.x) {
+        const int2 ik = src.col_at(w);
+        const VecArgs &va = src.vec(ik.x);
+        vector_item<VK>(va.n, va.n1, va.key, va.spk, va.z, va.zrow, va.alpha, va.sgn,
+                        src.scr(ik.x), va.out, ik.y, CtaTeam<8>{(int)threadIdx.x, red, 0});
+        __syncthreads();
     }
 }
 

@@ -36,7 +36,8 @@ enum {
     C_OLDTK = 22,     // their work ticket
     C_NMORE = 23,     // eigenpairs k_fmore evaluates: after k_fstep, after k_ffix
     C_NMORE1 = 24,
-    C_COUNT = 25
+    C_NCOL = 25,      // columns k_vectors writes
+    C_COUNT = 26
 };
 enum { C64_ITERS = 0, C64_MAXKB = 1, C64_MAXKNU = 2, C64_ITERS_FIX = 3, C64_DERIV = 4,
        C64_F32 = 5,     // O(n) passes in FP32 (midpoint tests, FP32 steps and brackets)
@@ -70,16 +71,19 @@ enum {
 // values of its sums, and its state.  p == null: the path is not used.
 struct FastPtrs {
     double *p, *plo;                      // reduced poles (double-double)
-    unsigned long long *P, *z;
+    unsigned long long *P, *P2, *z, *zh, *zl;   // (P2: in units of 2^-140; zh, zl: 128 bits)
     int *ez;
-    double *rp;                           // input rows
+    double *rp;                           // input rows (rP: SVD only)
     unsigned long long *rP;
-    double *mu, *mulo, *lhi, *N, *M2u;
-    unsigned long long *lmod;
+    double *mu, *mulo, *lhi, *llo, *N, *Nlo, *M2u;
+    unsigned long long *lmod, *lmod2;
     int *K1, *K2, *er;
     long long *s1, *s3, *s5;
     unsigned long long *s2, *s4;
-    int *n1, *n2;
+    long long *l1;                        // 32 bits below s1, s2, summed apart
+    unsigned long long *l2;
+    unsigned long long *cm, *cm2;         // column scales: significands, exponents
+    int *ce, *ce2, *l32;
     int *st, *old, *more;
 };
 
@@ -104,7 +108,7 @@ struct Scratch {
     double *es_sigma, *es_mu, *es_lam, *es_b, *es_Kb, *es_Knu, *es_fixshift;
     int *es_pole, *es_iters, *es_flags, *es_fixpole, *fixlist;
     int *pos;       // output position of computed (first m+1) and deflated items
-    int *pos0;      // computed item: the position its column was first written at
+    int *cols;      // items whose columns k_vectors writes
     double2 *wbuf;  // optional: one (delta_j, c_j) slice per eig team, wstride apart
     long long wstride;
 };

@@ -101,10 +101,15 @@ struct ae_server {
     int worker_error = cudaSuccess;
 
     long long merged = 0;             // requests solved in merged batched passes
+    // mean time between submissions of mergeable requests (seconds, halved
+    // towards each new gap), and the last one's time
+    double gap = 1.0;
+    clk::time_point t_small;
 
     void loop();
     bool admit_locked(Req *r);
     int admit_merged_locked();
+    bool worth_holding_locked() const;
     void retire_locked(Req *r);
 };
 
@@ -202,6 +207,15 @@ int ae_server::admit_merged_locked() {
     }
     slot_busy[slot] = cnt;          // freed as its requests retire
     return cnt;
+}
+
+// A lone small arrowhead waits for a second one (a merged pass of two costs
+// about what one alone does) while they come less than a millisecond apart:
+// for at most two such gaps from its submission.
+bool ae_server::worth_holding_locked() const {
+    if (queue.size() != 1 || !mergeable(queue.front()->in) || gap > 1e-3) return false;
+    const double age = std::chrono::duration<double>(clk::now() - queue.front()->t_submit).count();
+    return age < 2.0 * gap;
 }
 
 bool ae_server::admit_locked(Req *r) {
@@ -306,6 +320,7 @@ void ae_server::loop() {
         // 2. admit in FIFO order (a run of small arrowheads at the head as one)
         while (!queue.empty()) {
             if (admit_merged_locked() > 0) continue;
+            if (worth_holding_locked()) break;
             if (!admit_locked(queue.front())) break;
             queue.pop_front();
         }
@@ -387,6 +402,11 @@ int ae_serve_submit(ae_server *s, const ae_request *req, unsigned long long *tic
     if (!s->started) {
         s->started = true;
         s->t_first = r->t_submit;
+    }
+    if (mergeable(r->in)) {
+        const double dt = std::chrono::duration<double>(r->t_submit - s->t_small).count();
+        s->gap = 0.5 * (s->gap + std::min(dt, 0.01));
+        s->t_small = r->t_submit;
     }
     s->reqs[r->id] = r;
     s->queue.push_back(r);

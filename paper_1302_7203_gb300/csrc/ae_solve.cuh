@@ -118,42 +118,6 @@ __global__ void __launch_bounds__(256) k_fix_solve(Scratch S, SolveOpts o, int n
 }
 
 // ---------------------------------------------------------------------------
-// output placement and vectors
-// ---------------------------------------------------------------------------
-static __global__ void k_place(Scratch S) {
-    const PartRange P = part_range(S);
-    const int ncomp = S.cnt[C_M] + 1;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int nk = P.k1 - P.k0;
-    if (i < nk) place_item(S, P.k0 + i);
-    else if (i < nk + P.u1 - P.u0) place_item(S, ncomp + P.u0 + (i - nk));
-}
-
-// 8 items a CTA: their scalar outputs by a thread each, and by the CTA the
-// columns k_fcols does not write -- those of deflated rows and of eigenpairs the
-// FP64 solver took.
-template <Kind K>
-__global__ void __launch_bounds__(256) k_vectors(VecArgs va, Scratch S) {
-    __shared__ double red[16];
-    const int ncomp = S.cnt[C_M] + 1;
-    const PartRange P = part_range(S);
-    const int nk = P.k1 - P.k0;
-    const int nitems = nk + P.u1 - P.u0;
-    auto item_at = [&](int i) { return i < nk ? P.k0 + i : ncomp + P.u0 + (i - nk); };
-    const int i0 = blockIdx.x * 8;
-    if (threadIdx.x < 8 && i0 + (int)threadIdx.x < nitems)
-        scalar_item<K>(va.n, va.key, va.sgn, S, va.out, item_at(i0 + threadIdx.x));
-    if (!va.out.V) return;
-    for (int i = i0; i < i0 + 8 && i < nitems; ++i) {
-        const int item = item_at(i);
-        if (item < ncomp && S.f.p && S.f.st[item] == FST_DONE) continue;
-        vector_item<K>(va.n, va.n1, va.key, va.spk, va.z, va.zrow, va.alpha, va.sgn, S, va.out,
-                       item, CtaTeam<8>{(int)threadIdx.x, red, 0});
-        __syncthreads();
-    }
-}
-
-// ---------------------------------------------------------------------------
 // host orchestration
 // ---------------------------------------------------------------------------
 static int sm_count() {
@@ -165,6 +129,15 @@ static int sm_count() {
         if (cached <= 0) cached = 1;
     }
     return cached;
+}
+
+// Segments of the poles (rows) that k_feval (k_fcols) CTAs of 8 eigenpairs take:
+// enough for 8 waves of 3 CTAs an SM, so that the last one is at most an eighth
+// of the time (n = 8192 alone is 2.25 waves), but no less than a tile each.
+static int segments(int n, int rows) {
+    const int units = (n + 7) / 8, want = (24 * sm_count() + units - 1) / units;
+    const int tiles = (rows + kTile - 1) / kTile;
+    return want < 1 ? 1 : want < tiles ? want : tiles < 1 ? 1 : tiles;
 }
 
 // K: the arrowhead the kernels solve; VK: the kind of the vector epilogue
@@ -182,7 +155,7 @@ static void launch_pipeline(int n, int grid, Scratch S, const SolveOpts &so,
     if (S.f.p) {
         const int diag = va.out.dg_b || va.out.dg_Kb || va.out.dg_flags;
         k_fopen<K><<<g32, 256, 0, st>>>(src, so);
-        k_feval<<<g8, 256, 0, st>>>(src);
+        k_feval<<<dim3(g8, segments(n, va.n1)), 256, 0, st>>>(src);
         k_fstep<K><<<gt, 64, 0, st>>>(src, so, diag);
         k_fmore<K><<<gm, 256, 0, st>>>(src, so, 0, diag);
         k_fold<K><<<grid, 256, 0, st>>>(src, so);
@@ -207,9 +180,11 @@ static void launch_pipeline(int n, int grid, Scratch S, const SolveOpts &so,
         k_fix_solve<K><<<fgrid, 256, 0, st>>>(S, so, n);
     }
     if (ro.ev[3]) cudaEventRecord(ro.ev[3], st);
-    k_place<<<(n + 255) / 256, 256, 0, st>>>(S);
-    if (S.f.p && va.out.V) k_fcols<VK><<<g8, 256, 0, st>>>(src);
-    k_vectors<VK><<<g8, 256, 0, st>>>(va, S);
+    k_fout<VK><<<gt, 64, 0, st>>>(src);
+    if (va.out.V) {
+        if (S.f.p) k_fcols<VK><<<dim3(g8, segments(n, va.n1)), 256, 0, st>>>(src);
+        k_vectors<VK><<<n < 4 * sms ? n : 4 * sms, 256, 0, st>>>(src);
+    }
 }
 
 // The pipeline for each kind other than the arrowhead, one translation unit

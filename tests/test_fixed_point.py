@@ -49,13 +49,13 @@ int main() {
         const double sc = std::ldexp(1.0, -(int)(g() % 40));
         const double p = U(g) * (it % 3 ? 1 : sc);
         double lh = U(g) * sc;
-        if (it % 5 == 0) lh = p * (1 + std::ldexp((double)(g() % 1000) - 500, -14));
+        if (it % 5 == 0) lh = p * (1 + std::ldexp((double)(g() % 1000) - 500, -14 - (int)(g() % 12)));
         const double ll = 0.999 * U(g) * std::ldexp(std::fabs(lh), -53);
         const double D = p - lh;
         const uint64_t b = f64_bits(D);
         const uint32_t dh = (uint32_t)(b >> 32), dl = (uint32_t)b, eb = (dh << 1) >> 21;
         const uint32_t el = (uint32_t)((f64_bits(lh) << 1) >> 53);
-        if (eb < kFixMinExp || eb + 6 < el) continue;
+        if (eb < kFixMinExp || eb + kTailSpan < el) continue;
         ++n;
         const uint64_t L = fix_mod(lh) + fix_mod(ll);
         const int tl = tail_of(fix_mod(p) - L, dh, dl, eb);
