@@ -6,124 +6,159 @@
 //   DPR1   M = diag(d) + rho u u^T, via A = L^{-1} M L        (Sec. 6.3)
 //   SVD    B = [diag(d) z; 0 alpha], via A = B^T B            (Sec. 6.2)
 //
-//   k_check      validity / ordering flags; transformed keys and spikes
-//   k_rank       stable descending order (ties: lower input row)   (Eq. order)
-//   k_reduce     zero spikes deflated, equal poles folded, reduced poles
-//                compacted (single CTA, block scans)               (Sec. 1)
-//   k_post<K>    kind-specific arrowhead data (DPR1: spikes and corner of
-//                L^{-1} M L; SVD: exact (d_j z_j)^2 and alpha^2 + z^T z), FP32 copies
-//   k_eig<P>     one warp per eigenpair: Algorithm 1 shift, Algorithm 2 inverse
-//                with b in double-double (Theorem 6), Algorithm 3 bisection
-//   k_fix_decide / k_fix_solve<P>
-//                Theorem C1 quotient > 3 -> Remark 1; K_nu (Eq. K0) above the
-//                threshold -> Remark 2(a) other pole or 2(b) DPR1 shift; DPR1:
-//                the last eigenvalue is re-solved next to the last pole
-//   k_place      output positions (merge with deflated values)
-//   k_vectors<K> one warp per column: v = x/||x|| (Eq. eigenvecAi / Algorithm 4),
-//                DPR1 q ~ (D - lambda)^{-1} u, SVD right and left vectors
+// Preparation (ae_prep.cuh): k_prep, or k_check, k_rank, k_order, k_heads,
+// k_reduce, k_kind, k_post, k_forms over the rows.  Eigenpairs, remedies and
+// columns: ae_fast.cuh, launched by ae_solve.cuh.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
 
 #include "ae_internal.h"
 #include "ae_pipeline.cuh"
+#include "ae_prep.cuh"
 #include "ae_solve.cuh"
 
 namespace ae {
 
 // ---------------------------------------------------------------------------
-// input checks, transformed keys/spikes, ordering
+// checks, order, reduction, forms: over the rows by a grid (ae_prep.cuh)
 // ---------------------------------------------------------------------------
-// ARROW: key d, spike z.  DPR1: key sgn d (sgn = sign of rho), spike u.
-// SVD: key d (> 0 required), spike d z.
-// HERM: spike |zeta_r| of the complex (z[2r], z[2r+1]).  NSYM: spike
-// sqrt(zc_r zr_r) of the pair (z[r], zrow[r]), which must share a sign or both
-// be zero (the Remark of Sec. 6.1).
-__global__ void k_check(Kind kind, int n1, const double *__restrict__ d,
-                        const double *__restrict__ z, const double *__restrict__ zrow,
-                        double sgn, Scratch S) {
+template <Kind K>
+__global__ void __launch_bounds__(256) k_check(PrepArgs A, Scratch S) {
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
     int flags = 0;
-    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n1; r += gridDim.x * blockDim.x) {
-        const double dr = d[r];
-        const double zr = kind == KIND_HERM ? z[2 * r] : z[r];
-        if (!isfinite(dr) || !isfinite(zr)) flags |= CF_BAD;
-        double key = dr, spk = zr;
-        if (kind == KIND_DPR1) {
-            key = sgn * dr;
-            S.key[r] = key;
-        } else if (kind == KIND_TSVD) {
-            if (!(dr > 0.0)) flags |= CF_BAD;
-            spk = dr * zr;
-            S.spk[r] = spk;
-        } else if (kind == KIND_HERM) {
-            const double zi = z[2 * r + 1];
-            if (!isfinite(zi)) flags |= CF_BAD;
-            spk = hypot(zr, zi);
-            S.spk[r] = spk;
-        } else if (kind == KIND_NSYM) {
-            const double zw = zrow[r];
-            if (!isfinite(zw)) flags |= CF_BAD;
-            if ((zr == 0.0) != (zw == 0.0) || (zr != 0.0 && (zr > 0.0) != (zw > 0.0)))
-                flags |= CF_BAD;
-            spk = sqrt(fabs(zr)) * sqrt(fabs(zw));
-            S.spk[r] = spk;
-        }
-        if (spk == 0.0) flags |= CF_ZERO;
-        if (key == 0.0) flags |= CF_ZEROPOLE;
-        if (r + 1 < n1) {
-            const double kn = kind == KIND_DPR1 ? sgn * d[r + 1] : d[r + 1];
-            if (!(key > kn)) flags |= CF_UNSORTED;
-        }
+    if (r < A.n1) {
+        flags = check_item<K>(A, S, r);
+        S.spos[r] = 0;                              // (k_rank counts there)
     }
     flags = __reduce_or_sync(FULL, flags);
     if ((threadIdx.x & 31) == 0 && flags) atomicOr(S.cnt + C_FLAGS, flags);
 }
 
-// perm[s] = input row at sorted position s (descending, ties by lower row)
-__global__ void k_rank(int n1, const double *__restrict__ key, const int *cnt, int *perm) {
-    __shared__ double tile[1024];
-    const bool sorted = !(cnt[C_FLAGS] & CF_UNSORTED);
+// Sorted input without zero spikes: reduced as it stands.  Else the rows' ranks
+// (descending, ties by lower row), each CTA counting 256 rows against one tile
+// of 1024 keys (blockIdx.y).
+__global__ void __launch_bounds__(256) k_rank(int n1, const double *__restrict__ key,
+                                              const double *__restrict__ spk, Scratch S) {
+    __shared__ unsigned long long tile[1024];
+    const int flags = S.cnt[C_FLAGS];
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (sorted) {
-        if (r < n1) perm[r] = r;
+    if (!(flags & CF_UNSORTED)) {
+        if (blockIdx.y) return;
+        if (flags & CF_ZERO) {
+            if (r < n1) S.spos[r] = r;
+            return;
+        }
+        if (r < n1) identity_row(S, key, spk, r);
+        if (r == 0) {
+            S.cnt[C_M] = n1;
+            S.cnt[C_ND] = 0;
+        }
         return;
     }
-    // NaN compares as -inf here so that ranks always form a permutation (the
-    // input is rejected later, but no index may leave its array meanwhile)
-    const double dr = r < n1 ? (isnan(key[r]) ? -INFINITY : key[r]) : 0.0;
+    const int base = blockIdx.y * 1024, lim = min(1024, n1 - base);
+    for (int t = threadIdx.x; t < lim; t += 256) tile[t] = order_key(key[base + t]);
+    __syncthreads();
+    if (r >= n1) return;
+    const unsigned long long kr = order_key(key[r]);
     int rank = 0;
-    for (int base = 0; base < n1; base += 1024) {
-        __syncthreads();
-        for (int t = threadIdx.x; t < 1024; t += blockDim.x) {
-            const double v = base + t < n1 ? key[base + t] : 0.0;
-            tile[t] = isnan(v) ? -INFINITY : v;
-        }
-        __syncthreads();
-        const int lim = min(1024, n1 - base);
-        if (r < n1) {
-            for (int t = 0; t < lim; ++t) {
-                const double dq = tile[t];
-                const int q = base + t;
-                rank += (dq > dr) || (dq == dr && q < r);
-            }
-        }
+#pragma unroll 4
+    for (int t = 0; t < lim; ++t) {
+        const unsigned long long q = tile[t];
+        rank += (q > kr) || (q == kr && base + t < r);
     }
-    if (r < n1) perm[rank] = r;
+    if (rank) atomicAdd(S.spos + r, rank);
 }
 
-// Reduction (single CTA of 1024 threads) and the kind-specific arrowhead data.
-__global__ void __launch_bounds__(1024) k_reduce(int n1, const double *__restrict__ key,
-                                                 const double *__restrict__ spk,
-                                                 const int *__restrict__ perm, Scratch S) {
-    reduce_block(n1, key, spk, perm, S);
+__global__ void __launch_bounds__(256) k_order(int n1, Scratch S) {
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r < n1 && (S.cnt[C_FLAGS] & (CF_UNSORTED | CF_ZERO))) S.perm[S.spos[r]] = r;
+}
+
+// heads of runs in each CTA's 256 sorted positions (counted in fixlist, which
+// nothing uses before the remedies)
+__global__ void __launch_bounds__(256) k_heads(int n1, const double *__restrict__ key,
+                                               const double *__restrict__ spk, Scratch S) {
+    if (!(S.cnt[C_FLAGS] & (CF_UNSORTED | CF_ZERO))) return;
+    const int s = blockIdx.x * 256 + threadIdx.x;
+    const bool head = s < n1 && is_head(key, spk, S.perm, s);
+    const int c = __syncthreads_count(head);
+    if (threadIdx.x == 0) S.fixlist[blockIdx.x] = c;
+}
+
+__global__ void __launch_bounds__(256) k_reduce(int n1, const double *__restrict__ key,
+                                                const double *__restrict__ spk, Scratch S) {
+    __shared__ int wh[8], before;
+    if (!(S.cnt[C_FLAGS] & (CF_UNSORTED | CF_ZERO))) return;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    // heads before this CTA's positions, then before this thread's
+    if (wid == 0) {
+        int c = 0;
+        for (int b = lane; b < (int)blockIdx.x; b += 32) c += S.fixlist[b];
+        c = __reduce_add_sync(FULL, c);
+        if (lane == 0) before = c;
+    }
+    const int s = blockIdx.x * 256 + threadIdx.x;
+    const bool in = s < n1, head = in && is_head(key, spk, S.perm, s);
+    const unsigned bal = __ballot_sync(FULL, head);
+    if (lane == 0) wh[wid] = __popc(bal);
+    __syncthreads();
+    int jk = before + __popc(bal & ((1u << lane) - 1u));
+    for (int w = 0; w < wid; ++w) jk += wh[w];
+    if (in) reduce_item(S, key, spk, n1, s, head, jk, s - jk);
+    if (s == n1 - 1) {
+        S.cnt[C_M] = jk + (head ? 1 : 0);
+        S.cnt[C_ND] = n1 - S.cnt[C_M];
+    }
 }
 
 template <Kind K>
-__global__ void __launch_bounds__(1024) k_post(int n1, const double *__restrict__ d,
-                                               const double *__restrict__ z,
-                                               const double *__restrict__ zrow, double alpha,
-                                               double rho_abs, Scratch S) {
-    post_block<K>(n1, d, z, zrow, alpha, rho_abs, S);
+__global__ void __launch_bounds__(kChunk) k_kind(PrepArgs A, Scratch S) {
+    __shared__ PoleShare sh[kChunk / 32];
+    kind_chunk<K>(A, S, S.cnt[C_M], blockIdx.x, threadIdx.x, sh, 0);
+}
+template <Kind K>
+__global__ void __launch_bounds__(32) k_post(PrepArgs A, Scratch S) {
+    prep_finish<K>(A, S, threadIdx.x);
+}
+template <Kind K>
+__global__ void __launch_bounds__(256) k_forms(Scratch S, VecArgs va) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < va.n1) forms_item<K>(S, va, t);
+}
+
+// all of it by one CTA
+template <Kind K>
+__global__ void __launch_bounds__(1024) k_prep(PrepArgs A, Scratch S, VecArgs va) {
+    prep_block<K>(A, S, va);
+}
+
+// Up to this many rows one CTA prepares an instance (one launch instead of ten
+// operations on the stream).  A whole solve, one CTA against the grid kernels:
+// n = 64 99 / 120 us, n = 400 115 / 135 (rows in no order: 175 / 184),
+// n = 1000 163 / 177 (226 / 204), n = 1500 222 / 231 (581 / 430).
+constexpr int kPrepRows = 640;
+
+template <Kind K>
+static cudaError_t launch_prep(const PrepArgs &A, const Scratch &S, const VecArgs &va,
+                               cudaStream_t st) {
+    if (A.n1 <= kPrepRows) {
+        k_prep<K><<<1, 1024, 0, st>>>(A, S, va);
+        return cudaSuccess;
+    }
+    cudaError_t e = cudaMemsetAsync(S.cnt, 0, sizeof(int) * C_COUNT, st);
+    if (!e) e = cudaMemsetAsync(S.cnt64, 0, sizeof(unsigned long long) * C64_COUNT, st);
+    if (e) return e;
+    const int n1 = A.n1, g = (n1 + 255) / 256;
+    k_check<K><<<g, 256, 0, st>>>(A, S);
+    k_rank<<<dim3(g, (n1 + 1023) / 1024), 256, 0, st>>>(n1, va.key, va.spk, S);
+    k_order<<<g, 256, 0, st>>>(n1, S);
+    k_heads<<<g, 256, 0, st>>>(n1, va.key, va.spk, S);
+    k_reduce<<<g, 256, 0, st>>>(n1, va.key, va.spk, S);
+    k_kind<K><<<g, kChunk, 0, st>>>(A, S);
+    k_post<K><<<1, 32, 0, st>>>(A, S);
+    k_forms<K><<<g, 256, 0, st>>>(S, va);
+    return cudaSuccess;
 }
 
 // One part of a split solve: its eigenpair range (an even split of the m + 1
@@ -336,47 +371,36 @@ cudaError_t launch_solve(Kind kind, int n, const double *d, const double *z, dou
     const bool rho0 = kind == KIND_DPR1 && rho == 0.0;   // M = D: every row deflates
     const bool own_spk = kind == KIND_TSVD || kind == KIND_HERM || kind == KIND_NSYM || rho0;
     const double *spk = own_spk ? S.spk : z;
-    cudaError_t e;
-    e = cudaMemsetAsync(S.cnt, 0, sizeof(int) * C_COUNT, st);
-    if (e) return e;
-    if (rho0 && n1 > 0) {
-        e = cudaMemsetAsync(S.spk, 0, sizeof(double) * n1, st);
-        if (e) return e;
-    }
-    e = cudaMemsetAsync(S.cnt64, 0, sizeof(unsigned long long) * C64_COUNT, st);
-    if (e) return e;
-    if (ro.ev[0]) cudaEventRecord(ro.ev[0], st);
-    if (n1 > 0) {
-        const int g = (n1 + 255) / 256;
-        k_check<<<g, 256, 0, st>>>(kind, n1, d, z, zrow, sgn, S);
-        k_rank<<<g, 256, 0, st>>>(n1, key, S.cnt, S.perm);
-    }
-    k_reduce<<<1, 1024, 0, st>>>(n1, key, spk, S.perm, S);
-    SolveOpts so{ro.max_iter, ro.precision, ro.finish, ro.bgate, ro.kb_max};
-    VecArgs va{n, n1, key, spk, z, zrow, kind == KIND_DPR1 ? rho : alpha, sgn, out};
+    if (ro.max_iter < kMinIterCap) S.f = FastPtrs{};
+    const SolveOpts so{ro.max_iter, ro.precision, ro.finish, ro.bgate, ro.kb_max};
+    const VecArgs va{n, n1, key, spk, z, zrow, kind == KIND_DPR1 ? rho : alpha, sgn, out};
+    const PrepArgs A{n1, d, z, zrow, alpha, rho, sgn};
     const int grid = eig_grid(n);
+    cudaError_t e = cudaSuccess;
+    if (ro.ev[0]) cudaEventRecord(ro.ev[0], st);
     switch (kind) {
         case KIND_ARROW:
-            k_post<KIND_ARROW><<<1, 1024, 0, st>>>(n1, d, z, zrow, alpha, 0.0, S);
-            launch_pipeline<KIND_ARROW, KIND_ARROW>(n, grid, S, so, ro, va, st);
+            e = launch_prep<KIND_ARROW>(A, S, va, st);
+            if (!e) launch_pipeline<KIND_ARROW, KIND_ARROW>(n, grid, S, so, ro, va, st);
             break;
         case KIND_DPR1:
-            k_post<KIND_DPR1><<<1, 1024, 0, st>>>(n1, d, z, zrow, alpha, fabs(rho), S);
-            launch_pipeline_dpr1(n, grid, S, so, ro, va, st);
+            e = launch_prep<KIND_DPR1>(A, S, va, st);
+            if (!e) launch_pipeline_dpr1(n, grid, S, so, ro, va, st);
             break;
         case KIND_TSVD:
-            k_post<KIND_TSVD><<<1, 1024, 0, st>>>(n1, d, z, zrow, alpha, 0.0, S);
-            launch_pipeline_tsvd(n, grid, S, so, ro, va, st);
+            e = launch_prep<KIND_TSVD>(A, S, va, st);
+            if (!e) launch_pipeline_tsvd(n, grid, S, so, ro, va, st);
             break;
         case KIND_HERM:
-            k_post<KIND_HERM><<<1, 1024, 0, st>>>(n1, d, z, zrow, alpha, 0.0, S);
-            launch_pipeline_herm(n, grid, S, so, ro, va, st);
+            e = launch_prep<KIND_HERM>(A, S, va, st);
+            if (!e) launch_pipeline_herm(n, grid, S, so, ro, va, st);
             break;
         case KIND_NSYM:
-            k_post<KIND_NSYM><<<1, 1024, 0, st>>>(n1, d, z, zrow, alpha, 0.0, S);
-            launch_pipeline_nsym(n, grid, S, so, ro, va, st);
+            e = launch_prep<KIND_NSYM>(A, S, va, st);
+            if (!e) launch_pipeline_nsym(n, grid, S, so, ro, va, st);
             break;
     }
+    if (e) return e;
     if (ro.ev[4]) cudaEventRecord(ro.ev[4], st);
     return cudaGetLastError();
 }
@@ -385,17 +409,12 @@ cudaError_t launch_arrow_part(int n, const double *d, const double *z, double al
                               int nparts, int cap, const Outputs &out, const RunOpts &ro,
                               Scratch S, cudaStream_t st, int *pos0, int *count) {
     const int n1 = n - 1;
-    cudaError_t e = cudaMemsetAsync(S.cnt, 0, sizeof(int) * C_COUNT, st);
-    if (!e) e = cudaMemsetAsync(S.cnt64, 0, sizeof(unsigned long long) * C64_COUNT, st);
-    if (e) return e;
+    if (ro.max_iter < kMinIterCap) S.f = FastPtrs{};
+    const VecArgs va{n, n1, d, z, z, nullptr, alpha, 1.0, out};
     if (ro.ev[0]) cudaEventRecord(ro.ev[0], st);
-    if (n1 > 0) {
-        const int g = (n1 + 255) / 256;
-        k_check<<<g, 256, 0, st>>>(KIND_ARROW, n1, d, z, nullptr, 1.0, S);
-        k_rank<<<g, 256, 0, st>>>(n1, d, S.cnt, S.perm);
-    }
-    k_reduce<<<1, 1024, 0, st>>>(n1, d, z, S.perm, S);
-    k_post<KIND_ARROW><<<1, 1024, 0, st>>>(n1, d, z, nullptr, alpha, 0.0, S);
+    cudaError_t e =
+        launch_prep<KIND_ARROW>(PrepArgs{n1, d, z, nullptr, alpha, 0.0, 1.0}, S, va, st);
+    if (e) return e;
     k_part<<<1, 32, 0, st>>>(S, part, nparts);
     int h[C_COUNT];
     e = cudaMemcpyAsync(h, S.cnt, sizeof(h), cudaMemcpyDeviceToHost, st);
@@ -405,7 +424,6 @@ cudaError_t launch_arrow_part(int n, const double *d, const double *z, double al
     *count = (h[C_K1] - h[C_K0]) + (h[C_U1] - h[C_U0]);
     if (!out.lambda || *count > cap) return cudaSuccess;   // size query, or no room
     const SolveOpts so{ro.max_iter, ro.precision, ro.finish, ro.bgate, ro.kb_max};
-    const VecArgs va{n, n1, d, z, z, nullptr, alpha, 1.0, out};
     launch_pipeline<KIND_ARROW, KIND_ARROW>(n, eig_grid(n), S, so, ro, va, st);
     if (ro.ev[4]) cudaEventRecord(ro.ev[4], st);
     return cudaGetLastError();

@@ -32,6 +32,7 @@
 
 #include "ae_fast.cuh"
 #include "ae_pipeline.cuh"
+#include "ae_prep.cuh"
 
 namespace ae {
 
@@ -149,59 +150,10 @@ struct SrcMany {
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(1024) k_batch_prep(const BatchInst *__restrict__ I,
                                                      BatchCtl *ctl) {
-    __shared__ double tile[1024];
-    __shared__ int sflags;
     const BatchInst &B = I[blockIdx.x];
-    const Scratch &S = B.S;
-    const int n1 = B.n1;
     if (blockIdx.x == 0 && threadIdx.x == 0) *ctl = BatchCtl{};
-    if (threadIdx.x < C_COUNT) S.cnt[threadIdx.x] = 0;
-    if (threadIdx.x < C64_COUNT) S.cnt64[threadIdx.x] = 0ull;
-    if (threadIdx.x == 0) sflags = 0;
-    __syncthreads();
-    int flags = 0;
-    for (int r = threadIdx.x; r < n1; r += blockDim.x) {
-        const double dr = B.d[r], zr = B.z[r];
-        if (!isfinite(dr) || !isfinite(zr)) flags |= CF_BAD;
-        if (zr == 0.0) flags |= CF_ZERO;
-        if (dr == 0.0) flags |= CF_ZEROPOLE;
-        if (r + 1 < n1 && !(dr > B.d[r + 1])) flags |= CF_UNSORTED;
-    }
-    flags = __reduce_or_sync(FULL, flags);
-    if ((threadIdx.x & 31) == 0 && flags) atomicOr(&sflags, flags);
-    __syncthreads();
-    flags = sflags;
-    if (threadIdx.x == 0) S.cnt[C_FLAGS] = flags;
-    // order: identity when sorted, else ranks counted against tiles of the poles
-    if (!(flags & CF_UNSORTED)) {
-        for (int r = threadIdx.x; r < n1; r += blockDim.x) S.perm[r] = r;
-    } else {
-        for (int rb = 0; rb < n1; rb += blockDim.x) {
-            const int r = rb + threadIdx.x;
-            const double dr = r < n1 ? (isnan(B.d[r]) ? -INFINITY : B.d[r]) : 0.0;
-            int rank = 0;
-            for (int base = 0; base < n1; base += 1024) {
-                __syncthreads();
-                const double v = base + (int)threadIdx.x < n1 ? B.d[base + threadIdx.x] : 0.0;
-                tile[threadIdx.x] = isnan(v) ? -INFINITY : v;
-                __syncthreads();
-                const int lim = min(1024, n1 - base);
-                if (r < n1)
-                    for (int t = 0; t < lim; ++t) {
-                        const double dq = tile[t];
-                        rank += (dq > dr) || (dq == dr && base + t < r);
-                    }
-            }
-            if (r < n1) S.perm[rank] = r;
-        }
-    }
-    __syncthreads();
-    reduce_block(n1, B.d, B.z, S.perm, S);
-    __syncthreads();
-    post_block<KIND_ARROW>(n1, B.d, B.z, nullptr, *B.alpha, 0.0, S);
-    __syncthreads();
-    if (S.f.p)
-        for (int t = threadIdx.x; t < n1; t += blockDim.x) fprep_item<KIND_ARROW>(S, B.va, t);
+    const PrepArgs A{B.n1, B.d, B.z, nullptr, *B.alpha, 0.0, 1.0};
+    prep_block<KIND_ARROW>(A, B.S, B.va);
 }
 
 // buf: this warp's 4 slices of stored (delta_j, c_j) pairs, `stride` apart

@@ -137,6 +137,14 @@ __device__ __forceinline__ int fast_scale(const Scratch &S) {
 __device__ __forceinline__ double pow2(int e) {          // 2^e, -1022 <= e <= 1023
     return __longlong_as_double((long long)(1023 + e) << 52);
 }
+__device__ __forceinline__ double pow2_or(int e) {       // any e
+    return e >= -1022 && e <= 1023 ? pow2(e) : ldexp(1.0, e);
+}
+// x 2^e for |e| <= 2000 (two products, where ldexp takes some twenty operations)
+__device__ __forceinline__ double scalb2(double x, int e) {
+    const int h = e >> 1;
+    return x * pow2(h) * pow2(e - h);
+}
 
 // ---------------------------------------------------------------------------
 // k_fprep
@@ -149,7 +157,7 @@ __device__ __forceinline__ dd fast_pole(double d, int es) {
         const dd q = two_prod(s, s);
         return dd{q.hi * 0.125, q.lo * 0.125};
     }
-    return dd{ldexp(d, es), 0.0};
+    return dd{d * pow2(es), 0.0};
 }
 
 // One thread per pole and row.  Whatever falls outside the ranges the fixed-
@@ -179,13 +187,13 @@ __device__ __forceinline__ void fprep_item(const Scratch &S, const VecArgs &va, 
         if (!bad) {
             const unsigned long long b = (unsigned long long)__double_as_longlong(z2);
             unsigned long long Z = ((b & 0xfffffffffffffull) | 0x10000000000000ull) << 11;
-            Z += (unsigned long long)__double2ll_rn(ldexp(zl, 63 - e));
+            Z += (unsigned long long)__double2ll_rn(zl * pow2(63 - e));
             if (!(Z >> 63)) Z = ~0ull;               // a low part that rounds below 2^63, or over
             S.f.z[t] = Z;
             // and in 128 bits
             const unsigned __int128 W =
                 ((unsigned __int128)((b & 0xfffffffffffffull) | 0x10000000000000ull) << 75) +
-                (unsigned __int128)((__int128)(long long)ldexp(zl, 115 - e) << 12);
+                (unsigned __int128)((__int128)(long long)(zl * pow2(115 - e)) << 12);
             S.f.zh[t] = (unsigned long long)(W >> 64);
             S.f.zl[t] = (unsigned long long)W;
             S.f.ez[t] = e + 2 * es;
@@ -196,7 +204,7 @@ __device__ __forceinline__ void fprep_item(const Scratch &S, const VecArgs &va, 
         S.f.rp[t] = p.hi;
         if (K == KIND_TSVD) S.f.rP[t] = fix_mod(p.hi) + fix_mod(p.lo);
     }
-    if (t == 0) bad |= !(fabs(ldexp(S.prm[P_ALPHA_HI], es)) < 0x1p300);
+    if (t == 0) bad |= !(fabs(S.prm[P_ALPHA_HI] * pow2(es)) < 0x1p300);
     if (bad) atomicOr(S.cnt + C_FLAGS, CF_NOFAST);
 }
 
@@ -261,7 +269,7 @@ template <Kind K>
 __device__ __forceinline__ dd fast_sigma(const Scratch &S, int k, int es) {
     const int i = S.es_pole[k];
     if (i >= 0) return dd{S.f.p[i], S.f.plo[i]};
-    return dd{ldexp(S.es_sigma[k], es), 0.0};
+    return dd{S.es_sigma[k] * pow2(es), 0.0};
 }
 
 // ---------------------------------------------------------------------------
@@ -549,7 +557,7 @@ __global__ void __launch_bounds__(256) k_fopen(const __grid_constant__ Src src, 
     S.es_iters[k] = 0;
     const int es = fast_scale<K>(S);
     const int eL = ilogb(Ld), ezs = ilogb(R.zs);
-    const double mu = ldexp((double)ul, es - eL);
+    const double mu = scalb2((double)ul, es - eL);
     if (gersh) {
         // steps of Algorithm 3 from its Gershgorin bracket (1/mu inside it) to
         // the width 2 eps |1/mu|; after an FP32 bracket, from that one's width
@@ -752,7 +760,7 @@ __device__ __forceinline__ dd sum2(unsigned long long a, unsigned long long l, i
     const double h = (double)a;
     const double r = (double)(long long)(a - (unsigned long long)h) + (double)l * 0x1p-32;
     const dd v = fast_two_sum(h, r);
-    const double u = ldexp(1.0, K2 - 60);
+    const double u = scalb2(1.0, K2 - 60);
     return dd{v.hi * u, v.lo * u};
 }
 
@@ -986,12 +994,12 @@ __global__ void __launch_bounds__(64) k_fstep(const __grid_constant__ Src src, S
         const int K3 = K2 - er, K4 = K3 - er, K5 = K4 - er;
         FastSums q;
         const dd v = dd_add(dd_of_ll(S.f.s1[k]), dd{(double)S.f.l1[k] * 0x1p-32, 0.0});
-        const double us = ldexp(1.0, K1 - 62);
+        const double us = scalb2(1.0, K1 - 62);
         q.M1 = dd{v.hi * us, v.lo * us};
         q.M2 = sum2(S.f.s2[k], S.f.l2[k], K2);
-        q.M3 = -ldexp((double)S.f.s3[k], K3 - 57);
-        q.M4 = ldexp((double)S.f.s4[k], K4 - 55);
-        q.M5 = -ldexp((double)S.f.s5[k], K5 - 53);
+        q.M3 = -scalb2((double)S.f.s3[k], K3 - 57);
+        q.M4 = scalb2((double)S.f.s4[k], K4 - 55);
+        q.M5 = -scalb2((double)S.f.s5[k], K5 - 53);
         const int st = fast_advance<K>(S, k, q, kErrTerm, -1.0);
         S.f.st[k] = st;
         if (st == FST_OLD) src.push_old(inst, k);
@@ -1192,14 +1200,14 @@ __global__ void __launch_bounds__(256) k_fmore(const __grid_constant__ Src src, 
                 const int K3 = K2 - er, K4 = K3 - er, K5 = K4 - er;
                 FastSums q;
                 const dd v = dd_of_i128(a1);
-                const double us = ldexp(1.0, K1 - 124);
+                const double us = scalb2(1.0, K1 - 124);
                 q.M1 = dd{v.hi * us, v.lo * us};
                 q.M2 = sum2(a2, l2, K2);
-                q.M3 = -ldexp((double)a3, K3 - 57);
-                q.M4 = ldexp((double)a4, K4 - 55);
-                q.M5 = -ldexp((double)a5, K5 - 53);
+                q.M3 = -scalb2((double)a3, K3 - 57);
+                q.M4 = scalb2((double)a4, K4 - 55);
+                q.M5 = -scalb2((double)a5, K5 - 53);
                 const double ct = dr.tails ? kErrTermWide : kErrTerm;
-                int v2 = fast_advance<K>(S, k, q, ct, dr.tails ? ldexp((double)a2u, K2 - 60) : 0.0);
+                int v2 = fast_advance<K>(S, k, q, ct, dr.tails ? scalb2((double)a2u, K2 - 60) : 0.0);
                 if (v2 == FST_MORE && round + 1 == kMoreRounds) v2 = FST_OLD;
                 if (phase == 0) {
                     if (v2 == FST_DONE) {
@@ -1383,7 +1391,7 @@ __device__ __forceinline__ dd dd_rsqrt(dd x) {
 __device__ __forceinline__ void scale_of(dd x, unsigned long long &m, int &e) {
     const Mant h = mant_of(x.hi);
     e = h.e - 1023;
-    m = h.m + (unsigned long long)__double2ll_rn(ldexp(x.lo, 63 - e));
+    m = h.m + (unsigned long long)__double2ll_rn(scalb2(x.lo, 63 - e));
     if (!(m >> 63)) m = h.m;                                   // (the low part crossed a power of 2)
 }
 
@@ -1592,12 +1600,6 @@ __global__ void __launch_bounds__(256) k_vectors(const __grid_constant__ Src src
                         src.scr(ik.x), va.out, ik.y, CtaTeam<8>{(int)threadIdx.x, red, 0});
         __syncthreads();
     }
-}
-
-template <Kind K>
-__global__ void __launch_bounds__(256) k_fprep(Scratch S, VecArgs va) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < va.n1) fprep_item<K>(S, va, t);
 }
 
 }  // namespace ae

@@ -42,239 +42,6 @@ __device__ __forceinline__ int block_exscan(int v, int *warp_tot, int &total) {
     return res;
 }
 
-// Reduction (single CTA of 1024 threads, loops over chunks of the sorted order).
-static __device__ void reduce_block(int n1, const double *__restrict__ key,
-                             const double *__restrict__ spk, const int *__restrict__ perm,
-                             const Scratch &S) {
-    __shared__ int wt[33];
-    int carry_keep = 0, carry_defl = 0;
-    for (int base = 0; base < n1; base += 1024) {
-        const int s = base + threadIdx.x;
-        int keep = 0, defl = 0;
-        int r = -1;
-        double dr = 0.0, zr = 0.0;
-        bool zero = false, head = false;
-        if (s < n1) {
-            r = perm[s];
-            dr = key[r];
-            zr = spk[r];
-            zero = (zr == 0.0);
-            if (!zero) {
-                head = true;   // the first nonzero row of its run of equal poles
-                for (int q = s - 1; q >= 0; --q) {
-                    const int rq = perm[q];
-                    if (key[rq] != dr) break;
-                    if (spk[rq] != 0.0) { head = false; break; }
-                }
-            }
-            keep = head ? 1 : 0;
-            defl = head ? 0 : 1;
-        }
-        int tk, td;
-        const int jk = block_exscan(keep, wt, tk) + carry_keep;
-        const int jd = block_exscan(defl, wt, td) + carry_defl;
-        if (s < n1) {
-            S.spos[r] = s;
-            if (head) {
-                // reduced spike: sqrt of the sum of squares over the run
-                double acc = fabs(zr);
-                for (int q = s + 1; q < n1; ++q) {
-                    const int rq = perm[q];
-                    if (key[rq] != dr) break;
-                    acc = hypot(acc, spk[rq]);
-                }
-                S.pd[jk] = dr;
-                S.pv[jk] = dr;
-                S.pz[jk] = acc;
-                const double a2 = acc * acc;
-                S.pz2[jk] = a2;
-                S.pz2lo[jk] = fma(acc, acc, -a2);
-                S.prow[jk] = r;
-                S.kind[r] = 0;
-            } else {
-                S.kind[r] = zero ? 1 : 2;
-                S.drow[jd] = r;
-                S.dval[jd] = dr;
-                if (!zero) {
-                    // Helmert-type vector data: R_{m-1} over earlier nonzero
-                    // members of the run, R_m including this row
-                    double Rm1 = 0.0;
-                    int q = s - 1;
-                    for (; q >= 0; --q) {
-                        const int rq = perm[q];
-                        if (key[rq] != dr) break;
-                        Rm1 = hypot(Rm1, spk[rq]);
-                    }
-                    S.run_s0[r] = q + 1;
-                    S.run_R[2 * r] = Rm1;
-                    S.run_R[2 * r + 1] = hypot(Rm1, zr);
-                }
-            }
-        }
-        carry_keep += tk;
-        carry_defl += td;
-    }
-    if (threadIdx.x == 0) {
-        S.cnt[C_M] = carry_keep;
-        S.cnt[C_ND] = carry_defl;
-    }
-}
-
-// block reductions for the single-CTA post kernel (blockDim = 1024)
-__device__ __forceinline__ double block_max(double v, double *sh) {
-    v = warp_max(v);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double r = sh[0];
-        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) r = fmax(r, sh[w]);
-        sh[0] = r;
-    }
-    __syncthreads();
-    return sh[0];
-}
-
-// (the warp partials are combined by thread 0 alone and broadcast: on the one
-// SM a single-CTA kernel runs on, every redundant FP64 instruction counts)
-__device__ __forceinline__ dd block_sum_dd(dd v, double *sh) {
-    v = warp_sum_dd(v);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) {
-        sh[threadIdx.x >> 5] = v.hi;
-        sh[32 + (threadIdx.x >> 5)] = v.lo;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        dd r = {sh[0], sh[32]};
-        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) r = dd_add(r, dd{sh[w], sh[32 + w]});
-        sh[0] = r.hi;
-        sh[32] = r.lo;
-    }
-    __syncthreads();
-    return dd{sh[0], sh[32]};
-}
-
-__device__ __forceinline__ double block_sum(double v, double *sh) {
-    v = warp_sum(v);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double r = sh[0];
-        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) r += sh[w];
-        sh[0] = r;
-    }
-    __syncthreads();
-    return sh[0];
-}
-
-// Kind-specific arrowhead data after the reduction, then the FP32 copies
-// (single CTA of 1024 threads).
-template <Kind K>
-__device__ void post_block(int n1, const double *__restrict__ d, const double *__restrict__ z,
-                           const double *__restrict__ zrow, double alpha, double rho_abs,
-                           const Scratch &S) {
-    __shared__ double sh[64];
-    int m = S.cnt[C_M];
-    dd al = {alpha, 0.0};
-    if (K == KIND_DPR1) {
-        // Sec. 6.3: the reduced DPR1 poles p_0 > ... > p_{m-1} with weights u'_j;
-        // the arrowhead L^{-1} M L has poles p_0..p_{m-2}, spikes
-        // zeta_j = u'_j sqrt(rho (p_j - p_{m-1})) and corner p_{m-1} + rho u'^T u'
-        // (after u <- sqrt(rho) u); zeta_j^2 and the corner in double-double.
-        dd uu = {0.0, 0.0};
-        for (int j = threadIdx.x; j < m; j += blockDim.x) uu = dd_add_same(uu, two_prod(S.pz[j], S.pz[j]));
-        uu = block_sum_dd(uu, sh);
-        const double plast = m > 0 ? S.pd[m - 1] : 0.0;
-        __syncthreads();
-        for (int j = threadIdx.x; j < m - 1; j += blockDim.x) {
-            const dd z2 = dd_mul(dd_mul_d(two_prod(S.pz[j], S.pz[j]), rho_abs),
-                                 two_sum(S.pd[j], -plast));
-            S.pz2[j] = z2.hi;
-            S.pz2lo[j] = z2.lo;
-            S.pz[j] = dd_sqrt(z2).hi;
-        }
-        al = dd_add(dd{plast, 0.0}, dd_mul_d(uu, rho_abs));
-        if (threadIdx.x == 0) {
-            S.prm[P_PLAST] = plast;
-            S.cnt[C_M] = m - 1;      // arrowhead poles; m - 1 = -1: nothing to solve
-        }
-        m = m - 1;
-    } else if (K == KIND_TSVD) {
-        // Sec. 6.2: B^T B has poles d_j^2, spikes d_j z_j, corner alpha^2 + z^T z
-        // (the corner over all rows; runs of equal d keep their folded spike).
-        dd zz = {0.0, 0.0};
-        for (int r = threadIdx.x; r < n1; r += blockDim.x) zz = dd_add_same(zz, two_prod(z[r], z[r]));
-        zz = block_sum_dd(zz, sh);
-        al = dd_add(two_prod(alpha, alpha), zz);
-        __syncthreads();
-        for (int j = threadIdx.x; j < m; j += blockDim.x) {
-            const double dj = S.pd[j];
-            S.pv[j] = dj * dj;
-            const int r = S.prow[j];
-            // a single-row pole: (d_j z_j)^2 exactly in double-double
-            const bool single = (j + 1 == m || S.pd[j + 1] != dj) &&
-                                S.pz[j] == fabs(S.spk[r]);
-            if (single) {
-                const dd dz = two_prod(dj, z[r]);
-                const dd z2 = dd_mul(dz, dz);
-                S.pz2[j] = z2.hi;
-                S.pz2lo[j] = z2.lo;
-            }
-        }
-        const int nd = S.cnt[C_ND];
-        for (int t = threadIdx.x; t < nd; t += blockDim.x) S.dval[t] = S.dval[t] * S.dval[t];
-    } else if (K == KIND_HERM || K == KIND_NSYM) {
-        // a single-row pole's spike^2 exactly in double-double: |zeta|^2 =
-        // re^2 + im^2 (Sec. 6.1), resp. zc zr (its Remark), as the paper asks
-        // for the moduli in doubled precision when b is computed so
-        for (int j = threadIdx.x; j < m; j += blockDim.x) {
-            const int r = S.prow[j];
-            if (S.pz[j] != S.spk[r]) continue;      // another row was folded in
-            const dd z2 = K == KIND_HERM
-                              ? dd_add(two_prod(z[2 * r], z[2 * r]),
-                                       two_prod(z[2 * r + 1], z[2 * r + 1]))
-                              : two_prod(z[r], zrow[r]);
-            S.pz2[j] = z2.hi;
-            S.pz2lo[j] = z2.lo;
-            S.pz[j] = dd_sqrt(z2).hi;
-        }
-    }
-    if (threadIdx.x == 0) {
-        S.prm[P_ALPHA_HI] = al.hi;
-        S.prm[P_ALPHA_LO] = al.lo;
-    }
-    // Algorithm 5's spike ratio needs sum_j |zeta_j| over the reduced poles
-    __syncthreads();
-    double zsum = 0.0;
-    for (int j = threadIdx.x; j < m; j += blockDim.x) zsum += S.pz[j];
-    zsum = block_sum(zsum, sh);
-    if (threadIdx.x == 0) S.prm[P_ZSUM] = zsum;
-    // FP32 copies: keys and spike^2 scaled by powers of two so that the
-    // largest of each is O(1)
-    double mxd = 0.0, mxz = 0.0;
-    for (int j = threadIdx.x; j < m; j += blockDim.x) {
-        mxd = fmax(mxd, fabs(S.pd[j]));
-        mxz = fmax(mxz, S.pz2[j]);
-    }
-    mxd = block_max(mxd, sh);
-    mxz = block_max(mxz, sh);
-    const double ds = (mxd > 0.0 && isfinite(mxd)) ? ldexp(1.0, -ilogb(mxd)) : 1.0;
-    const double zs = (mxz > 0.0 && isfinite(mxz)) ? ldexp(1.0, -ilogb(mxz)) : 1.0;
-    for (int j = threadIdx.x; j < m; j += blockDim.x) {
-        const double v = S.pd[j] * ds;
-        const float h = (float)v;
-        S.pdh[j] = h;
-        S.pdl[j] = (float)(v - (double)h);
-        S.pz2f[j] = (float)(S.pz2[j] * zs);
-    }
-    if (threadIdx.x == 0) {
-        S.prm[P_DS] = ds;
-        S.prm[P_ZS] = zs;
-    }
-}
-
 template <Kind K>
 struct PolesOf;
 template <>

@@ -148,9 +148,7 @@ static void launch_pipeline(int n, int grid, Scratch S, const SolveOpts &so,
                             const RunOpts &ro, const VecArgs &va, cudaStream_t st) {
     const int sms = sm_count();
     const int gt = (n + 63) / 64, gm = n < 2 * sms ? n : 2 * sms, g8 = (n + 7) / 8, g32 = (n + 31) / 32;
-    if (so.max_iter < kMinIterCap) S.f = FastPtrs{};
     const SrcOne src{S, va};
-    if (S.f.p && va.n1 > 0) k_fprep<VK><<<(va.n1 + 255) / 256, 256, 0, st>>>(S, va);
     if (ro.ev[1]) cudaEventRecord(ro.ev[1], st);
     if (S.f.p) {
         const int diag = va.out.dg_b || va.out.dg_Kb || va.out.dg_flags;
