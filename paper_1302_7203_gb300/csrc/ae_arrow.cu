@@ -286,6 +286,7 @@ static size_t fast_layout(uintptr_t base, int n, FastPtrs *F) {
     };
     using u64 = unsigned long long;
     FastPtrs T;
+    T.grp = (GroupData *)take(sizeof(GroupData) * (nn / kGroup + 2));
     T.p = (double *)take(8 * n1);
     T.plo = (double *)take(8 * n1);
     T.P = (u64 *)take(8 * n1);

@@ -383,7 +383,7 @@ static std::vector<long long> prefix_tables(int count, const int *ns, const int 
         e[i + 1] = e[i] + n;
         u[i + 1] = u[i] + (n + epw - 1) / epw;
         a[i + 1] = a[i] + (n + 7) / 8;
-        b[i + 1] = b[i] + (n + 31) / 32;
+        b[i + 1] = b[i] + (n + 31) / 32 + 1;          // (unit 0: the outermost two)
     }
     P.total_n = e[count];
     P.n8 = a[count];
@@ -404,6 +404,7 @@ static void enqueue(const Plan &P, cudaStream_t st) {
                       P.wbuf, 4 * P.wstride};
     k_batch_prep<<<P.count, 1024, 0, st>>>(P.d_inst, P.d_ctl);
     if (P.fast) {
+        if (P.wstride > kFarFrom) k_fgroup<KIND_ARROW><<<(unsigned)P.n32, 256, 0, st>>>(src);
         k_fopen<KIND_ARROW><<<(unsigned)P.n32, 256, 0, st>>>(src, P.so);
         k_feval<<<(unsigned)P.n8, 256, 0, st>>>(src);
         k_fstep<KIND_ARROW><<<g1, 64, 0, st>>>(src, P.so, 0);

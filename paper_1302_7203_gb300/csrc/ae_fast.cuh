@@ -11,6 +11,9 @@
 // the eigenpair takes the FP64 / double-double solver (k_fold, ae_solver.cuh).
 //
 //   k_fprep   poles, spikes and rows in scaled and fixed-point form
+//   k_fgroup  the poles far from 32 consecutive eigenvalues as 20 moments about
+//             their middle, in fixed point: O(n) work a group instead of an
+//             eigenpair
 //   k_fopen   FP32: midpoint test (Algorithm 1), K_b (Algorithm 5's gate
 //             counters), model steps to |error| < 2^-16 of the distance to the
 //             nearest pole; a warp holds 4 eigenpairs, so that a pole read
@@ -126,6 +129,10 @@ __device__ __forceinline__ void fast_range(const Scratch &S, int &lo, int &hi) {
         hi = S.cnt[C_KHI];
     }
 }
+
+// Groups of 32 eigenpairs start at multiples of 32 whatever a part's range, so
+// that a part forms the sums the whole solve forms.
+constexpr int kGroup = 32;
 
 // power of two that scales the poles below 1/2 (see k_fprep)
 template <Kind K>
@@ -272,6 +279,231 @@ __device__ __forceinline__ dd fast_sigma(const Scratch &S, int k, int es) {
     return dd{S.es_sigma[k] * pow2(es), 0.0};
 }
 
+__device__ __forceinline__ float sqrt_f32(float x) {
+    float r;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+__device__ __forceinline__ dd dd_of_ll(long long v) {
+    const double h = (double)v;
+    return fast_two_sum(h, (double)(v - (long long)h));
+}
+
+// ---------------------------------------------------------------------------
+// k_fgroup: far poles as moments
+// ---------------------------------------------------------------------------
+// For the eigenvalues of a group, all inside an interval with middle c and half
+// length r, a pole with |p - c| >= 8 r contributes
+//     zeta^2 / (p - lambda) = sum_q t^q zeta^2 / (p - c)^(q+1),   t = lambda - c,
+// with |t / (p - c)| <= 1/8: 20 terms leave 8^-20 = 2^-60 of it.  The moments
+// A_q = sum zeta^2 / (p - c)^(q+1) are summed in fixed point as k_feval's sums
+// are (order q needs 60 - 3 q bits: 62-bit products up to q = 9, 32-bit ones
+// beyond; the bits below the last place, whose loss is a bias of n / 2 last
+// places, up to q = 4), ~250 instructions a pole for 32 eigenpairs, where opening and
+// evaluating at each pole takes 32 x 250.  8 balances the two parts: the near
+// poles (~ 8 groups' worth, 256) and the moments (n / 32 a pair).
+// Stored per group: A_q 2^(q e) with 2^e <= 8 r, the first three as
+// double-doubles; the opening's FP32 copies; the indices [jlo, jhi) of the
+// poles left to the passes (all of them where fewer than kMinFar would go).
+// Bound by issue slots.  Graded n = 16384: 0.17 ms here; opening 0.72 -> 0.07,
+// k_feval 1.81 -> 0.08 ms.  DPR1 n = 8192: 0.05 here; 0.27 -> 0.04, 0.47 -> 0.03.
+// Fewer than kFarFrom poles form no groups, and their outermost eigenpairs are
+// opened by a warp like the others: one solve at n = 64 / 256 / 1000 takes 97 /
+// 109 / 179 us so, and 116 / 126 / 184 us with groups and an opening by CTA
+// (two latencies more); at 1500 it is 225 against 219, and a batch, bound by
+// issue slots, gains from about 700 on.
+constexpr int kMoments = 20, kMomWide = 10, kMom32 = 10, kMomLow = 5;
+constexpr int kMinFar = 256, kFarFrom = 768;
+
+struct GroupData {
+    double A[kMoments], Al[3];
+    double c;
+    float fa[kMom32];       // A_q 2^(q e) in the opening's units
+    float T, W;             // sum |zeta^2/(p-c)|, sum |zeta/(p-c)| in those units
+    float ku;               // t 2^-e = tau0 + u ku for an offset u in those units
+    int e, jlo, jhi;
+};
+
+// sum A_q tau^q and its derivative by u, in the opening's units
+__device__ __forceinline__ float far32(const GroupData &G, float tau, float &d) {
+    float v = 0.f, w = 0.f;
+#pragma unroll
+    for (int q = kMom32 - 1; q >= 0; --q) {
+        w = fmaf(w, tau, v);
+        v = fmaf(v, tau, G.fa[q]);
+    }
+    d = w * G.ku;
+    return v;
+}
+
+// |x| as a float from the high word of a double x with 2^-120 < |x| < 2
+__device__ __forceinline__ float f32_of_bits(unsigned h) {
+    return __uint_as_float(((h & 0x7fffffffu) - (896u << 20)) << 3);
+}
+
+template <Kind K, class Src>
+__global__ void __launch_bounds__(256, 2) k_fgroup(const __grid_constant__ Src src) {
+    __shared__ float rt[8], rw[8];
+    __shared__ int jb[2];
+    __shared__ unsigned long long acc[8][kMoments + kMomLow];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int inst, first;
+    if (!src.unit(blockIdx.x, kGroup, inst, first) || first == 0) return;
+    const Scratch &S = src.scr(inst);
+    const int m = S.cnt[C_M];
+    int klo, khi;
+    fast_range(S, klo, khi);
+    const int k0 = (klo & ~(kGroup - 1)) + first - kGroup;
+    if (k0 >= khi || (S.cnt[C_FLAGS] & CF_NOFAST) || m < kFarFrom) return;
+    GroupData &G = S.f.grp[k0 / kGroup];
+    // the group's interior eigenvalues lie between these poles (k0 = m: none)
+    const int ka = k0 > 1 ? k0 : 1, kb = min(k0 + kGroup - 1, m - 1);
+    const double top = S.f.p[min(ka - 1, m - 1)], bot = S.f.p[max(kb, 0)];
+    const double c = 0.5 * (top + bot), r = fmax(top - c, c - bot);
+    const int e = (int)bexp(8.0 * r) - 1023;
+    if (threadIdx.x < 2) {
+        // poles >= c + 8 r, poles > c - 8 r
+        const double x = threadIdx.x ? c - 8.0 * r : c + 8.0 * r;
+        int lo = 0, hi = m;
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            const double p = S.f.p[mid];
+            if (threadIdx.x ? p > x : p >= x) lo = mid + 1;
+            else hi = mid;
+        }
+        jb[threadIdx.x] = lo;
+    }
+    __syncthreads();
+    const int jlo = jb[0] & ~31, jhi = min((jb[1] + 31) & ~31, m);
+    if (kb < ka || !(r > 0.0) || e < -100 || m - (jhi - jlo) < kMinFar) {
+        if (threadIdx.x == 0) {
+            G.jlo = 0;
+            G.jhi = m;
+        }
+        return;
+    }
+    const double one = unit_reg();
+    // bound of the sums, and the Gershgorin share, in FP32
+    float T = 0.f, Wf = 0.f;
+    for (int j = threadIdx.x; j < m; j += 256) {
+        if (j >= jlo && j < jhi) continue;
+        const float q = rcp_f32(f32_of_bits(hi32(fma(S.f.p[j], one, -c))));
+        const float z = S.pz2f[j];
+        T = fmaf(z, q, T);
+        Wf = fmaf(sqrt_f32(z), q, Wf);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        T += __shfl_xor_sync(FULL, T, o);
+        Wf += __shfl_xor_sync(FULL, Wf, o);
+    }
+    if (lane == 0) {
+        rt[wid] = T;
+        rw[wid] = Wf;
+    }
+    __syncthreads();
+    T = rt[0];
+    Wf = rw[0];
+    for (int w = 1; w < 8; ++w) {
+        T += rt[w];
+        Wf += rw[w];
+    }
+    const int es = fast_scale<K>(S), ezs = ilogb(S.prm[P_ZS]);
+    const int eL = K == KIND_TSVD ? 2 * ilogb(S.prm[P_DS]) : ilogb(S.prm[P_DS]);
+    const int K0 = T > 0.f ? ilogbf(T * 1.02f) + 1 + 2 * es - ezs : 0;
+    const DiffRange dr = diff_range(c);
+    const unsigned long long L = fix_mod(c), L2 = fix_mod<kFixFrac2>(c);
+    const int c1 = K0 + 1 - 1023, cs = 1 - e - 1023;
+    unsigned long long a[kMoments], l[kMomLow];
+#pragma unroll
+    for (int q = 0; q < kMoments; ++q) a[q] = 0;
+#pragma unroll
+    for (int q = 0; q < kMomLow; ++q) l[q] = 0;
+    auto add = [&](int j) {
+        const double p = S.f.p[j];
+        double D = fma(p, one, -c);
+        int tl;
+        unsigned dh = hi32(D), dl = (unsigned)__double2loint(D);
+        unsigned eb = (dh << 1) >> 21;
+        if (eb - dr.lo >= dr.span) {
+            const dd Dd = near_diff(dd{p, S.f.plo[j]}, dd{c, 0.0}, dd{0.0, 0.0});
+            D = Dd.hi;
+            tl = near_tail(Dd);
+            dh = hi32(D);
+            dl = (unsigned)__double2loint(D);
+            eb = (dh << 1) >> 21;
+        } else if (eb < kFixMinExp && dr.tails) {
+            tl = tail_of<kFixFrac2>(S.f.P2[j] - L2, dh, dl, eb);
+        } else {
+            tl = tail_of(S.f.P[j] - L, dh, dl, eb) & dr.tails;
+        }
+        const unsigned seed = hi32(rcp_seed(__hiloint2double(
+            (int)((dh & 0xfffffu) | 0x3ff00000u), 0)));
+        // (2^64 / m, so that a product keeps its place: 2^63 of the term)
+        unsigned long long R = recip63<true>(dh, dl, tl, seed);
+        R = R >> 63 ? ~0ull : R + R;
+        unsigned long long q = mul_hi3(S.f.z[j], R);
+        unsigned s = (unsigned)(c1 + (int)eb - S.f.ez[j]);
+        a[0] += shr64(q, s);
+        l[0] += low32(q, s);
+#pragma unroll
+        for (int i = 1; i < kMoments; ++i) {
+            q = i < kMomWide ? mul_hi3(q, R)
+                             : (unsigned long long)(unsigned)(q >> 32) * (unsigned)(R >> 32);
+            s += eb + cs;
+            a[i] += shr64(q, s);
+            if (i < kMomLow) l[i] += low32(q, s);
+        }
+    };
+    for (int j = threadIdx.x; j < jlo; j += 256) add(j);
+    // (odd powers change sign below c)
+#pragma unroll
+    for (int q = 0; q < kMoments; q += 2) a[q] = 0ull - a[q];
+#pragma unroll
+    for (int q = 0; q < kMomLow; q += 2) l[q] = 0ull - l[q];
+    for (int j = jhi + threadIdx.x; j < m; j += 256) add(j);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+        for (int q = 0; q < kMoments; ++q) a[q] += __shfl_xor_sync(FULL, a[q], o);
+#pragma unroll
+        for (int q = 0; q < kMomLow; ++q) l[q] += __shfl_xor_sync(FULL, l[q], o);
+    }
+    if (lane == 0) {
+#pragma unroll
+        for (int q = 0; q < kMoments; ++q) acc[wid][q] = a[q];
+#pragma unroll
+        for (int q = 0; q < kMomLow; ++q) acc[wid][kMoments + q] = l[q];
+    }
+    __syncthreads();
+    if (threadIdx.x < kMoments) {
+        const int q = threadIdx.x;
+        unsigned long long v = 0, y = 0;
+        for (int w = 0; w < 8; ++w) {
+            v += acc[w][q];
+            if (q < kMomLow) y += acc[w][kMoments + q];
+        }
+        // A_q 2^(q e): the unit of order q is 2^(K0 - q e - (62 - q))
+        dd x = dd_of_ll((long long)v);
+        if (q < kMomLow) x = dd_add(x, dd{(double)(long long)y * 0x1p-32, 0.0});
+        const double u = scalb2(q & 1 ? 1.0 : -1.0, K0 - 62 + q);
+        G.A[q] = x.hi * u;
+        if (q < 3) G.Al[q] = x.lo * u;
+        if (q < kMom32) G.fa[q] = (float)scalb2(x.hi * u, ezs - eL - es);
+    }
+    if (threadIdx.x == 0) {
+        const float f = (float)pow2(es - eL) * (8.f / 7.f);
+        G.c = c;
+        G.T = T * f;
+        G.W = Wf * f;
+        G.ku = (float)pow2(es - eL - e);
+        G.e = e;
+        G.jlo = jlo;
+        G.jhi = jhi;
+    }
+}
+
 // ---------------------------------------------------------------------------
 // k_fopen
 // ---------------------------------------------------------------------------
@@ -304,12 +536,6 @@ __device__ __forceinline__ float reduce4max(const float (&v)[4], int lane) {
     return k;
 }
 
-__device__ __forceinline__ float sqrt_f32(float x) {
-    float r;
-    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-
 // Zero of the model Phi(mu) ~ A + B / (dn - mu) = w / mu fitted to (Phi, Phi')
 // at u, as |mu|: with e = |dn| the distance to the interval's other pole (0:
 // none, then Phi is linear), s the side, everything scaled by a power of two
@@ -337,29 +563,32 @@ __device__ __forceinline__ float model_root(float s, float Phi, float dPhi, floa
     return A >= 0.f ? __fdividef(2.f * w, A + rt) : __fdividef(rt - A, 2.f * B);
 }
 
-template <Kind K, class Src>
-__global__ void __launch_bounds__(256) k_fopen(const __grid_constant__ Src src, SolveOpts o) {
+// NW warps share 4 eigenpairs (kc: eigenpair of this lane group, or some valid
+// one where have is false), each over its share of the poles [jlo, jhi); G: the
+// far poles' moments, or null.  red: 4 NW floats.
+template <Kind K, int NW, class Src>
+__device__ __forceinline__ void open_items(const Src &src, int inst, const Scratch &S,
+                                           const SolveOpts &o, int kc, bool have, int jlo,
+                                           int jhi, const GroupData *G, float *red) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    int inst, first;
-    if (!src.unit(blockIdx.x, 32, inst, first)) return;
-    const Scratch &S = src.scr(inst);
-    const int m = S.cnt[C_M];
-    int klo, khi;
-    fast_range(S, klo, khi);
-    const int k0 = klo + first + 4 * wid;
-    if (k0 >= khi) return;
-    const int g = lane >> 3;                          // this lane group's eigenpair
-    const int k = k0 + g;
-    const bool have = k < khi;
-    if ((S.cnt[C_FLAGS] & CF_NOFAST) || m < 2) {
-        if (have && (lane & 7) == 0) {
-            S.f.st[k] = FST_OLD;
-            src.push_old(inst, k);
+    const int m = S.cnt[C_M], k = kc;
+    const int js = jlo + lane + (NW > 1 ? 32 * wid : 0);
+    constexpr int JS = 32 * NW;
+    // a lane group's sum (maximum) over the team, from its warp's
+    auto team = [&](float v, bool mx) {
+        if (NW == 1) return v;
+        __syncthreads();
+        if ((lane & 7) == 0) red[wid * 4 + (lane >> 3)] = v;
+        __syncthreads();
+        float r = red[lane >> 3];
+        for (int w = 1; w < NW; ++w) {
+            const float x = red[w * 4 + (lane >> 3)];
+            r = mx ? fmaxf(r, x) : r + x;
         }
-        return;
-    }
+        return r;
+    };
+    const int es = fast_scale<K>(S);
     const auto R = PolesOf<K>::make(S, m);
-    const int kc = have ? k : khi - 1;
     const bool lowx = kc == 0, upx = kc == m;         // outermost eigenvalues
     const double Ld = R.f32_scale();
     const double g1 = R.zs / Ld;                      // scales f to the FP32 sums
@@ -382,7 +611,7 @@ __global__ void __launch_bounds__(256) k_fopen(const __grid_constant__ Src src, 
             mfe[e] = __shfl_sync(FULL, mf, 8 * e);
             tf[e] = af[e] = bf[e] = df[e] = 0.f;
         }
-        for (int j = lane; j < m; j += 32) {
+        for (int j = js; j < jhi; j += JS) {
             const float z = R.z2f(j);
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
@@ -400,10 +629,21 @@ __global__ void __launch_bounds__(256) k_fopen(const __grid_constant__ Src src, 
 #pragma unroll
         for (int e = 0; e < 4; ++e)
             if (bad[e]) bf[e] = INFINITY;
-        tm = reduce4(tf, lane);
-        am = reduce4(af, lane);
-        bm = reduce4(bf, lane);
-        dm = reduce4(df, lane);
+        tm = team(reduce4(tf, lane), false);
+        am = team(reduce4(af, lane), false);
+        bm = team(reduce4(bf, lane), false);
+        dm = team(reduce4(df, lane), false);
+    }
+    // far poles: their sum at this lane group's pole + u
+    float tau0 = 0.f;
+    auto far = [&](float u, float &d) { return far32(*G, fmaf(u, G->ku, tau0), d); };
+    auto set_tau = [&](int i) { tau0 = (float)((S.f.p[i] - G->c) * pow2(-G->e)); };
+    if (G) {
+        set_tau(i);
+        float d;
+        tm += far(mf, d);
+        dm += d;
+        am += G->T;
     }
     bool ok = true, mid64 = false;
     int passes = 0;
@@ -428,6 +668,7 @@ __global__ void __launch_bounds__(256) k_fopen(const __grid_constant__ Src src, 
     // ---- the chosen pole: model steps ----
     const double sig = R.pole(i);
     R.f32_shift(sig, i, sh, sl);
+    if (G) set_tau(i);
     const int jn = side > 0 ? i - 1 : i + 1;          // the interval's other pole
     const float en = (jn >= 0 && jn < m) ? (float)(fabs(R.shifted(jn, sig, i)) * Ld) : 0.f;
     const double a64 = R.a_dd(sig, i).hi;
@@ -468,7 +709,7 @@ __global__ void __launch_bounds__(256) k_fopen(const __grid_constant__ Src src, 
                 sd[e] = __shfl_sync(FULL, s, 8 * e);
                 ws[e] = wx[e] = 0.f;
             }
-            for (int j = lane; j < m; j += 32) {
+            for (int j = js; j < jhi; j += JS) {
                 const float z = R.z2f(j), q = sqrt_f32(z);
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
@@ -483,10 +724,11 @@ __global__ void __launch_bounds__(256) k_fopen(const __grid_constant__ Src src, 
                     wx[e] = fmaxf(wx[e], fmaf(sd[e], r, aw));
                 }
             }
-            wsum = reduce4(ws, lane);
-            wmax = reduce4max(wx, lane);
+            wsum = team(reduce4(ws, lane), false);
+            wmax = team(reduce4max(wx, lane), true);
+            if (G) wsum = fmaf(G->W, iw, wsum);
         } else {
-            for (int j = lane; j < m; j += 32) {
+            for (int j = js; j < jhi; j += JS) {
                 const float z = R.z2f(j);
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
@@ -500,9 +742,15 @@ __global__ void __launch_bounds__(256) k_fopen(const __grid_constant__ Src src, 
                 }
             }
         }
-        const float t = reduce4(tf, lane);
-        const float a = reduce4(af, lane);
-        const float d = reduce4(df, lane);
+        float t = team(reduce4(tf, lane), false);
+        float a = team(reduce4(af, lane), false);
+        float d = team(reduce4(df, lane), false);
+        if (G) {
+            float fd;
+            t += far(u, fd);
+            d += fd;
+            a += G->T;
+        }
         if (!done) {
             ++passes;
             const float Phi = -Af + gam * u + t, dPhi = gam + d;
@@ -537,7 +785,7 @@ __global__ void __launch_bounds__(256) k_fopen(const __grid_constant__ Src src, 
         if (__all_sync(FULL, done || !ok)) break;
     }
     ok &= done && isfinite(ul) && ul != 0.f && isfinite(Tabs) && Tabs > 0.f && isfinite(dsum);
-    if (!have || (lane & 7) != 0) return;
+    if (!have || (lane & 7) != 0 || (NW > 1 && wid != 0)) return;
     int flags = 0;
     if (o.precision == 1) {
         atomicAdd(S.cnt64 + C64_F32, (unsigned long long)passes);
@@ -555,7 +803,6 @@ __global__ void __launch_bounds__(256) k_fopen(const __grid_constant__ Src src, 
     S.es_b[k] = (double)num / (double)w * R.f32_scale();
     S.es_Kb[k] = (double)bm;
     S.es_iters[k] = 0;
-    const int es = fast_scale<K>(S);
     const int eL = ilogb(Ld), ezs = ilogb(R.zs);
     const double mu = scalb2((double)ul, es - eL);
     if (gersh) {
@@ -585,19 +832,61 @@ __global__ void __launch_bounds__(256) k_fopen(const __grid_constant__ Src src, 
     S.f.s2[k] = S.f.s4[k] = 0;
     S.f.l1[k] = 0;
     S.f.l2[k] = 0;
-    S.f.st[k] = ok ? FST_EVAL : FST_OLD;
+    // (the outermost ones, which no group holds, are evaluated by k_fmore)
+    S.f.st[k] = !ok ? FST_OLD : NW > 1 ? FST_MORE : FST_EVAL;
     if (!ok) src.push_old(inst, k);
+    else if (NW > 1) src.push_more(0, inst, k);
+}
+
+template <Kind K, class Src>
+__global__ void __launch_bounds__(256) k_fopen(const __grid_constant__ Src src, SolveOpts o) {
+    __shared__ float red[32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int inst, first;
+    if (!src.unit(blockIdx.x, kGroup, inst, first)) return;
+    const Scratch &S = src.scr(inst);
+    const int m = S.cnt[C_M];
+    int klo, khi;
+    fast_range(S, klo, khi);
+    if ((S.cnt[C_FLAGS] & CF_NOFAST) || m < 2) {
+        const int k = (klo & ~(kGroup - 1)) + first - kGroup + lane;
+        if (first && wid == 0 && k >= klo && k < khi) {
+            S.f.st[k] = FST_OLD;
+            src.push_old(inst, k);
+        }
+        return;
+    }
+    const int g = lane >> 3;                          // this lane group's eigenpair
+    const bool groups = m >= kFarFrom;
+    if (first == 0) {
+        if (!groups) return;
+        // the instance's outermost eigenpairs: all poles, by the CTA
+        const int k = g == 0 ? 0 : m;
+        const bool have = g < 2 && k >= klo && k < khi;
+        if (__syncthreads_or(have))
+            open_items<K, 8>(src, inst, S, o, k, have, 0, m, nullptr, red);
+        return;
+    }
+    const int k0 = (klo & ~(kGroup - 1)) + first - kGroup, k = k0 + 4 * wid + g;
+    const int x = groups ? 1 : 0;                     // (unit 0 has the outermost ones)
+    const bool have = k >= klo && k < khi && k >= x && k <= m - x;
+    if (!__any_sync(FULL, have)) return;
+    const GroupData *G = groups ? S.f.grp + k0 / kGroup : nullptr;
+    const int jlo = groups ? G->jlo : 0, jhi = groups ? G->jhi : m;
+    open_items<K, 1>(src, inst, S, o, min(max(k, x), m - x), have, jlo, jhi,
+                     jhi - jlo < m ? G : nullptr, red);
 }
 
 // ---------------------------------------------------------------------------
 // k_feval
 // ---------------------------------------------------------------------------
 // Five sums over the poles at each eigenpair's point: zeta^2/(p - lambda)^r for
-// r = 1..5, a warp per eigenpair (and segment of the poles, blockIdx.y: the sums
-// are integers, so that segments add up in any order), the 8 warps of a CTA
-// sharing tiles of poles in shared memory.  Bound by issue slots: ~90 a term (FP64: one subtraction, 64
-// clocks of that pipe, behind them); the r = 4, 5 sums are skipped, warp by
-// warp, where no lane's term reaches 2^-44 of their bound.
+// r = 1..5, over the poles near its group, a warp per eigenpair (and segment of
+// the poles, blockIdx.y: the sums are integers, so that segments add up in any
+// order), the 8 warps of a CTA sharing tiles of poles in shared memory.  Bound
+// by issue slots: ~90 a term (FP64: one subtraction, 64 clocks of that pipe,
+// behind them); the r = 4, 5 sums are skipped, warp by warp, where no lane's
+// term reaches 2^-44 of their bound.
 constexpr int kTile = 256;
 
 template <class Src>
@@ -611,12 +900,18 @@ __global__ void __launch_bounds__(256, 3) k_feval(const __grid_constant__ Src sr
     const Scratch &S = src.scr(inst);
     int klo, khi;
     fast_range(S, klo, khi);
-    if (klo + first >= khi) return;
-    const int k = klo + first + wid;
-    const bool act = k < khi && S.f.st[k] == FST_EVAL;
+    const int kf = (klo & ~7) + first;               // (8 eigenpairs of one group)
+    if (kf >= khi) return;
+    const int k = kf + wid;
+    const bool act = k >= klo && k < khi && S.f.st[k] == FST_EVAL;
     if (!__syncthreads_or(act)) return;
-    const int m = S.cnt[C_M];
-    const int ka = act ? k : klo + first;
+    const int ka = act ? k : kf >= klo ? kf : klo;
+    int jlo = 0, m = S.cnt[C_M];                     // the near poles: [jlo, m)
+    if (m >= kFarFrom) {
+        const GroupData &G = S.f.grp[kf / kGroup];
+        jlo = G.jlo;
+        m = G.jhi;
+    }
     const double lhi = S.f.lhi[ka];
     const unsigned long long L = S.f.lmod[ka];
     const DiffRange dr = diff_range(lhi);
@@ -626,12 +921,12 @@ __global__ void __launch_bounds__(256, 3) k_feval(const __grid_constant__ Src sr
     unsigned long long a1 = 0, a2 = 0, a3 = 0, a4 = 0, a5 = 0;
     unsigned long long l1 = 0, l2 = 0;       // 32 bits below a1, a2 (summed apart)
     // this segment's poles: whole tiles
-    const int all_tiles = (m + kTile - 1) / kTile;
+    const int all_tiles = (m - jlo + kTile - 1) / kTile;
     const int t0 = (int)((long long)blockIdx.y * all_tiles / gridDim.y);
     const int tiles = (int)((long long)(blockIdx.y + 1) * all_tiles / gridDim.y);
-    bool flip = k >= t0 * kTile;
+    bool flip = k >= jlo + t0 * kTile;
     auto load = [&](int t, double &p, unsigned long long &P, unsigned long long &z, int &e) {
-        const int j = t * kTile + threadIdx.x;
+        const int j = jlo + t * kTile + threadIdx.x;
         p = 4.0; P = 0; z = 0; e = -8192;               // padding: terms of 0
         if (j < m) {
             p = S.f.p[j];
@@ -653,12 +948,12 @@ __global__ void __launch_bounds__(256, 3) k_feval(const __grid_constant__ Src sr
         __syncthreads();
         if (t + 1 < tiles) load(t + 1, lp, lP, lz, le);
         if (!act) continue;
-        const int left = m - t * kTile;
+        const int left = m - jlo - t * kTile;
         const int nc = left >= kTile ? kTile / 32 : (left + 31) / 32;
 #pragma unroll 1
         for (int c = 0; c < nc; ++c) {
             const int x = c * 32 + lane;
-            const int j0 = t * kTile + c * 32;
+            const int j0 = jlo + t * kTile + c * 32;
             double D = fma(tp[bsel][x], one, -lhi);    // (an FMA: 2.0 lanes a clock, DADD 1.7)
             int tl;
             unsigned dh = hi32(D), dl = (unsigned)__double2loint(D);
@@ -750,11 +1045,6 @@ __global__ void __launch_bounds__(256, 3) k_feval(const __grid_constant__ Src sr
 // ---------------------------------------------------------------------------
 // k_fstep
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ dd dd_of_ll(long long v) {
-    const double h = (double)v;
-    return fast_two_sum(h, (double)(v - (long long)h));
-}
-
 // M2 from its fixed-point sum and the 32 bits a term below
 __device__ __forceinline__ dd sum2(unsigned long long a, unsigned long long l, int K2) {
     const double h = (double)a;
@@ -792,6 +1082,32 @@ struct FastSums {
     dd M1, M2;
     double M3, M4, M5;
 };
+
+// The far poles' share at lambda = c + t: the moments' polynomial and its Taylor
+// coefficients (order 0 to more than double: the first three moments in
+// double-double, the rest weighs at most 8^-3).
+__device__ __forceinline__ void add_far(const GroupData &G, dd t, FastSums &s) {
+    const double sc = pow2(-G.e);
+    const dd x = {t.hi * sc, t.lo * sc};
+    double b0 = 0.0, b1 = 0.0, b2 = 0.0, b3 = 0.0, b4 = 0.0, p3 = 0.0;
+#pragma unroll
+    for (int q = kMoments - 1; q >= 0; --q) {
+        b4 = fma(b4, x.hi, b3);
+        b3 = fma(b3, x.hi, b2);
+        b2 = fma(b2, x.hi, b1);
+        b1 = fma(b1, x.hi, b0);
+        b0 = fma(b0, x.hi, G.A[q]);
+        if (q == 3) p3 = b0;
+    }
+    dd v = dd_add(dd{G.A[2], G.Al[2]}, two_prod(x.hi, p3));
+    v = dd_add(dd{G.A[1], G.Al[1]}, dd_mul(x, v));
+    v = dd_add(dd{G.A[0], G.Al[0]}, dd_mul(x, v));
+    s.M1 = dd_add(s.M1, dd_neg(v));
+    s.M2 = dd_add(s.M2, dd{b1 * sc, 0.0});
+    s.M3 += b2 * sc * sc;
+    s.M4 += b3 * sc * sc * sc;
+    s.M5 += (b4 * sc) * sc * (sc * sc);
+}
 
 // The zero from an evaluation, by one thread.  cterm: the weight of the terms'
 // error (kErrTerm...); M2u: the sum the unit's error counts over (negative:
@@ -1000,6 +1316,13 @@ __global__ void __launch_bounds__(64) k_fstep(const __grid_constant__ Src src, S
         q.M3 = -scalb2((double)S.f.s3[k], K3 - 57);
         q.M4 = scalb2((double)S.f.s4[k], K4 - 55);
         q.M5 = -scalb2((double)S.f.s5[k], K5 - 53);
+        const GroupData &G = S.f.grp[k / kGroup];
+        if (S.cnt[C_M] >= kFarFrom && G.jhi - G.jlo < S.cnt[C_M]) {
+            const int i = S.es_pole[k];
+            dd tt = dd_add(dd{S.f.p[i], S.f.plo[i]}, dd{-G.c, 0.0});
+            tt = dd_add(tt, dd{S.f.mu[k], S.f.mulo[k]});
+            add_far(G, tt, q);
+        }
         const int st = fast_advance<K>(S, k, q, kErrTerm, -1.0);
         S.f.st[k] = st;
         if (st == FST_OLD) src.push_old(inst, k);

@@ -69,7 +69,9 @@ enum {
 // a power of two, as doubles and modulo 2^64 in units of 2^-106; spikes^2 as
 // significand and exponent; per eigenpair the evaluation point, the bounds and
 // values of its sums, and its state.  p == null: the path is not used.
+struct GroupData;
 struct FastPtrs {
+    GroupData *grp;                       // far poles of each group of 32 eigenpairs
     double *p, *plo;                      // reduced poles (double-double)
     unsigned long long *P, *P2, *z, *zh, *zl;   // (P2: in units of 2^-140; zh, zl: 128 bits)
     int *ez;

@@ -152,8 +152,11 @@ static void launch_pipeline(int n, int grid, Scratch S, const SolveOpts &so,
     if (ro.ev[1]) cudaEventRecord(ro.ev[1], st);
     if (S.f.p) {
         const int diag = va.out.dg_b || va.out.dg_Kb || va.out.dg_flags;
-        k_fopen<K><<<g32, 256, 0, st>>>(src, so);
-        k_feval<<<dim3(g8, segments(n, va.n1)), 256, 0, st>>>(src);
+        // (one unit more for a part that starts inside a group, and unit 0)
+        if (va.n1 >= kFarFrom) k_fgroup<K><<<g32 + 2, 256, 0, st>>>(src);
+        k_fopen<K><<<g32 + 2, 256, 0, st>>>(src, so);
+        k_feval<<<dim3(g8 + 1, segments(n, va.n1 < 2 * kTile ? va.n1 : 2 * kTile)), 256, 0,
+                  st>>>(src);
         k_fstep<K><<<gt, 64, 0, st>>>(src, so, diag);
         k_fmore<K><<<gm, 256, 0, st>>>(src, so, 0, diag);
         k_fold<K><<<grid, 256, 0, st>>>(src, so);

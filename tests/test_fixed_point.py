@@ -7,7 +7,8 @@ product), seeds off by an ulp included.
 GPU: eigenpairs at the passes' edges -- tile and chunk boundaries, outermost
 eigenvalues far from all poles, poles in tight clusters, a DPR1 whose last pole
 lies far out, spectra that need the 128-bit evaluations, inputs whose exponents
-the passes refuse, an iteration cap that sends a solve to the FP64 kernels --
+the passes refuse, an iteration cap that sends a solve to the FP64 kernels, far poles taken
+as moments (768 poles and more, groups of 32 eigenpairs) --
 against the oracle at the suite's bar, 10 n eps64.
 """
 import os
@@ -203,3 +204,48 @@ def test_svd_edges(ae, n):
         assert_parity(r["s"].cpu().numpy(), r[key].cpu().numpy(),
                       {"lam": ref["s"], "abserr": np.zeros(n), "V": ref[key]}, n,
                       what=f"svd {n} {key}")
+
+
+def far_case(case):
+    rng = np.random.default_rng(6)
+    if case[1:].isdigit():
+        return W.uniform_arrow(int(case[1:]), seed=int(case[1:]))
+    if case == "graded":
+        return W.graded_arrow(900, seed=31)
+    if case == "gap":                    # a group straddles a gap: no pole is far from it
+        d = np.concatenate([rng.uniform(4, 5, 432), rng.uniform(-3, -2, 433)])
+    elif case == "clusters":             # one group's poles agree to 1e-10
+        c = np.linspace(-5, 5, 30) + rng.uniform(-0.1, 0.1, 30)
+        d = (c[:, None] * (1 + 1e-10 * np.arange(1, 33))).ravel()
+    else:                                # "zero": eigenvalues next to 0 and large spikes
+        d = np.concatenate([rng.uniform(-5, 5, 800), 10.0 ** rng.uniform(-9, -1, 100)])
+    d = np.sort(d)[::-1].copy()
+    z = 1.0 - rng.random(d.size)
+    return d, z * (100.0 if case == "zero" else 1.0), 0.5
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("form", sorted(FORMS))
+@pytest.mark.parametrize("case", ["n768", "n769", "n770", "n800", "n801", "n802", "n1025",
+                                  "graded", "gap", "clusters", "zero"])
+def test_far_poles_as_moments(ae, case, form):
+    d, z, a = far_case(case)
+    r = ae.arrow_eig(t(d), t(z), a, opts=ae.default_opts(**FORMS[form]), info=True)
+    assert_parity(r["lam"].cpu().numpy(), r["V"].cpu().numpy(), oracle.arrow_eig(d, z, a),
+                  len(d) + 1, what=f"far poles {case} {form}")
+
+
+@pytest.mark.gpu
+def test_far_poles_dpr1_and_svd(ae):
+    d, u, rho = W.uniform_dpr1(900, seed=5)
+    ref = oracle.dpr1_eig(d, u, rho)
+    r = ae.dpr1_eig(t(d), t(u), rho)
+    assert_parity(r["lam"].cpu().numpy(), r["Q"].cpu().numpy(),
+                  {"lam": ref["lam"], "abserr": np.zeros(900), "V": ref["Q"]}, 900, what="dpr1")
+    d, z, a = W.uniform_tsvd(900, seed=5)
+    ref = oracle.tsvd(d, z, a)
+    r = ae.tri_arrow_svd(t(d), t(z), a)
+    for key in ("V", "U"):
+        assert_parity(r["s"].cpu().numpy(), r[key].cpu().numpy(),
+                      {"lam": ref["s"], "abserr": np.zeros(900), "V": ref[key]}, 900,
+                      what=f"svd {key}")
