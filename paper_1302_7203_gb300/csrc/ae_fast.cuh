@@ -563,6 +563,23 @@ __device__ __forceinline__ float model_root(float s, float Phi, float dPhi, floa
     return A >= 0.f ? __fdividef(2.f * w, A + rt) : __fdividef(rt - A, 2.f * B);
 }
 
+// An outermost eigenvalue beyond its pole, |mu| = x: s Phi = -s Af + gam x - R
+// with the other poles' R (dR its slope) at offset x.  Own pole plus R's tangent,
+// and one pole c / (x + dl) fitted to the whole sum, both lie below the sum, so
+// that the larger zero is the better one; far from the pole the tangent alone
+// creeps (of 336 such eigenvalues, n = 5 to 3000, 2 to 32 steps; both: at most 7).
+__device__ __forceinline__ float model_root_outer(float A, float gam, float R, float dR, float x,
+                                                  float w) {
+    const float lin = model_root(1.f, A + gam * x - R, gam + dR, x, 0.f, w);
+    const float q = __fdividef(w, x), S = q + R, dS = __fdividef(q, x) + dR;
+    const float h = __fdividef(S, dS), dl = h - x, c = S * h;
+    const float b = fmaf(gam, dl, A), a = fmaf(-gam, dl, A);
+    const float rt = sqrt_f32(fmaf(4.f * gam, c, a * a));
+    const float m = b < 0.f ? __fdividef(rt - b, 2.f * gam)
+                            : __fdividef(2.f * (c - A * dl), b + rt);
+    return dS < 1e36f && m > lin && m < 1e36f ? m : lin;
+}
+
 // NW warps share 4 eigenpairs (kc: eigenpair of this lane group, or some valid
 // one where have is false), each over its share of the poles [jlo, jhi); G: the
 // far poles' moments, or null.  red: 4 NW floats.
@@ -690,7 +707,9 @@ __device__ __forceinline__ void open_items(const Src &src, int inst, const Scrat
     float u = 0.f, ul = 0.f, wsum = 0.f, wmax = 0.f, num = 0.f, Tabs = 0.f, dsum = 0.f;
     bool done = false;
     const bool gersh = o.finish == 0;
-    for (int it = 0; it < 9; ++it) {
+    // (3 to 5 passes nearly always; one eigenpair in some thousands takes over 9,
+    // and one that ran out of passes costs the FP64 solver's 220 us)
+    for (int it = 0; it < 24; ++it) {
         float she[4], sle[4], ue[4], wi[4], sd[4], ws[4], wx[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
@@ -762,8 +781,9 @@ __device__ __forceinline__ void open_items(const Src &src, int inst, const Scrat
                 const float r0 = model_root(s, Phi, dPhi, 0.f, en, w);
                 u = (!lowx && !upx) ? s * 0.5f * (r0 + rm) : s * r0;
             } else {
-                const float mn = model_root(s, Phi, dPhi, u, en, w);
                 const float mo = fabsf(u);
+                const float mn = lowx || upx ? model_root_outer(-s * Af, gam, -s * t, d, mo, w)
+                                             : model_root(s, Phi, dPhi, u, en, w);
                 const float rho = en > 0.f ? fminf(mn, en - mn) : mn;
                 if (!(mn > 0.f) || (en > 0.f && !(mn < en))) { ok = false; done = true; }
                 else if (fabsf(mn - mo) <= 0x1p-8f * rho) {

@@ -154,7 +154,7 @@ def t(x):
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("form", sorted(FORMS))
-@pytest.mark.parametrize("case", ["n3", "n32", "n33", "n34", "n256", "n257", "n258", "n514",
+@pytest.mark.parametrize("case", ["n3", "n32", "n33", "n34", "n256", "n257", "n258", "n514", "n700",
                                   "far_corner", "long_spikes", "clusters", "zero_pole",
                                   "near_zero", "tiny_spikes", "cancelling", "huge", "small"])
 def test_edges_of_the_passes(ae, case, form):
