@@ -423,7 +423,7 @@ static void enqueue(const Plan &P, cudaStream_t st) {
     }
     k_fout<KIND_ARROW><<<g1, 64, 0, st>>>(src);
     if (P.vectors) {
-        if (P.fast) k_fcols<KIND_ARROW><<<(unsigned)P.n8, 256, 0, st>>>(src);
+        if (P.fast) k_fcols<KIND_ARROW><<<(unsigned)P.n32, 256, 0, st>>>(src);
         k_vectors<KIND_ARROW><<<gm, 256, 0, st>>>(src);
     }
     if (P.status) k_batch_status<<<(P.count + 255) / 256, 256, 0, st>>>(P.d_inst, P.count, P.status);

@@ -33,6 +33,8 @@
 //   k_fcols   columns: one difference, one reciprocal and two products a
 //             component, normalised in the same step and written once
 #pragma once
+#include <type_traits>
+
 #include "ae_fixed.cuh"
 #include "ae_pipeline.cuh"
 
@@ -318,7 +320,7 @@ constexpr int kMinFar = 256, kFarFrom = 768;
 
 struct GroupData {
     double A[kMoments], Al[3];
-    double c;
+    double c, r8;           // the middle, and 8 r (infinite: no interval)
     float fa[kMom32];       // A_q 2^(q e) in the opening's units
     float T, W;             // sum |zeta^2/(p-c)|, sum |zeta/(p-c)| in those units
     float ku;               // t 2^-e = tau0 + u ku for an offset u in those units
@@ -376,7 +378,13 @@ __global__ void __launch_bounds__(256, 2) k_fgroup(const __grid_constant__ Src s
     }
     __syncthreads();
     const int jlo = jb[0] & ~31, jhi = min((jb[1] + 31) & ~31, m);
-    if (kb < ka || !(r > 0.0) || e < -100 || m - (jhi - jlo) < kMinFar) {
+    const bool none = kb < ka || !(r > 0.0) || e < -100;
+    if (threadIdx.x == 0) {
+        G.c = c;
+        G.e = e;
+        G.r8 = none ? INFINITY : 8.0 * r;
+    }
+    if (none || m - (jhi - jlo) < kMinFar) {
         if (threadIdx.x == 0) {
             G.jlo = 0;
             G.jhi = m;
@@ -494,11 +502,9 @@ __global__ void __launch_bounds__(256, 2) k_fgroup(const __grid_constant__ Src s
     }
     if (threadIdx.x == 0) {
         const float f = (float)pow2(es - eL) * (8.f / 7.f);
-        G.c = c;
         G.T = T * f;
         G.W = Wf * f;
         G.ku = (float)pow2(es - eL - e);
-        G.e = e;
         G.jlo = jlo;
         G.jhi = jhi;
     }
@@ -1681,7 +1687,7 @@ __global__ void __launch_bounds__(64) k_ffix(const __grid_constant__ Src src) {
 // k_fcols
 // ---------------------------------------------------------------------------
 // significand (64 bits, top bit set), biased exponent and sign of a double;
-// a zero has significand 0
+// a zero has significand 0 and an exponent below all others
 struct Mant {
     unsigned long long m;
     int e;                // bit 31: the sign, low bits: the biased exponent
@@ -1697,25 +1703,27 @@ __device__ __forceinline__ Mant mant_of(double x) {
     }
     Mant r;
     r.m = e ? ((b & 0xfffffffffffffull) | 0x10000000000000ull) << 11 : 0ull;
-    r.e = (int)(((unsigned)(e - off) & 0xffffu) | sg);
+    r.e = (int)(((unsigned)(e ? e - off : -8192) & 0xffffu) | sg);
     return r;
 }
 
-// a G / 2^61 2^(be - 1023) rounded to double, G in (2^61, 2^63], a's
-// significand in [2^63, 2^64); sgn: the sign bit
+// a G / 2^61 2^(be - 1023) rounded to double, a G / 2^64 in (2^58, 2^63), a's
+// significand in [2^63, 2^64) or 0 with be < -1000; sgn: the sign bit.  CHECK:
+// the result may lie outside the normal range.
+template <bool CHECK>
 __device__ __forceinline__ double pack_prod(unsigned long long a, unsigned long long G, int be,
                                             unsigned sgn) {
     const unsigned long long H0 = mul_hi3(a, G);
     const unsigned h = (unsigned)(H0 >> 32);
-    const int lz = __clz(h);                            // 1..3
+    const int lz = __clz(h);                            // 1..5
     const unsigned long long H = (H0 << (lz - 1)) + 0x200ull;
-    const int e = be + 2 - lz;
+    const int e1 = be + 1 - lz;                         // exponent - 1
     const unsigned lo = (unsigned)(H >> 10);
-    unsigned hi = (unsigned)(H >> 42) + ((unsigned)(e - 1) << 20);
-    if (a == 0) return __hiloint2double((int)sgn, 0);
-    if ((unsigned)(e - 1) >= 2045u) {
+    const unsigned hi = (unsigned)(H >> 42) + ((unsigned)e1 << 20);
+    if (CHECK && (unsigned)e1 >= 2045u) {
+        if (a == 0) return __hiloint2double((int)sgn, 0);
         // below the normal range (or above it): in FP64
-        const double v = ldexp((double)(H >> 10), e - 1075);
+        const double v = ldexp((double)(H >> 10), e1 - 1074);
         return sgn ? -v : v;
     }
     return __hiloint2double((int)(hi | sgn), (int)lo);
@@ -1774,66 +1782,135 @@ __global__ void __launch_bounds__(64) k_fout(const __grid_constant__ Src src) {
     // scaled multipliers: spikes and poles both scale by 2^es (DPR1: see nrm)
     const dd inv = dd_rsqrt(nrm);
     scale_of(inv, S.f.cm[k], S.f.ce[k]);
-    if (VK != KIND_DPR1) S.f.ce[k] += es;
+    if (VK != KIND_DPR1) {
+        S.f.ce[k] += es;
+        // the last component
+        const int pos = out_pos<VK>(S, va.n, va.sgn, k);
+        double *col = va.out.V + (size_t)pos * va.out.ldv;
+        double *ucol = va.out.U ? va.out.U + (size_t)pos * va.out.ldu : nullptr;
+        const double vn = -inv.hi;
+        if (VK == KIND_HERM) {
+            col[2 * va.n1] = vn;
+            col[2 * va.n1 + 1] = 0.0;
+        } else {
+            col[va.n1] = vn;
+            if (VK == KIND_TSVD && ucol) ucol[va.n1] = va.alpha * vn / sv_of(S, k);
+            if (VK == KIND_NSYM && ucol) ucol[va.n1] = vn;
+        }
+    }
     if (VK == KIND_TSVD) {
         scale_of(dd_mul_d(inv, sv_of(S, k)), S.f.cm2[k], S.f.ce2[k]);
         S.f.ce2[k] += es;
     }
     // lambda's own tail, as an integer of 2^-30 last places of lambda
     const double lhi = S.f.lhi[k];
+    if (S.cnt[C_M] >= kFarFrom) {
+        // its offset from the group's middle, in 2^(e - 64) (s1 is free by now)
+        const GroupData &G = S.f.grp[k / kGroup];
+        if (G.r8 < 1e300) {
+            const dd x = two_sum(lhi, -G.c);
+            const double u = pow2(64 - G.e);
+            S.f.s1[k] = __double2ll_rn(x.hi * u) + __double2ll_rn((x.lo + S.f.llo[k]) * u);
+        }
+    }
     S.f.l32[k] = fabs(lhi) < 2.5
                      ? (int)rint(S.f.llo[k] * pow2(min(1075 - (int)bexp(lhi) + 30, 1023)))
                      : 0;
 }
 
-// Columns of the eigenpairs the fast path solved, a warp each; the CTA's 8
-// warps share tiles of input rows, blockIdx.y is the segment of rows.
+// Columns of the eigenpairs the fast path solved: a CTA has a group of 32 of
+// them and a segment of the rows (blockIdx.y), a warp 32 rows at a time, a lane
+// one row for all columns (few rows: the warps share the columns out).
 // Component a_r / ((d_r - sigma) - mu) / ||x||, for the second matrix (SVD: U,
-// NSYM: Y) or the imaginary part (HERM) with its own multiplier.  The difference
-// is fl(d_r - lambda) with lambda's tail taken into its reciprocal (SVD, whose
-// poles d^2 are no doubles: the exact tail): a component's error is that of
-// one subtraction and one rounding.
+// NSYM: Y) or the imaginary part (HERM) with its own multiplier.
+// Rows whose poles are far from the group's middle c (|p - c| >= 8 r, a warp's 32
+// rows all): the significand of p - c, formed once a row, less lambda - c shifted
+// to its place is the difference to 2^-62 with no FP64 operation, and its
+// reciprocal starts from an FP32 one: ~70 instructions an entry.  Other rows: the
+// difference is fl(d_r - lambda) with lambda's tail taken into its reciprocal
+// (SVD, whose poles d^2 are no doubles: the exact tail), ~115 an entry.  Either
+// way a component's error is that of one subtraction and one rounding.
+// Bound by issue slots and the wide multiplies' pipe (59 % and 53 % busy).  All
+// entries by ~115 instructions -> now: DPR1 n = 8192 331 -> 214 us, graded n =
+// 16384 1223 -> 787 us (2.7 TB/s written), a batch of 512 4.1 -> 2.6 ms.
+// rows a CTA takes at least: few rows are split further, for latency
+__host__ __device__ constexpr int col_rows(int n1) { return n1 < kFarFrom ? 32 : 128; }
+
 template <Kind VK, class Src>
 __global__ void __launch_bounds__(256, 3) k_fcols(const __grid_constant__ Src src) {
     constexpr bool CPLX = VK == KIND_HERM;
     constexpr bool TWO = VK == KIND_HERM || VK == KIND_NSYM || VK == KIND_TSVD;
     constexpr bool SVD = VK == KIND_TSVD;
-    __shared__ double tp[2][kTile];
-    __shared__ unsigned long long ta[2][kTile], tb[2][TWO ? kTile : 1], tP[2][SVD ? kTile : 1];
-    __shared__ int ea[2][kTile], eb2[2][TWO ? kTile : 1];
+    __shared__ ulonglong2 sA[2][kGroup];       // +-(lambda - c), scale
+    struct alignas(16) Out { double *v; int e, pad; };
+    __shared__ Out so[kGroup];                 // column, scale's exponent
+    __shared__ double *su[TWO && !CPLX ? kGroup : 1];
+    __shared__ double sl[kGroup];
+    __shared__ int4 sd[kGroup];                // diff_range, l32
+    __shared__ int se2[SVD ? kGroup : 1];
+    __shared__ unsigned long long sm2[SVD ? kGroup : 1], sL[SVD ? kGroup : 1];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     int inst, first;
-    if (!src.unit(blockIdx.x, 8, inst, first)) return;
+    if (!src.unit(blockIdx.x, kGroup, inst, first)) return;
     const Scratch &S = src.scr(inst);
     const VecArgs &va = src.vec(inst);
     const PartRange P = part_range(S);
-    if (!va.out.V || P.k0 + first >= P.k1) return;
-    const int k = P.k0 + first + wid;
-    const bool act = k < P.k1 && S.f.st[k] == FST_DONE;
-    if (!__syncthreads_or(act)) return;
-    const int ka = act ? k : P.k0 + first;
-    const int n1 = va.n1;
-    const double lhi = S.f.lhi[ka];
-    DiffRange dr = diff_range(lhi);
-    if (!SVD) dr = {dr.lo0, 4096u, dr.lo0, dr.tails};  // (no unit to mind)
-    const int l32 = S.f.l32[ka], el = (int)bexp(lhi) - 23;
-    const unsigned long long L = SVD ? S.f.lmod[ka] : 0ull;
-    const double one = unit_reg();
-    const unsigned long long mi = S.f.cm[ka], mi2 = SVD ? S.f.cm2[ka] : 0ull;
-    const int ei = S.f.ce[ka] + 1023, ei2 = SVD ? S.f.ce2[ka] + 1023 : ei;
-    const int pos = out_pos<VK>(S, va.n, va.sgn, ka);
+    const int kf = (P.k0 & ~(kGroup - 1)) + first;
+    if (!va.out.V || kf >= P.k1) return;
+    // every warp looks at the columns, the first prepares them
+    const int kl = kf + lane;
+    const bool act = kl >= P.k0 && kl < P.k1 && S.f.st[kl] == FST_DONE;
+    const unsigned cols = __ballot_sync(FULL, act);
+    if (!cols) return;
+    const int n1 = va.n1, m = S.cnt[C_M], es = fast_scale<VK>(S);
+    const GroupData &G = S.f.grp[kf / kGroup];
+    const bool groups = m >= kFarFrom && G.r8 < 1e300;
+    // (the outermost eigenvalues are in no group)
+    const unsigned fcol = __ballot_sync(FULL, groups && act && kl > 0 && kl < m);
+    if (wid == 0 && act) {
+        const int k = kl;
+        const double lhi = S.f.lhi[k];
+        DiffRange dr = diff_range(lhi);
+        if (!SVD) dr = {dr.lo0, 4096u, dr.lo0, dr.tails};  // (no unit to mind)
+        sl[lane] = lhi;
+        sd[lane] = make_int4((int)dr.lo, (int)dr.span, dr.tails, S.f.l32[k]);
+        const unsigned long long t = groups ? (unsigned long long)S.f.s1[k] : 0ull;
+        sA[0][lane] = make_ulonglong2(t, S.f.cm[k]);
+        sA[1][lane] = make_ulonglong2(0ull - t, S.f.cm[k]);
+        if (SVD) {
+            sL[lane] = S.f.lmod[k];
+            sm2[lane] = S.f.cm2[k];
+            se2[lane] = S.f.ce2[k] + 1023;
+        }
+        const int pos = out_pos<VK>(S, va.n, va.sgn, k);
+        double *col = va.out.V + (size_t)pos * va.out.ldv;
+        double *ucol = (TWO && !CPLX && va.out.U) ? va.out.U + (size_t)pos * va.out.ldu : nullptr;
+        so[lane] = Out{col, S.f.ce[k] + 1023, 0};
+        if (TWO && !CPLX) su[lane] = ucol;
+    }
+    // the range of the scales' exponents
+    const int ce = act ? S.f.ce[kl] + 1023 : 1023, ce2 = SVD && act ? S.f.ce2[kl] + 1023 : ce;
+    const int emin = __reduce_min_sync(FULL, min(ce, ce2)), emax = __reduce_max_sync(FULL, max(ce, ce2));
+    __syncthreads();
     const unsigned vsg = (VK == KIND_DPR1 && va.sgn < 0.0) ? 0x80000000u : 0u;
-    double *col = va.out.V + (size_t)pos * va.out.ldv;
-    double *ucol = (TWO && !CPLX && va.out.U) ? va.out.U + (size_t)pos * va.out.ldu : nullptr;
-    double lp;
-    unsigned long long lP = 0;
-    Mant la, lb;
-    auto load = [&](int t) {
-        const int r = t * kTile + threadIdx.x;
-        lp = 4.0; la = lb = Mant{0, 0};
-        if (r < n1) {
-            lp = S.f.rp[r];
-            if (SVD) lP = S.f.rP[r];
+    const double one = unit_reg();
+    // this segment's rows, whole tiles
+    const int tile = col_rows(n1), all_tiles = (n1 + tile - 1) / tile;
+    const int r0 = (int)((long long)blockIdx.y * all_tiles / gridDim.y) * tile;
+    const int r1 = min((int)((long long)(blockIdx.y + 1) * all_tiles / gridDim.y) * tile, n1);
+    const int nch = (r1 - r0 + 31) / 32;
+    const int parts = nch >= 5 ? 1 : nch >= 3 ? 2 : nch == 2 ? 4 : 8;
+    const int per = kGroup / parts, x0 = (wid % parts) * per;
+    const unsigned mine = (per == 32 ? ~0u : ((1u << per) - 1u) << x0) & cols;
+    for (int ch = wid / parts; ch < nch; ch += 8 / parts) {
+        const int r = r0 + ch * 32 + lane;
+        const bool in = r < r1;
+        double p = 4.0;
+        unsigned long long rP = 0;
+        Mant la = {0, -8192}, lb = {0, -8192};
+        if (in) {
+            p = S.f.rp[r];
+            if (SVD) rP = S.f.rP[r];
             if (CPLX) {
                 la = mant_of(va.z[2 * r]);
                 lb = mant_of(va.z[2 * r + 1]);
@@ -1847,39 +1924,82 @@ __global__ void __launch_bounds__(256, 3) k_fcols(const __grid_constant__ Src sr
                 la = mant_of(va.spk[r]);
             }
         }
-    };
-    const int all_tiles = (n1 + kTile - 1) / kTile;
-    const int t0 = (int)((long long)blockIdx.y * all_tiles / gridDim.y);
-    const int tiles = (int)((long long)(blockIdx.y + 1) * all_tiles / gridDim.y);
-    load(t0);
-    for (int t = t0; t < tiles; ++t) {
-        const int b = t & 1;
-        tp[b][threadIdx.x] = lp;
-        ta[b][threadIdx.x] = la.m;
-        ea[b][threadIdx.x] = la.e;
-        if (SVD) tP[b][threadIdx.x] = lP;
-        if (TWO) {
-            tb[b][threadIdx.x] = lb.m;
-            eb2[b][threadIdx.x] = lb.e;
+        const int e1 = (int)(short)(la.e & 0xffff), e2 = (int)(short)(lb.e & 0xffff);
+        // the entry of column x from the reciprocal R (2^63 / significand) of a
+        // difference with biased exponent ed and sign bit dsg
+        auto put = [&](auto chk, int x, unsigned long long cm, unsigned long long R, int ed,
+                       unsigned dsg) {
+            constexpr bool C = decltype(chk)::value;
+            const unsigned long long Gp = mul_hi3(cm, R);
+            const Out o = so[x];
+            const double v = pack_prod<C>(la.m, Gp, (e1 - ed) + o.e,
+                                          ((unsigned)(la.e ^ dsg) & 0x80000000u) ^ vsg);
+            if (CPLX) {
+                const double vi = pack_prod<C>(lb.m, Gp, (e2 - ed) + o.e,
+                                               (unsigned)(lb.e ^ dsg) & 0x80000000u);
+                if (in) {
+                    o.v[2 * r] = v;
+                    o.v[2 * r + 1] = vi;
+                }
+            } else {
+                if (in) o.v[r] = v;
+                if (TWO && su[x]) {
+                    const unsigned long long G2 = SVD ? mul_hi3(sm2[x], R) : Gp;
+                    const double vu = pack_prod<C>(lb.m, G2, (e2 - ed) + (SVD ? se2[x] : o.e),
+                                                   (unsigned)(lb.e ^ dsg) & 0x80000000u);
+                    if (in) su[x][r] = vu;
+                }
+            }
+        };
+        unsigned far = 0;
+        if (groups) {
+            dd D = two_sum(p, -G.c);
+            if (SVD && in) D = near_diff(fast_pole<VK>(va.key[r], es), dd{G.c, 0.0}, dd{0.0, 0.0});
+            if (__all_sync(FULL, fabs(D.hi) >= G.r8)) {
+                far = fcol & mine;
+                // |p - c| in 2^(e0 - 62)
+                const int e0 = (int)bexp(D.hi);
+                const unsigned long long b = (unsigned long long)__double_as_longlong(D.hi);
+                const unsigned long long Dm =
+                    (((b & 0xfffffffffffffull) | 0x10000000000000ull) << 10) +
+                    (unsigned long long)__double2ll_rd((D.hi < 0.0 ? -D.lo : D.lo) *
+                                                       pow2(10 + 1075 - e0));
+                const int sh = min(e0 - 1023 - G.e + 2, 63);
+                const unsigned dsg = (unsigned)(b >> 32);
+                const ulonglong2 *A = sA[dsg >> 31];
+                auto entry = [&](auto chk, int x) {
+                    const ulonglong2 a = A[x];
+                    const unsigned long long M =
+                        Dm - (unsigned long long)((long long)a.x >> sh);
+                    const float y = fmaf(rcp_f32((float)(unsigned)(M >> 32)), 0x1p30f, 2.f);
+                    put(chk, x, a.y, recip62(M, __float_as_uint(y) - 0x40000000u), e0 - 1, dsg);
+                };
+                // all of this warp's columns, no result near the ends of the range
+                const int lo = min(e1, TWO ? e2 : e1) - e0 + emin,
+                          hi = max(e1, TWO ? e2 : e1) - e0 + emax;
+                if (far == (per == 32 ? ~0u : ((1u << per) - 1u) << x0) &&
+                    __all_sync(FULL, (lo > 8 && hi < 2030) || !in)) {
+#pragma unroll 4
+                    for (int x = x0; x < x0 + per; ++x) entry(std::false_type{}, x);
+                } else {
+                    for (unsigned left = far; left; left &= left - 1)
+                        entry(std::true_type{}, __ffs(left) - 1);
+                }
+            }
         }
-        __syncthreads();
-        if (t + 1 < tiles) load(t + 1);
-        if (!act) continue;
-        const int left = n1 - t * kTile;
-        const int nc = left >= kTile ? kTile / 32 : (left + 31) / 32;
-#pragma unroll 2
-        for (int c = 0; c < nc; ++c) {
-            const int x = c * 32 + lane;
-            const int r = t * kTile + x;
-            double D = fma(tp[b][x], one, -lhi);       // (an FMA: 2.0 lanes a clock, DADD 1.7)
+        for (unsigned left = mine & ~far; left; left &= left - 1) {
+            const int x = __ffs(left) - 1;
+            const double lhi = sl[x];
+            const int4 q = sd[x];
+            double D = fma(p, one, -lhi);              // (an FMA: 2.0 lanes a clock, DADD 1.7)
             int tl;
             unsigned dh = hi32(D), dl = (unsigned)__double2loint(D);
             unsigned ed = (dh << 1) >> 21;
-            if (ed - dr.lo >= dr.span && r < n1) {
-                const int es = fast_scale<VK>(S);
+            if (ed - (unsigned)q.x >= (unsigned)q.y && in) {
+                const int k = kf + x;
                 const dd pr = fast_pole<VK>(va.key[r], es);
                 const dd Dd =
-                    near_diff(pr, fast_sigma<VK>(S, ka, es), dd{S.f.mu[ka], S.f.mulo[ka]});
+                    near_diff(pr, fast_sigma<VK>(S, k, es), dd{S.f.mu[k], S.f.mulo[k]});
                 D = Dd.hi;
                 tl = near_tail(Dd);
                 dh = hi32(D);
@@ -1887,45 +2007,12 @@ __global__ void __launch_bounds__(256, 3) k_fcols(const __grid_constant__ Src sr
                 ed = (dh << 1) >> 21;
             } else {
                 // -lambda's tail for p above, + below, in 2^-7 of D's last place
-                tl = SVD ? tail_of(tP[b][x] - L, dh, dl, ed) & dr.tails
-                         : sar32(l32 ^ ~((int)dh >> 31), ed - el);
+                tl = SVD ? tail_of(rP - sL[x], dh, dl, ed) & q.z
+                         : sar32(q.w ^ ~((int)dh >> 31), ed - ((int)bexp(lhi) - 23));
             }
             const unsigned seed = hi32(rcp_seed(__hiloint2double(
                 (int)((dh & 0xfffffu) | 0x3ff00000u), 0)));
-            const unsigned long long Rr = recip63<false>(dh, dl, tl, seed);
-            const unsigned long long G = mul_hi3(mi, Rr);
-            const int e1 = ea[b][x];
-            const unsigned sg = (((unsigned)e1 ^ dh) & 0x80000000u) ^ vsg;
-            const double v = pack_prod(ta[b][x], G, (int)(short)(e1 & 0xffff) - (int)ed + ei, sg);
-            if (CPLX) {
-                const int e2 = eb2[b][x];
-                const double vi = pack_prod(tb[b][x], G, (int)(short)(e2 & 0xffff) - (int)ed + ei,
-                                            ((unsigned)e2 ^ dh) & 0x80000000u);
-                if (r < n1) {
-                    col[2 * r] = v;
-                    col[2 * r + 1] = vi;
-                }
-            } else {
-                if (r < n1) col[r] = v;
-                if (TWO && ucol) {
-                    const unsigned long long G2 = SVD ? mul_hi3(mi2, Rr) : G;
-                    const int e2 = eb2[b][x];
-                    const double vu = pack_prod(tb[b][x], G2,
-                                                (int)(short)(e2 & 0xffff) - (int)ed + ei2,
-                                                ((unsigned)e2 ^ dh) & 0x80000000u);
-                    if (r < n1) ucol[r] = vu;
-                }
-            }
-        }
-    }
-    if (act && lane == 0 && VK != KIND_DPR1 && blockIdx.y == 0) {
-        const double vn = -dd_rsqrt(dd{S.f.N[ka], S.f.Nlo[ka]}).hi;
-        if (CPLX) {
-            col[2 * n1] = vn;
-            col[2 * n1 + 1] = 0.0;
-        } else {
-            col[n1] = vn;
-            if (ucol) ucol[n1] = SVD ? va.alpha * vn / sv_of(S, ka) : vn;
+            put(std::true_type{}, x, sA[0][x].y, recip63<false>(dh, dl, tl, seed), (int)ed, dh);
         }
     }
 }

@@ -126,4 +126,19 @@ AE_HD uint64_t recip63(uint32_t dh, uint32_t dl, int t, uint32_t seed) {
     return ((uint64_t)(R0 << 10) << 32) + (uint64_t)(c >> 7);
 }
 
+// 2^124 / m for m in [0.87 2^62, 1.13 2^63), from R0 = 2^84 / m to less than one
+// part in 2^21 (an FP32 reciprocal, rounded to an integer: 2^-21.2): with m R0 =
+// 2^84 (1 + e) modulo 2^64 it is R0 (1 - e + e^2) to 2^-60 (e^3 < 2^-63; the last
+// place is 2^-62 of 0.44 to 1.15).
+AE_HD uint64_t recip62(uint64_t m, uint32_t R0) {
+    const uint64_t w = (uint64_t)(uint32_t)m * R0;
+    const uint32_t xh = (uint32_t)(m >> 32) * R0 + (uint32_t)(w >> 32);
+    const uint64_t X = ((uint64_t)xh << 32) | (uint32_t)w;                  // e 2^84
+    const uint32_t sq = (uint32_t)((uint64_t)((int64_t)(int)xh * (int)xh) >> 32);  // e^2 2^72
+    const uint64_t C = X - (uint64_t)sq * 4096u;
+    const uint64_t m0 = (uint64_t)(uint32_t)C * R0;
+    const int64_t c = (int64_t)(int)(uint32_t)(C >> 32) * (int64_t)(int)R0 + (int64_t)(m0 >> 32);
+    return ((uint64_t)(R0 << 8) << 32) - (uint64_t)(c >> 12);
+}
+
 }  // namespace ae

@@ -131,12 +131,13 @@ static int sm_count() {
     return cached;
 }
 
-// Segments of the poles (rows) that k_feval (k_fcols) CTAs of 8 eigenpairs take:
-// enough for 8 waves of 3 CTAs an SM, so that the last one is at most an eighth
-// of the time (n = 8192 alone is 2.25 waves), but no less than a tile each.
-static int segments(int n, int rows) {
-    const int units = (n + 7) / 8, want = (24 * sm_count() + units - 1) / units;
-    const int tiles = (rows + kTile - 1) / kTile;
+// Segments of the poles (rows) that k_feval (k_fcols) CTAs of a unit of 8 (32)
+// eigenpairs take: enough for 8 waves of 3 CTAs an SM, so that the last one is at
+// most an eighth of the time (n = 8192 alone is 2.25 waves of 8), but no less than
+// a tile each.
+static int segments(int units, int rows, int tile) {
+    const int want = (24 * sm_count() + units - 1) / units;
+    const int tiles = (rows + tile - 1) / tile;
     return want < 1 ? 1 : want < tiles ? want : tiles < 1 ? 1 : tiles;
 }
 
@@ -155,7 +156,7 @@ static void launch_pipeline(int n, int grid, Scratch S, const SolveOpts &so,
         // (one unit more for a part that starts inside a group, and unit 0)
         if (va.n1 >= kFarFrom) k_fgroup<K><<<g32 + 2, 256, 0, st>>>(src);
         k_fopen<K><<<g32 + 2, 256, 0, st>>>(src, so);
-        k_feval<<<dim3(g8 + 1, segments(n, va.n1 < 2 * kTile ? va.n1 : 2 * kTile)), 256, 0,
+        k_feval<<<dim3(g8 + 1, segments(g8, va.n1 < 2 * kTile ? va.n1 : 2 * kTile, kTile)), 256, 0,
                   st>>>(src);
         k_fstep<K><<<gt, 64, 0, st>>>(src, so, diag);
         k_fmore<K><<<gm, 256, 0, st>>>(src, so, 0, diag);
@@ -183,7 +184,7 @@ static void launch_pipeline(int n, int grid, Scratch S, const SolveOpts &so,
     if (ro.ev[3]) cudaEventRecord(ro.ev[3], st);
     k_fout<VK><<<gt, 64, 0, st>>>(src);
     if (va.out.V) {
-        if (S.f.p) k_fcols<VK><<<dim3(g8, segments(n, va.n1)), 256, 0, st>>>(src);
+        if (S.f.p) k_fcols<VK><<<dim3(g32 + 1, segments(g32 + 1, va.n1, col_rows(va.n1))), 256, 0, st>>>(src);
         k_vectors<VK><<<n < 4 * sms ? n : 4 * sms, 256, 0, st>>>(src);
     }
 }

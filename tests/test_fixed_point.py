@@ -2,13 +2,13 @@
 
 CPU: the reciprocal, the modular tail and the high product, compiled for the
 host, against exact integers; the bounds are those the header derives (2^-56
-for the quadratic reciprocal, 2^-58.5 for the cubic one, 2 units for the
-product), seeds off by an ulp included.
+for the quadratic reciprocal, 2^-58.5 for the cubic one, 2^-60 for the columns'
+one, 2 units for the product), seeds off by an ulp included.
 GPU: eigenpairs at the passes' edges -- tile and chunk boundaries, outermost
 eigenvalues far from all poles, poles in tight clusters, a DPR1 whose last pole
 lies far out, spectra that need the 128-bit evaluations, inputs whose exponents
 the passes refuse, an iteration cap that sends a solve to the FP64 kernels, far poles taken
-as moments (768 poles and more, groups of 32 eigenpairs) --
+as moments and their rows' components (768 poles and more, groups of 32) --
 against the oracle at the suite's bar, 10 n eps64.
 """
 import os
@@ -44,7 +44,7 @@ static i128 fix128(double x) {          // floor(x 2^106)
 int main() {
     std::mt19937_64 g(7);
     std::uniform_real_distribution<> U(-0.5, 0.5);
-    double w2 = 0, w3 = 0;
+    double w2 = 0, w3 = 0, w6 = 0;
     int prod = 0, n = 0;
     for (int it = 0; it < 2000000; ++it) {
         const double sc = std::ldexp(1.0, -(int)(g() % 40));
@@ -81,8 +81,18 @@ int main() {
         const uint64_t ex = (uint64_t)(((u128)z * R3) >> 64);
         const int64_t df = (int64_t)(ex - mul_hi3(z, R3));
         if (df < 0 || df > 2) ++prod;
+        // recip62 from an FP32 reciprocal an ulp off
+        const uint64_t mm = (uint64_t)((0.872 + 1.384 * (double)(g() >> 11) * 0x1p-53) * 0x1p62);
+        float r1 = 1.0f / (float)(uint32_t)(mm >> 32);
+        uint32_t rb;
+        memcpy(&rb, &r1, 4);
+        rb += (int)(g() % 3) - 1;
+        memcpy(&r1, &rb, 4);
+        const uint32_t R0 = (uint32_t)std::lrint((double)r1 * 0x1p52);
+        const i128 pr = (i128)((u128)mm * recip62(mm, R0)) - ((i128)1 << 124);
+        w6 = std::fmax(w6, std::fabs((double)pr / 0x1p124));
     }
-    std::printf("%d %.3f %.3f %d\n", n, std::log2(w2), std::log2(w3), prod);
+    std::printf("%d %.3f %.3f %d %.3f\n", n, std::log2(w2), std::log2(w3), prod, std::log2(w6));
     return 0;
 }
 """
@@ -96,9 +106,10 @@ def test_fixed_point_arithmetic_on_the_host(tmp_path):
     subprocess.check_call(["g++", "-O2", "-std=c++17", "-I",
                            os.path.join(root, "paper_1302_7203_gb300", "csrc"), str(src), "-o",
                            str(exe)])
-    n, w2, w3, prod = subprocess.check_output([str(exe)]).split()
+    n, w2, w3, prod, w6 = subprocess.check_output([str(exe)]).split()
     assert int(n) > 500000
     assert float(w2) <= -55.5 and float(w3) <= -58.5 and int(prod) == 0
+    assert float(w6) <= -60.0
 
 
 FORMS = {"plain": {}, "fast": dict(precision=1, finish=1, bgate=1)}
@@ -249,3 +260,25 @@ def test_far_poles_dpr1_and_svd(ae):
         assert_parity(r["s"].cpu().numpy(), r[key].cpu().numpy(),
                       {"lam": ref["s"], "abserr": np.zeros(900), "V": ref[key]}, 900,
                       what=f"svd {key}")
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("order", ["sorted", "permuted"])
+def test_columns_of_far_rows(ae, order):
+    # zero and tiny spikes among the far rows (components of 0 and down to 1e-140),
+    # a last segment of few rows; permuted: no 32 rows are far together
+    rng = np.random.default_rng(8)
+    d, z, a = W.uniform_arrow(933, seed=8)
+    z = z.copy()
+    z[[3, 40, 500, 931]] = 0.0
+    z[100:140] *= 1e-130
+    p = rng.permutation(d.size) if order == "permuted" else np.arange(d.size)
+    r = ae.arrow_eig(t(d[p]), t(z[p]), a)
+    assert_parity(r["lam"].cpu().numpy(), r["V"].cpu().numpy(), oracle.arrow_eig(d[p], z[p], a),
+                  933, what=f"far rows {order}")
+    zr = z * (0.5 + rng.random(d.size))
+    r = ae.nsym_arrow_eig(t(d[p]), t(z[p]), t(zr[p]), a)
+    ref = oracle.nsym_eig(d[p], z[p], zr[p], a)
+    for key in ("X", "Y"):
+        assert_parity(r["lam"].cpu().numpy(), r[key].cpu().numpy(), {**ref, "V": ref[key]}, 933,
+                      what=f"far rows, {key} {order}")
