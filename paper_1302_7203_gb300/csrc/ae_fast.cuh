@@ -1408,14 +1408,20 @@ __device__ __forceinline__ dd dd_of_i128(__int128 v) {
 
 // One CTA per listed eigenpair: evaluations with f in 128 bits (a term to
 // ~2^-85, D's fixed-point unit 2^-106 permitting) and the other sums as
-// k_feval forms them, until the zero is accurate enough.  Phase 1 (after
+// k_feval forms them, until the zero is accurate enough.  A few items are bound by
+// a thread's own chain of ~300 instructions a term, so a single solve gives each
+// 16 warps (graded n = 16384: 584 -> 457 us for both phases, DPR1 n = 8192: 177 ->
+// 116); a batch, with many short ones, 8 (84 us for a batch of 512, 153 with 16).  Phase 1 (after
 // k_ffix): one evaluation at a flagged eigenpair's zero, then its remedy.
+constexpr int kMoreWarps = 16;                // at most
+
 template <Kind K, class Src>
-__global__ void __launch_bounds__(256) k_fmore(const __grid_constant__ Src src, SolveOpts o,
+__global__ void __launch_bounds__(32 * kMoreWarps) k_fmore(const __grid_constant__ Src src, SolveOpts o,
                                                int phase, int diag) {
-    __shared__ unsigned long long sh1[8], sh1h[8], sh2[8], sh2u[8], sh4[8];
-    __shared__ long long sh3[8], sh5[8];
-    __shared__ unsigned long long sh2l[8];
+    constexpr int NW = kMoreWarps;
+    __shared__ unsigned long long sh1[NW], sh1h[NW], sh2[NW], sh2u[NW], sh4[NW];
+    __shared__ long long sh3[NW], sh5[NW];
+    __shared__ unsigned long long sh2l[NW];
     __shared__ int verdict, verdict_unit;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int cnt = src.more_count(phase);
@@ -1446,7 +1452,7 @@ __global__ void __launch_bounds__(256) k_fmore(const __grid_constant__ Src src, 
             unsigned long long a2 = 0, a2u = 0, a4 = 0;
             long long a3 = 0, a5 = 0;
             unsigned long long l2 = 0;
-            for (int j = threadIdx.x; j < m; j += 256) {
+            for (int j = threadIdx.x; j < m; j += blockDim.x) {
                 const double p = S.f.p[j];
                 double D = p - lhi;
                 unsigned dh = hi32(D), eb = (dh << 1) >> 21;
@@ -1537,7 +1543,7 @@ __global__ void __launch_bounds__(256) k_fmore(const __grid_constant__ Src src, 
             }
             __syncthreads();
             if (threadIdx.x == 0) {
-                for (int x = 1; x < 8; ++x) {
+                for (int x = 1; x < (int)(blockDim.x >> 5); ++x) {
                     a1 += (__int128)(((unsigned __int128)sh1h[x] << 64) | sh1[x]);
                     a2 += sh2[x];
                     a2u += sh2u[x];

@@ -159,7 +159,7 @@ static void launch_pipeline(int n, int grid, Scratch S, const SolveOpts &so,
         k_feval<<<dim3(g8 + 1, segments(g8, va.n1 < 2 * kTile ? va.n1 : 2 * kTile, kTile)), 256, 0,
                   st>>>(src);
         k_fstep<K><<<gt, 64, 0, st>>>(src, so, diag);
-        k_fmore<K><<<gm, 256, 0, st>>>(src, so, 0, diag);
+        k_fmore<K><<<gm, 32 * kMoreWarps, 0, st>>>(src, so, 0, diag);
         k_fold<K><<<grid, 256, 0, st>>>(src, so);
         if (diag) k_fdiag<K><<<g8, 256, 0, st>>>(src, so);
     } else {
@@ -169,7 +169,7 @@ static void launch_pipeline(int n, int grid, Scratch S, const SolveOpts &so,
     if (ro.fixup) {
         k_fix_decide<<<(n + 255) / 256, 256, 0, st>>>(K, S, ro.knu_max);
         k_ffix<K><<<gt, 64, 0, st>>>(src);
-        if (S.f.p) k_fmore<K><<<gm, 256, 0, st>>>(src, so, 1, 0);
+        if (S.f.p) k_fmore<K><<<gm, 32 * kMoreWarps, 0, st>>>(src, so, 1, 0);
         // every CTA resident at once (the remedies are assigned statically)
         static int fix_per_sm = 0;
         if (!fix_per_sm) {
