@@ -25,6 +25,7 @@ namespace ae {
 // ---------------------------------------------------------------------------
 template <Kind K>
 __global__ void __launch_bounds__(256) k_check(PrepArgs A, Scratch S) {
+    after_previous();
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     int flags = 0;
     if (r < A.n1) {
@@ -40,6 +41,7 @@ __global__ void __launch_bounds__(256) k_check(PrepArgs A, Scratch S) {
 // of 1024 keys (blockIdx.y).
 __global__ void __launch_bounds__(256) k_rank(int n1, const double *__restrict__ key,
                                               const double *__restrict__ spk, Scratch S) {
+    after_previous();
     __shared__ unsigned long long tile[1024];
     const int flags = S.cnt[C_FLAGS];
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
@@ -71,6 +73,7 @@ __global__ void __launch_bounds__(256) k_rank(int n1, const double *__restrict__
 }
 
 __global__ void __launch_bounds__(256) k_order(int n1, Scratch S) {
+    after_previous();
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r < n1 && (S.cnt[C_FLAGS] & (CF_UNSORTED | CF_ZERO))) S.perm[S.spos[r]] = r;
 }
@@ -79,6 +82,7 @@ __global__ void __launch_bounds__(256) k_order(int n1, Scratch S) {
 // nothing uses before the remedies)
 __global__ void __launch_bounds__(256) k_heads(int n1, const double *__restrict__ key,
                                                const double *__restrict__ spk, Scratch S) {
+    after_previous();
     if (!(S.cnt[C_FLAGS] & (CF_UNSORTED | CF_ZERO))) return;
     const int s = blockIdx.x * 256 + threadIdx.x;
     const bool head = s < n1 && is_head(key, spk, S.perm, s);
@@ -88,6 +92,7 @@ __global__ void __launch_bounds__(256) k_heads(int n1, const double *__restrict_
 
 __global__ void __launch_bounds__(256) k_reduce(int n1, const double *__restrict__ key,
                                                 const double *__restrict__ spk, Scratch S) {
+    after_previous();
     __shared__ int wh[8], before;
     if (!(S.cnt[C_FLAGS] & (CF_UNSORTED | CF_ZERO))) return;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -114,15 +119,18 @@ __global__ void __launch_bounds__(256) k_reduce(int n1, const double *__restrict
 
 template <Kind K>
 __global__ void __launch_bounds__(kChunk) k_kind(PrepArgs A, Scratch S) {
+    after_previous();
     __shared__ PoleShare sh[kChunk / 32];
     kind_chunk<K>(A, S, S.cnt[C_M], blockIdx.x, threadIdx.x, sh, 0);
 }
 template <Kind K>
 __global__ void __launch_bounds__(32) k_post(PrepArgs A, Scratch S) {
+    after_previous();
     prep_finish<K>(A, S, threadIdx.x);
 }
 template <Kind K>
 __global__ void __launch_bounds__(256) k_forms(Scratch S, VecArgs va) {
+    after_previous();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t < va.n1) forms_item<K>(S, va, t);
 }
@@ -130,6 +138,7 @@ __global__ void __launch_bounds__(256) k_forms(Scratch S, VecArgs va) {
 // all of it by one CTA
 template <Kind K>
 __global__ void __launch_bounds__(1024) k_prep(PrepArgs A, Scratch S, VecArgs va) {
+    after_previous();
     prep_block<K>(A, S, va);
 }
 
@@ -151,13 +160,13 @@ static cudaError_t launch_prep(const PrepArgs &A, const Scratch &S, const VecArg
     if (e) return e;
     const int n1 = A.n1, g = (n1 + 255) / 256;
     k_check<K><<<g, 256, 0, st>>>(A, S);
-    k_rank<<<dim3(g, (n1 + 1023) / 1024), 256, 0, st>>>(n1, va.key, va.spk, S);
-    k_order<<<g, 256, 0, st>>>(n1, S);
-    k_heads<<<g, 256, 0, st>>>(n1, va.key, va.spk, S);
-    k_reduce<<<g, 256, 0, st>>>(n1, va.key, va.spk, S);
-    k_kind<K><<<g, kChunk, 0, st>>>(A, S);
-    k_post<K><<<1, 32, 0, st>>>(A, S);
-    k_forms<K><<<g, 256, 0, st>>>(S, va);
+    launch_after(k_rank, dim3(g, (n1 + 1023) / 1024), 256, st, n1, va.key, va.spk, S);
+    launch_after(k_order, g, 256, st, n1, S);
+    launch_after(k_heads, g, 256, st, n1, va.key, va.spk, S);
+    launch_after(k_reduce, g, 256, st, n1, va.key, va.spk, S);
+    launch_after(k_kind<K>, g, kChunk, st, A, S);
+    launch_after(k_post<K>, 1, 32, st, A, S);
+    launch_after(k_forms<K>, g, 256, st, S, va);
     return cudaSuccess;
 }
 

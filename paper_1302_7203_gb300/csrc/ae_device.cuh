@@ -38,6 +38,13 @@ __device__ __forceinline__ double rcp(double x) {
 static __device__ double g_unit = 1.0;
 __device__ __forceinline__ double unit_reg() { return __ldcg(&g_unit); }
 
+// First statement of the kernels of a solve's chain (launch_after): waits until the
+// kernel before is complete and its writes are visible.  A no-op in a kernel that
+// was launched plainly.
+__device__ __forceinline__ void after_previous() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 __device__ __forceinline__ double rcp_o(double x, double one) {
     double r = rcp_seed(x);
     double e = fma(-x, r, one);

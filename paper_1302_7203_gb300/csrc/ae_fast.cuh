@@ -346,6 +346,7 @@ __device__ __forceinline__ float f32_of_bits(unsigned h) {
 
 template <Kind K, class Src>
 __global__ void __launch_bounds__(256, 2) k_fgroup(const __grid_constant__ Src src) {
+    after_previous();
     __shared__ float rt[8], rw[8];
     __shared__ int jb[2];
     __shared__ unsigned long long acc[8][kMoments + kMomLow];
@@ -866,6 +867,7 @@ __device__ __forceinline__ void open_items(const Src &src, int inst, const Scrat
 
 template <Kind K, class Src>
 __global__ void __launch_bounds__(256) k_fopen(const __grid_constant__ Src src, SolveOpts o) {
+    after_previous();
     __shared__ float red[32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     int inst, first;
@@ -917,6 +919,7 @@ constexpr int kTile = 256;
 
 template <class Src>
 __global__ void __launch_bounds__(256, 3) k_feval(const __grid_constant__ Src src) {
+    after_previous();
     __shared__ double tp[2][kTile];
     __shared__ unsigned long long tP[2][kTile], tz[2][kTile];
     __shared__ int te[2][kTile];
@@ -1319,6 +1322,7 @@ __device__ __forceinline__ void fast_count(const Scratch &S, int k, const SolveO
 template <Kind K, class Src>
 __global__ void __launch_bounds__(64) k_fstep(const __grid_constant__ Src src, SolveOpts o,
                                               int diag) {
+    after_previous();
     int inst = 0, idx = 0, klo = 0, khi = 0, k = 0;
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     bool act = src.item(t, inst, idx);
@@ -1418,6 +1422,7 @@ constexpr int kMoreWarps = 16;                // at most
 template <Kind K, class Src>
 __global__ void __launch_bounds__(32 * kMoreWarps) k_fmore(const __grid_constant__ Src src, SolveOpts o,
                                                int phase, int diag) {
+    after_previous();
     constexpr int NW = kMoreWarps;
     __shared__ unsigned long long sh1[NW], sh1h[NW], sh2[NW], sh2u[NW], sh4[NW];
     __shared__ long long sh3[NW], sh5[NW];
@@ -1607,6 +1612,7 @@ __global__ void __launch_bounds__(32 * kMoreWarps) k_fmore(const __grid_constant
 // takes for a whole eigenpair), or a warp each when there are many.
 template <Kind K, class Src>
 __global__ void __launch_bounds__(256) k_fold(const __grid_constant__ Src src, SolveOpts o) {
+    after_previous();
     __shared__ double red[16];
     __shared__ int tick;
     const int cnt = src.old_count();
@@ -1644,6 +1650,7 @@ __global__ void __launch_bounds__(256) k_fold(const __grid_constant__ Src src, S
 // FP64 solver forms them (a warp per eigenpair)
 template <Kind K, class Src>
 __global__ void __launch_bounds__(256) k_fdiag(const __grid_constant__ Src src, SolveOpts o) {
+    after_previous();
     const int lane = threadIdx.x & 31;
     const WarpTeam T{lane};
     int inst, first;
@@ -1673,6 +1680,7 @@ __global__ void __launch_bounds__(256) k_fdiag(const __grid_constant__ Src src, 
 // serves, else on to k_fmore, or (those the FP64 solver took) to k_fix_solve.
 template <Kind K, class Src>
 __global__ void __launch_bounds__(64) k_ffix(const __grid_constant__ Src src) {
+    after_previous();
     int inst = 0, idx = 0;
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (!src.item(t, inst, idx)) return;
@@ -1758,6 +1766,7 @@ __device__ __forceinline__ void scale_of(dd x, unsigned long long &m, int &e) {
 // items' columns are listed for k_vectors.
 template <Kind VK, class Src>
 __global__ void __launch_bounds__(64) k_fout(const __grid_constant__ Src src) {
+    after_previous();
     int inst = 0, idx = 0;
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (!src.item(t, inst, idx)) return;
@@ -1844,6 +1853,7 @@ __host__ __device__ constexpr int col_rows(int n1) { return n1 < kFarFrom ? 32 :
 
 template <Kind VK, class Src>
 __global__ void __launch_bounds__(256, 3) k_fcols(const __grid_constant__ Src src) {
+    after_previous();
     constexpr bool CPLX = VK == KIND_HERM;
     constexpr bool TWO = VK == KIND_HERM || VK == KIND_NSYM || VK == KIND_TSVD;
     constexpr bool SVD = VK == KIND_TSVD;
@@ -2027,6 +2037,7 @@ __global__ void __launch_bounds__(256, 3) k_fcols(const __grid_constant__ Src sr
 // eigenpairs the FP64 solver took -- by a CTA each.
 template <Kind VK, class Src>
 __global__ void __launch_bounds__(256) k_vectors(const __grid_constant__ Src src) {
+    after_previous();
     __shared__ double red[16];
     const int cnt = src.col_count();
     for (int w = blockIdx.x; w < cnt; w += gridDim.x) {

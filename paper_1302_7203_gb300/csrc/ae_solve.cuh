@@ -51,6 +51,7 @@ __global__ void __launch_bounds__(256, 3) k_eig(Scratch S, SolveOpts o) {
 // others from its back, so that the remedy kernel deals the costlier ones out
 // first, one per SM in turn.
 static __global__ void k_fix_decide(Kind kind, Scratch S, double knu_max) {
+    after_previous();
     const PartRange P = part_range(S);
     const int k = P.k0 + blockIdx.x * blockDim.x + threadIdx.x;
     if (k < P.k1) fix_decide_item(kind, S, k, knu_max);
@@ -90,6 +91,7 @@ __device__ __forceinline__ void fix_solve_teams(const Scratch &S, const SolveOpt
 // warp w / CTAs of CTA w mod CTAs: spread over all SMs.
 template <Kind K>
 __global__ void __launch_bounds__(256) k_fix_solve(Scratch S, SolveOpts o, int n) {
+    after_previous();
     __shared__ double red[16];
     const int nfix = S.cnt[C_NFIX] + S.cnt[C_NFIX2];
     const long long nwarps = (long long)gridDim.x * (blockDim.x >> 5);
@@ -131,6 +133,26 @@ static int sm_count() {
     return cached;
 }
 
+// A kernel that begins with after_previous(), set up while the one before it on the
+// stream drains: some 15 to 22 short kernels make up a small solve, ~2 us each
+// between them (us plainly / so: n = 64 100 / 72, n = 1000 182 / 137, n = 1500
+// 218 / 170).  No kernel lets the next one start before its own end: waiting CTAs
+// then sit on the SMs and the few busy CTAs of the kernels between crowd together
+// (n = 64 76, n = 1000 274, DPR1 n = 8192 502 -> 620).
+template <class... P, class... A>
+static void launch_after(void (*k)(P...), dim3 grid, int block, cudaStream_t st, A... a) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = dim3(block);
+    c.stream = st;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    cudaLaunchKernelEx(&c, k, P(a)...);
+}
+
 // Segments of the poles (rows) that k_feval (k_fcols) CTAs of a unit of 8 (32)
 // eigenpairs take: enough for 8 waves of 3 CTAs an SM, so that the last one is at
 // most an eighth of the time (n = 8192 alone is 2.25 waves of 8), but no less than
@@ -154,22 +176,23 @@ static void launch_pipeline(int n, int grid, Scratch S, const SolveOpts &so,
     if (S.f.p) {
         const int diag = va.out.dg_b || va.out.dg_Kb || va.out.dg_flags;
         // (one unit more for a part that starts inside a group, and unit 0)
-        if (va.n1 >= kFarFrom) k_fgroup<K><<<g32 + 2, 256, 0, st>>>(src);
-        k_fopen<K><<<g32 + 2, 256, 0, st>>>(src, so);
-        k_feval<<<dim3(g8 + 1, segments(g8, va.n1 < 2 * kTile ? va.n1 : 2 * kTile, kTile)), 256, 0,
-                  st>>>(src);
-        k_fstep<K><<<gt, 64, 0, st>>>(src, so, diag);
-        k_fmore<K><<<gm, 32 * kMoreWarps, 0, st>>>(src, so, 0, diag);
-        k_fold<K><<<grid, 256, 0, st>>>(src, so);
-        if (diag) k_fdiag<K><<<g8, 256, 0, st>>>(src, so);
+        if (va.n1 >= kFarFrom) launch_after(k_fgroup<K, SrcOne>, g32 + 2, 256, st, src);
+        launch_after(k_fopen<K, SrcOne>, g32 + 2, 256, st, src, so);
+        launch_after(k_feval<SrcOne>,
+                     dim3(g8 + 1, segments(g8, va.n1 < 2 * kTile ? va.n1 : 2 * kTile, kTile)), 256,
+                     st, src);
+        launch_after(k_fstep<K, SrcOne>, gt, 64, st, src, so, diag);
+        launch_after(k_fmore<K, SrcOne>, gm, 32 * kMoreWarps, st, src, so, 0, diag);
+        launch_after(k_fold<K, SrcOne>, grid, 256, st, src, so);
+        if (diag) launch_after(k_fdiag<K, SrcOne>, g8, 256, st, src, so);
     } else {
         k_eig<K><<<grid, 256, 0, st>>>(S, so);
     }
     if (ro.ev[2]) cudaEventRecord(ro.ev[2], st);
     if (ro.fixup) {
-        k_fix_decide<<<(n + 255) / 256, 256, 0, st>>>(K, S, ro.knu_max);
-        k_ffix<K><<<gt, 64, 0, st>>>(src);
-        if (S.f.p) k_fmore<K><<<gm, 32 * kMoreWarps, 0, st>>>(src, so, 1, 0);
+        launch_after(k_fix_decide, (n + 255) / 256, 256, st, K, S, ro.knu_max);
+        launch_after(k_ffix<K, SrcOne>, gt, 64, st, src);
+        if (S.f.p) launch_after(k_fmore<K, SrcOne>, gm, 32 * kMoreWarps, st, src, so, 1, 0);
         // every CTA resident at once (the remedies are assigned statically)
         static int fix_per_sm = 0;
         if (!fix_per_sm) {
@@ -179,13 +202,15 @@ static void launch_pipeline(int n, int grid, Scratch S, const SolveOpts &so,
         int fgrid = sms * fix_per_sm;
         fgrid = fgrid < grid ? fgrid : grid;
         fgrid = n < fgrid ? n : fgrid;
-        k_fix_solve<K><<<fgrid, 256, 0, st>>>(S, so, n);
+        launch_after(k_fix_solve<K>, fgrid, 256, st, S, so, n);
     }
     if (ro.ev[3]) cudaEventRecord(ro.ev[3], st);
-    k_fout<VK><<<gt, 64, 0, st>>>(src);
+    launch_after(k_fout<VK, SrcOne>, gt, 64, st, src);
     if (va.out.V) {
-        if (S.f.p) k_fcols<VK><<<dim3(g32 + 1, segments(g32 + 1, va.n1, col_rows(va.n1))), 256, 0, st>>>(src);
-        k_vectors<VK><<<n < 4 * sms ? n : 4 * sms, 256, 0, st>>>(src);
+        if (S.f.p)
+            launch_after(k_fcols<VK, SrcOne>,
+                         dim3(g32 + 1, segments(g32 + 1, va.n1, col_rows(va.n1))), 256, st, src);
+        launch_after(k_vectors<VK, SrcOne>, n < 4 * sms ? n : 4 * sms, 256, st, src);
     }
 }
 
