@@ -11,20 +11,15 @@ value      eigenpairs/s of the whole job, inputs resident in HBM, device time of
            Between steps a 512 MiB buffer is written to flush L2 (129 MB).
 e2e        the same metric through arrow_eig_host: pinned host d, z in, lambda
            and V (2 GiB) out, copies inside the timed region.
-roofline   the eigenvalue kernel (k_eig): algorithmic FP64 flops per launch
-           (3 per term per evaluation of the secular function: subtract,
-           divide, add, as in Algorithm 3; 3 more per Newton evaluation that
-           forms the derivative; 3 per term for the shift choice where it ran
-           in FP64; 20 per term for the double-double element b, or 3 for a
-           standard-precision b under Algorithm 5's gate; 6 per eigenvector
-           component, which k_eig writes as soon as each eigenvalue is known)
-           over its event-timed duration, against the FP64 FMA throughput
-           measured on this GPU at the start of the run (ae_fma_peaks).  Also
-           reported: the FP64 instructions the kernel retires per term (from
-           the per-pass instruction counts and the solver's counters) and the
-           FP64-pipe busy fraction they imply; a mixed FP32 + FP64 roofline
-           for the forms that work in FP32 and double-float; and the all-FP64
-           bisection's algorithmic work over the headline form's k_eig time.
+roofline   the columns, the longest phase (k_fout, k_fcols, k_vectors): the bytes
+           of V over its event-timed duration, against the measured HBM copy
+           rate.  Beside it, for each form, the FP64 flops the method as
+           published spends on these eigenpairs (3 per term per evaluation of
+           the secular function, 3 more with the derivative, 3 per term for a
+           shift choice in FP64, 20 or 3 per term for b, 6 per component) over
+           the eigenvalue phase, as a multiple of the FP64 FMA throughput
+           measured at the start of the run (ae_fma_peaks): far above 1, as the
+           terms are formed in integers and far poles enter as moments.
 forms      fp32_newton_gated (default headline): FP32 model steps open the
            search, then the bracketed Newton finish in FP64 (same Pick
            function, bracket and stop test as Algorithm 3), with Algorithm 5's
@@ -68,12 +63,15 @@ UNIT = "eigenpairs/s"
 N_DEFAULT = 16384
 EPS64 = 2.0 ** -53
 ERR_BOUND = 10.0            # the acceptance bar, in units of n eps64
-# k_check k_rank k_reduce k_post k_eig k_fix_decide k_fix_solve k_place k_vectors
-LAUNCHES_PER_STEP = 9
+# k_check k_rank k_order k_heads k_reduce k_kind k_post k_forms, k_fgroup k_fopen
+# k_feval k_fstep k_fmore k_fold, k_fix_decide k_ffix k_fmore k_fix_solve, k_fout
+# k_fcols k_vectors (an order above 768; the forms of the bench take the same path)
+LAUNCHES_PER_STEP = 21
 # nominal FP64 rate, for context only (the roofline uses the measured one)
 FP64_NOMINAL_TFLOPS = 152 * 4 * 2070e6 / 1e12
 
-# FP64 instructions a term of each O(n) pass of k_eig retires (per lane):
+# FP64 instructions a term of each O(n) pass of the FP64 solver (csrc/ae_solver.cuh:
+# eigenpairs the fixed-point passes leave over, arrow_eig_noalloc) retires, per lane:
 # Algorithm 1's midpoint test in FP64 (difference, reciprocal 3, accumulate);
 # pass A with a standard-precision b (difference 1, reciprocal 3, quotient 1,
 # sum 1, sum of squares 1, stores' address arithmetic 1); with a double-double
@@ -93,26 +91,18 @@ INSTR_PER_TERM = {"mid": 6, "b_std": 8, "b_dd": 21, "eval": 5, "deriv": 3, "vect
 FP32_FLOPS_PER_TERM = {"f32": 6, "df": 45}
 
 
-# ncu dram__bytes_read.sum + dram__bytes_write.sum of one full-size k_eig
-# launch (graded n = 16384, fp32_newton_gated form; a 1-pass capture), with the hash
-# of the CUDA sources it was measured on.  The bench reports it as the
-# roofline's traffic only while the form, n and sources match.
-KEIG_TRAFFIC = {"form": "fp32_newton_gated", "n": 16384,
-                "read": 15391182336, "write": 8560969728,
-                "src_sha256": "9489edb4e9a5e1dee06e85a7d58353c99dcb4c0b624319cdff3c9a6801bf74d8"}
+# ncu dram__bytes_write.sum of one k_fcols launch (graded n = 16384; V is 2147483648
+# bytes, of which the last lines were still in L2)
+KFCOLS_WRITTEN = 2085399552
 
 
-def csrc_sha256():
-    import hashlib
-    d = os.path.join(ROOT, "paper_1302_7203_gb300", "csrc")
-    h = hashlib.sha256()
-    for f in sorted(os.listdir(d)):
-        p = os.path.join(d, f)
-        if os.path.isfile(p):
-            h.update(f.encode())
-            with open(p, "rb") as fh:
-                h.update(fh.read())
-    return h.hexdigest()
+def hbm_peak():
+    """Measured HBM copy rate in GB/s (6800 where no measurement is recorded)."""
+    try:
+        with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as fh:
+            return float(json.load(fh)["hbm_gbs"])
+    except (OSError, KeyError, ValueError, TypeError):
+        return 6800.0
 
 
 # solver forms: (ae_opts.precision, ae_opts.finish, ae_opts.bgate)
@@ -228,7 +218,7 @@ class Clocks:
 # ---------------------------------------------------------------------------
 def eig_kernel_flops(n, ncomp, total_iter, fix_iter, n_ddb=None, total_deriv=0, vectors=True,
                      n_mid=None):
-    """Algorithmic FP64 flops of one k_eig launch (see module docstring).
+    """FP64 flops of the method as published (see module docstring).
 
     Per term: 3 flops for the shift choice (Algorithm 1's midpoint test) where
     it ran in FP64 (n_mid = the eigenpairs whose test did; None: all of them);
@@ -238,7 +228,7 @@ def eig_kernel_flops(n, ncomp, total_iter, fix_iter, n_ddb=None, total_deriv=0, 
     secular function (subtract, divide, add, as in Algorithm 3) and 3 more per
     Newton evaluation that also formed the derivative (total_deriv).  vectors:
     6 flops per eigenvector component (Eq. Aeigenvec: 2 subtractions and a
-    division; square, add and scale to normalise), which k_eig writes.  Work
+    division; square, add and scale to normalise).  Work
     done in FP32 (the opening model steps, the certified midpoint tests) is
     not counted."""
     terms = n - 2                    # each O(n) pass runs over the other poles
@@ -258,7 +248,7 @@ def form_flops(n, info, form):
 
 
 def fp64_instructions(n, info, form, terms=None, stored_diff=False):
-    """FP64 lane-instructions the O(n) passes of one k_eig launch retire, from
+    """FP64 lane-instructions the O(n) passes of the FP64 solver would retire, from
     INSTR_PER_TERM and the solver's counters (the Newton finish's scalar
     bookkeeping, O(1) per eigenpair, is not included).  `terms`: the terms
     of an O(n) pass (default n - 2); `stored_diff`: the eigenvector pass
@@ -428,8 +418,7 @@ def extras(arrowhead, W, dev, stream, flush, args, peaks):
         ins = fp64_instructions(n, info, form, terms, stored_diff=stored and
                                 info["n_deflated"] == 0)
         r = roofline_numbers(fl, ins, fp32_flops(n, info, terms), ms_eig / 1e3, peaks)
-        return {"frac_fp64": r["frac"], "fp64_pipe_busy_implied": r["fp64_pipe_busy_implied"],
-                "mixed_frac": r["mixed"]["frac"]}
+        return {"published_fp64_flops_over_peak": r["frac"]}
 
     # config 0: the plain method (all-FP64 bisection, Algorithm 3 as printed)
     # and the headline form on the n = 1000 uniform arrowhead; full oracle
@@ -568,15 +557,15 @@ def extras(arrowhead, W, dev, stream, flush, args, peaks):
                            "instances": len(inst), "eigenpairs": tot_n,
                            "sum_n2": int((B.n.astype(np.int64) ** 2).sum()),
                            "fp64_steps_per_eigenpair": binfo["total_iter"] / tot_n,
-                           "roofline": {"bound": "alu", "achieved": rb["achieved"],
-                                        "peak": peaks["fp64_tflops"], "unit": "TFLOP/s",
-                                        "frac": rb["frac"],
-                                        "fp64_pipe_busy_implied": rb["fp64_pipe_busy_implied"],
-                                        "mixed": rb["mixed"],
-                                        "note": "algorithmic FP64 flops of all eigenpairs "
-                                                "and of the remedy solves (average pass "
-                                                "length) over the whole plan's time, against "
-                                                "the measured FP64 rate"},
+                           "roofline": {"bound": "hbm",
+                                        "achieved": 8.0 * float((B.n.astype(np.float64) ** 2)
+                                                                .sum()) / ms / 1e6,
+                                        "peak": hbm_peak(), "unit": "GB/s",
+                                        "frac": 8.0 * float((B.n.astype(np.float64) ** 2)
+                                                            .sum()) / ms / 1e6 / hbm_peak(),
+                                        "published_fp64_flops_over_peak": rb["frac"],
+                                        "note": "bytes of all V over the whole plan's time, "
+                                                "against the measured copy rate"},
                            "remedies": int(binfo["n_dpr1shift"] + binfo["n_nearzero"] +
                                            binfo["n_otherpole"]),
                            "b_double_double": int(binfo["n_ddb"]),
@@ -970,31 +959,27 @@ def main():
     ins = fp64_instructions(n, info, primary, stored_diff=stored)
     rl = roofline_numbers(form_flops(n, info, primary), ins, fp32_flops(n, info), eig_ms / 1e3,
                           peaks)
-    rl["fp64_instr_per_term"] = ins / (n - 2) / info["n_reduced"]
     # the all-FP64 bisection's algorithmic work (its measured step count) over
-    # this form's k_eig time: the rate at which the paper's work gets done
+    # this form's eigenvalue phase: the rate at which the paper's work gets done
     eq = None
     if "fp64" in runs:
         i64 = runs["fp64"][1][-1]
         eq = eig_kernel_flops(n, i64["n_reduced"], i64["total_iter"],
                               i64["fix_iter"]) / (eig_ms / 1e3) / 1e12
-    traffic = None
-    if (KEIG_TRAFFIC["form"] == primary and KEIG_TRAFFIC["n"] == n
-            and KEIG_TRAFFIC["src_sha256"] == csrc_sha256()):
-        traffic = KEIG_TRAFFIC["read"] + KEIG_TRAFFIC["write"]
-    roof = {"bound": "alu", "achieved": rl["achieved"], "peak": peaks["fp64_tflops"],
-            "unit": "TFLOP/s", "frac": rl["frac"], "traffic": traffic,
-            "traffic_note": "bytes per k_eig launch: the per-warp stored (delta_j, "
-                            "zeta_j^2/delta_j) pairs (written once per eigenpair, re-read "
-                            "by each FP64 evaluation), the staged eigenvector column and "
-                            "the n x n V written once",
-            "kernel": "k_eig", "kernel_ms": eig_ms,
-            "fp64_instr_per_term": rl["fp64_instr_per_term"],
-            "fp64_pipe_busy_implied": rl["fp64_pipe_busy_implied"],
-            "mixed_fp32_fp64": rl["mixed"],
+    col_ms = float(np.mean([x["ms_vectors"] for x in infos]))
+    gbs = 8.0 * n * n / col_ms / 1e6
+    roof = {"bound": "hbm", "achieved": gbs, "peak": hbm_peak(), "unit": "GB/s",
+            "frac": gbs / hbm_peak(),
+            "traffic": KFCOLS_WRITTEN if n == N_DEFAULT else None,
+            "traffic_note": "bytes k_fcols writes: V once, in 256-byte pieces",
+            "kernel": "k_fcols", "kernel_ms": col_ms,
+            "note": "k_fcols is bound by issue slots and the wide multiplies' pipe "
+                    "(~70 instructions a component), not by the bytes",
+            "eigenvalue_phase_ms": eig_ms,
+            "published_fp64_flops_over_peak": rl["frac"],
             "fp64_bisection_equivalent_tflops": eq,
-            "peak_note": "measured FP64 FMA throughput of this GPU (ae_fma_peaks, of "
-                         f"measured); nominal 152 SMs x 4 flop/clk x 2070 MHz = "
+            "peak_note": "measured HBM copy rate; FP64 FMA throughput measured by "
+                         f"ae_fma_peaks, nominal 152 SMs x 4 flop/clk x 2070 MHz = "
                          f"{FP64_NOMINAL_TFLOPS:.3f} TFLOP/s",
             "peaks_measured": peaks}
 

@@ -54,7 +54,7 @@ extern "C" {
 
 /* precision of the bisection (see ae_opts.precision) */
 #define AE_FP64 0             /* all-FP64 bisection from the Gershgorin bracket */
-#define AE_FP32_BRACKET 1     /* FP32 opening bracket, verified and finished in FP64 */
+#define AE_FP32_BRACKET 1     /* FP32 where it only picks trial points or is certified */
 
 /* how the FP64 finish locates the zero (see ae_opts.finish) */
 #define AE_FINISH_BISECT 0    /* bisection, Algorithm 3 (default) */
@@ -72,6 +72,13 @@ extern "C" {
 #define AE_FLAG_MID64 256     /* with AE_FP32_BRACKET: Algorithm 1's midpoint test was
                                  not settled by its FP32 evaluation and ran in FP64 */
 
+/* The solves evaluate the secular function in fixed point (64-bit integers, exact
+   differences, terms to about 2^-59; 128-bit sums where they cancel), opened in
+   FP32, whatever precision, finish and bgate say: results are at least as accurate
+   as either form below.  The options choose what the counters report -- the work of
+   the form as described -- and how the eigenpairs are solved that those passes
+   leave over (inputs whose exponents they refuse, max_iter below 100,
+   arrow_eig_noalloc). */
 typedef struct ae_opts {
     int precision;     /* AE_FP64 (default): every step in FP64 (double-double
                           where the paper asks).  AE_FP32_BRACKET: FP32 where its
@@ -115,17 +122,20 @@ typedef struct ae_info {
     int n_dpr1shift;      /* Remark 2(b) recomputations */
     int n_capped;         /* eigenpairs that hit max_iter */
     int n_fp32_fallback;  /* FP32 brackets rejected by the FP64 check */
-    int max_iter_used;    /* largest FP64 step count (bisection or Newton) of any eigenpair */
-    long long total_iter; /* sum of FP64 step counts (FP64 evaluations of the zero finder) */
+    int max_iter_used;    /* largest step count (bisection or Newton) of any eigenpair */
+    long long total_iter; /* sum of step counts: evaluations of the zero finder; with
+                             bisection, the steps Algorithm 3 takes from its bracket to
+                             its stop test, whether taken or not */
     long long fix_iter;   /* the part of total_iter spent in remedies */
     double max_Kb;        /* largest K_b of Eq. (K2) met */
     double max_Knu;       /* largest K_nu of Eq. (K0) met (before remedies) */
     float ms_reduce;      /* with opts->profile: checks, ordering, reduction */
-    float ms_eig;         /* eigenvalue kernel (shift, b, bisection) */
+    float ms_eig;         /* eigenvalues (opening, evaluations, steps) */
     float ms_fix;         /* remedy decisions and recomputations */
     float ms_vectors;     /* placement and eigenvector columns */
-    int n_ddb;            /* with opts->bgate: eigenpairs whose b was recomputed in
-                             double-double */
+    int n_ddb;            /* with opts->bgate: eigenpairs whose b the gate sends to
+                             double-double (K_b from the FP32 opening; with diagnostics,
+                             from b itself) */
     long long total_deriv; /* Newton finish: the evaluations of total_iter - fix_iter
                               (the solves of Algorithm 1's shift) that also formed
                               the derivative */
@@ -134,7 +144,7 @@ typedef struct ae_info {
     long long n_f32_passes; /* with AE_FP32_BRACKET: O(n) passes evaluated in FP32
                              (midpoint tests, model steps, bracket bisection) */
     long long n_df_passes;  /* with AE_FP32_BRACKET: O(n) passes in double-float
-                             (the Newton finish's opening model steps) */
+                             (the FP64 solver's opening model steps) */
 } ae_info;
 
 /* Optional per-eigenpair diagnostics (device arrays of length n, any may be
@@ -144,7 +154,7 @@ typedef struct ae_diag {
                         also when a remedy recomputed the eigenvalue */
     double *Kb;      /* K_b of Eq. (K2) for that shift pole */
     double *Knu;     /* K_nu of Eq. (K0) estimated from the neighbouring eigenvalues */
-    int *iters;      /* FP64 bisection steps of the final solve */
+    int *iters;      /* steps of the final solve (as total_iter) */
     int *flags;      /* AE_FLAG_* bits */
 } ae_diag;
 

@@ -143,7 +143,8 @@ __global__ void __launch_bounds__(1024) k_prep(PrepArgs A, Scratch S, VecArgs va
 }
 
 // Up to this many rows one CTA prepares an instance (one launch instead of ten
-// operations on the stream).  A whole solve, one CTA against the grid kernels:
+// operations on the stream).  A whole solve, one CTA against the grid kernels
+// (launched plainly):
 // n = 64 99 / 120 us, n = 400 115 / 135 (rows in no order: 175 / 184),
 // n = 1000 163 / 177 (226 / 204), n = 1500 222 / 231 (581 / 430).
 constexpr int kPrepRows = 640;

@@ -4,8 +4,9 @@
 // ONE launch over every instance:
 //   k_batch_prep      one CTA per instance: checks, order, reduction, FP32 and
 //                     fixed-point copies
-//   k_fopen, k_feval, k_fstep, k_fold, k_ffix, k_fcols (ae_fast.cuh) on units of
-//                     32, 8 or 1 eigenpairs of one instance (SrcMany)
+//   k_fgroup, k_fopen, k_feval, k_fstep, k_fmore, k_fold, k_ffix, k_fcols
+//                     (ae_fast.cuh) on units of 32, 8 or 1 eigenpairs of one
+//                     instance (SrcMany)
 //   k_batch_eig       the FP64 solver instead, for options the fixed-point path
 //                     does not serve: global work queue of (instance, eigenpair)
 //                     units; a unit is 32/W eigenpairs of one instance solved by

@@ -18,20 +18,22 @@
 //             counters), model steps to |error| < 2^-16 of the distance to the
 //             nearest pole; a warp holds 4 eigenpairs, so that a pole read
 //             from L1/L2 serves 4
-//   k_feval   fixed point: f and its next four derivatives' sums in one pass
+//   k_feval   fixed point: f and its next four derivatives' sums over the near
+//             poles in one pass
 //   k_fstep   one thread per eigenpair: the zero from the quartic expansion
 //             (relative error eps^4 at a step eps of the pole distance), the
 //             vector's norm from the same sums, else a model step
 //   k_fmore   the few (1-4 %) whose opening was too far off or whose terms
-//             cancel too much: further evaluations, a CTA each, with f summed
-//             in 128 bits
+//             cancel too much, and the outermost two: further evaluations, a
+//             CTA each, with f summed in 128 bits
 //   k_fold    the FP64 solver for what is left, a CTA per eigenpair
 //   k_ffix    remedies (Remarks 1, 2): the zero is already known beyond double
 //             precision, so moving it to the remedy's shift is a subtraction;
 //             checked, else k_fmore evaluates f at the zero in 128 bits first,
 //             and what that does not settle is left to k_fix_solve
-//   k_fcols   columns: one difference, one reciprocal and two products a
-//             component, normalised in the same step and written once
+//   k_fcols   columns: one difference (for rows far from a group without FP64),
+//             one reciprocal and two products a component, normalised in the
+//             same step and written once
 #pragma once
 #include <type_traits>
 
@@ -311,8 +313,8 @@ __device__ __forceinline__ dd dd_of_ll(long long v) {
 // Bound by issue slots.  Graded n = 16384: 0.17 ms here; opening 0.72 -> 0.07,
 // k_feval 1.81 -> 0.08 ms.  DPR1 n = 8192: 0.05 here; 0.27 -> 0.04, 0.47 -> 0.03.
 // Fewer than kFarFrom poles form no groups, and their outermost eigenpairs are
-// opened by a warp like the others: one solve at n = 64 / 256 / 1000 takes 97 /
-// 109 / 179 us so, and 116 / 126 / 184 us with groups and an opening by CTA
+// opened by a warp like the others: one solve (kernels launched plainly) at n = 64
+// / 256 / 1000 takes 97 / 109 / 179 us so, and 116 / 126 / 184 us with groups and an opening by CTA
 // (two latencies more); at 1500 it is 225 against 219, and a batch, bound by
 // issue slots, gains from about 700 on.
 constexpr int kMoments = 20, kMomWide = 10, kMom32 = 10, kMomLow = 5;
