@@ -191,16 +191,13 @@ __device__ __forceinline__ void fprep_item(const Scratch &S, const VecArgs &va, 
         S.f.P[t] = fix_mod(p.hi) + fix_mod(p.lo);
         S.f.P2[t] = fix_mod<kFixFrac2>(p.hi) + fix_mod<kFixFrac2>(p.lo);
         bad |= !(fabs(p.hi) < 0.5) || (p.hi != 0.0 && fabs(p.hi) < 0x1p-900);
-        // zeta^2 as a 64-bit significand and exponent (scaled by 4^es)
+        // zeta^2 as a 64-bit significand and z2's exponent (scaled by 4^es)
         const double z2 = S.pz2[t], zl = S.pz2lo[t];
         const int e = (int)bexp(z2) - 1023;
         bad |= !(e > -900 && e < 900);
         if (!bad) {
             const unsigned long long b = (unsigned long long)__double_as_longlong(z2);
-            unsigned long long Z = ((b & 0xfffffffffffffull) | 0x10000000000000ull) << 11;
-            Z += (unsigned long long)__double2ll_rn(zl * pow2(63 - e));
-            if (!(Z >> 63)) Z = ~0ull;               // a low part that rounds below 2^63, or over
-            S.f.z[t] = Z;
+            S.f.z[t] = fix_mant(z2, __double2ll_rn(zl * pow2(63 - e)));
             // and in 128 bits
             const unsigned __int128 W =
                 ((unsigned __int128)((b & 0xfffffffffffffull) | 0x10000000000000ull) << 75) +

@@ -68,6 +68,15 @@ AE_HD uint64_t fix_mod(double x) {
     return sh <= -63 ? (uint64_t)(m >> 63) : (uint64_t)(m >> -sh);
 }
 
+// hi + lo in units of 2^(e - 63), e the exponent of hi > 0: lo is given in that
+// unit, at most half of hi's last place (2^10; 2^9 below a power of two).  The top
+// bit is 0 where a negative lo takes a power of two below itself (a spike of unit
+// modulus, a product z * (1 / z)): the products need no leading 1, so the value
+// stays as it is.  No carry: hi's significand is at most 2^64 - 2^11.
+AE_HD uint64_t fix_mant(double hi, int64_t lo) {
+    return (((f64_bits(hi) & 0xfffffffffffffull) | 0x10000000000000ull) << 11) + (uint64_t)lo;
+}
+
 // high 64 bits of a * b, at most 2 below the exact floor (on the device as one
 // carry chain: 5 instructions, where the 64-bit adds take 8)
 AE_HD uint64_t mul_hi3(uint64_t a, uint64_t b) {
