@@ -1886,7 +1886,13 @@ __global__ void __launch_bounds__(256, 3) k_fcols(const __grid_constant__ Src sr
         const int k = kl;
         const double lhi = S.f.lhi[k];
         DiffRange dr = diff_range(lhi);
-        if (!SVD) dr = {dr.lo0, 4096u, dr.lo0, dr.tails};  // (no unit to mind)
+        if (!SVD) {
+            dr = {dr.lo0, 4096u, dr.lo0, dr.tails};        // (no unit to mind)
+        } else if (dr.tails) {
+            // (the rows carry the unit 2^-106 alone)
+            const unsigned lo = max(dr.lo0, kFixMinExp);
+            dr = {lo, 1025u - lo, dr.lo0, dr.tails};
+        }
         sl[lane] = lhi;
         sd[lane] = make_int4((int)dr.lo, (int)dr.span, dr.tails, S.f.l32[k]);
         const unsigned long long t = groups ? (unsigned long long)S.f.s1[k] : 0ull;

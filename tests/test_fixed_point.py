@@ -217,6 +217,19 @@ def test_svd_edges(ae, n):
                       what=f"svd {n} {key}")
 
 
+@pytest.mark.gpu
+@pytest.mark.parametrize("m", [200, 800])
+def test_svd_columns_of_close_squares(ae, m):
+    # squares down to 1e-80: differences below the rows' fixed-point unit
+    d, z = 10.0 ** -np.linspace(0, 40, m), np.random.default_rng(m).standard_normal(m)
+    ref = oracle.tsvd(d, z, 0.5)
+    r = ae.tri_arrow_svd(t(d), t(z), 0.5)
+    for key in ("V", "U"):
+        assert_parity(r["s"].cpu().numpy(), r[key].cpu().numpy(),
+                      {"lam": ref["s"], "abserr": np.zeros(m + 1), "V": ref[key]}, m + 1,
+                      what=f"svd, close squares, {m} {key}")
+
+
 def far_case(case):
     rng = np.random.default_rng(6)
     if case[1:].isdigit():
