@@ -1143,9 +1143,11 @@ __device__ __forceinline__ void add_far(const GroupData &G, dd t, FastSums &s) {
 // Returns FST_DONE with
 // the result stored (when no round is left FST_OLD), or FST_MORE with the next
 // point set: the model's zero, or the zero found where only its accuracy is
-// wanting.
+// wanting (unit_bad: for the differences' unit alone).
 template <Kind K>
-__device__ int fast_advance(const Scratch &S, int k, const FastSums &q, double cterm, double M2u) {
+__device__ int fast_advance(const Scratch &S, int k, const FastSums &q, double cterm, double M2u,
+                            bool &unit_bad) {
+    unit_bad = false;
     const int m = S.cnt[C_M];
     const int es = fast_scale<K>(S);
     int i = S.es_pole[k];
@@ -1193,8 +1195,7 @@ __device__ int fast_advance(const Scratch &S, int k, const FastSums &q, double c
                        0x1p45 * pow2(K1));
         }
         if (!(pow2(K1) * cterm + M2u * kErrUnit <= Nf * fabs(mf.hi))) {
-            S.f.M2u[k] = M2u;
-            S.f.N[k] = Nf;
+            unit_bad = M2u * kErrUnit > 0.25 * Nf * fabs(mf.hi);
             set_point(S, k, sg, mf);
             return FST_MORE;
         }
@@ -1352,7 +1353,8 @@ __global__ void __launch_bounds__(64) k_fstep(const __grid_constant__ Src src, S
             tt = dd_add(tt, dd{S.f.mu[k], S.f.mulo[k]});
             add_far(G, tt, q);
         }
-        const int st = fast_advance<K>(S, k, q, kErrTerm, -1.0);
+        bool unit_bad;
+        const int st = fast_advance<K>(S, k, q, kErrTerm, -1.0, unit_bad);
         S.f.st[k] = st;
         if (st == FST_OLD) src.push_old(inst, k);
         else if (st == FST_MORE) src.push_more(0, inst, k);
@@ -1566,7 +1568,9 @@ __global__ void __launch_bounds__(32 * kMoreWarps) k_fmore(const __grid_constant
                 q.M4 = scalb2((double)a4, K4 - 55);
                 q.M5 = -scalb2((double)a5, K5 - 53);
                 const double ct = dr.tails ? kErrTermWide : kErrTerm;
-                int v2 = fast_advance<K>(S, k, q, ct, dr.tails ? scalb2((double)a2u, K2 - 60) : 0.0);
+                bool ub;
+                int v2 = fast_advance<K>(S, k, q, ct, dr.tails ? scalb2((double)a2u, K2 - 60) : 0.0,
+                                         ub);
                 if (v2 == FST_MORE && round + 1 == kMoreRounds) v2 = FST_OLD;
                 if (phase == 0) {
                     if (v2 == FST_DONE) {
@@ -1594,7 +1598,7 @@ __global__ void __launch_bounds__(32 * kMoreWarps) k_fmore(const __grid_constant
                     }
                 }
                 verdict = v2;
-                verdict_unit = v2 == FST_MORE && S.f.M2u[k] * kErrUnit > 0.25 * S.f.N[k] * fabs(S.f.mu[k]);
+                verdict_unit = v2 == FST_MORE && ub;
             }
             __syncthreads();
             st = verdict;
