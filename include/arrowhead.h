@@ -453,6 +453,11 @@ typedef struct ae_serve_stats_t {
     long long merged;           /* requests admitted in merged batched passes */
 } ae_serve_stats_t;
 
+/* Requests start in FIFO order as slots and memory allow; small arrowheads (n <=
+   1024) waiting together are solved in one merged pass.  A lone small arrowhead
+   starts at once, unless its caller submits ahead (earlier requests' ends not yet
+   seen through poll, result or release) and such requests come less than 0.3 ms
+   apart: then it waits for another, 0.3 ms from its submission at most. */
 typedef struct ae_server ae_server;
 /* budget: bytes of device memory for scratch + held results; queue_cap: bound
    on waiting requests (submit returns AE_EAGAIN beyond it). */

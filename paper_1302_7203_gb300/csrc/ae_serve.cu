@@ -16,7 +16,9 @@
 // as one: a single pass of the batched stages on one slot solves them all,
 // one 32-lane team per eigenpair, so that their results carry the
 // single-instance solve's bits (remedied eigenpairs agree within the
-// tolerance), while each keeps its own result buffers and completion.
+// tolerance), while each keeps its own result buffers and completion.  A lone one
+// is started at once, unless its caller submits ahead of the results it has
+// collected, less than 0.3 ms apart: then it waits that long at most for another.
 // Nothing on the device waits for the host.
 #include <cuda_runtime.h>
 #include <math.h>
@@ -51,6 +53,8 @@ struct Req {
     double *result = nullptr;   // lambda | V | U in one block
     double *lam = nullptr, *V = nullptr, *U = nullptr;
     int slot = -1;
+    bool ahead = false;         // submitted before the earlier results were collected
+    bool seen = false;          // its caller knows that it has finished
     cudaEvent_t done = nullptr;
     int *cnt_host = nullptr;    // pinned copy of the solve's counters
     clk::time_point t_submit, t_done;
@@ -63,6 +67,7 @@ size_t wbuf_bytes(int n) {
 constexpr int kSmallN = 1024;     // orders merged into one batched pass
 constexpr int kMergeMax = 256;    // requests per merged pass
 constexpr int kScan = 1024;       // queue entries searched for them
+constexpr double kHold = 300e-6;  // longest wait of a lone one for another (seconds)
 
 bool mergeable(const ae_request &r) {
     return r.kind == AE_KIND_ARROW && r.n >= 2 && r.n <= kSmallN;
@@ -105,12 +110,18 @@ struct ae_server {
     // towards each new gap), and the last one's time
     double gap = 1.0;
     clk::time_point t_small;
+    long long unseen = 0;             // requests whose end no caller has seen yet
 
     void loop();
     bool admit_locked(Req *r);
     int admit_merged_locked();
     bool worth_holding_locked() const;
     void retire_locked(Req *r);
+    void see_locked(Req *r) {
+        if (r->seen || r->state == AE_REQ_QUEUED || r->state == AE_REQ_RUNNING) return;
+        r->seen = true;
+        --unseen;
+    }
 };
 
 // Admit the small arrowhead requests among the first kScan of the queue (all
@@ -210,12 +221,15 @@ int ae_server::admit_merged_locked() {
 }
 
 // A lone small arrowhead waits for a second one (a merged pass of two costs
-// about what one alone does) while they come less than a millisecond apart:
-// for at most two such gaps from its submission.
+// about what one alone does) only where its caller submits ahead, without
+// collecting the earlier results first, less than kHold apart: for two such gaps
+// from its submission, kHold at most.  A caller that waits for each result before
+// it submits again is never held.
 bool ae_server::worth_holding_locked() const {
-    if (queue.size() != 1 || !mergeable(queue.front()->in) || gap > 1e-3) return false;
+    if (queue.size() != 1 || !mergeable(queue.front()->in) || !queue.front()->ahead || gap > kHold)
+        return false;
     const double age = std::chrono::duration<double>(clk::now() - queue.front()->t_submit).count();
-    return age < 2.0 * gap;
+    return age < std::min(2.0 * gap, kHold);
 }
 
 bool ae_server::admit_locked(Req *r) {
@@ -403,6 +417,8 @@ int ae_serve_submit(ae_server *s, const ae_request *req, unsigned long long *tic
         s->started = true;
         s->t_first = r->t_submit;
     }
+    r->ahead = s->unseen > 0;
+    ++s->unseen;
     if (mergeable(r->in)) {
         const double dt = std::chrono::duration<double>(r->t_submit - s->t_small).count();
         s->gap = 0.5 * (s->gap + std::min(dt, 0.01));
@@ -423,6 +439,7 @@ int ae_serve_poll(ae_server *s, unsigned long long ticket, int *state, double *l
     auto it = s->reqs.find(ticket);
     if (it == s->reqs.end()) return -2;
     Req *r = it->second;
+    s->see_locked(r);
     *state = r->state;
     if (latency_s)
         *latency_s = (r->state == AE_REQ_DONE || r->state == AE_REQ_ERROR)
@@ -438,6 +455,7 @@ int ae_serve_result(ae_server *s, unsigned long long ticket, const double **lamb
     auto it = s->reqs.find(ticket);
     if (it == s->reqs.end()) return -2;
     Req *r = it->second;
+    s->see_locked(r);
     if (r->state != AE_REQ_DONE) return r->state == AE_REQ_ERROR ? r->status : AE_EAGAIN;
     if (lambda) *lambda = r->lam;
     if (V) *V = r->V;
@@ -452,6 +470,7 @@ int ae_serve_release(ae_server *s, unsigned long long ticket) {
     if (it == s->reqs.end()) return -2;
     Req *r = it->second;
     if (r->state == AE_REQ_QUEUED || r->state == AE_REQ_RUNNING) return AE_EAGAIN;
+    s->see_locked(r);
     if (r->result) cudaFreeAsync(r->result, s->streams[r->slot >= 0 ? r->slot : 0]);
     if (r->charged) s->in_use -= r->bytes;
     cudaEventDestroy(r->done);
