@@ -178,11 +178,11 @@ __device__ __forceinline__ void batch_unit(const BatchInst &B, long long unit_in
 __global__ void __launch_bounds__(256, 3) k_batch_eig(const BatchInst *__restrict__ I, int count,
                                                    const long long *__restrict__ uoff,
                                                    BatchCtl *ctl, SolveOpts o, double2 *wbuf,
-                                                   long long wstride) {
+                                                   long long wstride, int slices) {
     const int lane = threadIdx.x & 31;
     const long long total = uoff[count];
     const long long gw = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    double2 *buf = wbuf ? wbuf + gw * 4 * wstride : nullptr;
+    double2 *buf = wbuf ? wbuf + gw * slices * wstride : nullptr;
     for (;;) {
         long long u = 0;
         if (lane == 0) u = atomicAdd(&ctl->tick_eig, 1);
@@ -212,10 +212,10 @@ __global__ void k_batch_fix_decide(const BatchInst *__restrict__ I, int count,
 __global__ void __launch_bounds__(256) k_batch_fix_solve(const BatchInst *__restrict__ I,
                                                          const int2 *fixlist, BatchCtl *ctl,
                                                          SolveOpts o, double2 *wbuf,
-                                                         long long wstride) {
+                                                         long long wstride, int slices) {
     const int lane = threadIdx.x & 31;
     const long long gw = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    double2 *buf = wbuf ? wbuf + gw * 4 * wstride : nullptr;
+    double2 *buf = wbuf ? wbuf + gw * slices * wstride : nullptr;
     for (;;) {
         int w = 0;
         if (lane == 0) w = atomicAdd(&ctl->tick_fix, 1);
@@ -347,8 +347,10 @@ static int batch_eig_grid() {
 struct Plan {
     int count = 0;
     long long total_n = 0;
-    double2 *wbuf = nullptr;     // 4 slices of stored pairs per warp of k_batch_eig
+    // `slices` slices of stored pairs per warp of the FP64 kernels (`grid` CTAs)
+    double2 *wbuf = nullptr;
     long long wstride = 0;
+    int slices = 4, grid = 0;
     BatchInst *d_inst = nullptr;
     // prefix tables: eigenpairs, FP64 team units, units of 8 and of 32 eigenpairs
     // (count + 1 entries each, one after another)
@@ -402,7 +404,7 @@ static void enqueue(const Plan &P, cudaStream_t st) {
     const unsigned g = (unsigned)((P.total_n + 255) / 256), g1 = (unsigned)((P.total_n + 63) / 64);
     const unsigned gm = (unsigned)std::min<long long>(P.total_n, 4 * sm_count_b());
     const SrcMany src{P.d_inst, P.count, P.d_eoff, P.d_off8, P.d_off32, P.d_ctl, P.d_old, P.d_fix, P.d_more,
-                      P.wbuf, 4 * P.wstride};
+                      P.wbuf, P.slices * P.wstride};
     k_batch_prep<<<P.count, 1024, 0, st>>>(P.d_inst, P.d_ctl);
     if (P.fast) {
         if (P.wstride > kFarFrom) k_fgroup<KIND_ARROW><<<(unsigned)P.n32, 256, 0, st>>>(src);
@@ -410,17 +412,17 @@ static void enqueue(const Plan &P, cudaStream_t st) {
         k_feval<<<(unsigned)P.n8, 256, 0, st>>>(src);
         k_fstep<KIND_ARROW><<<g1, 64, 0, st>>>(src, P.so, 0);
         k_fmore<KIND_ARROW><<<gm, 256, 0, st>>>(src, P.so, 0, 0);
-        k_fold<KIND_ARROW><<<batch_eig_grid(), 256, 0, st>>>(src, P.so);
+        k_fold<KIND_ARROW><<<P.grid, 256, 0, st>>>(src, P.so);
     } else {
-        k_batch_eig<<<batch_eig_grid(), 256, 0, st>>>(P.d_inst, P.count, P.d_uoff, P.d_ctl, P.so,
-                                                      P.wbuf, P.wstride);
+        k_batch_eig<<<P.grid, 256, 0, st>>>(P.d_inst, P.count, P.d_uoff, P.d_ctl, P.so, P.wbuf,
+                                            P.wstride, P.slices);
     }
     if (P.ro.fixup) {
         k_batch_fix_decide<<<g, 256, 0, st>>>(P.d_inst, P.count, P.d_eoff, P.ro.knu_max);
         k_ffix<KIND_ARROW><<<g1, 64, 0, st>>>(src);
         if (P.fast) k_fmore<KIND_ARROW><<<gm, 256, 0, st>>>(src, P.so, 1, 0);
-        k_batch_fix_solve<<<batch_eig_grid(), 256, 0, st>>>(P.d_inst, P.d_fix, P.d_ctl, P.so,
-                                                             P.wbuf, P.wstride);
+        k_batch_fix_solve<<<P.grid, 256, 0, st>>>(P.d_inst, P.d_fix, P.d_ctl, P.so, P.wbuf,
+                                                  P.wstride, P.slices);
     }
     k_fout<KIND_ARROW><<<g1, 64, 0, st>>>(src);
     if (P.vectors) {
@@ -497,8 +499,9 @@ static cudaError_t build_plan(Plan *P, int count, const long long *n_off, const 
     long long nmax = 1;
     for (int i = 0; i < count; ++i) nmax = std::max<long long>(nmax, ns[i]);
     P->wstride = (nmax + 1) & ~1LL;
-    if ((e = cudaMalloc(&P->wbuf, sizeof(double2) * P->wstride * 4 *
-                                      (size_t)batch_eig_grid() * 8)))
+    P->grid = batch_eig_grid();
+    if ((e = cudaMalloc(&P->wbuf, sizeof(double2) * P->wstride * P->slices *
+                                      (size_t)P->grid * 8)))
         return e;
     P->host.resize(count);
     long long vo = 0;
@@ -525,10 +528,13 @@ static cudaError_t build_plan(Plan *P, int count, const long long *n_off, const 
 // ---------------------------------------------------------------------------
 // Layout of the one device block a request batch needs: descriptors, prefix
 // tables, remedy list, control block, corners, per-instance scratch and the
-// stored-pair slices; every part 256-byte aligned.
+// stored-pair slices (one a warp, since a warp has one eigenpair, and no more
+// warps than eigenpairs: two requests of n = 1000 take 32 MB); every part 256-byte
+// aligned.
 struct ReqBatchLayout {
     size_t inst, tab, fix, old, more, ctl, alpha, scratch, wbuf, total;
     long long wstride;
+    int grid;
     std::vector<size_t> soff;
 };
 
@@ -552,7 +558,8 @@ static ReqBatchLayout req_batch_layout(int count, const int *ns) {
     L.ctl = p;  p += up(sizeof(BatchCtl));
     L.alpha = p; p += up(sizeof(double) * count);
     L.scratch = p; p += L.soff[count];
-    L.wbuf = p; p += sizeof(double2) * (size_t)L.wstride * 4 * (size_t)batch_eig_grid() * 8;
+    L.grid = (int)std::min<long long>(batch_eig_grid(), (total_n + 7) / 8);
+    L.wbuf = p; p += sizeof(double2) * (size_t)L.wstride * (size_t)L.grid * 8;
     L.total = p + 256;
     return L;
 }
@@ -584,6 +591,8 @@ cudaError_t launch_req_batch(int count, const int *ns, const double *const *d,
     P.d_ctl = (BatchCtl *)(b + L.ctl);
     P.wbuf = (double2 *)(b + L.wbuf);
     P.wstride = L.wstride;
+    P.slices = 1;
+    P.grid = L.grid;
     double *d_alpha = (double *)(b + L.alpha);
     std::vector<BatchInst> host(count);
     const std::vector<int> W(count, 32);
