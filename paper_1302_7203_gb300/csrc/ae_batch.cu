@@ -85,7 +85,7 @@ struct BatchInst {
 };
 
 struct BatchCtl {
-    int tick_eig, tick_fix, nfix, nold, tick_old, nmore[2], ncol;
+    int tick_eig, tick_fix, nfix, nold, tick_old[2], nmore[2], ncol;
 };
 
 // index i with off[i] <= t < off[i+1]
@@ -128,7 +128,7 @@ struct SrcMany {
     }
     __device__ int old_count() const { return ctl->nold; }
     __device__ int2 old_at(int w) const { return old[w]; }
-    __device__ int *old_ticket() const { return &ctl->tick_old; }
+    __device__ int *old_ticket(int ph) const { return ctl->tick_old + ph; }
     __device__ void push_more(int ph, int i, int k) const {
         more[atomicAdd(&ctl->nmore[ph], 1)] = make_int2(i, k);
     }

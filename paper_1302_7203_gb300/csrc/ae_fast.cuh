@@ -26,7 +26,7 @@
 //   k_fmore   the few (1-4 %) whose opening was too far off or whose terms
 //             cancel too much, and the outermost two: further evaluations, a
 //             CTA each, with f summed in 128 bits
-//   k_fold    the FP64 solver for what is left, a CTA per eigenpair
+//   k_fold    the FP64 solver for what is left, a warp or a CTA per eigenpair
 //   k_ffix    remedies (Remarks 1, 2): the zero is already known beyond double
 //             precision, so moving it to the remedy's shift is a subtraction;
 //             checked, else k_fmore evaluates f at the zero in 128 bits first,
@@ -100,7 +100,7 @@ struct SrcOne {          // one instance, by value
     __device__ void push_old(int, int k) const { S.f.old[atomicAdd(S.cnt + C_NOLD, 1)] = k; }
     __device__ int old_count() const { return S.cnt[C_NOLD]; }
     __device__ int2 old_at(int w) const { return make_int2(0, S.f.old[w]); }
-    __device__ int *old_ticket() const { return S.cnt + C_OLDTK; }
+    __device__ int *old_ticket(int ph) const { return S.cnt + (ph ? C_OLDTK2 : C_OLDTK); }
     // eigenpairs for k_fmore: phase 0 after k_fstep, phase 1 after k_ffix (the
     // list of phase 0 is done with by then)
     __device__ void push_more(int ph, int, int k) const {
@@ -206,6 +206,10 @@ __device__ __forceinline__ void fprep_item(const Scratch &S, const VecArgs &va, 
             S.f.zl[t] = (unsigned long long)W;
             S.f.ez[t] = e + 2 * es;
         }
+        // (k_fopen's tests of a shift pole and of the gap behind it)
+        if (!((float)(z2 * S.prm[P_ZS]) > 0x1p-100f) ||
+            (t + 1 < m && !(fabs(S.pd[t] - S.pd[t + 1]) > 0x1p-31 * fabs(S.pd[t]))))
+            atomicAdd(S.cnt + C_HARD, 1);
     }
     if (t < va.n1) {
         const dd p = fast_pole<K>(va.key[t], es);
@@ -1611,8 +1615,25 @@ __global__ void __launch_bounds__(32 * kMoreWarps) k_fmore(const __grid_constant
 // ---------------------------------------------------------------------------
 // k_fold: the FP64 solver for the eigenpairs left over
 // ---------------------------------------------------------------------------
-// A CTA of 8 warps each (a few stragglers must not run as long as a warp
-// takes for a whole eigenpair), or a warp each when there are many.
+// A warp each, as k_eig and k_batch_eig have it, or a CTA of 8 warps where that is
+// the shorter way.  The choice is the instance's (order, form and the poles that
+// k_fprep counted), never the pass's, so that an eigenpair has the same bits in a
+// solve alone, a part or a merged pass.  One pass over the poles is bound by the
+// SM's FP64 pipe, which a warp alone nearly fills: a CTA gains where few eigenpairs
+// are left and each is long.  A whole solve, a warp / a CTA each, uniform poles, us:
+// one spike of 1e-18, bisection: n = 200 553 / 605, 1000 1510 / 916, 4097 3566 /
+// 1658, 8192 7204 / 3188; Newton: 200 223 / 264, 1000 369 / 396, 4097 700 / 600, 8192
+// 1196 / 890.  A quarter of the poles (spikes over 20 decades), bisection: 1000 1590 /
+// 1433, 4097 6233 / 4432, 8192 18473 / 14185; Newton: 1000 402 / 498, 4097 983 / 1177,
+// 8192 2548 / 2676.  All (scaled by 2^500), bisection: 200 483 / 1699, 1000 1395 /
+// 2557, 4097 12102 / 14579.
+constexpr int kFoldCta = 768, kFoldCtaNewton = 2048;
+__device__ __forceinline__ bool fold_by_cta(const Scratch &S, const SolveOpts &o) {
+    const int m = S.cnt[C_M], hard = S.cnt[C_HARD];
+    if (S.cnt[C_FLAGS] & CF_NOFAST) return false;
+    return o.finish == 0 ? m >= kFoldCta && 2 * hard <= m : m >= kFoldCtaNewton && 64 * hard <= m;
+}
+
 template <Kind K, class Src>
 __global__ void __launch_bounds__(256) k_fold(const __grid_constant__ Src src, SolveOpts o) {
     after_previous();
@@ -1620,32 +1641,28 @@ __global__ void __launch_bounds__(256) k_fold(const __grid_constant__ Src src, S
     __shared__ int tick;
     const int cnt = src.old_count();
     if (cnt == 0) return;
-    if (cnt < 16 * (int)gridDim.x) {
-        const CtaTeam<8> T{(int)threadIdx.x, red, 0};
-        for (;;) {
-            __syncthreads();
-            if (threadIdx.x == 0) tick = atomicAdd(src.old_ticket(), 1);
-            __syncthreads();
-            if (tick >= cnt) break;
-            const int2 ik = src.old_at(tick);
-            const Scratch &S = src.scr(ik.x);
-            const auto R = PolesOf<K>::make(S, S.cnt[C_M]);
-            eig_item<K>(R, T, S, ik.y, o, src.slice((long long)blockIdx.x * 8));
-        }
-    } else {
-        const int lane = threadIdx.x & 31;
-        for (;;) {
-            int w = 0;
-            if (lane == 0) w = atomicAdd(src.old_ticket(), 1);
-            w = __shfl_sync(FULL, w, 0);
-            if (w >= cnt) break;
-            const int2 ik = src.old_at(w);
-            const Scratch &S = src.scr(ik.x);
-            const auto R = PolesOf<K>::make(S, S.cnt[C_M]);
-            eig_item<K>(R, WarpTeam{lane}, S, ik.y, o,
-                        src.slice(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5));
-            __syncwarp();
-        }
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (int w = blockIdx.x; w < cnt;) {
+        const int2 ik = src.old_at(w);
+        const Scratch &S = src.scr(ik.x);
+        if (fold_by_cta(S, o))
+            eig_item<K>(PolesOf<K>::make(S, S.cnt[C_M]), CtaTeam<8>{(int)threadIdx.x, red, 0}, S,
+                        ik.y, o, src.slice((long long)blockIdx.x * 8));
+        __syncthreads();
+        if (threadIdx.x == 0) tick = gridDim.x + atomicAdd(src.old_ticket(0), 1);
+        __syncthreads();
+        w = tick;
+    }
+    // (each warp's first one spreads them over the SMs)
+    double2 *buf = src.slice((long long)blockIdx.x * 8 + wid);
+    for (int w = wid * gridDim.x + blockIdx.x; w < cnt;) {
+        const int2 ik = src.old_at(w);
+        const Scratch &S = src.scr(ik.x);
+        if (!fold_by_cta(S, o))
+            eig_item<K>(PolesOf<K>::make(S, S.cnt[C_M]), WarpTeam{lane}, S, ik.y, o, buf);
+        __syncwarp();
+        if (lane == 0) w = 8 * gridDim.x + atomicAdd(src.old_ticket(1), 1);
+        w = __shfl_sync(FULL, w, 0);
     }
 }
 

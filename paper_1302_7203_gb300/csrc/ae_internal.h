@@ -33,11 +33,13 @@ enum {
     C_POS0 = 19,      // output position of the part's first item
     C_KHI = 20,       // end of the eigenpairs k_eig solves (the part's range and its edges)
     C_NOLD = 21,      // eigenpairs the fixed-point path leaves to the FP64 solver
-    C_OLDTK = 22,     // their work ticket
+    C_OLDTK = 22,     // their work tickets: CTAs' (C_OLDTK2: warps')
     C_NMORE = 23,     // eigenpairs k_fmore evaluates: after k_fstep, after k_ffix
     C_NMORE1 = 24,
     C_NCOL = 25,      // columns k_vectors writes
-    C_COUNT = 26
+    C_HARD = 26,      // poles the FP32 opening refuses as shifts (k_fprep)
+    C_OLDTK2 = 27,
+    C_COUNT = 28
 };
 enum { C64_ITERS = 0, C64_MAXKB = 1, C64_MAXKNU = 2, C64_ITERS_FIX = 3, C64_DERIV = 4,
        C64_F32 = 5,     // O(n) passes in FP32 (midpoint tests, FP32 steps and brackets)
