@@ -1626,7 +1626,8 @@ __global__ void __launch_bounds__(32 * kMoreWarps) k_fmore(const __grid_constant
 // 1196 / 890.  A quarter of the poles (spikes over 20 decades), bisection: 1000 1590 /
 // 1433, 4097 6233 / 4432, 8192 18473 / 14185; Newton: 1000 402 / 498, 4097 983 / 1177,
 // 8192 2548 / 2676.  All (scaled by 2^500), bisection: 200 483 / 1699, 1000 1395 /
-// 2557, 4097 12102 / 14579.
+// 2557, 4097 12102 / 14579.  Three CTAs an SM, as k_eig (128 registers and two: all of
+// n = 4097 12.1 ms and 2.70 by Newton instead of 11.5 and 2.42).
 constexpr int kFoldCta = 768, kFoldCtaNewton = 2048;
 __device__ __forceinline__ bool fold_by_cta(const Scratch &S, const SolveOpts &o) {
     const int m = S.cnt[C_M], hard = S.cnt[C_HARD];
@@ -1635,7 +1636,7 @@ __device__ __forceinline__ bool fold_by_cta(const Scratch &S, const SolveOpts &o
 }
 
 template <Kind K, class Src>
-__global__ void __launch_bounds__(256) k_fold(const __grid_constant__ Src src, SolveOpts o) {
+__global__ void __launch_bounds__(256, 3) k_fold(const __grid_constant__ Src src, SolveOpts o) {
     after_previous();
     __shared__ double red[16];
     __shared__ int tick;
@@ -2059,8 +2060,15 @@ __global__ void __launch_bounds__(256, 3) k_fcols(const __grid_constant__ Src sr
     }
 }
 
-// The columns k_fcols does not write -- those of deflated rows and of
-// eigenpairs the FP64 solver took -- by a CTA each.
+// The columns k_fcols does not write -- those of deflated rows and of eigenpairs the
+// FP64 solver took.  A CTA each, staged in a slice of stored pairs, so that V, which
+// may lie in host memory, is written once (arrow_eig_host, n = 4097, spikes over 20
+// decades: 6.3 -> 5.2 ms).  Fewer rows: a warp each; CTAs then wait on their barriers
+// (300 instances of n = 100 to 800, all columns here: 20.1 ms by CTAs, 18.6 with this
+// line at 256 rows, 18.1 at 512, 17.1 at 1024, where one column of n = 1000 takes
+// 25 us longer; 10000 of n = 2: 1.83 -> 1.60 ms).
+constexpr int kWarpCols = 512;
+
 template <Kind VK, class Src>
 __global__ void __launch_bounds__(256) k_vectors(const __grid_constant__ Src src) {
     after_previous();
@@ -2069,9 +2077,20 @@ __global__ void __launch_bounds__(256) k_vectors(const __grid_constant__ Src src
     for (int w = blockIdx.x; w < cnt; w += gridDim.x) {
         const int2 ik = src.col_at(w);
         const VecArgs &va = src.vec(ik.x);
+        if (va.n1 < kWarpCols) continue;
         vector_item<VK>(va.n, va.n1, va.key, va.spk, va.z, va.zrow, va.alpha, va.sgn,
-                        src.scr(ik.x), va.out, ik.y, CtaTeam<8>{(int)threadIdx.x, red, 0});
+                        src.scr(ik.x), va.out, ik.y, CtaTeam<8>{(int)threadIdx.x, red, 0},
+                        (double *)src.slice(blockIdx.x));
         __syncthreads();
+    }
+    const int lane = threadIdx.x & 31;
+    for (int w = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; w < cnt; w += 8 * gridDim.x) {
+        const int2 ik = src.col_at(w);
+        const VecArgs &va = src.vec(ik.x);
+        if (va.n1 < kWarpCols)
+            vector_item<VK>(va.n, va.n1, va.key, va.spk, va.z, va.zrow, va.alpha, va.sgn,
+                            src.scr(ik.x), va.out, ik.y, WarpTeam{lane});
+        __syncwarp();
     }
 }
 

@@ -342,7 +342,8 @@ __device__ void scalar_item(int n, const double *__restrict__ key, double sgn, c
 }
 
 // Column(s) of item `item` by one team in FP64: deflated rows, and eigenpairs
-// the FP64 solver took.  `key`/`spk` are the transformed inputs the reduction
+// the FP64 solver took.  stage: room for the column (two doubles a row for HERM)
+// that pass 1 fills instead of the column itself, which may lie in host memory.  `key`/`spk` are the transformed inputs the reduction
 // saw; z is the caller's spike array (SVD: for the left vectors; HERM: the
 // complex spikes; NSYM: the column spikes, zrow the row spikes).
 // HERM writes U = Phi V (Sec. 6.1) as complex columns, row r at doubles 2r,
@@ -354,7 +355,8 @@ template <Kind K, class Team>
 __device__ void vector_item(int n, int n1, const double *__restrict__ key,
                             const double *__restrict__ spk, const double *__restrict__ z,
                             const double *__restrict__ zrow, double alpha, double sgn,
-                            const Scratch &S, const Outputs &out, int item, const Team &T) {
+                            const Scratch &S, const Outputs &out, int item, const Team &T,
+                            double *stage = nullptr) {
     const int lane = T.rank;
     constexpr bool CPLX = K == KIND_HERM;
     constexpr bool TWO = K == KIND_NSYM;
@@ -391,10 +393,10 @@ __device__ void vector_item(int n, int n1, const double *__restrict__ key,
         };
         // component of row r of x = [(D - lambda I)^{-1} spikes; -1]
         auto comp = [&](int r) { return spk[r] * recip(r); };
-        // Pass 1 stores x (HERM, NSYM: the reciprocal t) in the column and sums
-        // x^2 in sorted order (so the norm does not depend on the order of the
-        // input rows); pass 2 scales in place.
-        double *keep = col;                      // pass-1 values, RS doubles a row
+        // Pass 1 stores x (HERM, NSYM: the reciprocal t) and sums x^2 in sorted
+        // order (so the norm does not depend on the order of the input rows);
+        // pass 2 scales.
+        double *keep = stage ? stage : col;      // pass-1 values, RS doubles a row
         // two rows a lane at a time, two independent sums (the same order for
         // every kind, so that real spikes give the real solver's bits)
         auto one = [&](int r, double &acc) {
