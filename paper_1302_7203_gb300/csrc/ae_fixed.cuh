@@ -90,7 +90,7 @@ AE_HD uint64_t mul_hi3(uint64_t a, uint64_t b) {
         "addc.u32 c, 0, 0;\n\t"
         "mad.lo.cc.u32 %0, %3, %5, t;\n\t"
         "madc.hi.u32 %1, %3, %5, c;\n\t}"
-        : "=r"(lo), "=r"(hi)
+        : "=&r"(lo), "=r"(hi)                        // (lo is written before the last reads)
         : "r"(al), "r"(ah), "r"(bl), "r"(bh));
     return ((uint64_t)hi << 32) | lo;
 #endif
