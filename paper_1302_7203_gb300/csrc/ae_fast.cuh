@@ -704,6 +704,7 @@ __device__ __forceinline__ void open_items(const Src &src, int inst, const Scrat
     const float s = (float)side;
     const int jb = side > 0 ? i + 1 : i - 1;          // the pole behind it
     if (jb >= 0 && jb < m) ok &= fabs(R.shifted(jb, sig, i)) > 0x1p-32 * fabs(sig);
+    ok &= lowx || upx || en > 0x1p-100f;              // (0: below FP32's range)
     ok &= w > 0x1p-100f && fabsf(Af) < 0x1p100f && gam < 0x1p60f;
     float rm = 0.f;
     if (!lowx && !upx) {
@@ -721,8 +722,10 @@ __device__ __forceinline__ void open_items(const Src &src, int inst, const Scrat
     // and one that ran out of passes costs the FP64 solver's 220 us)
     for (int it = 0; it < 24; ++it) {
         float she[4], sle[4], ue[4], wi[4], sd[4], ws[4], wx[4];
+        int ie[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
+            ie[e] = __shfl_sync(FULL, i, 8 * e);
             she[e] = __shfl_sync(FULL, sh, 8 * e);
             sle[e] = __shfl_sync(FULL, sl, 8 * e);
             ue[e] = __shfl_sync(FULL, u, 8 * e);
@@ -743,7 +746,7 @@ __device__ __forceinline__ void open_items(const Src &src, int inst, const Scrat
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     const float D = R.shifted_f32(j, she[e], sle[e]);
-                    const float r = D == 0.f ? 0.f : rcp_f32(D);
+                    const float r = fabsf(D) < 0x1p-60f ? 0.f : rcp_f32(D);
                     const float t = z * r;
                     tf[e] += t;
                     af[e] += fabsf(t);
@@ -763,7 +766,10 @@ __device__ __forceinline__ void open_items(const Src &src, int inst, const Scrat
                 for (int e = 0; e < 4; ++e) {
                     const float D = R.shifted_f32(j, she[e], sle[e]);
                     const float rr = rcp_f32(D - ue[e]);
-                    const float r = D == 0.f ? 0.f : rr;     // not the shift pole's own
+                    // not the shift pole's own (by index: poles closer to it than
+                    // FP32's range have D = 0 too, and count further off; at the
+                    // pole itself they are left out, their squares overflow)
+                    const float r = (it == 0 ? fabsf(D) < 0x1p-60f : j == ie[e]) ? 0.f : rr;
                     const float t = z * r;
                     tf[e] += t;
                     af[e] += fabsf(t);
