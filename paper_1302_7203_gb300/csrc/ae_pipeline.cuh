@@ -284,10 +284,16 @@ __device__ __forceinline__ void run_column(const Scratch &S, const double *spk, 
 }
 
 // output position of item `item` in the caller's arrays (a part's own block;
-// -M's order reversed for a DPR1 with rho < 0)
+// -M's order reversed for a DPR1 with rho < 0).  Inside the block also where an
+// eigenvalue is NaN (input that is rejected when the caller asks): no write may
+// leave the arrays meanwhile.
 template <Kind K>
 __device__ __forceinline__ int out_pos(const Scratch &S, int n, double sgn, int item) {
-    const int pos = S.pos[item] - (S.cnt[C_PART] ? S.cnt[C_POS0] : 0);
+    int pos = S.pos[item];
+    if (S.cnt[C_PART]) {
+        const PartRange P = part_range(S);
+        pos = min(max(pos - P.pos0, 0), (P.k1 - P.k0) + (P.u1 - P.u0) - 1);
+    }
     return K == KIND_DPR1 && sgn < 0.0 ? n - 1 - pos : pos;
 }
 
