@@ -1229,7 +1229,9 @@ __device__ int fast_advance(const Scratch &S, int k, const FastSums &q, double c
         S.es_lam[k] = sigma + muu;
         S.f.N[k] = Nf;
         S.f.Nlo[k] = Nd.lo;
-        S.f.M2u[k] = M2u;
+        // (for a remedy's shift nearer than this one: the step d, in double, is
+        // known to 2^-53 of itself)
+        S.f.M2u[k] = M2u + Nf * fabs(d) / kErrUnit;
         set_point(S, k, dd{S.f.p[i], S.f.plo[i]}, mf);
         S.f.mu[k] = mf.hi;           // (set_point may have moved it to the rounded lambda)
         S.f.mulo[k] = mf.lo;
@@ -1303,8 +1305,10 @@ __device__ bool fast_remedy(const Scratch &S, int k, double cterm) {
     const auto R = PolesOf<K>::make(S, m);
     const double lo = k < m ? R.pole(k) : (K == KIND_DPR1 ? S.prm[P_PLAST] : -INFINITY);
     const double hi = k > 0 ? R.pole(k - 1) : INFINITY;
-    if (!(pow2(S.f.K1[k]) * cterm + S.f.M2u[k] * kErrUnit <= S.f.N[k] * need && isfinite(mu2.hi) && l2 >= lo &&
-          l2 <= hi && (i < 0 || muu != 0.0)))
+    // (mu itself is a double-double: 2^-105 of it)
+    if (!(pow2(S.f.K1[k]) * cterm + S.f.M2u[k] * kErrUnit <= S.f.N[k] * need &&
+          0x1p-53 * fabs(mu.hi) <= need && isfinite(mu2.hi) && l2 >= lo && l2 <= hi &&
+          (i < 0 || muu != 0.0)))
         return false;
     S.es_pole[k] = i;
     S.es_sigma[k] = sv;
