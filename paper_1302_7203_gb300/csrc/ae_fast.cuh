@@ -718,14 +718,20 @@ __device__ __forceinline__ void open_items(const Src &src, int inst, const Scrat
     float u = 0.f, ul = 0.f, wsum = 0.f, wmax = 0.f, num = 0.f, Tabs = 0.f, dsum = 0.f;
     bool done = false;
     const bool gersh = o.finish == 0;
+    // At the pole itself closer terms are left out: their squares overflow.  Beyond
+    // the outermost pole, crowded ones nearby would start the steps where the models
+    // drown in rounding.
+    const float cut = lowx || upx ? 0x1p-30f : 0x1p-60f;
     // (3 to 5 passes nearly always; one eigenpair in some thousands takes over 9,
     // and one that ran out of passes costs the FP64 solver's 220 us)
     for (int it = 0; it < 24; ++it) {
         float she[4], sle[4], ue[4], wi[4], sd[4], ws[4], wx[4];
+        float ce[4];
         int ie[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
             ie[e] = __shfl_sync(FULL, i, 8 * e);
+            ce[e] = __shfl_sync(FULL, cut, 8 * e);
             she[e] = __shfl_sync(FULL, sh, 8 * e);
             sle[e] = __shfl_sync(FULL, sl, 8 * e);
             ue[e] = __shfl_sync(FULL, u, 8 * e);
@@ -746,7 +752,7 @@ __device__ __forceinline__ void open_items(const Src &src, int inst, const Scrat
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     const float D = R.shifted_f32(j, she[e], sle[e]);
-                    const float r = fabsf(D) < 0x1p-60f ? 0.f : rcp_f32(D);
+                    const float r = fabsf(D) < ce[e] ? 0.f : rcp_f32(D);
                     const float t = z * r;
                     tf[e] += t;
                     af[e] += fabsf(t);
@@ -767,9 +773,8 @@ __device__ __forceinline__ void open_items(const Src &src, int inst, const Scrat
                     const float D = R.shifted_f32(j, she[e], sle[e]);
                     const float rr = rcp_f32(D - ue[e]);
                     // not the shift pole's own (by index: poles closer to it than
-                    // FP32's range have D = 0 too, and count further off; at the
-                    // pole itself they are left out, their squares overflow)
-                    const float r = (it == 0 ? fabsf(D) < 0x1p-60f : j == ie[e]) ? 0.f : rr;
+                    // FP32's range have D = 0 too, and count further off)
+                    const float r = (it == 0 ? fabsf(D) < ce[e] : j == ie[e]) ? 0.f : rr;
                     const float t = z * r;
                     tf[e] += t;
                     af[e] += fabsf(t);

@@ -36,3 +36,18 @@ def test_poles_below_the_fp32_range(ae, k, sign, equal, alpha, form):
     r = ae.arrow_eig(t(d), t(z), alpha, opts=ae.default_opts(**form))
     assert_parity(r["lam"].cpu().numpy(), r["V"].cpu().numpy(), oracle.arrow_eig(d, z, alpha),
                   k + 4, what=f"{k} tiny poles, alpha {alpha}")
+
+
+@pytest.mark.parametrize("form", [{}, {"precision": 1, "finish": 1, "bgate": 1}])
+@pytest.mark.parametrize("alpha", [-1e6, -0.5])
+@pytest.mark.parametrize("ratio", [1.006, 1.2])
+def test_last_eigenvalue_far_below_crowded_poles(ae, ratio, alpha, form):
+    # (at the last pole itself FP32 sums of squares come near its largest number)
+    m = 942
+    d = np.maximum(ratio ** -np.arange(m, dtype=float), 1e-40)
+    d = np.sort(d * (1 + 1e-3 * np.random.default_rng(3).random(m)))[::-1].copy()
+    t = lambda x: torch.as_tensor(x, device="cuda")
+    r = ae.arrow_eig(t(d), t(np.ones(m)), alpha, opts=ae.default_opts(**form))
+    assert_parity(r["lam"].cpu().numpy(), r["V"].cpu().numpy(),
+                  oracle.arrow_eig(d, np.ones(m), alpha), m + 1,
+                  what=f"crowded poles, ratio {ratio} alpha {alpha}")
