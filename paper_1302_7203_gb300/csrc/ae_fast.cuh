@@ -206,10 +206,6 @@ __device__ __forceinline__ void fprep_item(const Scratch &S, const VecArgs &va, 
             S.f.zl[t] = (unsigned long long)W;
             S.f.ez[t] = e + 2 * es;
         }
-        // (k_fopen's tests of a shift pole and of the gap behind it)
-        if (!((float)(z2 * S.prm[P_ZS]) > 0x1p-100f) ||
-            (t + 1 < m && !(fabs(S.pd[t] - S.pd[t + 1]) > 0x1p-31 * fabs(S.pd[t]))))
-            atomicAdd(S.cnt + C_HARD, 1);
     }
     if (t < va.n1) {
         const dd p = fast_pole<K>(va.key[t], es);
@@ -703,7 +699,13 @@ __device__ __forceinline__ void open_items(const Src &src, int inst, const Scrat
     const float w = R.z2f(i);
     const float s = (float)side;
     const int jb = side > 0 ? i + 1 : i - 1;          // the pole behind it
-    if (jb >= 0 && jb < m) ok &= fabs(R.shifted(jb, sig, i)) > 0x1p-32 * fabs(sig);
+    bool close = en < 0x1p-100f && jn >= 0 && jn < m;   // poles closer than FP32's range?
+    if (jb >= 0 && jb < m) {
+        const double gap = fabs(R.shifted(jb, sig, i));
+        ok &= gap > 0x1p-32 * fabs(sig);
+        close |= gap * Ld < 0x1p-100;
+    }
+    close = __any_sync(FULL, close);
     ok &= lowx || upx || en > 0x1p-100f;              // (0: below FP32's range)
     ok &= w > 0x1p-100f && fabsf(Af) < 0x1p100f && gam < 0x1p60f;
     float rm = 0.f;
@@ -726,16 +728,33 @@ __device__ __forceinline__ void open_items(const Src &src, int inst, const Scrat
     // and one that ran out of passes costs the FP64 solver's 220 us)
     for (int it = 0; it < 24; ++it) {
         float she[4], sle[4], ue[4], wi[4], sd[4], ws[4], wx[4];
-        float ce[4];
-        int ie[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            ie[e] = __shfl_sync(FULL, i, 8 * e);
-            ce[e] = __shfl_sync(FULL, cut, 8 * e);
             she[e] = __shfl_sync(FULL, sh, 8 * e);
             sle[e] = __shfl_sync(FULL, sl, 8 * e);
             ue[e] = __shfl_sync(FULL, u, 8 * e);
             tf[e] = af[e] = df[e] = 0.f;
+        }
+        // tf, af, df over the poles j for which skip(j, e, D) is false
+        auto sums = [&](auto skip) {
+            for (int j = js; j < jhi; j += JS) {
+                const float z = R.z2f(j);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float D = R.shifted_f32(j, she[e], sle[e]);
+                    const float rr = rcp_f32(D - ue[e]);
+                    const float r = skip(j, e, D) ? 0.f : rr;
+                    const float t = z * r;
+                    tf[e] += t;
+                    af[e] += fabsf(t);
+                    df[e] = fmaf(t, r, df[e]);
+                }
+            }
+        };
+        float ce[4];
+        if (it == 0) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) ce[e] = __shfl_sync(FULL, cut, 8 * e);
         }
         if (it == 0 && gersh) {
             // with Algorithm 3's bracket: sum and extreme of the Gershgorin
@@ -765,22 +784,16 @@ __device__ __forceinline__ void open_items(const Src &src, int inst, const Scrat
             wsum = team(reduce4(ws, lane), false);
             wmax = team(reduce4max(wx, lane), true);
             if (G) wsum = fmaf(G->W, iw, wsum);
+        } else if (it == 0) {
+            sums([&](int, int e, float D) { return fabsf(D) < ce[e]; });
+        } else if (!close) {
+            sums([](int, int, float D) { return D == 0.f; });     // the shift pole's own
         } else {
-            for (int j = js; j < jhi; j += JS) {
-                const float z = R.z2f(j);
+            // (poles closer to it than FP32's range have D = 0 too, and count)
+            int ie[4];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const float D = R.shifted_f32(j, she[e], sle[e]);
-                    const float rr = rcp_f32(D - ue[e]);
-                    // not the shift pole's own (by index: poles closer to it than
-                    // FP32's range have D = 0 too, and count further off)
-                    const float r = (it == 0 ? fabsf(D) < ce[e] : j == ie[e]) ? 0.f : rr;
-                    const float t = z * r;
-                    tf[e] += t;
-                    af[e] += fabsf(t);
-                    df[e] = fmaf(t, r, df[e]);
-                }
-            }
+            for (int e = 0; e < 4; ++e) ie[e] = __shfl_sync(FULL, i, 8 * e);
+            sums([&](int j, int e, float) { return j == ie[e]; });
         }
         float t = team(reduce4(tf, lane), false);
         float a = team(reduce4(af, lane), false);
@@ -901,6 +914,20 @@ __global__ void __launch_bounds__(256) k_fopen(const __grid_constant__ Src src, 
     const int g = lane >> 3;                          // this lane group's eigenpair
     const bool groups = m >= kFarFrom;
     if (first == 0) {
+        // poles that open_items refuses as shifts, about: spikes below 2^-50 of the
+        // largest, gaps below 2^-31 (2^21 last places; for k_fold's teams)
+        int hard = 0;
+        for (int t = threadIdx.x; t < m; t += 256) {
+            bool h = !(S.pz2f[t] > 0x1p-100f);
+            if (t + 1 < m) {
+                const unsigned long long a = __double_as_longlong(S.pd[t]);
+                const unsigned long long b = __double_as_longlong(S.pd[t + 1]);
+                h |= (a > b ? a - b : b - a) <= 1ull << 21;
+            }
+            hard += h;
+        }
+        hard = __reduce_add_sync(FULL, hard);
+        if (lane == 0 && hard) atomicAdd(S.cnt + C_HARD, hard);
         if (!groups) return;
         // the instance's outermost eigenpairs: all poles, by the CTA
         const int k = g == 0 ? 0 : m;
@@ -1632,7 +1659,7 @@ __global__ void __launch_bounds__(32 * kMoreWarps) k_fmore(const __grid_constant
 // ---------------------------------------------------------------------------
 // A warp each, as k_eig and k_batch_eig have it, or a CTA of 8 warps where that is
 // the shorter way.  The choice is the instance's (order, form and the poles that
-// k_fprep counted), never the pass's, so that an eigenpair has the same bits in a
+// k_fopen counted), never the pass's, so that an eigenpair has the same bits in a
 // solve alone, a part or a merged pass.  One pass over the poles is bound by the
 // SM's FP64 pipe, which a warp alone nearly fills: a CTA gains where few eigenpairs
 // are left and each is long.  A whole solve, a warp / a CTA each, uniform poles, us:

@@ -37,7 +37,7 @@ enum {
     C_NMORE = 23,     // eigenpairs k_fmore evaluates: after k_fstep, after k_ffix
     C_NMORE1 = 24,
     C_NCOL = 25,      // columns k_vectors writes
-    C_HARD = 26,      // poles the FP32 opening refuses as shifts (k_fprep)
+    C_HARD = 26,      // poles the FP32 opening refuses as shifts (counted in k_fopen)
     C_OLDTK2 = 27,
     C_COUNT = 28
 };
