@@ -19,7 +19,10 @@ roofline   the columns, the longest phase (k_fout, k_fcols, k_vectors): the byte
            shift choice in FP64, 20 or 3 per term for b, 6 per component) over
            the eigenvalue phase, as a multiple of the FP64 FMA throughput
            measured at the start of the run (ae_fma_peaks): far above 1, as the
-           terms are formed in integers and far poles enter as moments.
+           terms are formed in integers and far poles enter as moments.  The
+           counts behind it are the solver's counters: evaluations done with a
+           Newton finish, and with bisection the steps Algorithm 3 would take
+           from its bracket (modelled from the FP32 sums, not run).
 forms      fp32_newton_gated (default headline): FP32 model steps open the
            search, then the bracketed Newton finish in FP64 (same Pick
            function, bracket and stop test as Algorithm 3), with Algorithm 5's
@@ -91,9 +94,25 @@ INSTR_PER_TERM = {"mid": 6, "b_std": 8, "b_dd": 21, "eval": 5, "deriv": 3, "vect
 FP32_FLOPS_PER_TERM = {"f32": 6, "df": 45}
 
 
-# ncu dram__bytes_write.sum of one k_fcols launch (graded n = 16384; V is 2147483648
-# bytes, of which the last lines were still in L2)
-KFCOLS_WRITTEN = 2085399552
+# ncu dram__bytes_write.sum of one k_fcols launch (graded n = 16384, a 1-pass
+# capture; V is 2147483648 bytes, of which the last lines were still in L2), with
+# the hash of the CUDA sources it was measured on.  Reported as the roofline's
+# traffic only while form, n and sources match.
+KFCOLS_TRAFFIC = {"form": "fp32_newton_gated", "n": 16384, "written": 2085399552,
+                  "src_sha256": "SRCHASH"}
+
+
+def csrc_sha256():
+    import hashlib
+    d = os.path.join(ROOT, "paper_1302_7203_gb300", "csrc")
+    h = hashlib.sha256()
+    for f in sorted(os.listdir(d)):
+        p = os.path.join(d, f)
+        if os.path.isfile(p):
+            h.update(f.encode())
+            with open(p, "rb") as fh:
+                h.update(fh.read())
+    return h.hexdigest()
 
 
 def hbm_peak():
@@ -437,7 +456,7 @@ def extras(arrowhead, W, dev, stream, flush, args, peaks):
                                             out={"lam": lam, "V": V}, stream=stream)["info"])
         ms = timed_device(f0, 10, 3, stream, flush)
         e = max_err_neps(lam.cpu().numpy(), V.t().cpu().numpy(), ref, n)
-        res0[form] = {"value": n / (ms / 1e3), "ms_per_step": ms, "k_eig_ms": info["ms_eig"],
+        res0[form] = {"value": n / (ms / 1e3), "ms_per_step": ms, "eig_phase_ms": info["ms_eig"],
                       "max_err_neps": e, **kernel_roof(n, form, info["ms_eig"], stored=True)}
     out["uniform_n1000"] = {"unit": UNIT, "forms": res0,
                             "note": "config 0; fp64 = the plain method (Algorithm 3's "
@@ -460,7 +479,7 @@ def extras(arrowhead, W, dev, stream, flush, args, peaks):
     e = max_err_neps(lam[kt].cpu().numpy(), Q[kt].t().cpu().numpy(),
                      {"lam": r["lam"], "V": r["Q"]}, n)
     out["dpr1_n8192"] = {"value": n / (ms / 1e3), "unit": UNIT, "ms_per_step": ms,
-                         "k_eig_ms": info["ms_eig"], "max_err_neps": e,
+                         "eig_phase_ms": info["ms_eig"], "max_err_neps": e,
                          **kernel_roof(n + 1, args.form, info["ms_eig"])}
     d, z, al = W.uniform_tsvd(n, seed=4)
     dt, zt = torch.as_tensor(d, device=dev), torch.as_tensor(z, device=dev)
@@ -476,7 +495,7 @@ def extras(arrowhead, W, dev, stream, flush, args, peaks):
     eU = max_err_neps(s, U[kt].t().cpu().numpy(), {"lam": r["s"], "V": r["U"]}, n)
     eV["vectors_U"] = eU["vectors"]
     out["svd_n8192"] = {"value": n / (ms / 1e3), "unit": "singular triplets/s", "ms_per_step": ms,
-                        "k_eig_ms": info["ms_eig"], "max_err_neps": eV,
+                        "eig_phase_ms": info["ms_eig"], "max_err_neps": eV,
                         **kernel_roof(n, args.form, info["ms_eig"])}
     # Hermitian arrowhead (Sec. 6.1), complex U
     d, z, al = W.uniform_herm(n, seed=8)
@@ -492,7 +511,7 @@ def extras(arrowhead, W, dev, stream, flush, args, peaks):
     r["V"] = r["U"]
     e = max_err_neps(lam[kt].cpu().numpy(), Uc[kt].t().cpu().numpy(), r, n)
     out["herm_n8192"] = {"value": n / (ms / 1e3), "unit": UNIT, "ms_per_step": ms,
-                         "k_eig_ms": info["ms_eig"], "max_err_neps": e,
+                         "eig_phase_ms": info["ms_eig"], "max_err_neps": e,
                          **kernel_roof(n, args.form, info["ms_eig"], stored=True)}
     del Uc
     # non-symmetric arrowhead (Remark of Sec. 6.1), right and left vectors
@@ -512,7 +531,7 @@ def extras(arrowhead, W, dev, stream, flush, args, peaks):
     r["V"] = r["Y"]
     e["vectors_Y"] = max_err_neps(lk, Y[kt].t().cpu().numpy(), r, n)["vectors"]
     out["nsym_n8192"] = {"value": n / (ms / 1e3), "unit": UNIT, "ms_per_step": ms,
-                         "k_eig_ms": info["ms_eig"], "max_err_neps": e,
+                         "eig_phase_ms": info["ms_eig"], "max_err_neps": e,
                          **kernel_roof(n, args.form, info["ms_eig"], stored=True)}
     del Q, Y
     # batched: 4096 instances, orders log-uniform in [32, 4096], one CUDA-graph plan
@@ -556,7 +575,7 @@ def extras(arrowhead, W, dev, stream, flush, args, peaks):
     out["batched_4096"] = {"value": tot_n / (ms / 1e3), "unit": UNIT, "ms_per_step": ms,
                            "instances": len(inst), "eigenpairs": tot_n,
                            "sum_n2": int((B.n.astype(np.int64) ** 2).sum()),
-                           "fp64_steps_per_eigenpair": binfo["total_iter"] / tot_n,
+                           "counted_steps_per_eigenpair": binfo["total_iter"] / tot_n,
                            "roofline": {"bound": "hbm",
                                         "achieved": 8.0 * float((B.n.astype(np.float64) ** 2)
                                                                 .sum()) / ms / 1e6,
@@ -959,25 +978,22 @@ def main():
     ins = fp64_instructions(n, info, primary, stored_diff=stored)
     rl = roofline_numbers(form_flops(n, info, primary), ins, fp32_flops(n, info), eig_ms / 1e3,
                           peaks)
-    # the all-FP64 bisection's algorithmic work (its measured step count) over
-    # this form's eigenvalue phase: the rate at which the paper's work gets done
-    eq = None
-    if "fp64" in runs:
-        i64 = runs["fp64"][1][-1]
-        eq = eig_kernel_flops(n, i64["n_reduced"], i64["total_iter"],
-                              i64["fix_iter"]) / (eig_ms / 1e3) / 1e12
     col_ms = float(np.mean([x["ms_vectors"] for x in infos]))
     gbs = 8.0 * n * n / col_ms / 1e6
+    traffic = None
+    if (KFCOLS_TRAFFIC["form"] == primary and KFCOLS_TRAFFIC["n"] == n
+            and KFCOLS_TRAFFIC["src_sha256"] == csrc_sha256()):
+        traffic = KFCOLS_TRAFFIC["written"]
     roof = {"bound": "hbm", "achieved": gbs, "peak": hbm_peak(), "unit": "GB/s",
             "frac": gbs / hbm_peak(),
-            "traffic": KFCOLS_WRITTEN if n == N_DEFAULT else None,
-            "traffic_note": "bytes k_fcols writes: V once, in 256-byte pieces",
-            "kernel": "k_fcols", "kernel_ms": col_ms,
+            "traffic": traffic,
+            "traffic_note": "bytes k_fcols writes: V once, in 256-byte pieces (null: "
+                            "not measured on these sources)",
+            "kernel": "column phase: k_fout, k_fcols, k_vectors", "kernel_ms": col_ms,
             "note": "k_fcols is bound by issue slots and the wide multiplies' pipe "
                     "(~70 instructions a component), not by the bytes",
             "eigenvalue_phase_ms": eig_ms,
             "published_fp64_flops_over_peak": rl["frac"],
-            "fp64_bisection_equivalent_tflops": eq,
             "peak_note": "measured HBM copy rate; FP64 FMA throughput measured by "
                          f"ae_fma_peaks, nominal 152 SMs x 4 flop/clk x 2070 MHz = "
                          f"{FP64_NOMINAL_TFLOPS:.3f} TFLOP/s",
@@ -1020,7 +1036,7 @@ def main():
             variants[form] = {
                 "value": world * n * args.steps / (tot / 1e3), "ms_per_step": tot / args.steps,
                 "ms_eig": me, "frac_fp64": fl / (me / 1e3) / 1e12 / peaks["fp64_tflops"],
-                "fp64_steps_per_eigenpair": inf[-1]["total_iter"] / n,
+                "counted_steps_per_eigenpair": inf[-1]["total_iter"] / n,
                 "fp32_fallbacks": inf[-1]["n_fp32_fallback"],
                 "b_double_double": inf[-1]["n_ddb"], "max_err_neps": er}
         errs = [v["max_err_neps"] for v in variants.values()]

@@ -68,9 +68,11 @@ extern "C" {
 #define AE_FLAG_CAPPED 16     /* bisection stopped at max_iter */
 #define AE_FLAG_SINGULAR 32   /* remedy found a zero denominator: lambda = sigma */
 #define AE_FLAG_FP32_FALLBACK 64 /* FP32 bracket failed its FP64 check */
-#define AE_FLAG_DDB 128       /* with opts->bgate: b recomputed in double-double */
+#define AE_FLAG_DDB 128       /* with opts->bgate: the gate asks for b in double-double */
 #define AE_FLAG_MID64 256     /* with AE_FP32_BRACKET: Algorithm 1's midpoint test was
-                                 not settled by its FP32 evaluation and ran in FP64 */
+                                 not settled by its FP32 evaluation.  The FP64 solver
+                                 then runs it in FP64; the fixed-point passes go on
+                                 from either side and move the zero to the nearer pole */
 
 /* The solves evaluate the secular function in fixed point (64-bit integers, exact
    differences, terms to about 2^-59; 128-bit sums where they cancel), opened in
@@ -361,8 +363,10 @@ int nsym_arrow_eig(int n, const double *d, const double *zc, const double *zr, d
  * Batched arrowheads: `count` independent instances of orders n_i >= 1, solved
  * together -- each stage of the arrow_eig pipeline is one persistent launch
  * over all instances (eigenpairs of every instance share one work queue and
- * are solved by teams of W = 8, 16 or 32 lanes, W chosen per order bucket by
- * ae_autotune and cached).  The method per instance is that of arrow_eig
+ * are solved by the fixed-point passes on units of 32, 8 or 1 of them; by teams
+ * of W = 8, 16 or 32 lanes, W chosen per order bucket by ae_autotune and cached,
+ * where max_iter below 100 takes the FP64 solver).  The method per instance is
+ * that of arrow_eig
  * (Algorithms 1-3, Theorem 6, Remarks 1-2); the batching is this library's.
  *
  * Layout (all device arrays except n_off / v_off, which are HOST arrays of
@@ -405,9 +409,10 @@ void ae_batch_destroy(ae_batch *plan);
 /* Time team widths 8, 16, 32 on synthetic instances for order buckets
    32..256 (larger buckets use 32) and store the fastest per bucket in the JSON
    cache $AE_TUNE_CACHE (default ~/.cache/arrowhead_tune.json), keyed by the
-   device name and the library build.  Plans created afterwards use it. */
+   device name and the library build.  Plans created afterwards use it for the
+   FP64 solver, which serves them only with max_iter below 100. */
 int ae_autotune(int n_max, void *stream);
-/* The team width the batched solver uses for an instance of order n. */
+/* The team width the batched FP64 solver uses for an instance of order n. */
 int ae_team_width(int n);
 
 /*
@@ -421,7 +426,7 @@ int ae_team_width(int n);
  * requests of order <= 1024 waiting among the first 1024 of the queue (up to
  * 256, in queue order, all with or all without vectors) are admitted together,
  * ahead of the larger requests between them: one pass of the batched stages
- * (one 32-lane team per eigenpair) on one stream solves them all, each into
+ * on one stream solves them all, each into
  * its own result buffers; their results have the bits arrow_eig gives, except
  * remedied eigenpairs (Remarks 1, 2), which agree within the tolerance.
  */

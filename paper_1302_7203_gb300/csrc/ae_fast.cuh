@@ -1910,7 +1910,8 @@ __global__ void __launch_bounds__(64) k_fout(const __grid_constant__ Src src) {
 // way a component's error is that of one subtraction and one rounding.
 // Bound by issue slots and the wide multiplies' pipe (59 % and 53 % busy).  All
 // entries by ~115 instructions -> now: DPR1 n = 8192 331 -> 214 us, graded n =
-// 16384 1223 -> 787 us (2.7 TB/s written), a whole batch of 512 8.5 -> 7.0 ms.
+// 16384 1223 -> 787 us (2.7 TB/s written), a whole batch of 512 8.5 -> 7.0 ms (both
+// sides in one run of the whole step; the columns alone had read 307 and 1130 us).
 // rows a CTA takes at least: few rows are split further, for latency
 __host__ __device__ constexpr int col_rows(int n1) { return n1 < kFarFrom ? 32 : 128; }
 

@@ -14,8 +14,7 @@
 // kScan of the queue (order at most kSmallN, up to kMergeMax of them, in
 // their queue order, ahead of the larger requests between them) are admitted
 // as one: a single pass of the batched stages on one slot solves them all,
-// one 32-lane team per eigenpair, so that their results carry the
-// single-instance solve's bits (remedied eigenpairs agree within the
+// so that their results carry the single-instance solve's bits (remedied eigenpairs agree within the
 // tolerance), while each keeps its own result buffers and completion.  A lone one
 // is started at once, unless its caller submits ahead of the results it has
 // collected, less than 0.3 ms apart: then it waits that long at most for another.

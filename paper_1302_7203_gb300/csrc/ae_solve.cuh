@@ -1,9 +1,11 @@
 // ae_solve.cuh -- the pipeline after the reduction, as templates over the
-// problem kind: one warp per eigenpair (Algorithm 1's shift, Algorithm 2's
-// inverse with b by Theorem 6 under Algorithm 5's gate, Algorithm 3's
-// bisection or the bracketed Newton finish, the column of Eq. (eigenvecAi)),
-// the remedies of Theorem C1 and Remarks 1-2, output placement and the
-// remaining columns.  ae_arrow.cu instantiates it for the arrowhead itself;
+// problem kind: the fixed-point passes of ae_fast.cuh (far poles' moments, FP32
+// opening, evaluation, step, further evaluations, the FP64 solver for what they
+// leave), or k_eig, the FP64 solver for all eigenpairs, a warp each (Algorithm 1's
+// shift, Algorithm 2's inverse with b by Theorem 6 under Algorithm 5's gate,
+// Algorithm 3's bisection or the bracketed Newton finish); then the remedies of
+// Theorem C1 and Remarks 1-2, output placement and the columns.  ae_arrow.cu
+// instantiates it for the arrowhead itself;
 // each other kind has a translation unit of its own (ae_solve_*.cu), so that
 // the kinds compile in parallel.
 #pragma once
